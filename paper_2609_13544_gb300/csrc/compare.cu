@@ -17,26 +17,34 @@
 // clears the accumulator.  All merged quantities are integers or exact
 // values, so the result depends neither on the grid nor on the order of the
 // atomics.  Per element pair:
-//   - bitwise-equal pairs are counted (whole warp tiles at once when equal);
-//   - unequal pairs of a tile are compacted into a per-warp queue (element
-//     order) and processed 32 at a time;
-//   - a "window" pair -- ULP distance u < 2^UB (so the signs agree and c is
-//     within a factor 2 of g: c - g is exact in float32, Sterbenz), |g| at
-//     least 2^(Lb+1-bias), |d| < 2^(Lexp+22) -- is finished in float32 and
-//     integer arithmetic: V = |d| / 2^Lexp is an integer below 2^22, read
-//     from the bits of |d| + 1.5 * 2^(Lexp+23), so sum |d|, sum d and sum d^2
-//     accumulate as integers; the log2-relative bin is the exponent
-//     difference of |d| and |g|; the tolerance test is one float32 fma, exact
-//     except at equality; a pair updates the exact maxima only when it lies
-//     strictly above the thread's current ones (its pairs arrive in index
-//     order, so ties keep the earlier index);
+//   - a "window" pair -- same sign, a small ULP distance (so c - g is exact,
+//     Sterbenz), |d| inside the window of the piece -- increments shared
+//     counters: one that names its log2-relative bin and ULP distance, and
+//     (16-bit types) one that names the value of d, from which the exact sums
+//     follow at the end of the piece; float32 differences are added as
+//     integers instead.  The tolerance test is one float32 fma rounded down.
+//     Every pair of a vector takes these steps without a branch; equal ones
+//     land in counters that are left out;
+//   - the maxima: a pair above the CTA's bounds so far (a few per piece) sends
+//     its warp through a slow path that updates the exact records, lowest
+//     index on ties;
 //   - every other pair (non-finite, sign change, zeros, wide gaps, outside
-//     the window, tolerance ties) is listed and evaluated exactly after the
-//     piece, with float32 error-free transforms and integer digits added to a
-//     CTA-wide carry-save fixed-point accumulator.
+//     the window) is found by the same checks, listed and evaluated exactly
+//     after the piece, with float32 error-free transforms and integer digits
+//     added to a CTA-wide carry-save fixed-point accumulator.
+// What bounds it: instruction issue.  Per vector of 8 pairs and lane the dense
+// 16-bit loop executes about 210 (bfloat16) to 255 (binary16) instructions, a
+// vector of equal pairs about 80; all but the FP32 adds and fmas issue at half
+// rate.  The kernel before it compacted unequal pairs into a queue and kept
+// histogram rows per thread, about 60 instructions per unequal pair and 30 per
+// pair.  Measured (back-to-back calls, one GB300): 67 M bfloat16 pairs of
+// which half differ 182 -> 94 us, 355 M binary16 pairs in 292 segments 1007 ->
+// 489 us, 268 M bfloat16 pairs of which 0.3 % differ 265 -> 211 us, 25.6 M
+// float32 pairs in 161 segments 216 -> 127 us.
 // Binary64 arithmetic is avoided per element (GB300 runs it at a small
 // fraction of float32 rate); binary64 values appear only as containers and
 // in the once-per-segment rounding.
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include <cstdint>
@@ -54,46 +62,36 @@ namespace {
 // element types
 // ---------------------------------------------------------------------------
 // UBMAX: the largest ULP-distance bit length the window's position allows
-// for (the window sits 20 - UB binades deep below the largest golden seen).
-// LBMIN and LBMAX bound the window's floor binade Lb so that 2^Lexp is a
-// normal float32 (Lexp = Lb - BIAS - MB) and 1.5 * 2^(Lexp+23) is finite.
+// for (the window's floor sits 40 - UB binades below the largest golden seen).
+// LBMIN and LBMAX bound the window's floor binade Lb so that 2^Lexp is at least
+// 2^-100 (Lexp = Lb - BIAS - MB) and 1.5 * 2^(Lexp+44) is finite.
 template <int DT>
 struct Tr;
 template <>
 struct Tr<PEAT_F32> {
   static constexpr int BYTES = 4, VEC = 4, MB = 23, BIAS = 127, EMAX = 255;
-  static constexpr int UBMAX = 12, LBMIN = 24, LBMAX = 221;
+  static constexpr int UBMAX = 20, LBMIN = 50, LBMAX = 221;
   static constexpr uint32_t SIGN = 0x80000000u, MAG = 0x7FFFFFFFu, INF = 0x7F800000u;
 };
 template <>
 struct Tr<PEAT_F16> {
-  static constexpr int BYTES = 2, VEC = 8, MB = 10, BIAS = 15, EMAX = 31;
-  static constexpr int UBMAX = 10, LBMIN = 1, LBMAX = 30;
+  static constexpr int BYTES = 2, VEC = 8, MB = 10, EMAX = 31;
   static constexpr uint32_t SIGN = 0x8000u, MAG = 0x7FFFu, INF = 0x7C00u;
 };
 template <>
 struct Tr<PEAT_BF16> {
-  static constexpr int BYTES = 2, VEC = 8, MB = 7, BIAS = 127, EMAX = 255;
-  static constexpr int UBMAX = 7, LBMIN = 8, LBMAX = 221;
+  static constexpr int BYTES = 2, VEC = 8, MB = 7, EMAX = 255;
   static constexpr uint32_t SIGN = 0x8000u, MAG = 0x7FFFu, INF = 0x7F80u;
 };
 
-// Private per-thread histogram rows (16-bit counters, two threads per word):
-// ULP bins 1..63 in rows 0..62, then the log2-relative bins window pairs
-// reach, k in [KLO, KHI] in rows 63 + k - KLO (fp16 goldens may be subnormal,
-// whose ratios reach 2^(MB-1)).
-constexpr int NUR = 63;  // ULP rows
+// CTA geometry: the 16-bit kernel keeps its tables once per SM (one CTA of 16
+// warps), the float32 kernel runs two CTAs of 8 warps.
 template <int DT>
-struct Rows {
-  static constexpr int KLO = -(Tr<DT>::MB + 1);
-  // a window pair has c within a factor 2 of g, so |d| < |g| (k <= -1) unless
-  // g is an fp16 subnormal (|d| up to 2^MB - 1 steps of it)
-  static constexpr int KHI = DT == PEAT_F16 ? Tr<DT>::MB - 1 : -1;
-  static constexpr int NPB = NUR + KHI - KLO + 1;
+struct Geo {
+  static constexpr int NT = DT == PEAT_F32 ? 256 : 512;
+  static constexpr int NW = NT / 32;
+  static constexpr int CTAS = DT == PEAT_F32 ? 2 : 1;
 };
-constexpr int HALF = BLOCK / 2;
-constexpr int ROWB = HALF * 4;  // bytes per private row
-constexpr int NPB_MAX = NUR + 24;  // float32: k in [-24, -1]
 
 template <int DT>
 __device__ __forceinline__ float to_f32(uint32_t b) {
@@ -219,33 +217,38 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // ---- bulk-copy (TMA) staging: mbarrier + cp.async.bulk, waits bounded -----
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
+}
+// true in one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
 }
 // global -> shared bulk copy of `bytes` (16-byte aligned, multiple of 16), completing on bar
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
-__device__ __forceinline__ bool mbar_test(unsigned long long* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
       : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
+      : "r"(bar), "r"(parity)
       : "memory");
   return ok != 0;
 }
 // wait for phase `parity` of bar to complete, giving up after `limit` polls
 // (limit 0: give up without polling)
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, uint32_t limit) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t limit) {
   for (uint32_t it = 0; it < limit; it++)
     if (mbar_test(bar, parity)) return true;
   return false;
@@ -383,17 +386,17 @@ struct GenRec {
   long long abs_idx, rel_idx, ulp_idx;
 };
 
-// Maxima of the window pairs one thread evaluated exactly (offsets from the
-// CTA's first element; ties to the lower offset).  The rel record keeps |d|
-// and |g| of its pair (rd = 0: none).
-struct WinRec {
-  float amax, rd, rg;
-  uint32_t aidx, umax, uidx, ridx, pad;
+// The exact relative-error record of one warp's window pairs: |d| = a and |g|
+// of the best ratio so far (a = 0: none) at offset li from the CTA's first
+// element.  q: the ratio rounded to float32 (16-bit types: distinct ratios
+// round apart, see rel_key).
+struct RelRec {
+  float a, g, q;
+  uint32_t li;
 };
 
 // Per-warp staging ring for the bulk copies: NSTAGE stages, each one warp
 // tile of CHV 16-byte vectors of each tensor (two vectors per lane).
-constexpr int NW = BLOCK / 32;
 
 // scratch of the mean and variance of |d|: S1 = sum |d| and S2 = sum d^2,
 // both NLIMB digits weighing 2^(32 j + LIMB_LSB) (two more after carrying)
@@ -404,20 +407,60 @@ static_assert(LIMB_LSB % 32 == 0, "the S2 shift is a whole number of digits");
 struct FinScratch {
   unsigned long long cnt[8];
   long long limbs[NSUM * NLIMB];
-  Partial wbest[NW];
+  Partial wbest[16];
   double sums[NSUM];
 };
 constexpr int NSTAGE = 2;  // a power of two: stage and phase are bit fields of the use count
-constexpr int RWMAX = 6;   // window moves per warp and piece
+constexpr int RWMAX = 6;   // window moves per warp and piece (float32)
 constexpr int CHV = 64;
-constexpr int GSM = 128;   // general pairs per piece kept in shared memory
 
-struct __align__(128) Smem {
-  union {  // the mean/variance scratch of a finalizing CTA reuses the (by then idle) staging ring
-    uint4 ring_g[NW][NSTAGE][CHV];
-    MV mv;
-  };
-  uint4 ring_c[NW][NSTAGE][CHV];
+// The window tables: shared counters that every window pair increments by
+// one.  An increment by the constant one costs a cycle per distinct address
+// of a bank (lanes with the same address are merged; measured: 32 lanes on
+// one address 1.2 cycles, on random addresses 2.6, while adding a variable
+// serialises equal addresses), so the counters need no private copies.
+//
+// Every pair of a vector increments them, equal ones too (a predicated
+// increment compiles to a branch, five instructions): equal pairs (d = 0) land
+// in cells of their own that are left out.
+//
+// T1 (16-bit types) counts pairs by the value of d.  |d| has at most 8
+// significant bits, so 1 + 6 + 7 bits (bfloat16: the sign, the exponent modulo
+// 64, the significand field; the window holds 64 exponents) or 1 + 5 + 7
+// (binary16 scaled by 2^s, see Win) name it.  The low five bits of the index
+// are exclusive-ored with those of the exponent, or powers of two would share
+// a bank.  The three exact sums are formed from the counters at the end of a
+// piece.  d = 0 shares bfloat16's cell of exponent 0 mod 64, significand 0;
+// its number is known from T2 and taken off.
+//
+// T2 gives the bins.  bfloat16: by (ULP steps + 64, the golden's significand
+// field), which fixes the ratio |d| / |g| and so the log2-relative bin, and
+// (with atol = 0) the class.  binary16 and float32: by (floor(log2(|d| / |g|))
+// modulo 32, ULP steps + 128 or min(ULP steps, 63)), the two bins themselves.
+template <int DT>
+struct Tab;
+template <>
+struct Tab<PEAT_F32> {
+  static constexpr int N1 = 0, N2 = 32 * 64, UMAX = (1 << 23) - 1;
+};
+template <>
+struct Tab<PEAT_F16> {
+  static constexpr int N1 = 2 * 32 * 128, N2 = 32 * 256, ROWS = 32, UMAX = 127;
+};
+template <>
+struct Tab<PEAT_BF16> {
+  static constexpr int N1 = 2 * 64 * 128, N2 = 128 * 128, ROWS = 64, UMAX = 63;
+};
+
+template <int NW>
+struct Ring {
+  uint4 g[NW][NSTAGE][CHV];
+  uint4 c[NW][NSTAGE][CHV];
+};
+
+// totals and scratch, the same for both geometries
+template <int NW>
+struct Common {
   unsigned long long bar[NW][NSTAGE];
   unsigned long long hist[HBINS];
   unsigned long long sacc[NSUM][NLIMB];
@@ -427,29 +470,54 @@ struct __align__(128) Smem {
   long long ff, fu;                // first finite pair, first pair without NaN (search result)
   uint32_t* glist;                 // this CTA's list of general pairs (offsets), GCAP entries
   uint32_t gn;                     // entries appended in this piece (may exceed GCAP)
-  // the first GSM entries of the list stay here, with the pairs' bits
-  uint32_t gs_off[GSM], gs_g[GSM], gs_c[GSM];
   uint32_t nfe;                    // bitwise-equal pairs holding NaN or Inf
   int last;                        // this CTA finished the last piece of a one-segment call
   unsigned pieces;                 // a one-segment call's pieces: the CTAs whose ranges are not empty
-  FinScratch fin;
   int lb, ub;
-  // each warp's windows in the current piece: window r applies from the warp's
-  // chunk wstart[w][r] on (r = 0: the piece's initial window, also for the head)
+  // the CTA's window maxima of the piece: value in the high word, the
+  // complement of the pair's offset in the low one (the larger key is the
+  // larger value, then the lower index; low word 0: a starting bound taken
+  // from the window sample, no pair yet).  kabs: float32 bits of |d|; kulp:
+  // the ULP distance; krel: float32 bits of the ratio (float32 operands: a
+  // lower bound of it, the pairs are in wrel).
+  unsigned long long kabs, kulp, krel;
+  RelRec wrel[NW];
+  uint4 edge_g[CHV], edge_c[CHV];  // the staged head or tail of a piece
+  uint32_t wem[NW], wum[NW];       // float32: largest golden exponent and ULP distance of the vectors slow_vec saw in a tile
+  // float32: each warp's windows in the current piece: window r applies from
+  // the warp's chunk wstart[w][r] on (r = 0: the piece's initial window)
   uint32_t nwin[NW];
   uint32_t wstart[NW][RWMAX + 1];
   int wlb[NW][RWMAX + 1];
-  WinRec rec[BLOCK];
-  uint32_t priv[NPB_MAX * HALF];   // per-thread 16-bit counters, two threads per word
-  unsigned short qp[NW][CHV * 8];  // per-warp queue: tile positions of the unequal pairs
+  FinScratch fin;
   // the general path's totals, one copy per warp (fewer threads contend for an
-  // address), folded into hist and sacc at the end of each piece
+  // address), folded into hist and sacc at the end of a piece that used them
   unsigned long long ghist[NW][HBINS];
   unsigned long long gsacc[NW][NSUM][NLIMB];
 };
 
-__device__ __forceinline__ void sacc_add(Smem& sm, int which, unsigned __int128 m, int e, bool neg) {
-  for_digits(m, e, neg, [&](int j, int64_t v) { atomicAdd(&sm.sacc[which][j], (unsigned long long)v); });
+template <int DT>
+struct __align__(128) Smem {
+  static constexpr int NW = Geo<DT>::NW;
+  uint32_t t1[Tab<DT>::N1 ? Tab<DT>::N1 : 32];
+  uint32_t t2[Tab<DT>::N2];
+  union {  // the mean/variance scratch of a finalizing CTA reuses the (by then idle) staging ring
+    Ring<NW> ring;
+    MV mv;
+  };
+  Common<NW> k;
+};
+static_assert(sizeof(Smem<PEAT_F32>) <= 113 * 1024, "two float32 CTAs per SM");
+static_assert(sizeof(Smem<PEAT_BF16>) <= 227 * 1024 && sizeof(Smem<PEAT_F16>) <= 227 * 1024, "one 16-bit CTA per SM");
+static_assert(sizeof(MV) <= sizeof(Ring<8>), "the scratch fits the ring");
+static_assert(offsetof(Smem<PEAT_BF16>, ring) % 128 == 0 && offsetof(Smem<PEAT_F16>, ring) % 128 == 0 &&
+                  offsetof(Smem<PEAT_F32>, ring) % 128 == 0,
+              "bulk copies into the ring");
+
+
+template <int DT>
+__device__ __forceinline__ void sacc_add(Smem<DT>& sm, int which, unsigned __int128 m, int e, bool neg) {
+  for_digits(m, e, neg, [&](int j, int64_t v) { atomicAdd(&sm.k.sacc[which][j], (unsigned long long)v); });
 }
 // General-path terms, one per lane of a converged warp, into the warp's copy
 // of the sum digits: lanes whose digit indices agree are summed in registers
@@ -458,14 +526,15 @@ __device__ __forceinline__ void sacc_add(Smem& sm, int which, unsigned __int128 
 // so that no group sum overflows), and one lane per group adds the total.
 // Without this, the lanes of a warp would serialise on 64-bit shared atomics
 // to the same few digits.
-__device__ __forceinline__ void wsacc_add(Smem& sm, int which, uint64_t m, int e, bool neg, bool on) {
+template <int DT>
+__device__ __forceinline__ void wsacc_add(Smem<DT>& sm, int which, uint64_t m, int e, bool neg, bool on) {
   on = on && m != 0;
   if (!__any_sync(0xFFFFFFFFu, on)) return;
   const int lane = threadIdx.x & 31;
   const int p = e - LIMB_LSB, j = p >> 5, r = p & 31;
   const uint32_t m0 = (uint32_t)m, m1 = (uint32_t)(m >> 32);
   const uint32_t out[3] = {m0 << r, (m1 << r) | (r ? m0 >> (32 - r) : 0u), r ? m1 >> (32 - r) : 0u};
-  unsigned long long* d = sm.gsacc[threadIdx.x >> 5][which];
+  unsigned long long* d = sm.k.gsacc[threadIdx.x >> 5][which];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     const bool ok = on && out[k] != 0u && (unsigned)(j + k) < (unsigned)NLIMB;
@@ -476,21 +545,24 @@ __device__ __forceinline__ void wsacc_add(Smem& sm, int which, uint64_t m, int e
     if (ok && lane == __ffs(grp) - 1) atomicAdd(d + j + k, (unsigned long long)((int64_t)shi * 65536 + slo));
   }
 }
-__device__ __forceinline__ void wsacc_add_f(Smem& sm, int which, float x, int sc, bool on) {
+template <int DT>
+__device__ __forceinline__ void wsacc_add_f(Smem<DT>& sm, int which, float x, int sc, bool on) {
   int e = 0;
   const uint32_t m = x != 0.0f ? split_float(x, e) : 0u;
   wsacc_add(sm, which, m, e + sc, x < 0.0f, on);
 }
-__device__ __forceinline__ void wsacc_add_prod_f(Smem& sm, int which, float x, float y, int sc, bool on) {
+template <int DT>
+__device__ __forceinline__ void wsacc_add_prod_f(Smem<DT>& sm, int which, float x, float y, int sc, bool on) {
   int ex = 0, ey = 0;
   const uint32_t mx = x != 0.0f ? split_float(x, ex) : 0u, my = y != 0.0f ? split_float(y, ey) : 0u;
   wsacc_add(sm, which, (uint64_t)mx * my, ex + ey + sc, (x < 0.0f) != (y < 0.0f), on);
 }
 // one histogram bin per lane (bin < 0: none), counted once per distinct bin
-__device__ __forceinline__ void whist_add(Smem& sm, int bin) {
+template <int DT>
+__device__ __forceinline__ void whist_add(Smem<DT>& sm, int bin) {
   const unsigned grp = __match_any_sync(0xFFFFFFFFu, bin);
   if (bin >= 0 && (threadIdx.x & 31) == __ffs(grp) - 1 && PEAT_CHECK(bin < HBINS))
-    atomicAdd(&sm.ghist[threadIdx.x >> 5][bin], (unsigned long long)__popc(grp));
+    atomicAdd(&sm.k.ghist[threadIdx.x >> 5][bin], (unsigned long long)__popc(grp));
 }
 
 // floor(log2(a / g)) for a = (hi + lo) 2^sc > 0 and g > 0 (float32 pair, any range)
@@ -620,7 +692,7 @@ __device__ __forceinline__ void general_pair(GenRec& cd, GenOut& o, uint32_t G, 
 // 2^sc, |d| = (hi + lo) 2^sc with (hi, lo) = +-(s, t), d^2 = (s^2 + 2st +
 // t^2) 4^sc, added by the whole warp.
 template <int DT>
-__device__ __forceinline__ void general_lane(Smem& sm, GenRec& cd, uint32_t G, uint32_t C, int64_t idx, float rtol,
+__device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, uint32_t G, uint32_t C, int64_t idx, float rtol,
                                              float atol, bool valid) {
   GenOut o{-1, -1, 0.0f, 0.0f, 0};
   if (valid) general_pair<DT>(cd, o, G, C, idx, rtol, atol);
@@ -641,34 +713,29 @@ __device__ __forceinline__ void general_lane(Smem& sm, GenRec& cd, uint32_t G, u
 // ---------------------------------------------------------------------------
 // per-thread window state and per-piece window constants (registers)
 // ---------------------------------------------------------------------------
+// mism: window pairs above the tolerance (a float32 count, exact below 2^24).
+// float32 only, since the last flush, with |d| = (V1 2^21 + V2) 2^Lexp: A the
+// sum of |d| and S of d in units of 2^Lexp, Q11, Q12, Q22 the sums of V1 V1,
+// V1 V2, V2 V2.
 struct Lane {
-  uint32_t sa, sn;   // this tile's sum of V, and of V over negative d
-  uint32_t within;   // window pairs within tolerance
-  uint32_t uneq;     // unequal pairs seen (the rest of the piece is bitwise equal)
-  uint32_t ndef;     // pairs sent to the general path in the current tile
-  uint64_t A, N, Q;  // this round's sums of V, of V over negative d, of V^2
+  float mism;
+  int64_t A, S, Q12;
+  uint64_t Q11, Q22;
 };
 
-// This thread's window maxima so far (its pairs come in increasing index
-// order): a later pair at or below them cannot be a maximum of the piece, so
-// only pairs strictly above one of them are evaluated exactly.
-struct Thr {
-  float ta;       // |d|
-  uint32_t tu;    // ud
-  float tra, trm; // ratio tra / trm
-};
-
-// The window (warp-uniform; a warp moves it when too many of a tile's pairs
-// fall outside): Lb is the floor binade, Lexp = Lb - BIAS - MB the weight of
-// V's unit.
+// float32: the window (warp-uniform; a warp moves it when too many of a
+// tile's pairs fall outside): Lb is the floor binade, Lexp = Lb - BIAS - MB,
+// |d| a multiple of 2^Lexp below 2^(Lexp + 42).  bfloat16: fe, the float32 exponent field of the
+// smallest |d|; T1 holds 64 exponents from there.  binary16: fe = s, the
+// values are scaled by 2^s (exactly), so that their differences are normal.
 struct Win {
-  float rtol, atol;
-  float gmin;       // smallest |g| of a window pair: 2^(Lb + 1 - BIAS)
-  float lim;        // |d| < 2^(Lexp + 22)
-  float M;          // 1.5 * 2^(Lexp + 23): bits(|d| + M) - bits(M) = |d| / 2^Lexp
-  int lb;           // Lb
-  uint32_t base;    // shared address of this thread's counter in private row 0
-  uint32_t inc;     // 1 (low half of the word) or 65536 (high half)
+  float rtol, atol;  // binary16: atol scaled by 2^s
+  float lim;         // 2^(Lexp + 42)
+  // 1.5 * 2^(23 + e): bits(x + M) - bits(M) is x / 2^e rounded to an integer,
+  // for |x| < 2^(e + 22); e = Lexp + 21 for M1, Lexp for M2
+  float M1, M2;
+  int lb;            // Lb
+  int fe;
 };
 
 // the window with floor binade lb
@@ -677,43 +744,41 @@ __device__ __forceinline__ void set_window_lb(Win& W, int lb) {
   using Ty = Tr<DT>;
   const int lexp = lb - Ty::BIAS - Ty::MB;
   W.lb = lb;
-  W.gmin = (DT == PEAT_F16 && lb == Ty::LBMIN) ? __uint_as_float((uint32_t)(127 - 24) << 23)
-                                                 : __uint_as_float((uint32_t)(lb + 1 - Ty::BIAS + 127) << 23);
-  W.lim = __uint_as_float((uint32_t)(lexp + 22 + 127) << 23);
-  W.M = __uint_as_float(((uint32_t)(lexp + 23 + 127) << 23) | 0x400000u);
+  W.lim = __uint_as_float((uint32_t)(lexp + 42 + 127) << 23);
+  W.M1 = __uint_as_float(((uint32_t)(lexp + 44 + 127) << 23) | 0x400000u);
+  W.M2 = __uint_as_float(((uint32_t)(lexp + 23 + 127) << 23) | 0x400000u);
 }
 // The window placed for data whose largest finite golden exponent is emax and
-// whose ULP distances have ubits bits: V = |d| / 2^Lexp < 2^22 for such pairs
-// with goldens up to 2 binades above emax (one bit to spare on u).
+// whose ULP distances have ubits bits: |d| < 2^(Lexp + 42) for such pairs with
+// goldens up to 2 binades above emax (one bit to spare on u).
 template <int DT>
 __device__ __forceinline__ int window_floor(int emax, int ubits) {
   using Ty = Tr<DT>;
   const int UB = min(ubits + 1, Ty::UBMAX);
-  const int lb = emax + UB - 20;
+  const int lb = emax + UB - 40;
   return lb < Ty::LBMIN ? Ty::LBMIN : (lb > Ty::LBMAX ? Ty::LBMAX : lb);
 }
 template <int DT>
 __device__ __forceinline__ int win_lexp(const Win& W) {
   return W.lb - Tr<DT>::BIAS - Tr<DT>::MB;
 }
+// The window of 16-bit data whose largest finite golden exponent field is
+// emax.  bfloat16: a difference of at most 63 steps lies below 2^1 times the
+// golden's binade, so T1 ends 4 binades above the largest golden seen and
+// covers 59 below it; |d| stays at or above 2^-100 (tolerance differences
+// are then normal numbers, see count_mismatch).  binary16: the scale takes
+// the largest golden seen to 2^13, two binades below overflow; s >= 0 loses no
+// bits, and from s = 10 on even the smallest subnormal becomes normal.
+template <int DT>
+__device__ __forceinline__ int window16(int emax) {
+  if constexpr (DT == PEAT_F16) return min(max(28 - emax, 0), 15);
+  else return min(max(emax + 4 - 63, 27), 254 - 63);
+}
 
 __device__ __forceinline__ void lane_init(Lane& L) {
-  L.sa = L.sn = 0;
-  L.within = L.uneq = L.ndef = 0;
-  L.A = L.N = L.Q = 0;
-}
-__device__ __forceinline__ void thr_init(Thr& T) {
-  T.ta = 0.0f;
-  T.tu = 0;
-  T.tra = 0.0f;
-  T.trm = 1.0f;
-}
-__device__ __forceinline__ void rec_init(WinRec& r) {
-  r.amax = r.rd = 0.0f;
-  r.rg = 1.0f;
-  r.aidx = r.uidx = r.ridx = 0xFFFFFFFFu;
-  r.umax = 0;
-  r.pad = 0;
+  L.mism = 0.0f;
+  L.A = L.S = L.Q12 = 0;
+  L.Q11 = L.Q22 = 0;
 }
 __device__ __forceinline__ void gen_init(GenRec& c) {
   c.abs_hi = c.abs_lo = 0.0f;
@@ -726,160 +791,75 @@ __device__ __forceinline__ void gen_init(GenRec& c) {
   c.abs_idx = c.rel_idx = c.ulp_idx = -1;
 }
 
-__device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
-// sign(an1 / m1 - an2 / m2) > 0 for the normalised ratios of window pairs
-template <int DT>
-__device__ __forceinline__ bool rel_greater(float an1, float m1, float an2, float m2) {
-  const float p = __fmul_rn(an1, m2), q = __fmul_rn(an2, m1);
-  if constexpr (DT == PEAT_F32) {
-    // an has at most UB + 2 significant bits, m 24: the products need an
-    // error term, which is exact (no underflow: both products exceed 2^-26)
-    const float ep = __fmaf_rn(an1, m2, -p), eq = __fmaf_rn(an2, m1, -q);
-    return p > q || (p == q && ep > eq);
-  } else {
-    // at most (UB + 2) + (MB + 1) <= 24 significant bits: both products exact
-    return p > q;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// one unequal pair
-// ---------------------------------------------------------------------------
-
-// The window test.  gr, cr: raw bits (bf16: the float32 bits, i.e. raw << 16);
-// gf, cf: the values.  Also returns ud (the ULP distance, bf16: scaled by
-// 2^16), s = c - g, a = |s| and thr.  u < 2^MB keeps c within a factor 2 of
-// g (so c - g is exact in float32, Sterbenz); |g| >= gmin makes g and c
-// multiples of 2^Lexp; |d| < lim bounds V below 2^22; a tolerance tie goes to
-// the general path.  No sign test is needed: a pair of opposite signs has
-// ud > 2^23 (float32, bf16 scaled) or > 2^10 (fp16), beyond the bound.
-template <int DT>
-__device__ __forceinline__ uint32_t ud_bound() {
-  return DT == PEAT_BF16 ? (1u << Tr<DT>::MB) << 16 : 1u << Tr<DT>::MB;
-}
-template <int DT>
-__device__ __forceinline__ bool in_window(uint32_t gr, uint32_t cr, float gf, float cf, const Win& W, uint32_t& ud,
-                                          float& s, float& a, float& thr) {
-  {
-    const uint32_t dd = DT == PEAT_F16 ? cr - gr : __float_as_uint(cf) - __float_as_uint(gf);
-    ud = (int32_t)dd < 0 ? 0u - dd : dd;
-  }
-  s = __fsub_rn(cf, gf);
-  a = fabsf(s);
-  const float ag = fabsf(gf);
-  thr = __fmaf_rn(W.rtol, ag, W.atol);
-  return ud < ud_bound<DT>() && ag >= W.gmin && a < W.lim && a != thr;
-}
-
-// normalised ratio |d| / |g| = an / mg, mg in [1, 2)
-__device__ __forceinline__ void norm_ratio(float a, float gf, float& an, float& mg) {
-  const uint32_t gb = __float_as_uint(gf);
+// a1 / g1 > a2 / g2 for window pairs (positive normal a, g): the ratios
+// normalised to g in [1, 2), then exact products
+__device__ __forceinline__ void norm_ratio(float a, float g, float& an, float& mg) {
+  const uint32_t gb = __float_as_uint(g);
   an = __uint_as_float(__float_as_uint(a) - (gb & 0x7F800000u) + 0x3F800000u);
   mg = __uint_as_float((gb & 0x007FFFFFu) | 0x3F800000u);
 }
+__device__ __forceinline__ bool rel_greater(float a1, float g1, float a2, float g2) {
+  if (a2 == 0.0f) return a1 > 0.0f;
+  if (a1 == 0.0f) return false;
+  float an1, m1, an2, m2;
+  norm_ratio(a1, g1, an1, m1);
+  norm_ratio(a2, g2, an2, m2);
+  const float p = __fmul_rn(an1, m2), q = __fmul_rn(an2, m1);
+  // error terms of the products, exact (no underflow: both products exceed 2^-26)
+  const float ep = __fmaf_rn(an1, m2, -p), eq = __fmaf_rn(an2, m1, -q);
+  return p > q || (p == q && ep > eq);
+}
+
+// ---------------------------------------------------------------------------
+// window pairs
+// ---------------------------------------------------------------------------
+// Whether a pair of unequal patterns is a window pair: a pure function of the
+// bits and the window, so that a rescan of the piece decides as the tiles did.
+// G, C: raw bits.
+//
+// 16-bit types: both finite, C - G at most UMAX steps of the pattern either way
+// (the signs then agree), the golden not zero.  c - g is then exact in the type
+// itself (Sterbenz; a subnormal pair's difference is a multiple of the
+// smallest step) with at most 8 significant bits.  bfloat16: |d| also inside
+// T1 (so that both operands are normal).  binary16: the golden scaled by 2^fe
+// finite, and the scaled golden and difference normal.
+//
+// float32: ULP distance below 2^23 (so the signs agree and c is within a
+// factor 2 of g: c - g is exact, Sterbenz), |d| < lim and |d| a multiple of
+// 2^Lexp: |d| rounded to a multiple of 2^(Lexp + 21) and the (exact) remainder
+// are then read as integers V1, V2 from the bits of sums with M1 and M2; with
+// the remainder of the first, 42 bits hold the distances of goldens 20 binades
+// apart and more, so few pairs are left out.  2^Lexp is a normal number, so a golden that is zero or
+// subnormal never passes (its |d| is below 2^23 2^-149).
+template <int DT>
+__device__ __forceinline__ bool pair_window(uint32_t G, uint32_t C, const Win& W, uint32_t& u, float& gf, float& a) {
+  using Ty = Tr<DT>;
+  gf = to_f32<DT>(G);
+  const float cf = to_f32<DT>(C);
+  const float d = __fsub_rn(cf, gf);
+  a = fabsf(d);
+  u = C > G ? C - G : G - C;
+  if constexpr (DT == PEAT_F32) {
+    const float l = __fsub_rn(a, __fsub_rn(__fadd_rn(a, W.M1), W.M1));
+    return u < (1u << 23) && a < W.lim && __fsub_rn(__fadd_rn(l, W.M2), W.M2) == l;
+  } else {
+    const uint32_t mg = G & Ty::MAG, mc = C & Ty::MAG;
+    const bool ok = mg < Ty::INF && mc < Ty::INF && mg != 0u && u <= (uint32_t)Tab<DT>::UMAX && ((G ^ C) & Ty::SIGN) == 0u;
+    if constexpr (DT == PEAT_BF16) {
+      return ok && ((__float_as_uint(a) >> 23) - (uint32_t)W.fe) < 64u;
+    } else {
+      const float lo = __uint_as_float((uint32_t)(127 - 14 - W.fe) << 23);  // 2^-14 before scaling
+      return ok && (int)(mg >> 10) + W.fe <= 30 && a >= lo && fabsf(gf) >= lo;
+    }
+  }
+}
 
 // a pair outside the window: append it to the CTA's general list (evaluated
-// at the end of the piece; past GCAP entries the piece is rescanned).  G, C:
-// the pair's raw bits, kept with the first GSM entries.
-__device__ __forceinline__ void defer_pair(uint32_t li, uint32_t G, uint32_t C, Smem& sm) {
-  const uint32_t slot = atomicAdd(&sm.gn, 1u);
-  if (slot < (uint32_t)GCAP) sm.glist[slot] = li;
-}
-
-
-// Everything of one unequal pair except its maxima; returns whether the pair
-// lies strictly above one of the warp's maxima (it is then evaluated exactly
-// by rescan_pair).
+// at the end of the piece; past GCAP entries the piece is rescanned)
 template <int DT>
-__device__ __forceinline__ bool pair_proc(Lane& L, const Thr& T, uint32_t gr, uint32_t cr, float gf, float cf,
-                                          uint32_t li, const Win& W, Smem& sm) {
-  uint32_t ud;
-  float s, a, thr;
-  if (!in_window<DT>(gr, cr, gf, cf, W, ud, s, a, thr)) {
-    defer_pair(li, DT == PEAT_BF16 ? gr >> 16 : gr, DT == PEAT_BF16 ? cr >> 16 : cr, sm);
-    L.ndef++;
-    return false;
-  }
-  L.within += a < thr ? 1u : 0u;
-  float an, mg;
-  norm_ratio(a, gf, an, mg);
-  const int k = (int)(__float_as_uint(an) - __float_as_uint(mg)) >> 23;  // floor(log2(|d| / |g|))
-  red_shared(W.base + (uint32_t)((NUR - Rows<DT>::KLO + k) * ROWB), W.inc);
-  const uint32_t u = min(DT == PEAT_BF16 ? ud >> 16 : ud, (uint32_t)NUR);  // ULP bin, 63 = 63 or more
-  red_shared(W.base + (u - 1) * ROWB, W.inc);
-  // exact sums in units of 2^Lexp
-  const uint32_t V = __float_as_uint(__fadd_rn(a, W.M)) - __float_as_uint(W.M);
-  L.sa += V;
-  L.sn += s < 0.0f ? V : 0u;
-  L.Q += (uint64_t)V * V;
-  return (a > T.ta) | (ud > T.tu) | rel_greater<DT>(an, mg, T.tra, T.trm);
-}
-
-// a candidate pair (a window pair strictly above one of this thread's maxima,
-// later in index than all of them): update the exact records and thresholds
-template <int DT>
-__device__ __forceinline__ void rescan_pair(uint32_t gr, uint32_t cr, float gf, float cf, uint32_t li, const Win& W,
-                                            WinRec& r, Thr& T) {
-  uint32_t ud;
-  float s, a, thr;
-  in_window<DT>(gr, cr, gf, cf, W, ud, s, a, thr);
-  float an, mg;
-  norm_ratio(a, gf, an, mg);
-  if (a > T.ta) {
-    T.ta = a;
-    r.amax = a;
-    r.aidx = li;
-  }
-  if (ud > T.tu) {
-    T.tu = ud;
-    r.umax = ud;
-    r.uidx = li;
-  }
-  if (rel_greater<DT>(an, mg, T.tra, T.trm)) {
-    T.tra = an;
-    T.trm = mg;
-    r.rd = a;
-    r.rg = fabsf(gf);
-    r.ridx = li;
-  }
-}
-
-// element j of a 16-byte vector: raw bits in the form pair_proc takes, and value
-template <int DT>
-__device__ __forceinline__ void elem(const uint4& v, int j, uint32_t& r, float& f) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  if constexpr (DT == PEAT_F32) {
-    r = w[j];
-    f = __uint_as_float(r);
-  } else if constexpr (DT == PEAT_BF16) {
-    const uint32_t x = w[j >> 1];
-    r = (j & 1) ? (x & 0xFFFF0000u) : (x << 16);
-    f = __uint_as_float(r);
-  } else {
-    const uint32_t x = w[j >> 1];
-    const __half2 h = *reinterpret_cast<const __half2*>(&x);
-    r = (j & 1) ? (x >> 16) : (x & 0xFFFFu);
-    f = (j & 1) ? __high2float(h) : __low2float(h);
-  }
-}
-
-// element at position pos of a staged tile
-template <int DT>
-__device__ __forceinline__ void elem_at(const uint4* t, uint32_t pos, uint32_t& r, float& f) {
-  if constexpr (DT == PEAT_F32) {
-    r = reinterpret_cast<const uint32_t*>(t)[pos];
-    f = __uint_as_float(r);
-  } else if constexpr (DT == PEAT_BF16) {
-    r = (uint32_t)reinterpret_cast<const unsigned short*>(t)[pos] << 16;
-    f = __uint_as_float(r);
-  } else {
-    const unsigned short x = reinterpret_cast<const unsigned short*>(t)[pos];
-    r = x;
-    f = __half2float(__ushort_as_half(x));
-  }
+__device__ __forceinline__ void defer_pair(uint32_t li, Smem<DT>& sm) {
+  const uint32_t slot = atomicAdd(&sm.k.gn, 1u);
+  if (slot < (uint32_t)GCAP) sm.k.glist[slot] = li;
 }
 
 // lanes of one vector whose golden value is NaN or Inf, as a bitmask
@@ -895,35 +875,33 @@ __device__ __forceinline__ uint32_t nonfinite_lanes(const uint4& v) {
 template <int DT>
 __device__ __forceinline__ bool any_nonfinite(const uint4& v) {
   using T = Tr<DT>;
-  if constexpr (T::BYTES == 2) {
-    constexpr uint32_t ADD = (0x8000u - T::INF) * 0x10001u;  // sets bit 15 of a half iff its magnitude >= INF
-    return ((((v.x & 0x7FFF7FFFu) + ADD) | ((v.y & 0x7FFF7FFFu) + ADD) | ((v.z & 0x7FFF7FFFu) + ADD) |
-             ((v.w & 0x7FFF7FFFu) + ADD)) & 0x80008000u) != 0u;
+  if constexpr (T::BYTES == 2) {  // x * 0 is NaN for NaN and infinity, else a zero
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t z = 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      if constexpr (DT == PEAT_BF16) {
+        const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]), __floats2bfloat162_rn(0.0f, 0.0f),
+                                         *reinterpret_cast<const __nv_bfloat162*>(&z));
+        z = *reinterpret_cast<const uint32_t*>(&r);
+      } else {
+        const __half2 r = __hfma2(*reinterpret_cast<const __half2*>(&w[i]), __floats2half2_rn(0.0f, 0.0f),
+                                  *reinterpret_cast<const __half2*>(&z));
+        z = *reinterpret_cast<const uint32_t*>(&r);
+      }
+    }
+    return (z & 0x7FFF7FFFu) != 0u;
   } else {
     uint32_t m = max(max(v.x & T::MAG, v.y & T::MAG), max(v.z & T::MAG, v.w & T::MAG));
     return m >= T::INF;
   }
 }
-// bitmask of the lanes whose bit patterns differ
-template <int DT>
-__device__ __forceinline__ uint32_t unequal_mask(const uint4& g, const uint4& c) {
-  const uint32_t x[4] = {g.x ^ c.x, g.y ^ c.y, g.z ^ c.z, g.w ^ c.w};
-  uint32_t m = 0;
-  if constexpr (Tr<DT>::BYTES == 4) {
-#pragma unroll
-    for (int j = 0; j < 4; j++) m |= (x[j] != 0u ? 1u : 0u) << j;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; j++) m |= ((x[j] & 0xFFFFu) != 0u ? 1u : 0u) << (2 * j) | (x[j] > 0xFFFFu ? 2u : 0u) << (2 * j);
-  }
-  return m;
-}
 
-// Equal lanes of one vector: every bitwise-equal pair is EXACT; the ones
-// holding NaN/Inf also count as non-finite pairs.
+// A vector of equal pairs: every one is EXACT; the ones holding NaN/Inf also
+// count as non-finite pairs.
 template <int DT>
-__device__ __forceinline__ void count_equal(const uint4& g, uint32_t eqm, Smem& sm) {
-  if (eqm && any_nonfinite<DT>(g)) atomicAdd(&sm.nfe, (uint32_t)__popc(nonfinite_lanes<DT>(g) & eqm));
+__device__ __forceinline__ void count_equal(const uint4& g, Smem<DT>& sm) {
+  if (any_nonfinite<DT>(g)) atomicAdd(&sm.k.nfe, (uint32_t)__popc(nonfinite_lanes<DT>(g)));
 }
 
 __device__ __forceinline__ uint64_t wsum64(uint64_t v) {
@@ -932,239 +910,558 @@ __device__ __forceinline__ uint64_t wsum64(uint64_t v) {
   return v;
 }
 
-// This warp's window sums (in units of 2^lexp) into the CTA's exact
-// accumulator: A, N < 2^38 and Q < 2^60 per thread between flushes; warp sums
-// in 128 bits.
-__device__ __forceinline__ void flush_sums(Lane& L, Smem& sm, int lexp) {
-  const uint64_t A = wsum64(L.A), N = wsum64(L.N);
-  const uint64_t qlo = wsum64(L.Q & 0xFFFFFFFFull), qhi = wsum64(L.Q >> 32);
-  if ((threadIdx.x & 31) == 0) {
-    const uint64_t P = A - N;  // sum of V over positive d
-    if (P >= N) sacc_add(sm, 0, (unsigned __int128)(P - N), lexp, false);
-    else sacc_add(sm, 0, (unsigned __int128)(N - P), lexp, true);
-    sacc_add(sm, 1, (unsigned __int128)A, lexp, false);
-    sacc_add(sm, 2, (unsigned __int128)qlo + ((unsigned __int128)qhi << 32), 2 * lexp, false);
-  }
-  L.A = L.N = L.Q = 0;
-}
-
-// When a tile sent many pairs (at least 32, and a quarter of its unequal
-// ones) to the general path, the warp moves its window to the tile's own data
-// -- largest finite golden exponent, largest same-sign ULP distance -- after
-// flushing the sums kept in the old window's units, and logs the move so that
-// a rescan of the piece applies to every pair the window it saw.  At most
-// RWMAX moves per warp and piece.
-// the window floor for the data of a staged tile (out of line: rarely run)
-template <int DT>
-__device__ __noinline__ int tile_window_floor(const uint4* gt, const uint4* ct, int nvalid) {
-  using Ty = Tr<DT>;
+// float32: this warp's window sums (in units of 2^lexp) into the CTA's exact
+// accumulator: |A|, |S| < 2^59, Q11, Q22 and |Q12| < 2^58 per thread between
+// flushes; combined in 128 bits.
+__device__ __forceinline__ void flush_sums(Lane& L, Smem<PEAT_F32>& sm, int lexp) {
+  const uint64_t A = wsum64((uint64_t)L.A), S = wsum64((uint64_t)L.S);
+  const uint64_t q11 = wsum64(L.Q11), q12 = wsum64((uint64_t)L.Q12), q22 = wsum64(L.Q22);
   const int lane = threadIdx.x & 31;
-  uint32_t emax = 0, umax = 0;
-#pragma unroll
-  for (int v = 0; v < 2; v++) {
-    if (lane + 32 * v >= nvalid) continue;
-    const uint4 gv = gt[lane + 32 * v], cv = ct[lane + 32 * v];
-#pragma unroll
-    for (int j = 0; j < Ty::VEC; j++) {
-      const uint32_t G = lane_bits<DT>(gv, j), C = lane_bits<DT>(cv, j);
-      const uint32_t e = (G & Ty::MAG) >> Ty::MB;
-      if (e < (uint32_t)Ty::EMAX && e > emax) emax = e;
-      if (((G ^ C) & Ty::SIGN) == 0u && (G & Ty::MAG) < Ty::INF && (C & Ty::MAG) < Ty::INF)
-        umax = max(umax, G > C ? G - C : C - G);
-    }
+  if (lane < NSUM) {  // a lane per sum
+    const bool neg = lane == 0 && (int64_t)S < 0;
+    const unsigned __int128 q = ((unsigned __int128)q11 << 42) + (unsigned __int128)((__int128)(int64_t)q12 << 22) + q22;
+    const unsigned __int128 m = lane == 0 ? (unsigned __int128)(neg ? 0ull - S : S) : (lane == 1 ? (unsigned __int128)A : q);
+    sacc_add<PEAT_F32>(sm, lane, m, lane == 2 ? 2 * lexp : lexp, neg);
   }
-  emax = __reduce_max_sync(0xFFFFFFFFu, emax);
-  umax = __reduce_max_sync(0xFFFFFFFFu, umax);
-  return window_floor<DT>((int)emax, 32 - __clz(umax));
+  L.A = L.S = L.Q12 = 0;
+  L.Q11 = L.Q22 = 0;
 }
 
-// nd: the warp's general pairs of this tile, total: its unequal pairs
-template <int DT>
-__device__ __forceinline__ void maybe_rewindow(Lane& L, Win& W, const uint4* gt, const uint4* ct, int nvalid,
-                                               uint32_t nd, uint32_t total, uint32_t ichunk, Smem& sm) {
-  if (nd < 32u || nd * 4u < total) return;
+// float32: when the slow path sent many pairs of a tile (at least 32, and a
+// quarter of the unequal ones it saw) to the general path, the warp moves its
+// window to the data it saw there -- largest finite golden exponent, largest
+// same-sign ULP distance (wem, wum) -- after flushing the sums kept in the old window's
+// units, and logs the move so that a rescan of the piece applies to every pair
+// the window it saw.  At most RWMAX moves per warp and piece.
+// (This part: the new floor binade, logged; -1: the window stays.)
+__device__ __noinline__ int next_window(int lb0, uint32_t ichunk, Smem<PEAT_F32>& sm) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t r = sm.nwin[warp];
-  if (r >= (uint32_t)RWMAX) return;
-  const int lb = tile_window_floor<DT>(gt, ct, nvalid);
-  if (lb == W.lb) return;
-  flush_sums(L, sm, win_lexp<DT>(W));
-  set_window_lb<DT>(W, lb);
+  const uint32_t r = sm.k.nwin[warp];
+  const int lb = window_floor<PEAT_F32>((int)sm.k.wem[warp], 32 - __clz(sm.k.wum[warp]));
+  if (r >= (uint32_t)RWMAX || lb == lb0) return -1;
   __syncwarp();
   if (lane == 0) {
-    sm.wstart[warp][r + 1] = ichunk + 1;
-    sm.wlb[warp][r + 1] = lb;
-    sm.nwin[warp] = r + 1;
+    sm.k.wstart[warp][r + 1] = ichunk + 1;
+    sm.k.wlb[warp][r + 1] = lb;
+    sm.k.nwin[warp] = r + 1;
   }
   __syncwarp();
+  return lb;
 }
 
-// One warp tile of CHV vectors staged in shared memory: lane L owns vectors L
-// and L + 32; tile element e sits at offset tli + e from the CTA's first
-// element.  Equal pairs are counted in place.  When at most a quarter of the
-// pairs differ, each lane works through its own unequal pairs (cheaper than
-// compacting a few); otherwise they are queued (in element order) and
-// processed 32 at a time, so every thread does useful work.  Pairs above the
-// thread's maxima are then evaluated exactly.
+// The bounds a tile's pairs are tested against, from the CTA's records.  A
+// pair above one of them takes the slow path; pairs at or below all of them
+// cannot be a maximum of the piece.  A record at or after the tile's first
+// element (another warp is ahead, or a starting bound) is lowered one step,
+// so that an equal value at a lower index is seen.  A starting bound may come
+// from a pair outside the window, so each is capped at the window's own.
+struct Bounds {
+  uint32_t ab;  // |d|: float32 bits, or the (scaled) 16-bit pattern in both halves
+  uint32_t ub;  // ULP distance
+  float r;      // ratio: a pair is above when |d| - |g| r > 0
+  bool low;     // one of them was lowered: read again before the next tile
+};
 template <int DT>
-__device__ __forceinline__ void do_tile(Lane& L, Thr& T, const uint4* gt, int nvalid, uint32_t tli, Win& W,
-                                        uint32_t ichunk, Smem& sm) {
-  // the candidate ring sits a fixed distance after the golden ring
-  const uint4* ct = gt + (offsetof(Smem, ring_c) - offsetof(Smem, ring_g)) / sizeof(uint4);
+__device__ __forceinline__ Bounds read_bounds(const Smem<DT>& sm, uint32_t tli, const Win& W) {
+  const unsigned long long ka = *(volatile const unsigned long long*)&sm.k.kabs;
+  const unsigned long long ku = *(volatile const unsigned long long*)&sm.k.kulp;
+  const unsigned long long kr = *(volatile const unsigned long long*)&sm.k.krel;
+  Bounds b;
+  b.ab = (uint32_t)(ka >> 32);
+  if constexpr (DT == PEAT_BF16) {
+    b.ab = min(b.ab, ((uint32_t)(W.fe + 64) << 23) - 0x10000u) >> 16;
+  } else if constexpr (DT == PEAT_F16) {
+    const float sc = __fmul_rn(__uint_as_float(b.ab), __uint_as_float((uint32_t)(127 + W.fe) << 23));
+    b.ab = sc < 65504.0f ? (uint32_t)__half_as_ushort(__float2half_rn(sc)) : 0x7BFFu;
+  } else {
+    b.ab = min(b.ab, __float_as_uint(W.lim) - 1u);
+  }
+  b.low = ~(uint32_t)ka >= tli && b.ab != 0u;
+  if (b.low) b.ab--;
+  if constexpr (DT != PEAT_F32) b.ab |= b.ab << 16;
+  b.ub = min((uint32_t)(ku >> 32), (uint32_t)Tab<DT>::UMAX);
+  const bool lu = ~(uint32_t)ku >= tli && b.ub != 0u, lr = ~(uint32_t)kr >= tli;
+  if (lu) b.ub--;
+  b.low = b.low || lu || (DT != PEAT_F32 && lr && kr != 0ull);
+  const float q = __uint_as_float((uint32_t)(kr >> 32));
+  // 16-bit types: q is the record's ratio rounded to nearest, and two distinct
+  // ratios of window pairs (|d| and |g| of at most 8 and 11 significant bits)
+  // differ by more than 2^-20 of their value, so a factor 1 +- 2^-22 separates
+  // them exactly.  float32: always lowered (q is a lower bound already).
+  b.r = __fmul_rn(q, DT == PEAT_F32 || lr ? 0.99999976158142090f : 1.0000002384185791f);
+  return b;
+}
+
+// One vector position of a staged tile, all lanes of the warp, when some pair
+// of it is out of the window or above a bound: pairs out of the window go to
+// the general list, the window maxima into the CTA's records, and the tile's
+// pairs that the table phase must not see (general pairs, equal pairs holding
+// NaN or Inf) are zeroed in the stage.  Returns the lane's general pairs and
+// (high half) unequal pairs.  Out of line: it runs a few times per warp on
+// ordinary data.
+template <int DT>
+__device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t li0, int lb, int fe) {
   using Ty = Tr<DT>;
-  constexpr int VEC = Ty::VEC;
-  constexpr uint32_t FULL = (1u << VEC) - 1u;
+  using E = typename std::conditional<Ty::BYTES == 4, uint32_t, unsigned short>::type;
+  Win W;
+  if constexpr (DT == PEAT_F32) set_window_lb<DT>(W, lb);
+  else W.lim = W.M1 = W.M2 = 0.0f, W.lb = 0;
+  W.rtol = W.atol = 0.0f;
+  W.fe = fe;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool okA = lane < nvalid, okB = lane + 32 < nvalid;
-  uint4 gA, cA, gB, cB;
-  if (nvalid == CHV) {  // a full tile (all but the last of a piece)
-    gA = gt[lane];
-    cA = ct[lane];
-    gB = gt[lane + 32];
-    cB = ct[lane + 32];
-  } else {
-    const uint4 z = make_uint4(0, 0, 0, 0);
-    gA = okA ? gt[lane] : z;
-    cA = okA ? ct[lane] : z;
-    gB = okB ? gt[lane + 32] : z;
-    cB = okB ? ct[lane + 32] : z;
-  }
-  const bool diff = ((gA.x ^ cA.x) | (gA.y ^ cA.y) | (gA.z ^ cA.z) | (gA.w ^ cA.w) | (gB.x ^ cB.x) | (gB.y ^ cB.y) |
-                     (gB.z ^ cB.z) | (gB.w ^ cB.w)) != 0u;
-  if (!__any_sync(0xFFFFFFFFu, diff)) {  // the whole warp tile is bitwise equal
-    if (okA) count_equal<DT>(gA, FULL, sm);
-    if (okB) count_equal<DT>(gB, FULL, sm);
-    return;
-  }
-  const uint32_t nA = okA ? unequal_mask<DT>(gA, cA) : 0u, nB = okB ? unequal_mask<DT>(gB, cB) : 0u;
-  if (okA) count_equal<DT>(gA, FULL & ~nA, sm);
-  if (okB) count_equal<DT>(gB, FULL & ~nB, sm);
-  // one scan of the packed counts gives the A-queue and B-queue offsets (10-bit
-  // fields: a warp tile has at most 512 pairs)
-  const uint32_t packed = __popc(nA) | (__popc(nB) << 10);
-  uint32_t incl = packed;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
-  const uint32_t totA = tot & 0x3FFu, total = totA + ((tot >> 10) & 0x3FFu);
-  L.uneq += __popc(nA) + __popc(nB);
-  if (total * 4u <= 64u * VEC) {
-    // sparse tile: each lane visits its own unequal pairs (slot s < VEC:
-    // element s of vector A, else element s - VEC of vector B; increasing index)
-    uint32_t m = nA | (nB << VEC), cm = 0;
-    while (m) {
-      const uint32_t sl = __ffs(m) - 1;
-      m &= m - 1u;
-      const uint32_t pos = sl < (uint32_t)VEC ? lane * VEC + sl : (lane + 32) * VEC + sl - VEC;
-      uint32_t gr, cr;
-      float gf, cf;
-      elem_at<DT>(gt, pos, gr, gf);
-      elem_at<DT>(ct, pos, cr, cf);
-      if (pair_proc<DT>(L, T, gr, cr, gf, cf, tli + pos, W, sm)) cm |= 1u << sl;
-    }
-    L.A += L.sa;
-    L.N += L.sn;
-    L.sa = L.sn = 0;
-    if (cm) {
-      WinRec& r = sm.rec[threadIdx.x];
-      do {
-        const uint32_t sl = __ffs(cm) - 1;
-        cm &= cm - 1u;
-        const uint32_t pos = sl < (uint32_t)VEC ? lane * VEC + sl : (lane + 32) * VEC + sl - VEC;
-        uint32_t gr, cr;
-        float gf, cf;
-        elem_at<DT>(gt, pos, gr, gf);
-        elem_at<DT>(ct, pos, cr, cf);
-        rescan_pair<DT>(gr, cr, gf, cf, tli + pos, W, r, T);
-      } while (cm);
-    }
-    L.ndef = 0;  // sparse tiles never move the window (a quarter of their pairs at most differ)
-    __syncwarp();
-    return;
-  }
-  uint32_t posA = (incl & 0x3FFu) - (packed & 0x3FFu);
-  uint32_t posB = totA + ((incl >> 10) & 0x3FFu) - ((packed >> 10) & 0x3FFu);
-  unsigned short* q = sm.qp[warp];
-#pragma unroll
-  for (int j = 0; j < VEC; j++) {
-    if ((nA >> j) & 1u) q[posA++] = (unsigned short)(lane * VEC + j);
-    if ((nB >> j) & 1u) q[posB++] = (unsigned short)((lane + 32) * VEC + j);
-  }
-  __syncwarp();
-  // two queue entries per iteration (e, e + 32: in index order per lane);
-  // bit o of cm marks this lane's o-th entry as a maxima candidate
-  uint32_t cm = 0;
-  uint32_t ob = 1;
-  for (uint32_t e = lane; e < total; e += 64, ob <<= 2) {
-    const uint32_t pos0 = q[e];
-    const bool two = e + 32 < total;
-    const uint32_t pos1 = two ? q[e + 32] : pos0;
-    uint32_t gr0, cr0, gr1, cr1;
-    float gf0, cf0, gf1, cf1;
-    elem_at<DT>(gt, pos0, gr0, gf0);
-    elem_at<DT>(ct, pos0, cr0, cf0);
-    elem_at<DT>(gt, pos1, gr1, gf1);
-    elem_at<DT>(ct, pos1, cr1, cf1);
-    if (pair_proc<DT>(L, T, gr0, cr0, gf0, cf0, tli + pos0, W, sm)) cm |= ob;
-    if (two && pair_proc<DT>(L, T, gr1, cr1, gf1, cf1, tli + pos1, W, sm)) cm |= ob << 1;
-  }
-  L.A += L.sa;
-  L.N += L.sn;
-  L.sa = L.sn = 0;
-  if (cm) {
-    WinRec& r = sm.rec[threadIdx.x];
-    do {
-      const uint32_t o = __ffs(cm) - 1;
-      cm &= cm - 1u;
-      const uint32_t pos = q[lane + 32 * o];
-      uint32_t gr, cr;
-      float gf, cf;
-      elem_at<DT>(gt, pos, gr, gf);
-      elem_at<DT>(ct, pos, cr, cf);
-      rescan_pair<DT>(gr, cr, gf, cf, tli + pos, W, r, T);
-    } while (cm);
-  }
+  E* g = reinterpret_cast<E*>(gt);
+  E* c = reinterpret_cast<E*>(ct);
+  float ba = 0.0f, rq = 0.0f, ra = 0.0f, rg = 1.0f;
+  uint32_t ai = 0, bu = 0, ui = 0, ri = 0, nd = 0, ne = 0, nf = 0, em = 0, um0 = 0;
   {
-    const uint32_t nd = __reduce_add_sync(0xFFFFFFFFu, L.ndef);
-    L.ndef = 0;
-    maybe_rewindow<DT>(L, W, gt, ct, nvalid, nd, total, ichunk, sm);
+#pragma unroll 1
+    for (int j = 0; j < Ty::VEC; j++) {
+      const uint32_t G = g[j], C = c[j];
+      if constexpr (DT == PEAT_F32) {  // what places the next window
+        const uint32_t mg = G & Ty::MAG;
+        if (mg < Ty::INF) em = max(em, mg >> Ty::MB);
+        if (((G ^ C) & Ty::SIGN) == 0u && mg < Ty::INF && (C & Ty::MAG) < Ty::INF) um0 = max(um0, G > C ? G - C : C - G);
+      }
+      if (G == C) {
+        if ((G & Ty::MAG) >= Ty::INF) {
+          nf++;
+          g[j] = 0;
+          c[j] = 0;
+        }
+        continue;
+      }
+      ne++;
+      uint32_t u;
+      float gf, a;
+      if (!pair_window<DT>(G, C, W, u, gf, a)) {
+        defer_pair<DT>(li0 + j, sm);
+        nd++;
+        g[j] = 0;
+        c[j] = 0;
+        continue;
+      }
+      const float ag = fabsf(gf);
+      if (a > ba) ba = a, ai = li0 + j;
+      if (u > bu) bu = u, ui = li0 + j;
+      if constexpr (DT == PEAT_F32) {
+        if (rel_greater(a, ag, ra, rg)) ra = a, rg = ag, ri = li0 + j;
+      } else {
+        const float q = __fdiv_rn(a, ag);
+        if (q > rq) rq = q, ra = a, rg = ag, ri = li0 + j;
+      }
+    }
   }
+  if (nf) atomicAdd(&sm.k.nfe, nf);
+  if constexpr (DT == PEAT_F32) {
+    em = __reduce_max_sync(0xFFFFFFFFu, em);
+    um0 = __reduce_max_sync(0xFFFFFFFFu, um0);
+    if (lane == 0) {
+      sm.k.wem[warp] = max(sm.k.wem[warp], em);
+      sm.k.wum[warp] = max(sm.k.wum[warp], um0);
+    }
+  }
+  // lanes hold consecutive elements, so the lowest lane has the lowest index
+  const uint32_t am = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(ba));
+  if (am) {
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, __float_as_uint(ba) == am);
+    if (lane == __ffs(who) - 1) atomicMax(&sm.k.kabs, ((unsigned long long)am << 32) | (uint32_t)~ai);
+  }
+  const uint32_t um = __reduce_max_sync(0xFFFFFFFFu, bu);
+  if (um) {
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, bu == um);
+    if (lane == __ffs(who) - 1) atomicMax(&sm.k.kulp, ((unsigned long long)um << 32) | (uint32_t)~ui);
+  }
+  if (am) {
+    RelRec& R = sm.k.wrel[warp];
+    if constexpr (DT == PEAT_F32) {
+      // the lanes near the best approximate ratio, in order, compared exactly
+      const float qa = ra > 0.0f ? __fdiv_rn(ra, rg) : 0.0f;
+      const float qm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(qa)));
+      unsigned cand = __ballot_sync(0xFFFFFFFFu, ra > 0.0f && qa >= __fmul_rn(qm, 0.999999f));
+      float xa = R.a, xg = R.g;
+      uint32_t xi = R.li;
+      bool up = false;
+      while (cand) {
+        const int s = __ffs(cand) - 1;
+        cand &= cand - 1u;
+        const float ya = __shfl_sync(0xFFFFFFFFu, ra, s), yg = __shfl_sync(0xFFFFFFFFu, rg, s);
+        const uint32_t yi = __shfl_sync(0xFFFFFFFFu, ri, s);
+        if (rel_greater(ya, yg, xa, xg)) xa = ya, xg = yg, xi = yi, up = true;
+      }
+      __syncwarp();
+      if (up && lane == 0) {
+        R.a = xa;
+        R.g = xg;
+        R.li = xi;
+        atomicMax(&sm.k.krel, (unsigned long long)__float_as_uint(__fdiv_rd(xa, xg)) << 32);
+      }
+    } else {
+      const uint32_t qm = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(rq));
+      const unsigned who = __ballot_sync(0xFFFFFFFFu, __float_as_uint(rq) == qm);
+      if (lane == __ffs(who) - 1 && rq > R.q) {
+        R.a = ra;
+        R.g = rg;
+        R.q = rq;
+        R.li = ri;
+        atomicMax(&sm.k.krel, ((unsigned long long)qm << 32) | (uint32_t)~ri);
+      }
+    }
+  }
+  fence_proxy_async();  // the zeroed pairs before the next bulk copy into the stage
   __syncwarp();
+  return nd | (ne << 16);
 }
 
-// one element outside the vector grid (li: offset from the CTA's first
-// element), with its maxima evaluated exactly
-template <int DT>
-__device__ __forceinline__ void do_scalar(Lane& L, Thr& T, uint32_t G, uint32_t C, uint32_t li, const Win& W,
-                                          Smem& sm) {
-  using Ty = Tr<DT>;
-  if (G == C) {
-    if ((G & Ty::MAG) >= Ty::INF) atomicAdd(&sm.nfe, 1u);
-    return;
-  }
-  L.uneq++;
-  uint32_t gr = G, cr = C;
-  float gf, cf;
-  if constexpr (DT == PEAT_F32) {
-    gf = __uint_as_float(G);
-    cf = __uint_as_float(C);
-  } else if constexpr (DT == PEAT_BF16) {
-    gr = G << 16;
-    cr = C << 16;
-    gf = __uint_as_float(gr);
-    cf = __uint_as_float(cr);
-  } else {
-    gf = __half2float(__ushort_as_half((unsigned short)G));
-    cf = __half2float(__ushort_as_half((unsigned short)C));
-  }
-  if (pair_proc<DT>(L, T, gr, cr, gf, cf, li, W, sm)) rescan_pair<DT>(gr, cr, gf, cf, li, W, sm.rec[threadIdx.x], T);
-  L.A += L.sa;
-  L.N += L.sn;
-  L.sa = L.sn = 0;
+// ---- the tile loops ---------------------------------------------------------
+// Per vector and lane: the checks of every pair (no branches), one vote, then
+// the table increments.  The checks flag a pair that is not a window pair or
+// lies above one of the bounds; a warp with a flagged pair runs slow_vec and
+// then the table phase on what is left.  Everything the signature needs comes
+// from the tables, except the tolerance count and (float32) the sums.
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ __half2 h2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+__device__ __forceinline__ __nv_bfloat162 b2(uint32_t v) { return *reinterpret_cast<const __nv_bfloat162*>(&v); }
+template <class T>
+__device__ __forceinline__ uint32_t bits2(const T& v) {
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// add one to the shared word at byte offset off of the dynamic shared memory
+// (constant plus a register: one instruction)
+extern __shared__ __align__(128) unsigned char smem_raw[];
+__device__ __forceinline__ void inc_shared(uint32_t base, uint32_t off) {
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(base + off));
+}
+// mism += |d| > atol + rtol |g|, exactly: |d| is a float32, so it exceeds the
+// bound when it exceeds the bound rounded down, and the difference (a normal
+// number, |d| >= 2^-100) times 2^127 saturates to 0 or 1.  All on the FP32
+// pipe, which has twice the rate of compares and integer adds.
+__device__ __forceinline__ void count_mismatch(float& mism, float d, float g, const Win& W) {
+  const float over = __fsub_rn(fabsf(d), __fmaf_rd(W.rtol, fabsf(g), W.atol));
+  mism += __saturatef(__fmul_rn(over, 0x1p127f));
+}
+
+// the two halves of a packed pair as float32
+__device__ __forceinline__ float lo_b(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float hi_b(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
+
+// NP packed pairs of pairs: what both phases use
+template <int NP>
+struct Vec16 {
+  uint32_t t[NP];  // packed ULP steps + UMAX + 1
+  uint32_t d[NP];  // packed (scaled) differences c - g
+  uint32_t g[NP];  // packed (scaled) goldens
+};
+// Packed pattern differences plus the bias: each half in (0, 2 bias) for a
+// window pair.  A borrow or a carry out of the low half means that the low pair
+// is flagged as well (out of range, or holding NaN or Inf).
+template <int DT, int NP>
+__device__ __forceinline__ void prep16(Vec16<NP>& v, const uint32_t (&g)[NP], const uint32_t (&c)[NP], uint32_t scale2) {
+  constexpr uint32_t BIAS = (uint32_t)(Tab<DT>::UMAX + 1) * 0x10001u;
+#pragma unroll
+  for (int i = 0; i < NP; i++) {
+    v.t[i] = c[i] - g[i] + BIAS;
+    if constexpr (DT == PEAT_BF16) {
+      v.g[i] = g[i];
+      v.d[i] = bits2(__hsub2(b2(c[i]), b2(g[i])));
+    } else {
+      const __half2 gs = __hmul2(h2(g[i]), h2(scale2));
+      v.g[i] = bits2(gs);
+      v.d[i] = bits2(__hfma2(h2(c[i]), h2(scale2), __hneg2(gs)));
+    }
+  }
+}
+// true when a pair of the vector is flagged
+template <int DT, int NP>
+__device__ __forceinline__ bool check16(const Vec16<NP>& v, const Win& W, const Bounds& B) {
+  // the biased step counts are binary16 subnormals: exact sums in units of 2^-24
+  constexpr uint32_t NBIAS = (uint32_t)(Tab<DT>::UMAX + 1) * 0x10001u | 0x80008000u;
+  __half2 um = h2(0u);
+  float xm = 0.0f;
+  bool bad;
+#pragma unroll
+  for (int i = 0; i < NP; i++) um = __hmax2_nan(um, __habs2(__hadd2(h2(v.t[i]), h2(NBIAS))));
+  bad = !__hble2(um, h2(B.ub * 0x10001u));
+  if constexpr (DT == PEAT_BF16) {
+    const __nv_bfloat162 fl = b2((uint32_t)W.fe * 0x00800080u);
+    __nv_bfloat162 am = b2(0u), tiny = b2(0u);
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+      const __nv_bfloat162 ad = __habs2(b2(v.d[i]));
+      am = __hmax2_nan(am, ad);
+      tiny = __hfma2(__hlt2(ad, fl), ad, tiny);  // a difference below T1 (but not zero)
+      xm = max3(xm, __fmaf_rn(-fabsf(lo_b(v.g[i])), B.r, fabsf(lo_b(v.d[i]))),
+                __fmaf_rn(-fabsf(hi_b(v.g[i])), B.r, fabsf(hi_b(v.d[i]))));
+    }
+    bad = bad || !__hble2(am, b2(B.ab)) || (bits2(tiny) & 0x7FFF7FFFu) != 0u;
+  } else {
+    __half2 am = h2(0u);
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+      am = __hmax2_nan(am, __habs2(h2(v.d[i])));
+      xm = max3(xm, __fmaf_rn(-fabsf(__low2float(h2(v.g[i]))), B.r, fabsf(__low2float(h2(v.d[i])))),
+                __fmaf_rn(-fabsf(__high2float(h2(v.g[i]))), B.r, fabsf(__high2float(h2(v.d[i])))));
+    }
+    bad = bad || !__hble2(am, h2(B.ab));
+    if (W.fe < 10) {  // a subnormal golden or difference (but not zero)
+      const __half2 fl = h2(0x04000400u);
+      __half2 tiny = h2(0u);
+#pragma unroll
+      for (int i = 0; i < NP; i++) {
+        const __half2 ad = __habs2(h2(v.d[i]));
+        tiny = __hmax2(tiny, __hmul2(__hlt2(__hmin2(ad, __habs2(h2(v.g[i]))), fl), ad));
+      }
+      bad = bad || (bits2(tiny) & 0x7FFF7FFFu) != 0u;
+    }
+  }
+  return bad || xm > 0.0f;
+}
+// the table phase
+template <int DT, int NP>
+__device__ __forceinline__ void count16(const Vec16<NP>& v, const Win& W, uint32_t t1, uint32_t t2, float& mism) {
+#pragma unroll
+  for (int i = 0; i < NP; i++) {
+    const uint32_t d = v.d[i];
+    uint32_t o1, o2;  // packed byte offsets
+    if constexpr (DT == PEAT_BF16) {
+      o1 = ((d & 0x1FFF1FFFu) * 4u) | (d & 0x80008000u);
+      o1 ^= (d >> 5) & 0x007C007Cu;
+      o2 = v.t[i] * 512u + (v.g[i] & 0x007F007Fu) * 4u;
+      if (W.atol != 0.0f) {
+        count_mismatch(mism, lo_b(d), lo_b(v.g[i]), W);
+        count_mismatch(mism, hi_b(d), hi_b(v.g[i]), W);
+      }
+    } else {
+      o1 = (d >> 1) & 0x7FFC7FFCu;
+      o1 ^= (d >> 8) & 0x007C007Cu;
+      // |d| - |g| as patterns: 1024 (floor(log2(|d| / |g|)) + 32) + a remainder
+      const uint32_t y = (d | 0x80008000u) - (v.g[i] & 0x7FFF7FFFu);
+      o2 = (y & 0x7C007C00u) | (v.t[i] * 4u);
+      count_mismatch(mism, __low2float(h2(d)), __low2float(h2(v.g[i])), W);
+      count_mismatch(mism, __high2float(h2(d)), __high2float(h2(v.g[i])), W);
+    }
+    inc_shared(t1, o1 & 0xFFFFu);
+    inc_shared(t1, o1 >> 16);
+    inc_shared(t2, o2 & 0xFFFFu);
+    inc_shared(t2, o2 >> 16);
+  }
+}
+
+// A vector of which few lanes hold an unequal pair: each lane visits its own
+// unequal words (two pairs at a time), the rest of the warp an equal one.
+// (Out of line of the dense path: late steps of a sweep and fault injections
+// leave most vectors with one or two unequal pairs.)
+template <int DT>
+__device__ __forceinline__ void sparse16(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t m, uint32_t li,
+                                         uint32_t next, const Win& W, Bounds& B, uint32_t t1, uint32_t t2, uint32_t scale2, float& mism) {
+  const uint32_t* g = reinterpret_cast<const uint32_t*>(gt);
+  const uint32_t* c = reinterpret_cast<const uint32_t*>(ct);
+  bool checked = false;
+  while (__any_sync(0xFFFFFFFFu, m != 0u)) {
+    const int i = __ffs(m | 8u) - 1;  // a lane without unequal words left takes word 3, as a pair of equal ones
+    uint32_t gw[1] = {g[i]}, cw[1] = {c[i]};
+    if (m == 0u) cw[0] = gw[0] = 0u;
+    Vec16<1> v;
+    prep16<DT, 1>(v, gw, cw, scale2);
+    if (!checked && __any_sync(0xFFFFFFFFu, check16<DT, 1>(v, W, B))) {
+      slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
+      B = read_bounds<DT>(sm, next, W);
+      checked = true;  // the whole vector
+      continue;        // general pairs are zero now
+    }
+    m &= m - 1u;
+    count16<DT, 1>(v, W, t1, t2, mism);
+  }
+}
+
+// vectors with at most this many lanes holding unequal pairs take sparse16
+// (a word costs about half of a whole vector)
+constexpr int SPARSE_LANES = 10;
+
+// A tile of CHV vectors (two per lane)
+template <int DT>
+__device__ __forceinline__ void tile16(Lane& L, Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t tli, const Win& W,
+                                       Bounds& B) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t t1 = smem_addr(smem_raw) + (uint32_t)offsetof(Smem<DT>, t1);
+  const uint32_t t2 = smem_addr(smem_raw) + (uint32_t)offsetof(Smem<DT>, t2);
+  const uint32_t scale2 = (uint32_t)(15 + W.fe) * 0x04000400u;  // binary16: 2^s in both halves
+  gt += lane;
+  ct += lane;
+  uint32_t li = tli + (uint32_t)lane * 8u;
+#pragma unroll 1
+  for (int i = 0; i < CHV / 32; i++, gt += 32, ct += 32, li += 256u) {
+    uint4 gv = *gt, cv = *ct;
+    const uint32_t x0 = gv.x ^ cv.x, x1 = gv.y ^ cv.y, x2 = gv.z ^ cv.z, x3 = gv.w ^ cv.w;
+    const unsigned lanes = __ballot_sync(0xFFFFFFFFu, (x0 | x1 | x2 | x3) != 0u);
+    if (__popc(lanes) <= SPARSE_LANES) {
+      // equal lanes: EXACT pairs; the ones holding NaN or Inf also count as non-finite
+      // (slow_vec when some lane has unequal words: it counts the equal pairs and zeroes them)
+      if (__any_sync(0xFFFFFFFFu, any_nonfinite<DT>(gv))) {
+        if (lanes == 0u) count_equal<DT>(gv, sm);
+        else slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
+      }
+      if (lanes) {
+        const uint32_t m = (x0 ? 1u : 0u) | (x1 ? 2u : 0u) | (x2 ? 4u : 0u) | (x3 ? 8u : 0u);
+        sparse16<DT>(sm, gt, ct, m, li, tli + (uint32_t)(i + 1) * 256u, W, B, t1, t2, scale2, L.mism);
+      }
+      continue;
+    }
+    Vec16<4> v;
+    uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w}, c[4] = {cv.x, cv.y, cv.z, cv.w};
+    prep16<DT, 4>(v, g, c, scale2);
+    if (__any_sync(0xFFFFFFFFu, check16<DT, 4>(v, W, B))) {
+      slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
+      gv = *gt;
+      cv = *ct;
+      const uint32_t gn[4] = {gv.x, gv.y, gv.z, gv.w}, cn[4] = {cv.x, cv.y, cv.z, cv.w};
+      prep16<DT, 4>(v, gn, cn, scale2);
+      B = read_bounds<DT>(sm, tli + (uint32_t)(i + 1) * 256u, W);
+    }
+    count16<DT, 4>(v, W, t1, t2, L.mism);
+  }
+}
+
+__device__ __forceinline__ void tile32(Lane& L, Smem<PEAT_F32>& sm, uint4* gt, uint4* ct, uint32_t tli, Win& W,
+                                       Bounds& B, uint32_t ichunk) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t t2 = smem_addr(smem_raw) + (uint32_t)offsetof(Smem<PEAT_F32>, t2);
+  uint32_t nd = 0, total = 0;
+  const uint32_t M1b = __float_as_uint(W.M1), M2b = __float_as_uint(W.M2);
+  // sums of the bits of |d| + M1, its remainder + M2, and the same of d: per
+  // tile 8 times the bits of M1 and M2 too many
+  uint32_t a1 = 0, a2 = 0, s1 = 0, s2 = 0;
+  gt += lane;
+  ct += lane;
+  uint32_t li = tli + (uint32_t)lane * 4u;
+#pragma unroll 1
+  for (int v = 0; v < CHV / 32; v++, gt += 32, ct += 32, li += 128u) {
+    uint4 gv = *gt, cv = *ct;
+    const bool diff = ((gv.x ^ cv.x) | (gv.y ^ cv.y) | (gv.z ^ cv.z) | (gv.w ^ cv.w)) != 0u;
+    if (!__any_sync(0xFFFFFFFFu, diff)) {
+      count_equal<PEAT_F32>(gv, sm);
+      a1 += 4u * M1b;
+      s1 += 4u * M1b;
+      a2 += 4u * M2b;
+      s2 += 4u * M2b;
+      continue;
+    }
+    float d[4];
+    int t[4];
+    auto prep = [&] {
+      const uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w}, c[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        d[j] = __fsub_rn(__uint_as_float(c[j]), __uint_as_float(g[j]));
+        t[j] = (int)(c[j] - g[j]);
+      }
+    };
+    prep();
+    {
+      const float g[4] = {__uint_as_float(gv.x), __uint_as_float(gv.y), __uint_as_float(gv.z), __uint_as_float(gv.w)};
+      float am = 0.0f, em = 0.0f, xm = 0.0f;
+      int tmx = 0, tmn = 0;
+      auto err = [&](float x) {  // d not a multiple of 2^Lexp
+        const float l = __fsub_rn(x, __fsub_rn(__fadd_rn(x, W.M1), W.M1));
+        return fabsf(__fsub_rn(__fsub_rn(__fadd_rn(l, W.M2), W.M2), l));
+      };
+#pragma unroll
+      for (int j = 0; j < 4; j += 2) {
+        tmx = max(tmx, max(t[j], t[j + 1]));
+        tmn = min(tmn, min(t[j], t[j + 1]));
+        am = max3_nan(am, fabsf(d[j]), fabsf(d[j + 1]));
+        em = max3(em, err(d[j]), err(d[j + 1]));
+        xm = max3(xm, __fmaf_rn(-fabsf(g[j]), B.r, fabsf(d[j])), __fmaf_rn(-fabsf(g[j + 1]), B.r, fabsf(d[j + 1])));
+      }
+      const bool bad = !(am <= __uint_as_float(B.ab)) || em != 0.0f || xm > 0.0f || tmx > (int)B.ub || tmn < -(int)B.ub;
+      if (__any_sync(0xFFFFFFFFu, bad)) {
+        if (total == 0 && lane == 0) sm.k.wem[threadIdx.x >> 5] = sm.k.wum[threadIdx.x >> 5] = 0;
+        const uint32_t r = slow_vec<PEAT_F32>(sm, gt, ct, li, W.lb, 0);
+        nd += __reduce_add_sync(0xFFFFFFFFu, r & 0xFFFFu);
+        total += __reduce_add_sync(0xFFFFFFFFu, r >> 16);
+        gv = *gt;
+        cv = *ct;
+        prep();
+        B = read_bounds<PEAT_F32>(sm, tli + (uint32_t)(v + 1) * 128u, W);
+      }
+    }
+    const uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      count_mismatch(L.mism, d[j], __uint_as_float(g[j]), W);
+      const float a = fabsf(d[j]);
+      const float x1 = __fadd_rn(d[j], W.M1), y1 = __fadd_rn(a, W.M1);
+      const float x2 = __fadd_rn(__fsub_rn(d[j], __fsub_rn(x1, W.M1)), W.M2);
+      const float y2 = __fadd_rn(__fsub_rn(a, __fsub_rn(y1, W.M1)), W.M2);
+      s1 += __float_as_uint(x1);
+      s2 += __float_as_uint(x2);
+      a1 += __float_as_uint(y1);
+      a2 += __float_as_uint(y2);
+      const int v1 = (int)(__float_as_uint(y1) - M1b), v2 = (int)(__float_as_uint(y2) - M2b);
+      L.Q11 += (uint64_t)((int64_t)v1 * v1);
+      L.Q12 += (int64_t)v1 * v2;
+      L.Q22 += (uint64_t)((int64_t)v2 * v2);
+      // row floor(log2(|d| / |g|)) mod 32: bits 23 .. 27 of the difference of
+      // the patterns (the signs only reach bit 31)
+      const uint32_t y = __float_as_uint(d[j]) - g[j];
+      inc_shared(t2, ((y >> 15) & 0x1F00u) | (uint32_t)(min(abs(t[j]), 63) * 4));
+    }
+  }
+  L.A += ((int64_t)(int32_t)(a1 - 8u * M1b) << 21) + (int32_t)(a2 - 8u * M2b);
+  L.S += ((int64_t)(int32_t)(s1 - 8u * M1b) << 21) + (int32_t)(s2 - 8u * M2b);
+  if (nd >= 32u && nd * 4u >= total) {
+    const int lb = next_window(W.lb, ichunk, sm);
+    if (lb >= 0) {
+      flush_sums(L, sm, win_lexp<PEAT_F32>(W));
+      set_window_lb<PEAT_F32>(W, lb);
+      B.low = true;  // the bound on |d| depends on the window
+    }
+  }
+}
+
+// The tile loop out of line: tiles staged by the warp's lanes and partial ones
+// (a second inlined copy would only cost registers and instruction cache; by
+// value, so that the caller's state stays in registers).
+struct ColdOut {
+  Lane L;
+  int lb;
+};
+template <int DT>
+__device__ __noinline__ ColdOut tile_cold(Lane L, Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t tli, Win W, int ichunk) {
+  fence_proxy_async();  // the lanes' stores to the stage, before a later bulk copy into it
+  __syncwarp();
+  Bounds B = read_bounds<DT>(sm, tli, W);
+  if constexpr (DT == PEAT_F32) tile32(L, sm, gt, ct, tli, W, B, (uint32_t)ichunk);
+  else tile16<DT>(L, sm, gt, ct, tli, W, B);
+  __syncwarp();
+  return ColdOut{L, W.lb};
+}
+
+// Elements [e0, e1) (at most a tile) staged by the warp's lanes; the rest of the
+// tile: pairs of zeros (EXACT, not counted).
+template <int DT, bool INJ>
+__device__ __noinline__ void stage_scalar(const CompareParams& p, uint4* gt, uint4* ct, int64_t e0, int64_t e1) {
+  using Ty = Tr<DT>;
+  using E = typename std::conditional<Ty::BYTES == 4, uint32_t, unsigned short>::type;
+  for (int e = threadIdx.x & 31; e < CHV * Ty::VEC; e += 32) {
+    uint32_t G = 0, C = 0;
+    if (e0 + e < e1) {
+      G = load_scalar<DT>(p.g, e0 + e);
+      C = cand_at<DT, INJ>(p, e0 + e, G);
+    }
+    reinterpret_cast<E*>(gt)[e] = (E)G;
+    reinterpret_cast<E*>(ct)[e] = (E)C;
+  }
+}
+
 
 // ---------------------------------------------------------------------------
 // CTA ranges: boundaries precomputed on the host
@@ -1287,7 +1584,8 @@ __device__ __forceinline__ void part_warp_reduce(Partial& x) {
 
 
 // warp sums of the general path's class counters into the CTA counters
-__device__ __forceinline__ void gen_counts(const GenRec& g, Smem& sm) {
+template <int DT>
+__device__ __forceinline__ void gen_counts(const GenRec& g, Smem<DT>& sm) {
   const int lane = threadIdx.x & 31;
   const uint32_t gen = g.n_gw + g.n_gm + g.n_ga + g.n_gf + g.n_geq;
   const uint32_t c[7] = {g.n_geq, gen, g.n_nf, g.n_gw, g.n_gm, g.n_ga, g.n_gf};
@@ -1295,46 +1593,47 @@ __device__ __forceinline__ void gen_counts(const GenRec& g, Smem& sm) {
 #pragma unroll
   for (int k = 0; k < 7; k++) v[k] = __reduce_add_sync(0xFFFFFFFFu, c[k]);
   if (lane == 0) {
-    if (v[0]) atomicAdd(&sm.cnt[0], (unsigned long long)v[0]);
-    if (v[1]) atomicAdd(&sm.cnt[1], 0ull - (unsigned long long)v[1]);  // general pairs are not window pairs
-    if (v[2]) atomicAdd(&sm.cnt[3], (unsigned long long)v[2]);
-    if (v[3]) atomicAdd(&sm.cnt[4], (unsigned long long)v[3]);
-    if (v[4]) atomicAdd(&sm.cnt[5], (unsigned long long)v[4]);
-    if (v[5]) atomicAdd(&sm.cnt[6], (unsigned long long)v[5]);
-    if (v[6]) atomicAdd(&sm.cnt[7], (unsigned long long)v[6]);
+    // EXACT: the piece length less the window pairs, less the general pairs that differ
+    if (v[1] != v[0]) atomicAdd(&sm.k.cnt[0], 0ull - (unsigned long long)(v[1] - v[0]));
+    if (v[2]) atomicAdd(&sm.k.cnt[3], (unsigned long long)v[2]);
+    if (v[3]) atomicAdd(&sm.k.cnt[4], (unsigned long long)v[3]);
+    if (v[4]) atomicAdd(&sm.k.cnt[5], (unsigned long long)v[4]);
+    if (v[5]) atomicAdd(&sm.k.cnt[6], (unsigned long long)v[5]);
+    if (v[6]) atomicAdd(&sm.k.cnt[7], (unsigned long long)v[6]);
   }
 }
 
 // The general pairs of a piece [pb, pe), evaluated exactly by every thread of
 // the CTA: from the list when it held them all, else found again by a rescan
 // of the piece with the same window test.  Out of line, so that the hot loop
-// carries no call.  Leaves each warp's general maxima in sm.wbest[warp].
+// carries no call.  Leaves each warp's general maxima in sm.k.wbest[warp].
 template <int DT, bool INJ>
-__device__ __noinline__ void run_general(Win W, Smem& sm, const CompareParams& p, int64_t pb, int64_t pe,
+__device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParams& p, int64_t pb, int64_t pe,
                                          int64_t vb, int64_t ve) {
+  constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   // entered only after a barrier and with at least one general pair (finish_piece)
-  const uint32_t n = sm.gn;
-  const int64_t lo = sm.lo;
+  const uint32_t n = sm.k.gn;
+  const int64_t lo = sm.k.lo;
   GenRec cd;
   gen_init(cd);
   // whole warps in every round (general_lane adds with the whole warp)
   const uint32_t lane = threadIdx.x & 31u, w0 = threadIdx.x & ~31u;
   if (n <= (uint32_t)GCAP) {
-    for (uint32_t b = w0; b < n; b += BLOCK) {
+    for (uint32_t b = w0; b < n; b += NT) {
       const uint32_t e = b + lane;
       const bool valid = e < n;
       int64_t i = 0;
       uint32_t G = 0, C = 0;
       if (valid) {
-        i = lo + sm.glist[e];
+        i = lo + sm.k.glist[e];
         if (!PEAT_CHECK(i >= 0 && i < p.n_total)) i = lo;  // a listed offset outside the tensor
         G = load_scalar<DT>(p.g, i);
         C = cand_at<DT, INJ>(p, i, G);
       }
-      general_lane<DT>(sm, cd, G, C, i, W.rtol, W.atol, valid);
+      general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, valid);
     }
   } else {
-    for (int64_t b = pb + w0; b < pe; b += BLOCK) {
+    for (int64_t b = pb + w0; b < pe; b += NT) {
       const int64_t i = b + lane;
       bool want = false;
       uint32_t G = 0, C = 0;
@@ -1344,38 +1643,34 @@ __device__ __noinline__ void run_general(Win W, Smem& sm, const CompareParams& p
         want = G != C;
       }
       if (want) {
-        uint32_t gr = G, cr = C;
-        if constexpr (DT == PEAT_BF16) {
-          gr = G << 16;
-          cr = C << 16;
-        }
-        // the window this pair was tested with: the head ran with the initial
-        // window, a body chunk with its warp's window of that time, the tail
-        // with its thread's warp's last window
-        int w = 0;
-        uint32_t ik = 0;
-        if (vb < ve && i >= vb) {
-          if (i >= ve) {
-            w = (int)(((i - ve) % BLOCK) >> 5);
-            ik = 0xFFFFFFFFu;
-          } else {
-            const int64_t k = (i - vb) / (CHV * Tr<DT>::VEC);
-            w = (int)(k % NW);
-            ik = (uint32_t)(k / NW);
-          }
-        }
-        int r = (int)sm.nwin[w];
-        while (r > 0 && sm.wstart[w][r] > ik) r--;
         Win Wi = W;
-        set_window_lb<DT>(Wi, sm.wlb[w][r]);
-        uint32_t ud;
-        float s, a, thr;
-        want = !in_window<DT>(gr, cr, to_f32<DT>(G), to_f32<DT>(C), Wi, ud, s, a, thr);
+        if constexpr (DT == PEAT_F32) {
+          // the window this pair was tested with: the head ran with the
+          // initial window, a body chunk with its warp's window of that time,
+          // the tail with warp 0's last window
+          int w = 0;
+          uint32_t ik = 0;
+          if (vb < ve && i >= vb) {
+            if (i >= ve) {
+              ik = 0xFFFFFFFFu;
+            } else {
+              const int64_t k = (i - vb) / (CHV * Tr<DT>::VEC);
+              w = (int)(k % NW);
+              ik = (uint32_t)(k / NW);
+            }
+          }
+          int r = (int)sm.k.nwin[w];
+          while (r > 0 && sm.k.wstart[w][r] > ik) r--;
+          set_window_lb<DT>(Wi, sm.k.wlb[w][r]);
+        }
+        uint32_t u;
+        float gf, a;
+        want = !pair_window<DT>(G, C, Wi, u, gf, a);
       }
-      general_lane<DT>(sm, cd, G, C, i, W.rtol, W.atol, want);
+      general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, want);
     }
   }
-  gen_counts(cd, sm);
+  gen_counts<DT>(cd, sm);
   Partial x;
   part_none(x);
   x.abs_hi = cd.abs_hi;
@@ -1390,234 +1685,380 @@ __device__ __noinline__ void run_general(Win W, Smem& sm, const CompareParams& p
   x.ulp = cd.ulp;
   x.ulp_idx = cd.ulp_idx;
   part_warp_reduce(x);
-  if ((threadIdx.x & 31) == 0) sm.wbest[threadIdx.x >> 5] = x;
+  if ((threadIdx.x & 31) == 0) sm.k.wbest[threadIdx.x >> 5] = x;
   __syncthreads();
-  if (threadIdx.x == 0) sm.gn = 0;
+  // the per-warp totals into the CTA's
+  for (int b = threadIdx.x; b < HBINS; b += NT) {
+    unsigned long long v = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) {
+      v += sm.k.ghist[w][b];
+      sm.k.ghist[w][b] = 0;
+    }
+    if (v) atomicAdd(&sm.k.hist[b], v);
+  }
+  for (int j = threadIdx.x; j < NSUM * NLIMB; j += NT) {
+    unsigned long long v = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) {
+      v += (&sm.k.gsacc[w][0][0])[j];
+      (&sm.k.gsacc[w][0][0])[j] = 0;
+    }
+    if (v) atomicAdd(&sm.k.sacc[0][0] + j, v);
+  }
 }
 
 // [pb, pe): the lowest index of a finite pair and of a pair without NaN
-// (the argmax when every error is zero), searched BLOCK elements at a time
+// (the argmax when every error is zero), searched NT elements at a time
 // (the piece's first pair, which settles both unless it holds NaN or Inf, is
 // tested when the piece starts; this search runs only when it did not)
 template <int DT, bool INJ>
-__device__ __noinline__ void first_pairs(Smem& sm, const CompareParams& p, int64_t pb, int64_t pe) {
+__device__ __noinline__ void first_pairs(Smem<DT>& sm, const CompareParams& p, int64_t pb, int64_t pe) {
   using Ty = Tr<DT>;
   constexpr long long NONE = 0x7FFFFFFFFFFFFFFFll;
-  for (int64_t base = pb;; base += BLOCK) {
+  for (int64_t base = pb;; base += Geo<DT>::NT) {
     __syncthreads();
-    if (base >= pe || (sm.ff != NONE && sm.fu != NONE)) break;
+    if (base >= pe || (sm.k.ff != NONE && sm.k.fu != NONE)) break;
     const int64_t i = base + threadIdx.x;
     if (i < pe) {
       const uint32_t Gi = load_scalar<DT>(p.g, i);
       const uint32_t ag = Gi & Ty::MAG, ac = cand_at<DT, INJ>(p, i, Gi) & Ty::MAG;
-      if (ag < Ty::INF && ac < Ty::INF) atomicMin(&sm.ff, (long long)i);
-      if (ag <= Ty::INF && ac <= Ty::INF) atomicMin(&sm.fu, (long long)i);
+      if (ag < Ty::INF && ac < Ty::INF) atomicMin(&sm.k.ff, (long long)i);
+      if (ag <= Ty::INF && ac <= Ty::INF) atomicMin(&sm.k.fu, (long long)i);
     }
   }
   __syncthreads();
 }
 
-// Fold the per-thread 16-bit histograms and the window sums into the CTA
-// totals.  All threads call it; it ends with the private counters zeroed.
+// Add n pairs of log2-relative exponent k, each lane its own (n = 0: none; the
+// whole warp calls it): one shared atomic per distinct k of the warp.
 template <int DT>
-__device__ void fold_round(Lane& L, Smem& sm, int lexp) {
-  constexpr int NPB = Rows<DT>::NPB;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  flush_sums(L, sm, lexp);  // lexp: this warp's window
-  __syncthreads();
-  // private rows: one warp per row
-  for (int r = warp; r < NPB; r += NW) {
-    uint32_t sum = 0;
-    for (int w = lane; w < HALF; w += 32) {
-      const uint32_t v = sm.priv[r * HALF + w];
-      sum += (v & 0xFFFFu) + (v >> 16);
-      sm.priv[r * HALF + w] = 0;
-    }
-    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
-    if (lane == 0 && sum) {
-      const int bin = r < NUR ? 64 + r + 1 : 48 + Rows<DT>::KLO + (r - NUR);
-      if (PEAT_CHECK(bin >= 0 && bin < HBINS)) sm.hist[bin] += sum;
-    }
+__device__ __forceinline__ void add_rel(Smem<DT>& sm, int k, uint32_t n) {
+  unsigned todo = __ballot_sync(0xFFFFFFFFu, n != 0u);
+  while (todo) {
+    const int k0 = __shfl_sync(0xFFFFFFFFu, k, __ffs(todo) - 1);
+    const bool mine = n != 0u && k == k0;
+    const uint32_t s = __reduce_add_sync(0xFFFFFFFFu, mine ? n : 0u);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sm.k.hist[min(max(48 + k0, 1), 62)], (unsigned long long)s);
+    todo &= ~__ballot_sync(0xFFFFFFFFu, mine);
   }
-  __syncthreads();
 }
 
-__device__ void finalize_segment(const CompareParams& p, int64_t s, FinScratch& f, MV& mv);
+// The window tables into the CTA's totals, leaving them zero (called by every
+// thread, between barriers).
+template <int DT>
+__device__ __forceinline__ void fold_tables(Smem<DT>& sm, const Win& W) {
+  constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t zeros = 0;  // bfloat16, warp 0: the pairs with d = 0 in T1
+  uint32_t nwin = 0, nover = 0;
+  if constexpr (DT == PEAT_BF16) {
+    // a warp per ULP distance row, cells by the golden's significand field
+    for (int t = warp; t < 128; t += NW) {
+      uint32_t n[4], any = 0;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        n[j] = sm.t2[t * 128 + lane + 32 * j];
+        any |= n[j];
+      }
+      if (!__any_sync(0xFFFFFFFFu, any != 0u)) continue;
+#pragma unroll
+      for (int j = 0; j < 4; j++) sm.t2[t * 128 + lane + 32 * j] = 0;
+      const uint32_t row = __reduce_add_sync(0xFFFFFFFFu, n[0] + n[1] + n[2] + n[3]);
+      if (t == 64) {
+        zeros = row;
+        continue;
+      }
+      const int u = t - 64;
+      if (lane == 0) atomicAdd(&sm.k.hist[64 + abs(u)], (unsigned long long)row);
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        // golden and candidate in half steps of the golden's binade [256, 512)
+        const int x = 128 + lane + 32 * j + u;
+        const int g2 = 2 * (128 + lane + 32 * j), c2 = x >= 256 ? 4 * x - 512 : (x < 128 ? 128 + x : 2 * x);
+        const int a2 = abs(c2 - g2);
+        const float fa = (float)a2, fg = (float)g2;
+        const int k = (int)(__float_as_uint(fa) - __float_as_uint(fg)) >> 23;
+        add_rel<DT>(sm, k, n[j]);
+        // atol = 0: |d| <= rtol |g| does not depend on the binade
+        if (W.atol == 0.0f && fa > __fmul_rd(W.rtol, fg)) nover += n[j];
+      }
+      nwin += lane == 0 ? row : 0u;
+    }
+  } else {
+    // T2: a thread holds every (NT / COLS)-th row of one column
+    constexpr int COLS = DT == PEAT_F32 ? 64 : 256, R = NT / COLS;
+    constexpr int ZERO = DT == PEAT_F32 ? 0 : 128;  // the column of d = 0
+    const int col = tid % COLS, r0 = tid / COLS;
+#pragma unroll 4
+    for (int i = 0; i < 32 / R; i++) {
+      const int row = r0 + i * R;
+      uint32_t* q = sm.t2 + row * COLS + col;
+      const uint32_t v = col == ZERO ? 0u : *q;
+      *q = 0;
+      if (!__any_sync(0xFFFFFFFFu, v != 0u)) continue;
+      nwin += v;
+      // (a warp covers 32 columns of one row; a piece has below 2^31 pairs)
+      const uint32_t s = __reduce_add_sync(0xFFFFFFFFu, v);
+      const int k = row < 16 && DT == PEAT_F16 ? row : (row == 0 ? 0 : row - 32);
+      if (lane == 0) atomicAdd(&sm.k.hist[min(max(48 + k, 1), 62)], (unsigned long long)s);
+    }
+    if (nwin) atomicAdd(&sm.k.hist[64 + (DT == PEAT_F32 ? col : min(abs(col - 128), 63))], (unsigned long long)nwin);
+  }
+  nwin = __reduce_add_sync(0xFFFFFFFFu, nwin);
+  nover = __reduce_add_sync(0xFFFFFFFFu, nover);
+  if (lane == 0 && nwin) {
+    atomicAdd(&sm.k.cnt[1], (unsigned long long)nwin);            // window pairs
+    atomicAdd(&sm.k.cnt[2], (unsigned long long)nwin - nover);    // of them within tolerance (mismatches taken off)
+    atomicAdd(&sm.k.cnt[0], 0ull - (unsigned long long)nwin);     // are not EXACT
+  }
+  // T1: a warp per exponent; each counter adds count * v to sum |d| and sum d
+  // and count * v^2 to sum d^2, v = 128 + M in units of the exponent's step
+  if constexpr (DT != PEAT_F32) {
+    constexpr int ROWS = Tab<DT>::ROWS;
+    for (int r = warp; r < ROWS; r += NW) {
+      uint32_t* tp = sm.t1 + r * 128;
+      uint32_t* tn = tp + ROWS * 128;
+      uint32_t cp[4], cn[4];
+      uint32_t any = 0;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        cp[j] = tp[lane + 32 * j];
+        cn[j] = tn[lane + 32 * j];
+      }
+      if (r == 0) {  // d = 0 (warp 0, lane 0, j = 0)
+        if (lane == 0) cp[0] -= DT == PEAT_BF16 ? zeros : cp[0];
+        tp[lane] = 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) any |= cp[j] | cn[j];
+      if (!__any_sync(0xFFFFFFFFu, any != 0u)) continue;
+      uint64_t sp = 0, sn = 0, q = 0;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const uint32_t m = 128u + (uint32_t)((lane ^ (r & 31)) + 32 * j);
+        sp += (uint64_t)cp[j] * m;
+        sn += (uint64_t)cn[j] * m;
+        q += (uint64_t)cp[j] * (m * m) + (uint64_t)cn[j] * (m * m);
+        tp[lane + 32 * j] = 0;
+        tn[lane + 32 * j] = 0;
+      }
+      sp = wsum64(sp);
+      sn = wsum64(sn);
+      q = wsum64(q);
+      if (lane < NSUM) {  // a lane per sum
+        const int u = DT == PEAT_BF16 ? W.fe + ((r - W.fe) & 63) - 134 : r - 22 - W.fe;
+        const uint64_t m = lane == 0 ? (sp >= sn ? sp - sn : sn - sp) : (lane == 1 ? sp + sn : q);
+        sacc_add<DT>(sm, lane, (unsigned __int128)m, lane == 2 ? 2 * u : u, lane == 0 && sp < sn);
+      }
+    }
+  }
+}
+
+// The window maxima of the CTA's piece, for lane 0 of warp 0 (the whole warp
+// calls it).
+template <int DT>
+__device__ __forceinline__ void window_best(Smem<DT>& sm, Partial& x) {
+  constexpr int NW = Geo<DT>::NW;
+  const int lane = threadIdx.x & 31;
+  part_none(x);
+  const int64_t lo = sm.k.lo;
+  if ((uint32_t)sm.k.kabs) {
+    x.abs_hi = __uint_as_float((uint32_t)(sm.k.kabs >> 32));
+    x.abs_idx = lo + (uint32_t)~(uint32_t)sm.k.kabs;
+  }
+  if ((uint32_t)sm.k.kulp) {
+    x.ulp = sm.k.kulp >> 32;
+    x.ulp_idx = lo + (uint32_t)~(uint32_t)sm.k.kulp;
+  }
+  RelRec r{0.0f, 1.0f, 0.0f, 0u};
+  if (lane < NW) r = sm.k.wrel[lane];
+  if constexpr (DT == PEAT_F32) {
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) {
+      const float ya = __shfl_down_sync(0xFFFFFFFFu, r.a, o), yg = __shfl_down_sync(0xFFFFFFFFu, r.g, o);
+      const uint32_t yi = __shfl_down_sync(0xFFFFFFFFu, r.li, o);
+      if (ya > 0.0f && (rel_greater(ya, yg, r.a, r.g) || (yi < r.li && !rel_greater(r.a, r.g, ya, yg))))
+        r.a = ya, r.g = yg, r.li = yi;
+    }
+  } else {
+    // the CTA's key names the winning pair: its warp holds it
+    const uint32_t kl = (uint32_t)sm.k.krel;
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, kl != 0u && r.a > 0.0f && r.li == ~kl);
+    const int s = who ? __ffs(who) - 1 : 0;
+    r.a = __shfl_sync(0xFFFFFFFFu, who ? r.a : 0.0f, s);
+    r.g = __shfl_sync(0xFFFFFFFFu, r.g, s);
+    r.li = __shfl_sync(0xFFFFFFFFu, r.li, s);
+  }
+  if (r.a > 0.0f) {
+    x.rel_hi = r.a;
+    x.rel_g = r.g;
+    x.rel_idx = lo + r.li;
+  }
+}
+
+template <int NT>
+__device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, FinScratch& f, MV& mv);
 __device__ void write_empty_segments(const CompareParams& p);
+
+// the window maxima, class counters and list of a new piece
+template <int DT>
+__device__ __forceinline__ void piece_init(Smem<DT>& sm) {
+  const int tid = threadIdx.x;
+  if (tid < Geo<DT>::NW) sm.k.wrel[tid] = RelRec{0.0f, 1.0f, 0.0f, 0xFFFFFFFFu};
+  if (tid == 32) sm.k.kabs = sm.k.kulp = sm.k.krel = 0ull;
+  if (tid == 33) {
+    sm.k.gn = 0;
+    sm.k.nfe = 0;
+    sm.k.lb = sm.k.ub = 0;
+  }
+  if (tid >= 64 && tid < 72) sm.k.cnt[tid - 64] = 0;
+}
 
 // End of one segment piece [pb, pe): the integer totals go to the segment's
 // accumulator (global atomics), the maxima to the CTA's partial slot.  The
 // CTA that finishes the segment's last piece then finalizes the segment.
 template <int DT, bool INJ>
-__device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem& sm, const CompareParams& p,
+__device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm, const CompareParams& p,
                                              int64_t seg, int64_t pb, int64_t pe, int64_t vb, int64_t ve) {
+  constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   Partial* out = p.partials + seg + blockIdx.x;
   SegAcc* acc = p.acc + seg;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if constexpr (DT == PEAT_F32) flush_sums(L, sm, win_lexp<DT>(W));
+  {
+    const uint32_t over = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)L.mism);
+    if (lane == 0 && over) atomicAdd(&sm.k.cnt[2], 0ull - (unsigned long long)over);
+  }
+  lane_init(L);
+  __syncthreads();  // every tile is in the tables, the list and the records
   // the piece's general pairs, if any: the out-of-line call (and its register
   // traffic) only when there is one
-  __syncthreads();
-  if (sm.gn != 0) {
-    run_general<DT, INJ>(W, sm, p, pb, pe, vb, ve);
-  } else if ((threadIdx.x & 31) == 0) {
-    part_none(sm.wbest[threadIdx.x >> 5]);
-  }
-  fold_round<DT>(L, sm, win_lexp<DT>(W));  // ends with a barrier: the general path's per-warp totals are complete
-  for (int b = threadIdx.x; b < HBINS; b += BLOCK) {
-    unsigned long long v = 0;
-#pragma unroll
-    for (int w = 0; w < NW; w++) {
-      v += sm.ghist[w][b];
-      sm.ghist[w][b] = 0;
-    }
-    sm.hist[b] += v;
-  }
-  for (int j = threadIdx.x; j < NSUM * NLIMB; j += BLOCK) {
-    unsigned long long v = 0;
-#pragma unroll
-    for (int w = 0; w < NW; w++) {
-      v += (&sm.gsacc[w][0][0])[j];
-      (&sm.gsacc[w][0][0])[j] = 0;
-    }
-    (&sm.sacc[0][0])[j] += v;
-  }
-  if (sm.ff == 0x7FFFFFFFFFFFFFFFll || sm.fu == 0x7FFFFFFFFFFFFFFFll) first_pairs<DT, INJ>(sm, p, pb, pe);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t lo = sm.lo;
-  // window pairs = unequal pairs - general pairs; EXACT = the piece length -
-  // unequal pairs + general pairs found equal (64-bit wrapping adds; the
-  // totals are non-negative)
-  {
-    const uint32_t vu = __reduce_add_sync(0xFFFFFFFFu, L.uneq), vw = __reduce_add_sync(0xFFFFFFFFu, L.within);
-    if (lane == 0) {
-      if (vu) {
-        atomicAdd(&sm.cnt[1], (unsigned long long)vu);
-        atomicAdd(&sm.cnt[0], 0ull - (unsigned long long)vu);
-      }
-      if (vw) atomicAdd(&sm.cnt[2], (unsigned long long)vw);
-    }
-    if (threadIdx.x == 0) {
-      atomicAdd(&sm.cnt[0], (unsigned long long)(pe - pb));
-      atomicAdd(&sm.cnt[3], (unsigned long long)sm.nfe);
-    }
-  }
-  // maxima: this thread's window record, then the warp's, merged with the
-  // warp's general best
-  {
-    const WinRec r = sm.rec[threadIdx.x];
-    Partial w;
-    part_none(w);
-    if (r.amax > 0.0f) {
-      w.abs_hi = r.amax;
-      w.abs_idx = lo + r.aidx;
-    }
-    if (r.rd > 0.0f) {
-      w.rel_hi = r.rd;
-      w.rel_g = r.rg;
-      w.rel_idx = lo + r.ridx;
-    }
-    if (r.umax > 0u) {
-      w.ulp = DT == PEAT_BF16 ? r.umax >> 16 : r.umax;
-      w.ulp_idx = lo + r.uidx;
-    }
-    part_warp_reduce(w);
-    if (lane == 0) {
-      Partial x = sm.wbest[warp];
-      part_merge(x, w);
-      sm.wbest[warp] = x;
-    }
-  }
-  __syncthreads();
+  const bool gen = sm.k.gn != 0;
+  if (gen) run_general<DT, INJ>(W, sm, p, pb, pe, vb, ve);
+  if (sm.k.ff == 0x7FFFFFFFFFFFFFFFll || sm.k.fu == 0x7FFFFFFFFFFFFFFFll) first_pairs<DT, INJ>(sm, p, pb, pe);
   if (warp == 0) {
     Partial x;
-    if (lane < NW) x = sm.wbest[lane];
-    else part_none(x);
-    part_warp_reduce(x);
+    window_best<DT>(sm, x);
+    if (gen) {
+      Partial y;
+      if (lane < NW) y = sm.k.wbest[lane];
+      else part_none(y);
+      part_warp_reduce(y);
+      if (lane == 0) part_merge(x, y);
+    }
     if (lane == 0) {
       constexpr long long NONE = 0x7FFFFFFFFFFFFFFFll;
-      x.first_fin = sm.ff == NONE ? -1 : sm.ff;
-      x.first_ulp = sm.fu == NONE ? -1 : sm.fu;
+      x.first_fin = sm.k.ff == NONE ? -1 : sm.k.ff;
+      x.first_ulp = sm.k.fu == NONE ? -1 : sm.k.fu;
       if (PEAT_CHECK(seg >= 0 && seg < p.nseg && seg + (int64_t)blockIdx.x < p.nseg + p.nctas && pb <= pe &&
                      pe <= p.n_total))
         *out = x;
+      atomicAdd(&sm.k.cnt[0], (unsigned long long)(pe - pb));
+      atomicAdd(&sm.k.cnt[3], (unsigned long long)sm.k.nfe);
     }
   }
-  for (int b = threadIdx.x; b < HBINS; b += BLOCK)
-    if (sm.hist[b]) atomicAdd(&acc->hist[b], sm.hist[b]);
-  if (threadIdx.x < 8 && sm.cnt[threadIdx.x]) atomicAdd(&acc->cnt[threadIdx.x], sm.cnt[threadIdx.x]);
-  for (int j = threadIdx.x; j < NSUM * NLIMB; j += BLOCK) {
-    const unsigned long long v = (&sm.sacc[0][0])[j];
+  fold_tables<DT>(sm, W);
+  __syncthreads();  // the totals are complete
+  for (int b = tid; b < HBINS; b += NT) {
+    if (sm.k.hist[b]) atomicAdd(&acc->hist[b], sm.k.hist[b]);
+    sm.k.hist[b] = 0;
+  }
+  if (tid >= 128 && tid < 136 && sm.k.cnt[tid - 128]) atomicAdd(&acc->cnt[tid - 128], sm.k.cnt[tid - 128]);
+  for (int j = tid - 160; j >= 0 && j < NSUM * NLIMB; j += NT) {
+    const unsigned long long v = (&sm.k.sacc[0][0])[j];
     if (v) atomicAdd(reinterpret_cast<unsigned long long*>(&acc->limbs[0][0]) + j, v);
+    (&sm.k.sacc[0][0])[j] = 0;
   }
   // publish, then count this piece: the segment's pieces are the CTAs whose
   // ranges meet it (a multi-segment call finalizes in a second launch, after
   // this one)
-  if (p.nseg == 1) __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    sm.last = 0;
-    if (p.nseg == 1) {  // one segment: its last CTA finalizes it (else a second launch does, in parallel)
-      sm.last = atomicAdd(&acc->done, 1u) == sm.pieces - 1u;
-    }
-  }
-  // reset the CTA totals for the next piece
-  for (int b = threadIdx.x; b < HBINS; b += BLOCK) sm.hist[b] = 0;
-  for (int j = threadIdx.x; j < NSUM * NLIMB; j += BLOCK) (&sm.sacc[0][0])[j] = 0;
-  if (threadIdx.x < 8) sm.cnt[threadIdx.x] = 0;
-  if (threadIdx.x == 0) sm.nfe = 0;
-  rec_init(sm.rec[threadIdx.x]);
-  lane_init(L);
-  __syncthreads();
-  if (sm.last) {
+  if (p.nseg == 1) {
     __threadfence();
-    finalize_segment(p, seg, sm.fin, sm.mv);
+    __syncthreads();
+    if (tid == 0) sm.k.last = atomicAdd(&acc->done, 1u) == sm.k.pieces - 1u;
+    __syncthreads();
+    if (sm.k.last) {
+      __threadfence();
+      finalize_segment<NT>(p, seg, sm.k.fin, sm.mv);
+    }
+  } else {
+    __syncthreads();
   }
 }
 
 // ---------------------------------------------------------------------------
 // stage 1
 // ---------------------------------------------------------------------------
-constexpr int CTAS_PER_SM = 2;
+// The window sample: VEC (or one) pairs per thread from the start of the
+// piece give the largest finite golden exponent and the largest ULP distance
+// of a pair of one sign (they place the window), and starting bounds for the
+// three maxima.  A starting bound is the value of some pair of the piece, so
+// no maximum lies below it.
+template <int DT, int NV>
+__device__ __forceinline__ void sample_pairs(const uint32_t (&g)[NV], const uint32_t (&c)[NV], uint32_t& emax,
+                                             uint32_t& umax, uint32_t& ab, uint32_t& qb) {
+  using Ty = Tr<DT>;
+  float am = 0.0f, qm = 0.0f;
+#pragma unroll
+  for (int j = 0; j < NV; j++) {
+    const uint32_t G = g[j], C = c[j], mg = G & Ty::MAG, mc = C & Ty::MAG;
+    const uint32_t e = mg >> Ty::MB;
+    if (e < (uint32_t)Ty::EMAX && e > emax) emax = e;
+    if (((G ^ C) & Ty::SIGN) == 0u && mg < Ty::INF && mc < Ty::INF && G != C) {
+      const uint32_t u = G > C ? G - C : C - G;
+      umax = max(umax, u);
+      if (u <= (uint32_t)Tab<DT>::UMAX && mg != 0u) {
+        const float gf = fabsf(to_f32<DT>(G)), a = fabsf(__fsub_rn(to_f32<DT>(C), to_f32<DT>(G)));
+        am = fmaxf(am, a);
+        qm = fmaxf(qm, DT == PEAT_F32 ? __fdiv_rd(a, gf) : __fdiv_rn(a, gf));
+      }
+    }
+  }
+  ab = __float_as_uint(am);
+  qb = __float_as_uint(qm);
+}
 
 template <int DT, bool INJ>
-__global__ void __launch_bounds__(BLOCK, CTAS_PER_SM) compare_stage1(CompareParams p) {
+__global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(CompareParams p) {
   using Ty = Tr<DT>;
-  using R = Rows<DT>;
-  constexpr int VEC = Ty::VEC;
-  // pairs per thread per round stay below 2^16 (16-bit private counters): each
-  // warp tile gives a thread at most 2 VEC pairs
-  constexpr int64_t ROUND_CHUNKS = (int64_t)NW * (65535 / (2 * VEC));
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  constexpr int VEC = Ty::VEC, NT = Geo<DT>::NT, NW = Geo<DT>::NW;
+  constexpr int64_t TILE = (int64_t)CHV * VEC;
+  Smem<DT>& sm = *reinterpret_cast<Smem<DT>*>(smem_raw);
   pdl_trigger();  // a multi-segment call's finalize kernel may start launching (it waits for this grid)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int b = tid; b < HBINS; b += BLOCK) sm.hist[b] = 0;
-  for (int j = tid; j < NSUM * NLIMB; j += BLOCK) (&sm.sacc[0][0])[j] = 0;
-  for (int j = tid; j < R::NPB * HALF; j += BLOCK) sm.priv[j] = 0;
-  for (int j = tid; j < NW * HBINS; j += BLOCK) (&sm.ghist[0][0])[j] = 0;
-  for (int j = tid; j < NW * NSUM * NLIMB; j += BLOCK) (&sm.gsacc[0][0][0])[j] = 0;
-  if (tid < 8) sm.cnt[tid] = 0;
-  rec_init(sm.rec[tid]);
+  // (the shuffle tells the compiler that the warp's number is the same in all
+  // its lanes: addresses derived from it stay in uniform registers, as the
+  // bulk copies want them)
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+  for (int b = tid; b < HBINS; b += NT) sm.k.hist[b] = 0;
+  for (int j = tid; j < NSUM * NLIMB; j += NT) (&sm.k.sacc[0][0])[j] = 0;
+  {  // the tables, 16 bytes per store
+    uint4* tz = reinterpret_cast<uint4*>(sm.t2);
+    for (int j = tid; j < Tab<DT>::N2 / 4; j += NT) tz[j] = make_uint4(0, 0, 0, 0);
+    tz = reinterpret_cast<uint4*>(sm.t1);
+    for (int j = tid; j < Tab<DT>::N1 / 4; j += NT) tz[j] = make_uint4(0, 0, 0, 0);
+  }
+  for (int j = tid; j < NW * HBINS; j += NT) (&sm.k.ghist[0][0])[j] = 0;
+  for (int j = tid; j < NW * NSUM * NLIMB; j += NT) (&sm.k.gsacc[0][0][0])[j] = 0;
   const int64_t lo = p.bounds[blockIdx.x], hi = p.bounds[blockIdx.x + 1];
   if (tid == 0) {
-    sm.lo = lo;
-    sm.gn = 0;
-    sm.nfe = 0;
-    sm.glist = p.glist + (size_t)blockIdx.x * GCAP;
+    sm.k.lo = lo;
+    sm.k.glist = p.glist + (size_t)blockIdx.x * GCAP;
   }
   if (lane == 0) {
-    for (int st = 0; st < NSTAGE; st++) mbar_init(&sm.bar[warp][st], 1);
+    for (int st = 0; st < NSTAGE; st++) mbar_init(smem_addr(&sm.k.bar[warp][st]), 1);
     mbar_init_fence();
   }
   Win W;
   W.rtol = p.rtol;
   W.atol = p.atol;
-  W.base = smem_addr(&sm.priv[tid & (HALF - 1)]);
-  W.inc = tid < HALF ? 1u : 65536u;
+  W.lim = W.M1 = W.M2 = 0.0f;
+  W.lb = W.fe = 0;
   Lane L;
   lane_init(L);
   if (p.nseg == 1 && p.n_total > 0 && warp == 0) {  // (counted here, off the tail of the last piece)
     const int b1 = cta_of_warp(p.n_total - 1, p), b0 = cta_of_warp(0, p);
-    if (lane == 0) sm.pieces = (unsigned)(b1 - b0 + 1);
+    if (lane == 0) sm.k.pieces = (unsigned)(b1 - b0 + 1);
   }
   __syncthreads();
   if (blockIdx.x == 0 && p.has_empty) write_empty_segments(p);
@@ -1630,138 +2071,189 @@ __global__ void __launch_bounds__(BLOCK, CTAS_PER_SM) compare_stage1(ComparePara
   while (pb < hi) {
     while (p.offsets[s + 1] <= pb) s++;  // skip empty segments
     const int64_t pe = min(hi, p.offsets[s + 1]);
-    // vector body [vb, ve) on the aligned grid, scalar head and tail
+    // the body [vb, ve): on the aligned vector grid, with a head and a tail of
+    // fewer than VEC elements; without a common grid (p0 < 0) the whole piece,
+    // staged element by element
+    const bool scalar = !(p.p0 >= 0 && p.p0 < p.n_total);
     int64_t vb = pe, ve = pe;
-    if (p.p0 >= 0 && p.p0 < p.n_total) {
+    if (!scalar) {
       int64_t a0 = pb <= p.p0 ? p.p0 : p.p0 + ((pb - p.p0 + VEC - 1) / VEC) * VEC;
       int64_t a1 = pe <= p.p0 ? p.p0 : p.p0 + ((pe - p.p0) / VEC) * VEC;
       if (a0 < a1) vb = a0, ve = a1;
     }
-    const int64_t nvec = (ve - vb) / VEC;
+    const bool body_scalar = scalar || vb >= ve;  // also a piece inside one vector
+    if (body_scalar) vb = pb, ve = pe;
+    const int64_t nvec = (ve - vb + VEC - 1) / VEC;
     const int64_t nchunk = (nvec + CHV - 1) / CHV;
-    // start this warp's copies (chunk k = warp + NW * i) before anything else
-    auto issue = [&](uint32_t sq, int64_t k) {
-      const int st = (int)(sq % NSTAGE);
-      const int64_t v0 = k * CHV;
-      const uint32_t bytes = (uint32_t)(min((int64_t)CHV, nvec - v0) * 16);
-      const int64_t off = (vb + v0 * VEC) * Ty::BYTES;
-      fence_proxy_async();
-      mbar_expect_tx(&sm.bar[warp][st], INJ ? bytes : 2 * bytes);
-      bulk_load(&sm.ring_g[warp][st][0], gbase + off, bytes, &sm.bar[warp][st]);
-      if (!INJ) bulk_load(&sm.ring_c[warp][st][0], cbase + off, bytes, &sm.bar[warp][st]);
+    // this warp's chunks: warp + NW i, i < nmy; only the piece's last chunk is partial
+    const int nmy = nchunk > warp ? (int)((nchunk - warp + NW - 1) / NW) : 0;
+    const uint32_t lastv = (uint32_t)(nvec - (nchunk - 1) * CHV);  // its vectors
+    const int ilast = (int)((nchunk - 1) % NW) == warp ? nmy - 1 : -2;
+    // start this warp's copies before anything else
+    const char* gnext = gbase + (vb + warp * TILE) * Ty::BYTES;
+    const char* cnext = cbase + (vb + warp * TILE) * Ty::BYTES;
+    const uint32_t bar0 = smem_addr(&sm.k.bar[warp][0]);
+    const uint32_t rg0 = smem_addr(&sm.ring.g[warp][0][0]), rc0 = smem_addr(&sm.ring.c[warp][0][0]);
+    constexpr uint32_t STAGEB = CHV * 16u;
+    auto issue = [&](uint32_t sq, int i) {  // chunk i, at gnext, into stage sq % NSTAGE, by one lane
+      const uint32_t st = sq % NSTAGE;
+      const uint32_t bytes = i == ilast ? lastv * 16u : STAGEB;
+      if (elect_one()) {  // (the stage was only read since the last copy, or its writers fenced)
+        mbar_expect_tx(bar0 + 8u * st, INJ ? bytes : 2 * bytes);
+        bulk_load(rg0 + STAGEB * st, gnext, bytes, bar0 + 8u * st);
+        if (!INJ) bulk_load(rc0 + STAGEB * st, cnext, bytes, bar0 + 8u * st);
+      }
     };
-    const int64_t my_chunks = nchunk > warp ? (nchunk - warp + NW - 1) / NW : 0;
-    if (lane == 0 && !failed)
-      for (int64_t i = 0; i < NSTAGE && i < my_chunks; i++) issue(seq + (uint32_t)i, warp + NW * i);
-    // the window from a sample of the piece: the largest finite golden
-    // exponent and the largest same-sign ULP distance of the first vectors
-    if (tid == 0) sm.lb = sm.ub = 0;
-    __syncthreads();
-    // the piece's first pair (its loads overlap the sample's)
+    constexpr uint32_t STEP = (uint32_t)NW * STAGEB;  // bytes between a warp's chunks
+    if (!failed && !body_scalar)
+      for (int i = 0; i < NSTAGE && i < nmy; i++, gnext += STEP, cnext += STEP) issue(seq + (uint32_t)i, i);
+    piece_init<DT>(sm);
+    // the sample's loads and the piece's first pair
+    uint32_t emax = 0, umax = 0, ab = 0, qb = 0;
     uint32_t G0 = 0, C0 = 0;
     if (tid == 0) {
       G0 = load_scalar<DT>(p.g, pb);
       C0 = cand_at<DT, INJ>(p, pb, G0);
     }
-    if (tid < nvec) {
-      const uint4 gv = load_vec(p.g, (vb + (int64_t)tid * VEC) * Ty::BYTES);
-      const uint4 cv = INJ ? inj_one<DT>(p, gv, vb + (int64_t)tid * VEC)
-                           : load_vec(p.c, (vb + (int64_t)tid * VEC) * Ty::BYTES);
-      uint32_t emax = 0, umax = 0;
-#pragma unroll
-      for (int j = 0; j < VEC; j++) {
-        const uint32_t G = lane_bits<DT>(gv, j), C = lane_bits<DT>(cv, j);
-        const uint32_t e = (G & Ty::MAG) >> Ty::MB;
-        if (e < (uint32_t)Ty::EMAX && e > emax) emax = e;
-        if (((G ^ C) & Ty::SIGN) == 0u && (G & Ty::MAG) < Ty::INF && (C & Ty::MAG) < Ty::INF) {
-          const uint32_t u = G > C ? G - C : C - G;
-          umax = u > umax ? u : umax;
-        }
+    if (!body_scalar) {
+      if (tid < nvec) {
+        const uint4 gv = load_vec(p.g, (vb + (int64_t)tid * VEC) * Ty::BYTES);
+        const uint4 cv = INJ ? inj_one<DT>(p, gv, vb + (int64_t)tid * VEC)
+                             : load_vec(p.c, (vb + (int64_t)tid * VEC) * Ty::BYTES);
+        uint32_t ge[VEC], ce[VEC];
+        unpack_vec<DT>(gv, ge);
+        unpack_vec<DT>(cv, ce);
+        sample_pairs<DT, VEC>(ge, ce, emax, umax, ab, qb);
       }
-      atomicMax(&sm.lb, (int)emax);
-      atomicMax(&sm.ub, (int)(32 - __clz(umax)));
+    } else if (vb + tid < ve) {
+      uint32_t ge[1], ce[1];
+      ge[0] = load_scalar<DT>(p.g, vb + tid);
+      ce[0] = cand_at<DT, INJ>(p, vb + tid, ge[0]);
+      sample_pairs<DT, 1>(ge, ce, emax, umax, ab, qb);
+    }
+    emax = __reduce_max_sync(0xFFFFFFFFu, emax);
+    umax = __reduce_max_sync(0xFFFFFFFFu, umax);
+    ab = __reduce_max_sync(0xFFFFFFFFu, ab);
+    qb = __reduce_max_sync(0xFFFFFFFFu, qb);
+    __syncthreads();  // piece_init is visible
+    if (lane == 0) {
+      if (emax) atomicMax(&sm.k.lb, (int)emax);
+      if (umax) atomicMax(&sm.k.ub, (int)(32 - __clz(umax)));
+      if (ab) atomicMax(&sm.k.kabs, (unsigned long long)ab << 32);
+      if (umax) atomicMax(&sm.k.kulp, (unsigned long long)min(umax, (1u << 23) - 1u) << 32);
+      if (qb) atomicMax(&sm.k.krel, (unsigned long long)qb << 32);
     }
     if (tid == 0) {
       constexpr long long NONE = 0x7FFFFFFFFFFFFFFFll;
       const bool fin = (G0 & Ty::MAG) < Ty::INF && (C0 & Ty::MAG) < Ty::INF;
-      sm.ff = fin ? pb : NONE;
-      sm.fu = fin ? pb : NONE;
+      sm.k.ff = fin ? pb : NONE;
+      sm.k.fu = fin ? pb : NONE;
     }
     __syncthreads();
-    // the piece's initial window, the first entry of every warp's window log
-    {
-      const int lb0 = window_floor<DT>(sm.lb, sm.ub);
+    if constexpr (DT == PEAT_F32) {
+      // the piece's initial window, the first entry of every warp's window log
+      const int lb0 = window_floor<DT>(sm.k.lb, sm.k.ub);
       set_window_lb<DT>(W, lb0);
       if (lane == 0) {
-        sm.nwin[warp] = 0;
-        sm.wstart[warp][0] = 0;
-        sm.wlb[warp][0] = lb0;
+        sm.k.nwin[warp] = 0;
+        sm.k.wstart[warp][0] = 0;
+        sm.k.wlb[warp][0] = lb0;
       }
+      __syncwarp();
+    } else {
+      W.fe = window16<DT>(sm.k.lb);
+      if constexpr (DT == PEAT_F16) W.atol = __fmul_rn(p.atol, __uint_as_float((uint32_t)(127 + W.fe) << 23));
     }
-    Thr T;
-    thr_init(T);
-    auto scalar_range = [&](int64_t b0, int64_t b1) {
-      for (int64_t i = b0 + tid; i < b1; i += BLOCK) {
-        const uint32_t G = load_scalar<DT>(p.g, i);
-        do_scalar<DT>(L, T, G, cand_at<DT, INJ>(p, i, G), (uint32_t)(i - lo), W, sm);
+    // Tiles: warp w takes chunks w, w + NW, ... of CHV vectors from its
+    // staging ring (NSTAGE chunks in flight ahead of the one processed);
+    // warp 0 also the head (i = -1, before its chunks) and the tail (after).
+    uint32_t tli = (uint32_t)(vb - lo) + (uint32_t)warp * (uint32_t)TILE;
+    Bounds B;
+    auto run_cold = [&](uint4* gt, uint4* ct, uint32_t li, int i) {
+      const ColdOut o = tile_cold<DT>(L, sm, gt, ct, li, W, i);
+      L = o.L;
+      if constexpr (DT == PEAT_F32) {
+        if (o.lb != W.lb) set_window_lb<DT>(W, o.lb);
       }
+      B.low = true;
     };
-    // scalar head: fewer than VEC elements, or the whole piece in scalar mode
-    // (then in rounds of at most 65535 elements per thread)
-    {
-      const int64_t h_end = vb < pe ? vb : pe;
-      constexpr int64_t ROUND_ELEMS = (int64_t)BLOCK * 65535;
-      for (int64_t r0 = pb; r0 < h_end; r0 += ROUND_ELEMS) {
-        const int64_t r1 = min(h_end, r0 + ROUND_ELEMS);
-        scalar_range(r0, r1);
-        if (r1 < h_end) fold_round<DT>(L, sm, win_lexp<DT>(W));
-      }
+    if (warp == 0 && pb < vb) {
+      stage_scalar<DT, INJ>(p, sm.k.edge_g, sm.k.edge_c, pb, vb);
+      run_cold(sm.k.edge_g, sm.k.edge_c, (uint32_t)(pb - lo), -1);
     }
-    // vector body: warp w takes chunks w, w + NW, ... of CHV vectors from its
-    // staging ring; NSTAGE chunks are in flight ahead of the one processed
-    int64_t i = 0;  // this warp's chunk counter within the piece
-    int64_t fail_i = -1;
+    B = read_bounds<DT>(sm, tli, W);
+    int fail_i = -1;
     uint32_t fail_seq = 0;
-    for (int64_t r0 = 0; r0 < nchunk; r0 += ROUND_CHUNKS) {
-      const int64_t r1 = min(nchunk, r0 + ROUND_CHUNKS);
-      for (int64_t k = warp + NW * i; k < r1; k = warp + NW * (++i)) {
-        const int st = (int)(seq % NSTAGE);
-        const uint32_t parity = (seq / NSTAGE) & 1u;
-        if (!failed && !mbar_wait(&sm.bar[warp][st], parity, p.wait_limit)) {
-          failed = true;  // chunks fail_i .. fail_i + NSTAGE - 1 may still be in flight
-          fail_i = i;
-          fail_seq = seq;
-          if (lane == 0) atomicOr(p.status, 1u);
-        }
-        if (!failed && PEAT_CHECK(k * CHV < nvec && vb + k * CHV * VEC - lo < ((int64_t)1 << 32))) {
-          const int64_t v0 = k * CHV;
-          const int nvalid = (int)min((int64_t)CHV, nvec - v0);
-          if constexpr (INJ) {
-            // the candidate tile, generated from the golden tile into the candidate ring
-            inj_chunk<DT>(p, sm.ring_g[warp][st], sm.ring_c[warp][st], nvalid, vb + v0 * VEC);
-            __syncwarp();
+    if (body_scalar) {
+#pragma unroll 1
+      for (int i = 0; i < nmy; i++, tli += (uint32_t)(NW * TILE)) {
+        const int64_t e0 = vb + (warp + (int64_t)NW * i) * TILE;
+        __syncwarp();
+        stage_scalar<DT, INJ>(p, sm.ring.g[warp][0], sm.ring.c[warp][0], e0, min(ve, e0 + TILE));
+        run_cold(sm.ring.g[warp][0], sm.ring.c[warp][0], tli, i);
+        if constexpr (DT == PEAT_F32)
+          if ((i & 8191) == 8191) flush_sums(L, sm, win_lexp<DT>(W));
+      }
+    } else if (!failed) {
+#pragma unroll 1
+      for (int i = 0; i < nmy; i++) {
+        const uint32_t st = seq % NSTAGE;
+        if (!mbar_test(bar0 + 8u * st, (seq / NSTAGE) & 1u) || p.wait_limit == 0) {
+          if (!mbar_wait(bar0 + 8u * st, (seq / NSTAGE) & 1u, p.wait_limit)) {
+            failed = true;  // chunks i .. i + NSTAGE - 1 may still be in flight
+            fail_i = i;
+            fail_seq = seq;
+            if (lane == 0) atomicOr(p.status, 1u);
+            break;
           }
-          do_tile<DT>(L, T, sm.ring_g[warp][st], nvalid, (uint32_t)(vb + v0 * VEC - lo), W, (uint32_t)i, sm);
-          if (lane == 0 && i + NSTAGE < my_chunks) issue(seq + NSTAGE, warp + NW * (i + NSTAGE));
+        }
+        uint4 *gt = sm.ring.g[warp][st], *ct = sm.ring.c[warp][st];
+        if (!PEAT_CHECK((warp + (int64_t)NW * i) * CHV < nvec && vb - lo + (warp + (int64_t)NW * i) * TILE < ((int64_t)1 << 32)))
+          break;
+        if constexpr (INJ) {
+          // the candidate tile, generated from the golden tile into the candidate ring
+          inj_chunk<DT>(p, gt, ct, i == ilast ? (int)lastv : CHV, vb + (warp + (int64_t)NW * i) * TILE);
+          __syncwarp();
+        }
+        if (i == ilast && lastv < (uint32_t)CHV) {  // a partial tile
+          for (int v = lane; v < CHV; v += 32)
+            if (v >= (int)lastv) gt[v] = ct[v] = make_uint4(0, 0, 0, 0);
+          run_cold(gt, ct, tli, i);
+        } else {
+          if (B.low || (i & 3) == 0) B = read_bounds<DT>(sm, tli, W);
+          if constexpr (DT == PEAT_F32) tile32(L, sm, gt, ct, tli, W, B, (uint32_t)i);
+          else tile16<DT>(L, sm, gt, ct, tli, W, B);
+        }
+        __syncwarp();
+        if (i + NSTAGE < nmy) {
+          issue(seq + NSTAGE, i + NSTAGE);
+          gnext += STEP;
+          cnext += STEP;
         }
         seq++;
+        tli += (uint32_t)(NW * TILE);
+        // V1, V2 < 2^21 and 8 pairs per lane and chunk: the products stay below 2^59 between flushes
+        if constexpr (DT == PEAT_F32)
+          if ((i & 8191) == 8191) flush_sums(L, sm, win_lexp<DT>(W));
       }
-      if (r1 < nchunk) fold_round<DT>(L, sm, win_lexp<DT>(W));
+    }
+    if (warp == 0 && ve < pe) {
+      stage_scalar<DT, INJ>(p, sm.k.edge_g, sm.k.edge_c, ve, pe);
+      run_cold(sm.k.edge_g, sm.k.edge_c, (uint32_t)(ve - lo), nmy);
     }
     if (fail_i >= 0) {
       // copies this warp issued but never consumed: wait for them before the
       // staging memory is reused or the CTA exits
-      for (int64_t j = fail_i; j < my_chunks && j < fail_i + NSTAGE; j++) {
+      for (int j = fail_i; j < nmy && j < fail_i + NSTAGE; j++) {
         const uint32_t sq = fail_seq + (uint32_t)(j - fail_i);
-        mbar_wait(&sm.bar[warp][sq % NSTAGE], (sq / NSTAGE) & 1u, DRAIN_LIMIT);
+        mbar_wait(bar0 + 8u * (sq % NSTAGE), (sq / NSTAGE) & 1u, DRAIN_LIMIT);
       }
     }
-    // scalar tail (fewer than VEC elements), after the body
-    if (vb < ve && ve < pe) scalar_range(ve, pe);
     finish_piece<DT, INJ>(L, W, sm, p, s, pb, pe, vb, ve);
     pb = pe;
   }
 }
+
 
 // ---------------------------------------------------------------------------
 // stage 2: one CTA per segment: merge the maxima of the segment's pieces,
@@ -1818,6 +2310,7 @@ __device__ __forceinline__ Partial load_partial(const Partial* src) {
 // maxima in CTA order, round the exact sums once, write the outputs and clear
 // the accumulator for the next call.  Uses the CTA's totals in shared memory
 // as scratch (they are zero on entry and on exit).
+template <int NT>
 __device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, FinScratch& f, MV& mv) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t s0 = p.offsets[s], s1 = p.offsets[s + 1];
@@ -1843,14 +2336,14 @@ __device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s,
   part_none(x);
   {
     const int b0 = cta_of_warp(s0, p), b1 = cta_of_warp(s1 - 1, p);
-    for (int b = b0 + tid; b <= b1; b += BLOCK) part_merge(x, load_partial(p.partials + s + b));
+    for (int b = b0 + tid; b <= b1; b += NT) part_merge(x, load_partial(p.partials + s + b));
   }
   part_warp_reduce(x);
   if (lane == 0) f.wbest[warp] = x;
   __syncthreads();
   if (warp == 1 && lane < NSUM) f.sums[lane] = limbs_to_double(limbs + lane * NLIMB);
   if (warp == 0) {
-    if (lane < NW) x = f.wbest[lane];
+    if (lane < NT / 32) x = f.wbest[lane];
     else part_none(x);
     part_warp_reduce(x);
   }
@@ -1910,12 +2403,12 @@ __global__ void __launch_bounds__(BLOCK) compare_finalize(CompareParams p) {
   __shared__ FinScratch f;
   __shared__ MV mv;
   pdl_wait();  // stage 1 complete
-  if (p.offsets[blockIdx.x] < p.offsets[blockIdx.x + 1]) finalize_segment(p, blockIdx.x, f, mv);
+  if (p.offsets[blockIdx.x] < p.offsets[blockIdx.x + 1]) finalize_segment<BLOCK>(p, blockIdx.x, f, mv);
 }
 
 // The outputs of every empty segment (no pairs): zero counts and sums, argmax -1.
 __device__ __noinline__ void write_empty_segments(const CompareParams& p) {
-  for (int64_t s = threadIdx.x; s < p.nseg; s += BLOCK) {
+  for (int64_t s = threadIdx.x; s < p.nseg; s += blockDim.x) {
     if (p.offsets[s] != p.offsets[s + 1]) continue;
     peat_stats_t r;
     memset(&r, 0, sizeof(r));
@@ -1932,8 +2425,8 @@ template <int DT>
 cudaError_t launch_t(const CompareParams& p, cudaStream_t st) {
   // NVTX ranges (host-side enqueue of each stage) for profilers; no cost without one attached
   nvtxRangePushA(p.inj_n > 0 ? "peat inject+compare stage 1" : "peat compare stage 1");
-  if (p.inj_n > 0) compare_stage1<DT, true><<<p.nctas, BLOCK, sizeof(Smem), st>>>(p);
-  else compare_stage1<DT, false><<<p.nctas, BLOCK, sizeof(Smem), st>>>(p);
+  if (p.inj_n > 0) compare_stage1<DT, true><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
+  else compare_stage1<DT, false><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
   cudaError_t e = cudaGetLastError();
   nvtxRangePop();
   if (e == cudaSuccess && p.stage1_event) e = cudaEventRecord(static_cast<cudaEvent_t>(p.stage1_event), st);
@@ -2009,8 +2502,8 @@ int64_t compare_cta_bound(int dtype, int64_t b, int nctas, int64_t n, int64_t p0
 template <int DT, bool INJ>
 cudaError_t prepare_one() {
   cudaError_t e =
-      cudaFuncSetAttribute(compare_stage1<DT, INJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
-  if (e == cudaSuccess)  // as much shared memory as the SM offers: CTAS_PER_SM CTAs of sizeof(Smem) each
+      cudaFuncSetAttribute(compare_stage1<DT, INJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<DT>));
+  if (e == cudaSuccess)  // as much shared memory as the SM offers: Geo<DT>::CTAS CTAs of sizeof(Smem<DT>) each
     e = cudaFuncSetAttribute(compare_stage1<DT, INJ>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
@@ -2027,7 +2520,7 @@ cudaError_t compare_prepare() {
   return e;
 }
 
-int compare_ctas_per_sm() { return CTAS_PER_SM; }
+int compare_ctas_per_sm(int dtype) { return dtype == PEAT_F32 ? Geo<PEAT_F32>::CTAS : Geo<PEAT_BF16>::CTAS; }
 size_t compare_partial_bytes() { return sizeof(Partial); }
 size_t compare_segacc_bytes() { return sizeof(SegAcc); }
 

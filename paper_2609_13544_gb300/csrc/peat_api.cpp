@@ -485,7 +485,7 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
     p.p0 = -1;
   // persistent grid; small inputs get about one CTA per 4K elements
   int64_t want = (n + 4095) / 4096;
-  p.nctas = (int)std::max<int64_t>(1, std::min<int64_t>(h->max_ctas, want));
+  p.nctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->nsm * peat::compare_ctas_per_sm(dtype), want));
   // stage 1 keeps element offsets within a CTA's range in 32 bits
   if (n / p.nctas >= ((int64_t)1 << 31) - 64)
     return fail(h, PEAT_ERR_UNSUPPORTED, "n is too large for one call (more than 2^31 elements per CTA)");
@@ -669,7 +669,7 @@ peat_status_t peat_signature_create(peat_handle_t* out, const peat_config_t* cfg
     delete h;
     return PEAT_ERR_CUDA;
   }
-  h->max_ctas = std::max(1, h->nsm * peat::compare_ctas_per_sm());
+  h->max_ctas = std::max(1, 2 * h->nsm);  // the most any element type's compare runs at once
   // segmented calls may use up to 2 * max_ctas CTAs (see segment_split)
   size_t slots = (size_t)h->max_segments + 2 * (size_t)h->max_ctas;
   size_t staging = (size_t)h->max_segments + 2 + 2 * (size_t)h->max_ctas;
@@ -1264,7 +1264,7 @@ peat_status_t peat_compare_noalloc(const void* golden, const void* candidate, in
     p.p0 = (int64_t)(((16 - ag % 16) % 16) / B);
   else
     p.p0 = -1;
-  const int max_ctas = std::min(NOALLOC_MAX_CTAS, D.nsm * peat::compare_ctas_per_sm());
+  const int max_ctas = std::min(NOALLOC_MAX_CTAS, D.nsm * peat::compare_ctas_per_sm(dtype));
   p.nctas = (int)std::max<int64_t>(1, std::min<int64_t>(max_ctas, (n + 4095) / 4096));
   // the per-CTA element offsets of stage 1 are 32-bit
   if (n / p.nctas >= ((int64_t)1 << 31) - 64)

@@ -46,7 +46,7 @@ constexpr int NLIMB = 24;
 constexpr int LIMB_LSB = -416;
 constexpr int NSUM = 3;  // 0: sum d, 1: sum |d|, 2: sum d^2
 
-constexpr int BLOCK = 256;    // threads per compare CTA
+constexpr int BLOCK = 256;    // threads of the small kernels (bounds, per-segment finalize)
 constexpr int GCAP = 16384;   // general-path pairs a CTA lists per segment piece (more: the piece is rescanned)
 constexpr int HBINS = 128;    // 64 rel bins + 64 ULP bins
 
@@ -127,7 +127,7 @@ struct CompareParams {
 
 // Host-side launchers (compare.cu / inject.cu).
 cudaError_t launch_compare(int dtype, const CompareParams& p, cudaStream_t s);
-int compare_ctas_per_sm();
+int compare_ctas_per_sm(int dtype);  // resident CTAs of the element type's stage 1 (at most 2)
 cudaError_t compare_prepare();
 // CTA b of a grid of nctas owns elements [bound(b), bound(b+1)); boundaries
 // lie on the 16-byte vector grid that starts at element p0 (p0 < 0: none)

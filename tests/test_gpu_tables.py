@@ -1,0 +1,96 @@
+"""The compare's window tables at the places where they can go wrong: tile and
+vector edges, vectors with a few unequal lanes, equal pairs that hold NaN or
+infinity inside them, ties of a maximum across the whole tensor, values at the
+ends of the window, and a nonzero atol.  Everything exact against the oracle."""
+import numpy as np
+import pytest
+
+from parity_util import NP_BITS, assert_hist_equal, assert_stats_equal, to_device
+
+pytestmark = pytest.mark.gpu
+DTYPES = ("f32", "f16", "bf16")
+
+
+def encode(x, dtype):
+    if dtype == "f32":
+        return np.asarray(x, np.float32).view(np.uint32)
+    if dtype == "f16":
+        return np.asarray(x, np.float16).view(np.uint16)
+    return (np.ascontiguousarray(np.asarray(x, np.float32)).view(np.uint32) >> 16).astype(np.uint16)
+
+
+def check(peat_gpu, oracle, gb, cb, dtype, rtol, atol, ctx, shift=0):
+    with peat_gpu.Handle(0) as h:
+        st, hist = peat_gpu.peat_compare(h, to_device(gb, dtype, shift), to_device(cb, dtype, shift), rtol, atol)
+    ost, oh = oracle.compare(gb, cb, dtype, rtol, atol)
+    assert_stats_equal(st, ost, ctx)
+    assert_hist_equal(hist, oh, ctx)
+
+
+def steps(gb, k):
+    """Patterns k steps away, inside the finite range and the same sign."""
+    w = gb.dtype.itemsize * 8
+    mag = gb & ((1 << (w - 1)) - 1)
+    return np.where(mag > 4096 if w == 32 else mag > 300, gb + k.astype(gb.dtype), gb).astype(gb.dtype)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n", (1, 7, 8, 9, 255, 256, 511, 512, 513, 8191, 8192, 8193, 65537))
+@pytest.mark.parametrize("shift", (0, 3))
+def test_edges(peat_gpu, oracle, dtype, n, shift):
+    rng = np.random.default_rng(n + shift)
+    gb = encode(rng.standard_normal(n), dtype)
+    cb = steps(gb, rng.integers(-3, 4, n))
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} n={n} shift={shift}", shift)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("share", (0.0, 0.0005, 0.01, 0.05, 0.3, 1.0))
+def test_shares_of_unequal_pairs(peat_gpu, oracle, dtype, share):
+    """Sparse and dense vectors, with NaN and infinity in equal and unequal pairs of both."""
+    rng = np.random.default_rng(int(share * 1e4))
+    n = 200_003
+    gb = encode(rng.standard_normal(n) * 3.0, dtype)
+    k = np.where(rng.random(n) < share, rng.integers(-2, 3, n), 0)
+    cb = steps(gb, k)
+    special = [np.nan, np.inf, -np.inf, 0.0, -0.0]
+    for i in rng.integers(0, n, 60):
+        gb[i] = cb[i] = encode([special[int(rng.integers(0, 5))]], dtype)[0]
+    for i in rng.integers(0, n, 20):
+        cb[i] = encode([special[int(rng.integers(0, 5))]], dtype)[0]
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} share={share}")
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("value", (1.0, 1.3, -777.0, 3e-5, 60000.0))
+def test_one_value_everywhere(peat_gpu, oracle, dtype, value):
+    """Every pair ties for all three maxima: the first one wins."""
+    n = 150_001
+    gb = np.repeat(encode([value], dtype), n)
+    cb = gb.copy()
+    cb[1234:] += 1
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-2, 0.0, f"{dtype} value={value}")
+
+
+@pytest.mark.parametrize("dtype,lo,hi", (("f32", -120, 120), ("f32", -12, 3), ("f16", -24, -10), ("f16", -24, 15),
+                                         ("f16", 8, 15), ("bf16", -120, 120), ("bf16", -60, 4), ("bf16", -126, -100)))
+@pytest.mark.parametrize("width", (1, 20, 63, 64, 127, 128, 400))
+def test_window_ends(peat_gpu, oracle, dtype, lo, hi, width):
+    """Goldens over a range of binades, differences up to `width` steps: inside and outside of the window."""
+    rng = np.random.default_rng(width)
+    n = 60_000
+    x = np.exp2(rng.uniform(lo, hi, n)) * rng.choice([-1.0, 1.0], n)
+    gb = encode(x, dtype)
+    cb = (gb.astype(np.int64) + rng.integers(-width, width + 1, n)).clip(0, 2 ** (8 * gb.dtype.itemsize) - 1).astype(
+        NP_BITS[dtype])
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-2, 0.0, f"{dtype} 2^{lo}..2^{hi} width={width}")
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("rtol,atol", ((1e-3, 1e-5), (0.0, 1e-3), (2.0 ** -7, 2.0 ** -12), (0.0, 0.0), (1.0, 1e30)))
+def test_tolerances(peat_gpu, oracle, dtype, rtol, atol):
+    rng = np.random.default_rng(3)
+    n = 100_001
+    gb = encode(rng.standard_normal(n), dtype)
+    cb = steps(gb, rng.integers(-9, 10, n))
+    check(peat_gpu, oracle, gb, cb, dtype, rtol, atol, f"{dtype} rtol={rtol} atol={atol}")
