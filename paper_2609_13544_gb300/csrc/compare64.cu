@@ -2,8 +2,10 @@
 // histograms of the compare) for binary64 operands: the FP32-FP64 pairs of
 // Fig. 5 once the float32 side is widened (exactly) to binary64.
 //
-// d = c - g is an exact double-double (hi, lo) from Fast2Sum on the operands
-// ordered by magnitude, held halved with a scale of one when the difference
+// Most pairs (one sign, patterns less than 2^51 apart, zero atol) are finished
+// in integer arithmetic on the patterns (fast64).  For the others d = c - g is
+// an exact double-double (hi, lo) from Fast2Sum on the operands ordered by
+// magnitude, held halved with a scale of one when the difference
 // overflows binary64 (both operands are then large, so halving is exact).  Decisions that rounding could
 // flip (the tolerance, the relative maximum) take a binary64 or float32 test
 // with a margin first and otherwise the sign of an exact sum of integer
@@ -75,6 +77,21 @@ __device__ __forceinline__ float lg_diff(int xe, float xf, int ye, float yf) {
 __device__ bool rel_gt(const Rel& x, const Rel& y) {
   if (x.kind != y.kind) return x.kind > y.kind;
   if (x.kind != 1) return false;
+  if (x.a.lo == 0.0 && y.a.lo == 0.0 && x.a.sc == 0 && y.a.sc == 0) {
+    // single binary64 magnitudes: the cross products of the 53-bit
+    // significands (106 bits, leading bit 104 or 105), aligned
+    uint64_t xa, xg, ya, yg;
+    int exa, exg, eya, eyg;
+    norm_d(x.a.hi, xa, exa);
+    norm_d(x.g, xg, exg);
+    norm_d(y.a.hi, ya, eya);
+    norm_d(y.g, yg, eyg);
+    const uint64_t ONE = 1ull << 52;
+    const u128 l = (u128)(xa | ONE) * (yg | ONE), r = (u128)(ya | ONE) * (xg | ONE);
+    const int dl = (exa + eyg) - (eya + exg);
+    if (dl > 2 || dl < -2) return dl > 0;
+    return dl >= 0 ? (l << dl) > r : l > (r << -dl);
+  }
   XTerm t[4] = {prod_term(x.a.hi, y.g, x.a.sc, false), prod_term(fabs(x.a.lo), y.g, x.a.sc, x.a.lo < 0.0),
                 prod_term(y.a.hi, x.g, y.a.sc, true), prod_term(fabs(y.a.lo), x.g, y.a.sc, y.a.lo >= 0.0)};
   return xsign(t, 4) > 0;
@@ -280,6 +297,12 @@ __device__ __forceinline__ void pair64(const Cmp64Params& p, Acc64& t, unsigned*
   hist_add(H, ulpbin < 0 ? -1 : 64 + ulpbin);
 }
 
+// (out of line: the pairs that the integer path leaves)
+__device__ __noinline__ void pair64_slow(const Cmp64Params& p, Acc64& t, unsigned* H, long long* S, uint64_t G, uint64_t C,
+                                         bool ok, uint32_t off) {
+  pair64(p, t, H, S, G, C, ok, off);
+}
+
 // x better than y: larger, or equal at a lower index (-1: absent, worst)
 __device__ __forceinline__ bool better_mag(const Mag& x, long long ix, const Mag& y, long long iy) {
   if (ix < 0) return false;
@@ -324,125 +347,400 @@ __device__ __forceinline__ void rec_from_acc(Part64Rec& r, const Acc64& a, long 
   r.mu = a.mu, r.iu = a.iu ? ib + a.iu - 1 : -1;
 }
 
-// the CTA's records merged into thread 0's (every thread calls it)
+// the CTA's records merged into thread 0's (every thread calls it; buf holds
+// half of them)
 __device__ void block_merge(Part64Rec& r, Part64Rec* buf) {
-  buf[threadIdx.x] = r;
-  __syncthreads();
   for (int w = TB / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) rec_merge(buf[threadIdx.x], buf[threadIdx.x + w]);
+    if ((int)threadIdx.x >= w && (int)threadIdx.x < 2 * w) buf[threadIdx.x - w] = r;
+    __syncthreads();
+    if ((int)threadIdx.x < w) rec_merge(r, buf[threadIdx.x]);
     __syncthreads();
   }
-  r = buf[0];
-  __syncthreads();
 }
 
-// carry-normalise n limbs of 32-bit digits (thread 0): every limb in [0, 2^32), the top one signed
-__device__ void normalise(long long* d, int n) {
-  long long carry = 0;
-  for (int j = 0; j < n - 1; j++) {
-    const long long v = d[j] + carry;
-    carry = v >> 32;
-    d[j] = v & 0xFFFFFFFFll;
+__device__ __forceinline__ uint64_t wsum_u64(uint64_t v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
+// The integer path.  A window pair has patterns less than 2^51 apart (so one
+// sign, exponents at most one apart, c - g exact): with el the smaller
+// exponent field, |d| = a 2^(el - 1075) for the integer a = |C - G|, plus the
+// larger operand's fraction field when the exponents differ (its steps are
+// two units).  With s = el - base in [0, WS]:
+//   - sum |d| and the sum of the negative ones: a << s in 128-bit registers;
+//   - sum d^2: a * a shifted by 2 s, added as 32-bit digits to the thread's own
+//     64-bit counters in shared memory;
+//   - the two bins from shared counters by (floor(log2(|d| / |g|)) mod 64,
+//     min(ULP distance, 63)) (increments by one merge equal addresses; column
+//     0 takes the lanes without an unequal pair and is left out);
+//   - the tolerance (atol = 0) and the relative maximum from the ratio in
+//     float32, within 2^-21: closer calls take the slow path.
+// A pair outside the window, non-finite, or above one of the warp's maxima so
+// far goes to pair64.  The warp's iterations visit its pairs in index order, so a
+// pair equal to a maximum of an earlier round cannot win.
+//
+// What bounds it: integer instruction issue (no FP64 instruction, whose pipe
+// takes 64 cycles per warp here, and no local memory): about 250 instructions
+// per pair slot of a warp.  12.3 M pairs (a float32 rounding widened, rtol
+// 1e-7), one call: 2200 -> 207 us, of which the finalization 32; before, every
+// term went through binary64 Fast2Sum and local-memory windows (1070
+// instructions and 1.9 GB of local-memory traffic).
+constexpr int WS = 56, QD = 8;
+
+struct CtaBounds {  // the largest of the warps' bounds
+  unsigned long long kabs, ku;
+  unsigned rb;
+};
+struct Fast64 {
+  u128 s1, n1;         // sum |d|, sum of |d| over negative d, in units of 2^(base - 1075)
+  uint32_t mism;       // pairs above the tolerance
+  int base;            // -1: not placed yet (no unequal finite pair seen)
+  uint32_t miss;       // pairs of small distance outside the window since it was placed
+  // the warp's bounds: a pair above one of them takes the slow path.  Its own
+  // maxima, and the CTA's less one step (a pair of another warp may have the
+  // same value at a higher index).
+  uint64_t kabs, ku;   // |d| as a key (exponent, significand), ULP distance
+  float rb;            // ratio, lowered by 2^-19
+  // maxima seen in this round, bounds from the next one on (a lane's second
+  // pair precedes the next lane's first)
+  uint64_t pk, pu;
+  uint32_t nslow;      // pairs given to pair64 (the whole warp's)
+};
+
+// The integer path's sums into the item's digits (the whole warp calls it):
+// words summed over the warp, then added by one lane.
+// By value, so that the caller's state stays in registers.
+__device__ __noinline__ void fast_flush(int base, u128 s1, u128 n1, long long* S, unsigned long long* Q) {
+  const int lane = threadIdx.x & 31;
+  const int u = base - 1075;
+#pragma unroll 1
+  for (int w = 0; w < 4; w++) {
+    const uint64_t a1 = wsum_u64((uint32_t)(s1 >> (32 * w))), an = wsum_u64((uint32_t)(n1 >> (32 * w)));
+    if (lane == 0) {
+      sacc_add(S + SL, a1, u + 32 * w, false);
+      sacc_add(S, a1, u + 32 * w, false);  // sum d = sum |d| - 2 sum of the negative ones
+      sacc_add(S, (u128)an << 1, u + 32 * w, true);
+    }
   }
-  d[n - 1] += carry;
+#pragma unroll 1
+  for (int w = 0; w < QD; w++) {
+    const uint64_t qs = wsum_u64(Q[w * TB]);
+    Q[w * TB] = 0ull;
+    if (lane == 0) sacc_add(S + 2 * SL, qs, 2 * u + 32 * w, false);
+  }
+}
+
+// one pair slot of the warp (every lane calls it; a lane without a pair passes equal zeros and ok = false)
+__device__ __forceinline__ void fast64(const Cmp64Params& p, Fast64& f, Acc64& acc, unsigned* H, long long* S,
+                                       uint32_t t2, unsigned long long* Q, CtaBounds* cb, uint64_t G, uint64_t C,
+                                       bool ok, uint32_t off, float rlo, float rhi) {
+  constexpr uint64_t FRAC = 0xFFFFFFFFFFFFFull;
+  const int64_t U = (int64_t)(C - G);
+  const uint64_t au = U < 0 ? (uint64_t)-U : (uint64_t)U;
+  const bool nz = au != 0;
+  const uint64_t mx = (U > 0 ? C : G) & MAG64, mn = (U > 0 ? G : C) & MAG64;
+  const uint32_t eu = (uint32_t)(mx >> 52), el = (uint32_t)(mn >> 52);
+  const uint64_t a0 = au + (eu != el ? mx & FRAC : 0ull);
+  if (f.base < 0) {  // (warp-uniform) place the window by the first unequal pairs
+    const uint32_t em = __reduce_max_sync(0xFFFFFFFFu, nz && el < 0x7FFu ? el : 0u);
+    if (em) f.base = max((int)em - 40, 64);
+  }
+  const int s0 = (int)el - f.base;
+  const bool win = nz && au < (1ull << 51) && (unsigned)s0 <= (unsigned)WS && el < 0x7FFu && eu < 0x7FFu && f.base >= 0 && p.atol == 0.0;
+  bool exc = nz ? !win : (ok && el == 0x7FFu);
+  // |d| normalised: a << lz has its leading one at bit 63
+  const int lz = __clzll((long long)(a0 | 1ull));
+  const uint64_t am = a0 << lz;
+  const int ea = (int)el + 63 - lz;  // |d| = (am / 2^63) 2^(ea - 1075)
+  const int eg = (int)((uint32_t)(G >> 52) & 0x7FFu);
+  const uint64_t gn = (((G & FRAC) | (1ull << 52)) << 11);
+  const int dk = ea - eg - 52;
+  const int k = dk - (am < gn ? 1 : 0);
+  const uint64_t key = ((uint64_t)(uint32_t)ea << 52) + ((am << 1) >> 12);
+  const float fa = __uint_as_float(0x3F800000u | ((uint32_t)(am >> 40) & 0x7FFFFFu));
+  const float fg = __uint_as_float(0x3F800000u | ((uint32_t)(G >> 29) & 0x7FFFFFu));
+  float rc;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(rc) : "f"(fg));
+  const float rf = __uint_as_float(__float_as_uint(fa * rc) + ((uint32_t)dk << 23));
+  exc = exc || (win && (key > f.kabs || au > f.ku || rf >= f.rb || (rf > rlo && rf < rhi)));
+  const bool use = win && !exc;
+  const uint64_t a = use ? a0 : 0ull;
+  const int s = use ? s0 : 0;
+  f.mism += use && rf >= rhi ? 1u : 0u;
+  const uint32_t uc = use ? (uint32_t)(au < 63 ? au : 63) : 0u;
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(t2 + ((((uint32_t)k & 63u) << 6) | uc) * 4u));
+  const uint64_t vlo = a << s, vhi = (a >> 1) >> (63 - s);
+  const u128 v = ((u128)vhi << 64) | vlo;
+  f.s1 += v;
+  const bool neg = (U < 0) != ((int64_t)G < 0);
+  f.n1 += neg ? v : (u128)0;
+  {
+    const uint32_t alo = (uint32_t)a, ahi = (uint32_t)(a >> 32);
+    const uint32_t w = (uint32_t)(2 * s) >> 5, b = (uint32_t)(2 * s) & 31u;
+    unsigned long long* q = Q + w * TB;
+    if (!__any_sync(0xFFFFFFFFu, ahi != 0u)) {  // a < 2^32: three digits
+      const uint64_t pp = (uint64_t)alo * alo;
+      const uint32_t p0 = (uint32_t)pp, p1 = (uint32_t)(pp >> 32);
+      q[0] += p0 << b;
+      q[TB] += __funnelshift_l(p0, p1, b);
+      q[2 * TB] += __funnelshift_l(p1, 0u, b);
+    } else {
+      const u128 pp = (u128)a * a;
+      const uint32_t p0 = (uint32_t)pp, p1 = (uint32_t)(pp >> 32), p2 = (uint32_t)(pp >> 64), p3 = (uint32_t)(pp >> 96);
+      q[0] += p0 << b;
+      q[TB] += __funnelshift_l(p0, p1, b);
+      q[2 * TB] += __funnelshift_l(p1, p2, b);
+      q[3 * TB] += __funnelshift_l(p2, p3, b);
+      q[4 * TB] += __funnelshift_l(p3, 0u, b);
+    }
+  }
+  const unsigned who = __ballot_sync(0xFFFFFFFFu, exc);
+  if (who) {
+    pair64_slow(p, acc, H, S, G, C, exc, off);
+    f.nslow += (uint32_t)__popc(who);
+    // too many pairs outside the window: place it again by the next unequal ones
+    f.miss += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, exc && !win && au < (1ull << 51) && f.base >= 0 && p.atol == 0.0));
+    if (f.miss >= 256u) {
+      fast_flush(f.base, f.s1, f.n1, S, Q);
+      f.s1 = f.n1 = 0;
+      f.base = -1;
+      f.miss = 0;
+    }
+    // the warp's bounds (only window pairs raise them)
+    const bool up = exc && win;
+    const uint32_t kh = __reduce_max_sync(0xFFFFFFFFu, up ? (uint32_t)(key >> 32) : 0u);
+    const uint32_t kl = __reduce_max_sync(0xFFFFFFFFu, up && (uint32_t)(key >> 32) == kh ? (uint32_t)key : 0u);
+    const uint32_t uh = __reduce_max_sync(0xFFFFFFFFu, up ? (uint32_t)(au >> 32) : 0u);
+    const uint32_t ul = __reduce_max_sync(0xFFFFFFFFu, up && (uint32_t)(au >> 32) == uh ? (uint32_t)au : 0u);
+    const float rm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, up ? __float_as_uint(rf) : 0u));
+    f.pk = max(f.pk, ((uint64_t)kh << 32) | kl);
+    f.pu = max(f.pu, ((uint64_t)uh << 32) | ul);
+    f.rb = fmaxf(f.rb, rm * 0.999998f);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&cb->kabs, (unsigned long long)f.pk);
+      atomicMax(&cb->ku, (unsigned long long)f.pu);
+      atomicMax(&cb->rb, __float_as_uint(f.rb));
+    }
+  }
 }
 
 __global__ void __launch_bounds__(TB, 2) compare64_stage1(Cmp64Params p) {
   __shared__ unsigned H[PEAT_HIST_BINS];
   __shared__ long long S[3 * SL];
-  __shared__ Part64Rec buf[TB];
+  __shared__ unsigned long long tot[2];  // window pairs, of them above the tolerance; pairs given to pair64
+  __shared__ unsigned long long nsl;
+  __shared__ unsigned first;  // offset of the item's first equal finite pair (searched when it matters)
+  __shared__ int need;
+  __shared__ CtaBounds cb;
+  union Scratch {
+    struct {
+      uint32_t t2[64 * 64];
+      unsigned long long q[QD][TB];
+    } w;
+    Part64Rec buf[TB / 2];
+  };
+  __shared__ Scratch sc;
   pdl_trigger();  // the finalize kernel may start launching (it waits for this grid)
   const int lane = threadIdx.x & 31;
+  const uint32_t t2 = (uint32_t)__cvta_generic_to_shared(sc.w.t2);
+  // the tolerance on the float32 ratio: closer than 2^-18 to rtol takes the exact test
+  const float rt = (float)p.rtol, rlo = rt * 0.999996f, rhi = rt * 1.000004f;
+  Fast64 f;
+  long long prev = -1;
   for (long long item = blockIdx.x; item < p.nitems; item += gridDim.x) {
     const long long b = p.item_b[item], e = p.item_e[item], seg = p.item_seg[item];
     const long long base = p.offsets[seg];
     for (int k = threadIdx.x; k < PEAT_HIST_BINS; k += TB) H[k] = 0u;
     for (int k = threadIdx.x; k < 3 * SL; k += TB) S[k] = 0;
+    for (int k = threadIdx.x; k < 64 * 64; k += TB) sc.w.t2[k] = 0u;
+#pragma unroll
+    for (int k = 0; k < QD; k++) sc.w.q[k][threadIdx.x] = 0ull;
+    if (threadIdx.x < 2) tot[threadIdx.x] = 0ull;
+    if (threadIdx.x == 2) nsl = 0ull;
+    if (threadIdx.x == 3 && seg != prev) cb.kabs = cb.ku = 0ull, cb.rb = 0u;
     __syncthreads();
     Acc64 acc;
     acc64_init(acc);
-    // pairs of elements (one 16-byte vector of each tensor) on the absolute index grid
-    const long long q0 = b >> 1, q1 = (e + 1) >> 1;
-    for (long long q = q0 + threadIdx.x; __any_sync(0xFFFFFFFFu, q < q1); q += TB) {
-      const bool okq = q < q1;
-      const long long i0 = q << 1;
-      uint64_t gw[2] = {0, 0}, cw[2] = {0, 0};
-      if (okq && p.vec && i0 >= b && i0 + 2 <= e) {
-        const ulonglong2 gv = __ldg(reinterpret_cast<const ulonglong2*>(p.g) + q);
-        const ulonglong2 cv = __ldg(reinterpret_cast<const ulonglong2*>(p.c) + q);
-        gw[0] = gv.x, gw[1] = gv.y, cw[0] = cv.x, cw[1] = cv.y;
-      } else if (okq) {
-        for (int j = 0; j < 2; j++)
-          if (i0 + j >= b && i0 + j < e) {
-            gw[j] = __ldg(reinterpret_cast<const unsigned long long*>(p.g) + i0 + j);
-            cw[j] = __ldg(reinterpret_cast<const unsigned long long*>(p.c) + i0 + j);
-          }
+    f.s1 = f.n1 = 0;
+    f.mism = f.nslow = f.miss = 0;
+    f.base = -1;
+    // bounds carry over within a segment: its items come in index order
+    if (seg != prev) {
+      f.kabs = f.ku = f.pk = f.pu = 0ull;
+      f.rb = 0.0f;
+      prev = seg;
+    }
+    // pairs of elements (one 16-byte vector of each tensor) on the absolute
+    // index grid, the next ones loaded while these are processed
+    // (offsets in the item are 32-bit: it has at most 2^22 elements)
+    const int len = (int)(e - b), o0 = -(int)(b & 1);  // vector v holds the item's offsets o0 + 2 v, o0 + 2 v + 1
+    const int nq = (len - o0 + 1) >> 1;
+    const char* gp = reinterpret_cast<const char*>(p.g) + (b + o0) * 8;
+    const char* cp = reinterpret_cast<const char*>(p.c) + (b + o0) * 8;
+    auto load = [&](int v, ulonglong2& gv, ulonglong2& cv) {
+      gv = cv = make_ulonglong2(0ull, 0ull);
+      const int o = o0 + 2 * v;
+      if (p.vec && o >= 0 && o + 2 <= len) {
+        gv = __ldg(reinterpret_cast<const ulonglong2*>(gp) + v);
+        cv = __ldg(reinterpret_cast<const ulonglong2*>(cp) + v);
+      } else {
+        const unsigned long long* gq = reinterpret_cast<const unsigned long long*>(gp) + 2 * v;
+        const unsigned long long* cq = reinterpret_cast<const unsigned long long*>(cp) + 2 * v;
+        if (o >= 0 && o < len) gv.x = __ldg(gq), cv.x = __ldg(cq);
+        if (o + 1 < len) gv.y = __ldg(gq + 1), cv.y = __ldg(cq + 1);
       }
-#pragma unroll 1
-      for (int j = 0; j < 2; j++) {
-        const long long i = i0 + j;
-        pair64(p, acc, H, S, j ? gw[1] : gw[0], j ? cw[1] : cw[0], okq && i >= b && i < e, (uint32_t)(i - b));
+    };
+    ulonglong2 gn, cn;
+    int v = threadIdx.x;
+    load(v, gn, cn);
+    // whole warps in every round
+    for (int r = threadIdx.x & ~31; r < nq; r += TB, v += TB) {
+      const ulonglong2 gc = gn, cc = cn;
+      load(v + TB, gn, cn);
+      const int o = o0 + 2 * v;
+      {
+        const volatile CtaBounds* vb = &cb;
+        const uint64_t ka = (uint64_t)vb->kabs, ku = (uint64_t)vb->ku;
+        f.kabs = max(max(f.kabs, f.pk), ka - (ka ? 1 : 0));
+        f.ku = max(max(f.ku, f.pu), ku - (ku ? 1 : 0));
+        f.rb = fmaxf(f.rb, __uint_as_float(vb->rb));
       }
+      fast64(p, f, acc, H, S, t2, &sc.w.q[0][threadIdx.x], &cb, gc.x, cc.x, o >= 0 && o < len, (uint32_t)o, rlo, rhi);
+      fast64(p, f, acc, H, S, t2, &sc.w.q[0][threadIdx.x], &cb, gc.y, cc.y, o + 1 < len, (uint32_t)(o + 1), rlo, rhi);
     }
     win_flush(acc.sd, acc.bd, S);
     win_flush(acc.sa, acc.ba, S + SL);
     win3_flush(acc.sq, S + 2 * SL);
-    Part64Rec r;
-    rec_from_acc(r, acc, b - base);
-    block_merge(r, buf);
-    Part64* out = p.parts + item;
-    if (threadIdx.x == 0) {
-      out->rec = r;
-      for (int s = 0; s < 3; s++) normalise(S + s * SL, SL);
+    if (f.base >= 0) fast_flush(f.base, f.s1, f.n1, S, &sc.w.q[0][threadIdx.x]);
+    const uint32_t mism = __reduce_add_sync(0xFFFFFFFFu, f.mism);
+    if (lane == 0) {
+      if (mism) atomicAdd(&tot[1], (unsigned long long)mism);
+      if (f.nslow) atomicAdd(&nsl, (unsigned long long)f.nslow);
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < 3 * SL; k += TB) out->limbs[k] = S[k];
+    // the bins: a thread holds every fourth row of one column
+    {
+      const int col = threadIdx.x & 63;
+      uint32_t cs = 0;
+      for (int i = 0; i < 16; i++) {
+        const int row = (threadIdx.x >> 6) + 4 * i;
+        const uint32_t v = col == 0 ? 0u : sc.w.t2[row * 64 + col];
+        if (!__any_sync(0xFFFFFFFFu, v != 0u)) continue;
+        cs += v;
+        const uint32_t rs = __reduce_add_sync(0xFFFFFFFFu, v);
+        const int k = row == 0 ? 0 : row - 64;
+        if (lane == 0) atomicAdd(H + max(k + 48, 1), rs);
+      }
+      if (cs) atomicAdd(H + 64 + col, cs);
+      cs = __reduce_add_sync(0xFFFFFFFFu, cs);
+      if (lane == 0 && cs) atomicAdd(&tot[0], (unsigned long long)cs);
+    }
+    __syncthreads();
+    Part64Rec r;
+    rec_from_acc(r, acc, b - base);
+    block_merge(r, sc.buf);
+    Part64* out = p.parts + item;
+    const unsigned long long fast = (unsigned long long)(e - b) - nsl, same = fast - tot[0];
+    if (threadIdx.x == 0) {
+      // the integer path's pairs: finite, unequal ones within or above the
+      // tolerance (one sign: no flips), the rest bitwise equal
+      r.cnt[PEAT_EXACT] += same;
+      r.cnt[PEAT_WITHIN_TOL] += tot[0] - tot[1];
+      r.cnt[PEAT_MISMATCH] += tot[1];
+      r.nfin += fast;
+      H[0] += (unsigned)same;
+      H[64] += (unsigned)same;
+      // an equal pair has |d| = 0 and u = 0: it matters when nothing larger was recorded
+      need = same != 0ull && (r.ia < 0 || r.ahi == 0.0 || r.iu < 0 || r.mu == 0ull);
+      first = nsl == 0ull ? 0u : 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    if (need && nsl != 0ull) {
+      for (long long x = b; x < e && first == 0xFFFFFFFFu; x += TB) {
+        __syncthreads();
+        const long long i = x + threadIdx.x;
+        if (i < e) {
+          const uint64_t G = __ldg(reinterpret_cast<const unsigned long long*>(p.g) + i);
+          const uint64_t C = __ldg(reinterpret_cast<const unsigned long long*>(p.c) + i);
+          if (G == C && (G & MAG64) < INF64) atomicMin(&first, (unsigned)(i - b));
+        }
+        __syncthreads();
+      }
+    }
+    if (threadIdx.x == 0) {
+      if (need) {
+        const long long z = b - base + first;
+        if (r.ia < 0 || (r.ahi == 0.0 && z < r.ia)) r.ahi = r.alo = 0.0, r.asc = 0, r.ia = z;
+        if (r.ir < 0 || (r.rkind == 0 && z < r.ir)) r.rkind = 0, r.ir = z;
+        if (r.iu < 0 || (r.mu == 0ull && z < r.iu)) r.mu = 0ull, r.iu = z;
+      }
+      out->rec = r;
+    }
+    __syncthreads();
+    // one carry step (limbs below 2^33 in magnitude afterwards, the top one as it is)
+    for (int k = threadIdx.x; k < P64_MASK * 32; k += TB) {
+      const int j = k % SL;
+      const long long v = k < 3 * SL ? (j == SL - 1 ? S[k] : (S[k] & 0xFFFFFFFFll)) + (j > 0 ? S[k - 1] >> 32 : 0ll) : 0ll;
+      if (k < 3 * SL) out->limbs[k] = v;
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, v != 0);
+      if (lane == 0) out->mask[k >> 5] = m;
+    }
     if (p.hist)
       for (int k = threadIdx.x; k < PEAT_HIST_BINS; k += TB)
         if (H[k]) atomicAdd(p.hist + seg * PEAT_HIST_BINS + k, (unsigned long long)H[k]);
     __syncthreads();
   }
-  (void)lane;
 }
 
-// RN64 of a normalised limb sum (limbs in [0, 2^32), the top one signed), with
-// the subnormal grid below 2^-1022 and +-inf past the largest double
-__device__ double limbs_rn64(const long long* d) {
-  // magnitude limbs
-  unsigned long long m[SL];
-  const bool neg = d[SL - 1] < 0;
-  // a top limb of 32 bits or more is past 2^2080, far beyond the largest double
-  if (d[SL - 1] >= (1ll << 32) || d[SL - 1] < -(1ll << 32))
-    return neg ? -__longlong_as_double(0x7FF0000000000000ll) : __longlong_as_double(0x7FF0000000000000ll);
-  long long borrow = 0;
-  for (int j = 0; j < SL; j++) {
-    long long v = neg ? -d[j] - borrow : d[j];
-    if (neg) {
-      borrow = v < 0 ? 1 : 0;
-      v += borrow ? (1ll << 32) : 0;
+// RN64 of the carry-save digits d[0..n) (digit j weighs 2^(32 (lo + j) + SLSB);
+// all others are zero), with the subnormal grid below 2^-1022 and +-inf past the
+// largest double.  d has room for two more digits, which take the carry; it
+// is rewritten as the magnitude.
+__device__ double digits_rn64(long long* d, int n, int lo) {
+  auto carry_up = [&](int m) {
+    long long carry = 0;
+    for (int j = 0; j < m; j++) {
+      const long long v = d[j] + carry;
+      carry = v >> 32;
+      d[j] = v & 0xFFFFFFFFll;
     }
-    m[j] = (unsigned long long)v;
+    return carry;
+  };
+  d[n] = d[n + 1] = 0;
+  const bool neg = carry_up(n + 2) < 0;  // (a sum is below 2^64 of its top digit's weight)
+  if (neg) {
+    long long borrow = 0;
+    for (int j = 0; j < n + 2; j++) {
+      long long v = -d[j] - borrow;
+      borrow = v < 0 ? 1 : 0;
+      d[j] = v + (borrow ? (1ll << 32) : 0);
+    }
   }
-  int top = -1;
-  for (int j = SL - 1; j >= 0 && top < 0; j--)
-    if (m[j]) top = j * 32 + 31 - __clz((int)(uint32_t)m[j]);
-  if (top < 0) return 0.0;
-  auto bit = [&](int k) -> unsigned long long { return k < 0 ? 0ull : (m[k >> 5] >> (k & 31)) & 1ull; };
+  int t = n + 1;
+  while (t >= 0 && d[t] == 0) t--;
+  if (t < 0) return 0.0;
+  // the leading four digits as W, whose bit 0 weighs 2^(32 (lo + t - 3) + SLSB)
+  auto dig = [&](int j) -> u128 { return j >= 0 ? (u128)(uint32_t)d[j] : (u128)0; };
+  const u128 W = (dig(t) << 96) | (dig(t - 1) << 64) | (dig(t - 2) << 32) | dig(t - 3);
+  const int b0 = 32 * (lo + t - 3) + SLSB, top = b0 + 127 - __clz((int)(uint32_t)d[t]);
   int low = top - 52;
-  if (low + SLSB < -1074) low = -1074 - SLSB;
-  unsigned long long mant = 0;
-  for (int k = top; k >= low; k--) mant = (mant << 1) | bit(k);
-  const unsigned long long round = bit(low - 1);
-  bool sticky = false;
-  for (int k = low - 2; k >= 0 && !sticky; k--) sticky = bit(k) != 0;
+  if (low < -1074) low = -1074;
+  const int sh = low - b0;  // at least 96 - 52
+  unsigned long long mant = sh < 128 ? (unsigned long long)(W >> sh) : 0ull;
+  const bool round = sh <= 128 && ((W >> (sh - 1)) & 1) != 0;
+  bool sticky = sh > 128 ? W != 0 : (W << (129 - sh)) != 0;
+  for (int j = t - 4; j >= 0 && !sticky; j--) sticky = d[j] != 0;
   if (round && (sticky || (mant & 1ull))) mant++;
-  const double r = ldexp((double)mant, low + SLSB);
+  const double r = ldexp((double)mant, low);  // +inf past the largest double
   return neg ? -r : r;
 }
 
 // RN64 of (hi + lo) 2^sc / g (finite positive): the candidate around the
 // binary64 quotient whose neighbouring midpoints bracket the exact value
 __device__ double rel_value64(const Mag& a, double g) {
+  if (a.lo == 0.0 && a.sc == 0) return __ddiv_rn(a.hi, g);  // one binary64 number over another: correctly rounded
   // at or past (2^54 - 1) 2^970 (the rounding threshold of the largest double): +inf
   {
     uint64_t mg;
@@ -482,7 +780,7 @@ __device__ double rel_value64(const Mag& a, double g) {
 }
 
 __global__ void __launch_bounds__(TB) compare64_finalize(Cmp64Params p) {
-  __shared__ Part64Rec buf[TB];
+  __shared__ Part64Rec buf[TB / 2];
   __shared__ long long S[3 * SL];
   pdl_wait();  // stage 1 complete
   const long long seg = blockIdx.x;
@@ -495,19 +793,63 @@ __global__ void __launch_bounds__(TB) compare64_finalize(Cmp64Params p) {
   r.mu = 0, r.iu = -1;
   for (long long it = f0 + threadIdx.x; it < f1; it += TB) rec_merge(r, p.parts[it].rec);
   block_merge(r, buf);
-  for (int k = threadIdx.x; k < 3 * SL; k += TB) {
-    long long v = 0;
-    for (long long it = f0; it < f1; it++) v += p.parts[it].limbs[k];
-    S[k] = v;
-  }
-  __syncthreads();
+  // the items' digits: only the columns that some item has (a dozen of 408 on
+  // ordinary data), a warp per column; the range of each sum
+  __shared__ unsigned cols[P64_MASK];
+  __shared__ unsigned short list[3 * SL];
+  __shared__ int nlist, lo[3], hi[3];
+  __shared__ long long D[3 * (SL + 2)];
+  __shared__ double sums[3];
+  __shared__ unsigned long long nfin;
   // the mean and variance of |d| from S1 = sum |d| and S2 = sum d^2, both SL
   // digits weighing 2^(32 j + SLSB) (two more after carrying)
   __shared__ MeanVarScratch<SL + 2, SL + 2, -SLSB / 32> mv;
   static_assert(SLSB % 32 == 0, "the S2 shift is a whole number of digits");
-  if (threadIdx.x == 0) carry_to_digits(S + SL, SL, mv.A);
-  if (threadIdx.x == 32) carry_to_digits(S + 2 * SL, SL, mv.B);
-  mean_var_block(mv, r.nfin, SLSB);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = threadIdx.x; k < 3 * SL; k += TB) S[k] = 0;
+  for (int k = threadIdx.x; k < SL + 2; k += TB) mv.A[k] = mv.B[k] = 0u;
+  if (threadIdx.x < P64_MASK) cols[threadIdx.x] = 0u;
+  if (threadIdx.x < 3) lo[threadIdx.x] = SL, hi[threadIdx.x] = -1;
+  if (threadIdx.x == 0) nlist = 0, nfin = r.nfin;
+  __syncthreads();
+  for (long long it = f0 * P64_MASK + threadIdx.x; it < f1 * P64_MASK; it += TB) {
+    const unsigned m = p.parts[it / P64_MASK].mask[it % P64_MASK];
+    if (m) atomicOr(&cols[it % P64_MASK], m);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 3 * SL; k += TB)
+    if ((cols[k >> 5] >> (k & 31)) & 1u) {
+      list[atomicAdd(&nlist, 1)] = (unsigned short)k;
+      atomicMin(&lo[k / SL], k % SL);
+      atomicMax(&hi[k / SL], k % SL);
+    }
+  __syncthreads();
+  for (int x = warp; x < nlist; x += TB / 32) {
+    const int k = list[x];
+    long long v = 0;
+#pragma unroll 8
+    for (long long it = f0 + lane; it < f1; it += 32) v += p.parts[it].limbs[k];
+    v = (long long)wsum_u64((uint64_t)v);
+    if (lane == 0) S[k] = v;
+  }
+  __syncthreads();
+  // the digits of S1 and S2 carried (non-negative: two more take the carry), and
+  // the three sums rounded, a warp each
+  if (lane == 0 && warp < 2) {
+    const int q = warp + 1, n = hi[q] - lo[q] + 1;
+    if (n > 0) {
+      uint32_t* out = warp ? mv.B : mv.A;
+      // (at most SL + 2 digits: the carry of the top ones stays inside)
+      carry_to_digits(S + q * SL + lo[q], n, out + lo[q]);
+    }
+  }
+  if (lane == 0 && warp >= 2 && warp < 5) {
+    const int q = warp - 2, n = hi[q] - lo[q] + 1;
+    long long* d = D + q * (SL + 2);
+    for (int j = 0; j < n; j++) d[j] = S[q * SL + lo[q] + j];
+    sums[q] = n > 0 ? digits_rn64(d, n, lo[q]) : 0.0;
+  }
+  mean_var_block(mv, nfin, SLSB);
   if (threadIdx.x != 0) return;
   peat_stats_t o;
   o.n = (uint64_t)(p.offsets[seg + 1] - p.offsets[seg]);
@@ -521,10 +863,9 @@ __global__ void __launch_bounds__(TB) compare64_finalize(Cmp64Params p) {
   o.argmax_rel = r.ir;
   o.max_ulp = r.iu >= 0 ? r.mu : 0;
   o.argmax_ulp = r.iu;
-  for (int s = 0; s < 3; s++) normalise(S + s * SL, SL);
-  o.sum_signed = limbs_rn64(S);
-  o.sum_abs = limbs_rn64(S + SL);
-  o.sum_sq = limbs_rn64(S + 2 * SL);
+  o.sum_signed = sums[0];
+  o.sum_abs = sums[1];
+  o.sum_sq = sums[2];
   o.rtol_eff = p.rtol;
   o.atol_eff = p.atol;
   o.mean_abs = mv.mean;

@@ -227,7 +227,7 @@ static cudaError_t single_bounds(peat_handle_t h, int dtype, int nctas, int64_t 
 }
 
 // Work items for the 8-bit and binary64 compares: runs of at most `ch`
-// elements within one segment (about four per SM for one tensor), staged
+// elements within one segment (about per_sm per SM for one tensor), staged
 // with the offsets into the handle's workspace, followed by one record of
 // `part_bytes` per item.  Fills the item fields of p (any of the two
 // parameter structs) and returns the device base of the records.
@@ -237,9 +237,9 @@ struct Items {
   void* parts;
 };
 static peat_status_t stage_items(peat_handle_t h, const int64_t* offsets, int64_t nseg, size_t part_bytes,
-                                 cudaStream_t st, Items* out) {
+                                 int per_sm, cudaStream_t st, Items* out) {
   const int64_t n = offsets[nseg];
-  int64_t ch = (n + 4 * (int64_t)h->nsm - 1) / (4 * (int64_t)h->nsm);
+  int64_t ch = (n + per_sm * (int64_t)h->nsm - 1) / (per_sm * (int64_t)h->nsm);
   ch = std::min<int64_t>(std::max<int64_t>((ch + 15) / 16 * 16, 4096), (int64_t)1 << 22);
   int64_t nitems = 0;
   for (int64_t s = 0; s < nseg; s++) nitems += (offsets[s + 1] - offsets[s] + ch - 1) / ch;
@@ -346,7 +346,7 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
                                    int64_t nseg, int dtype, float rtol, float atol, peat_stats_t* stats,
                                    uint64_t* hist, cudaStream_t st) {
   Items it;
-  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part8), st, &it);
+  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part8), 4, st, &it);
   if (ps != PEAT_OK) return ps;
   cudaError_t e;
   if (hist) {
@@ -394,7 +394,7 @@ static peat_status_t compare64_impl(peat_handle_t h, const void* g, const void* 
                                     int64_t nseg, float rtol, float atol, peat_stats_t* stats, uint64_t* hist,
                                     cudaStream_t st) {
   Items it;
-  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part64), st, &it);
+  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part64), 2, st, &it);
   if (ps != PEAT_OK) return ps;
   cudaError_t e;
   if (hist) {

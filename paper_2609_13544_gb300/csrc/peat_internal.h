@@ -259,8 +259,8 @@ struct Cmp8Params {
 };
 cudaError_t launch_compare8(int dtype, const Cmp8Params& p, int nctas, cudaStream_t s);
 
-// binary64: one item's maxima and counts, and its three sums as normalised
-// 32-bit digits from 2^-2272 (the top limb signed)
+// binary64: one item's maxima and counts, and its three sums as carry-save
+// digits of 32 bits from 2^-2272 (below 2^34 in magnitude, the top one not)
 struct Part64Rec {
   unsigned long long cnt[PEAT_NCLASS], nfin;
   double ahi, alo;  // max |d| = (ahi + alo) 2^asc at ia
@@ -275,8 +275,10 @@ struct Part64Rec {
   long long iu;
 };
 constexpr int P64_LIMBS = 136;
+constexpr int P64_MASK = (3 * P64_LIMBS + 31) / 32;
 struct Part64 {
   Part64Rec rec;
+  unsigned int mask[P64_MASK + 1];  // which limbs are not zero
   long long limbs[3 * P64_LIMBS];  // sum d, sum |d|, sum d^2
 };
 struct Cmp64Params {
