@@ -226,7 +226,7 @@ static cudaError_t single_bounds(peat_handle_t h, int dtype, int nctas, int64_t 
   return cudaSuccess;
 }
 
-// Work items for the 8-bit and binary64 compares: runs of at most `ch`
+// Work items for the 8-bit and binary64 compares: runs of at most `most`
 // elements within one segment (about per_sm per SM for one tensor), staged
 // with the offsets into the handle's workspace, followed by one record of
 // `part_bytes` per item.  Fills the item fields of p (any of the two
@@ -237,10 +237,10 @@ struct Items {
   void* parts;
 };
 static peat_status_t stage_items(peat_handle_t h, const int64_t* offsets, int64_t nseg, size_t part_bytes,
-                                 int per_sm, cudaStream_t st, Items* out) {
+                                 int per_sm, int64_t most, cudaStream_t st, Items* out) {
   const int64_t n = offsets[nseg];
   int64_t ch = (n + per_sm * (int64_t)h->nsm - 1) / (per_sm * (int64_t)h->nsm);
-  ch = std::min<int64_t>(std::max<int64_t>((ch + 15) / 16 * 16, 4096), (int64_t)1 << 22);
+  ch = std::min<int64_t>(std::max<int64_t>((ch + 15) / 16 * 16, 4096), most);
   int64_t nitems = 0;
   for (int64_t s = 0; s < nseg; s++) nitems += (offsets[s + 1] - offsets[s] + ch - 1) / ch;
   // staging: offsets (nseg + 1), item_b, item_e, item_seg (nitems each), seg_first (nseg + 1)
@@ -346,7 +346,7 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
                                    int64_t nseg, int dtype, float rtol, float atol, peat_stats_t* stats,
                                    uint64_t* hist, cudaStream_t st) {
   Items it;
-  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part8), 4, st, &it);
+  peat_status_t ps = stage_items(h, offsets, nseg, 2 * sizeof(peat::Part8), 1, (int64_t)1 << 20, st, &it);
   if (ps != PEAT_OK) return ps;
   cudaError_t e;
   if (hist) {
@@ -383,7 +383,7 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
   p.parts = static_cast<peat::Part8*>(it.parts);
   p.stats = stats;
   p.hist = reinterpret_cast<unsigned long long*>(hist);
-  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>(it.nitems, 2 * (int64_t)h->nsm));
+  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>(it.nitems, (int64_t)h->nsm));
   e = peat::launch_compare8(dtype, p, nctas, st);
   if (e != cudaSuccess) return cuda_fail(h, e, "8-bit compare launch");
   return PEAT_OK;
@@ -394,7 +394,7 @@ static peat_status_t compare64_impl(peat_handle_t h, const void* g, const void* 
                                     int64_t nseg, float rtol, float atol, peat_stats_t* stats, uint64_t* hist,
                                     cudaStream_t st) {
   Items it;
-  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part64), 2, st, &it);
+  peat_status_t ps = stage_items(h, offsets, nseg, sizeof(peat::Part64), 2, (int64_t)1 << 22, st, &it);
   if (ps != PEAT_OK) return ps;
   cudaError_t e;
   if (hist) {
@@ -663,7 +663,7 @@ peat_status_t peat_signature_create(peat_handle_t* out, const peat_config_t* cfg
     delete h;
     return PEAT_ERR_CUDA;
   }
-  if (peat::compare_prepare() != cudaSuccess) {
+  if (peat::compare_prepare() != cudaSuccess || peat::compare8_prepare() != cudaSuccess) {
     cudaGetLastError();
     g_create_error = "could not configure the compare kernels";
     delete h;

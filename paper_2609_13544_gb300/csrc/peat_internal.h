@@ -253,10 +253,11 @@ struct Cmp8Params {
   // floor(rtol |g| 2^S + atol 2^S) (2^40 when it exceeds every possible difference)
   unsigned long long amax[128];
   int vec;                   // both bases 16-byte aligned
-  Part8* parts;              // nitems
+  Part8* parts;              // 2 nitems: the table's totals, and those of the pairs of opposite signs
   peat_stats_t* stats;       // nseg
   unsigned long long* hist;  // nseg x 128, zero before the launch; NULL: none
 };
+cudaError_t compare8_prepare();  // once per device, before the first launch
 cudaError_t launch_compare8(int dtype, const Cmp8Params& p, int nctas, cudaStream_t s);
 
 // binary64: one item's maxima and counts, and its three sums as carry-save
