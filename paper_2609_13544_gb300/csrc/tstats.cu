@@ -9,7 +9,8 @@
 // Stage 1 (tstats_stage1): CTA b owns the contiguous element range
 // [bounds[b], bounds[b+1]) and walks the segments it meets.  A finite element
 // x = +-m 2^(e-150) (m < 2^24, e the biased float32 exponent, 1 for
-// subnormals) inside its warp's window e - Lb in [0, WSPAN] adds m << (e - Lb)
+// subnormals) inside its warp's window e - Lb in [0, WSPAN] (float32 elements;
+// the 16-bit types have their own below) adds m << (e - Lb)
 // to one of two 128-bit integers (by sign) and m^2 << 2(e - Lb) to a third;
 // the window follows the data (placed 6 binades above the largest exponent a
 // warp tile holds, moved when a tile leaves it), elements outside it go to
@@ -37,10 +38,10 @@ constexpr int LB_UNSET = -1000;
 // with m below 2^(MB + 1) (the implicit bit for a normal value) and ee the
 // exponent field (1 for subnormals); EINF marks infinities and NaNs.  A
 // warp's window covers ee - Lb in [0, WSPAN].  Terms: t = m << (ee - Lb) and
-// t^2.  16-bit types: t < 2^28, t^2 < 2^56 (one 32 x 32 -> 64 multiply), the
-// signed sum of t in 64 bits and of t^2 in 128; float32: t < 2^54, t^2 <
-// 2^108, both sums in 128 bits (by sign for t).  FLUSH in-window elements per
-// lane at most between two flushes of the sums into digits.
+// t^2: t < 2^54, t^2 < 2^108, both sums in 128 bits (by sign for t).  FLUSH
+// in-window elements per lane at most between two flushes of the sums into
+// digits.  (The window is the float32 kernel's; the 16-bit types have ways of
+// their own below.)
 template <int DT>
 struct TS;
 template <>
@@ -50,8 +51,7 @@ struct TS<PEAT_F32> {
 };
 template <>
 struct TS<PEAT_F16> {
-  static constexpr int BYTES = 2, VEC = 8, BITS = 16, MB = 10, BM = 25, WSPAN = 16;
-  static constexpr uint32_t EMASK = 0x1Fu, EINF = 0x1Fu, FLUSH = 1u << 20;
+  static constexpr int BYTES = 2, BITS = 16, BM = 25;
 };
 template <>
 struct TS<PEAT_BF16> {
@@ -110,12 +110,8 @@ __device__ __forceinline__ void lim_add(long long* lim, int j, int64_t v) {
 template <int DT>
 struct TsLane {
   unsigned __int128 s1p = 0, s1n = 0;  // float32: sum of t by sign
-  int64_t s1 = 0;                      // 16-bit types: signed sum of t
+  int64_t s1 = 0;                      // fp16: signed sum of t
   unsigned __int128 s2 = 0;            // sum of t^2
-  // 16-bit types, within one round of at most 32 elements per lane (terms
-  // below 2^28 and 2^56): the sums as 64-bit multiply-adds, folded into s1
-  // and s2 after every round
-  uint64_t r1p = 0, r1n = 0, r2 = 0;
   uint32_t nnan = 0, ninf = 0, since = 0, slow = 0;
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0;  // raw-order keys
 };
@@ -129,16 +125,6 @@ __device__ __forceinline__ int64_t wsum_i64(int64_t v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
   return v;
-}
-
-// a round's 64-bit partial sums into the lane's totals (16-bit types)
-template <int DT>
-__device__ __forceinline__ void ts_fold(TsLane<DT>& L) {
-  if constexpr (TS<DT>::BYTES == 2) {
-    L.s1 += (int64_t)L.r1p - (int64_t)L.r1n;
-    L.s2 += L.r2;
-    L.r1p = L.r1n = L.r2 = 0;
-  }
 }
 
 // The warp's integers into the CTA's digits (lim: S1, lim + NLIMB: S2), by
@@ -203,18 +189,10 @@ __device__ __forceinline__ void ts_elem(TsLane<DT>& L, uint32_t r, int lb, long 
   const uint32_t m = mant | (e ? (1u << T::MB) : 0u);
   const int ee = e ? (int)e : 1, s = ee - lb;
   if ((unsigned)s <= (unsigned)T::WSPAN) {
-    if constexpr (T::BYTES == 4) {
-      const uint64_t t = (uint64_t)m << s;  // below 2^54
-      if (neg) L.s1n += t;
-      else L.s1p += t;
-      L.s2 += ((unsigned __int128)__umul64hi(t, t) << 64) | (t * t);
-    } else {
-      // multiply-adds (the FMA pipe) rather than shifts and carries (ALU)
-      const uint32_t t = m << s, ng = r >> 15;  // t below 2^28
-      L.r1n += (uint64_t)t * ng;
-      L.r1p += (uint64_t)t * (1u - ng);
-      L.r2 += (uint64_t)t * t;  // below 2^56
-    }
+    const uint64_t t = (uint64_t)m << s;  // below 2^54
+    if (neg) L.s1n += t;
+    else L.s1p += t;
+    L.s2 += ((unsigned __int128)__umul64hi(t, t) << 64) | (t * t);
   } else if (m != 0) {
     ts_slow<DT>(m, ee, neg, lim);
     L.slow++;
@@ -281,7 +259,6 @@ __device__ void ts_piece(const TsParams& p, int64_t a, int64_t b, long long* lim
         L.since += VEC;
       }
     }
-    ts_fold<DT>(L);
   }
   // the elements outside the vector grid: [a, a0) and [a0 + nv VEC, b), in
   // whole-CTA rounds as well
@@ -305,9 +282,153 @@ __device__ void ts_piece(const TsParams& p, int64_t a, int64_t b, long long* lim
       ts_elem<DT>(L, r, lb, lim);
       L.since++;
     }
-    ts_fold<DT>(L);
   }
   (void)lane;
+}
+
+// ---- fp16 elements ----
+// Every finite binary16 value is an integer below 2^40 in units of 2^-24:
+// x = (V1 2^20 + V2) 2^-24, where V1 is x rounded to a multiple of 2^-4 and V2
+// the exact remainder, both read from the bits of float32 sums (x + 1.5 2^19
+// has the unit 2^-4, the remainder + 1.5 2^-1 the unit 2^-24).  So no window
+// follows the data: sum x adds V1 and V2 as 32-bit integers, sum x^2 the
+// products V1 V1, V1 V2 and V2 V2 in 64 bits.  A warp's vector whose values all
+// lie below 1/4 (most of a checkpoint's) needs V2 alone.  The extremes come
+// from packed minima and maxima; NaN and infinities are found by them, counted,
+// and zeroed.
+//
+// What bounds it: memory latency and the ends of the pieces on such tensors
+// (4.2 TB/s), the multiply-adds on the others.  Measured: 355 M checkpoint values
+// in 292 segments 836 us with the integer window per element (35
+// instructions), 171 us now; 67 M values N(0, 4) in one tensor 133 -> 67 us.
+// Loading a round ahead with half the vectors per round: 195 us, not kept.
+constexpr float F16_M1 = 0x1.8p+19f, F16_M2 = 0x1.8p-1f;
+struct F16Sum {
+  uint32_t a1 = 0, a2 = 0;  // bits of x + M1 and of the remainder + M2, since the last fold
+  uint32_t n1 = 0, n2 = 0;  // how many of each
+  int64_t s = 0;            // sum x in units of 2^-24, folded
+  uint64_t q11 = 0, q22 = 0;
+  int64_t q12 = 0;
+  uint32_t since = 0;       // elements since the last flush
+};
+__device__ __forceinline__ void f16_small(F16Sum& L, float x) {
+  const uint32_t b = __float_as_uint(__fadd_rn(x, F16_M2));
+  L.a2 += b;
+  const int v = (int)(b - __float_as_uint(F16_M2));
+  L.q22 += (uint64_t)((int64_t)v * v);
+}
+__device__ __forceinline__ void f16_any(F16Sum& L, float x) {
+  const float x1 = __fadd_rn(x, F16_M1);
+  const float x2 = __fadd_rn(__fsub_rn(x, __fsub_rn(x1, F16_M1)), F16_M2);
+  L.a1 += __float_as_uint(x1);
+  L.a2 += __float_as_uint(x2);
+  const int v1 = (int)(__float_as_uint(x1) - __float_as_uint(F16_M1)), v2 = (int)(__float_as_uint(x2) - __float_as_uint(F16_M2));
+  L.q11 += (uint64_t)((int64_t)v1 * v1);
+  L.q12 += (int64_t)v1 * v2;
+  L.q22 += (uint64_t)((int64_t)v2 * v2);
+}
+// the 32-bit sums into 64 bits (at most 2^9 elements since the last time: below 2^31)
+__device__ __forceinline__ void f16_fold(F16Sum& L) {
+  L.s += ((int64_t)(int32_t)(L.a1 - L.n1 * __float_as_uint(F16_M1)) << 20) + (int32_t)(L.a2 - L.n2 * __float_as_uint(F16_M2));
+  L.a1 = L.a2 = L.n1 = L.n2 = 0;
+}
+// V1 < 2^20, V2 < 2^22 in size: at most 2^18 elements between flushes keep the products below 2^62
+__device__ __forceinline__ void f16_flush(F16Sum& L, TsLane<PEAT_F16>& T, long long* lim) {
+  f16_fold(L);
+  T.s1 = L.s;
+  T.s2 = ((unsigned __int128)L.q11 << 40) + (unsigned __int128)((__int128)L.q12 << 21) + L.q22;
+  ts_flush<PEAT_F16>(T, 1, lim);  // units of 2^(1 - BM) = 2^-24
+  L.s = L.q12 = 0;
+  L.q11 = L.q22 = 0;
+  L.since = 0;
+}
+__device__ __forceinline__ __half2 as_h2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+
+// one element: counts, extremes (packed in the low half) and sums
+__device__ __forceinline__ void f16_one(F16Sum& L, TsLane<PEAT_F16>& T, uint32_t r) {
+  if ((r & 0x7FFFu) >= 0x7C00u) {
+    if (r & 0x3FFu) T.nnan++;
+    else T.ninf++;
+    return;
+  }
+  const uint32_t k = raw_key<PEAT_F16>(r);
+  T.kmin = min(T.kmin, k);
+  T.kmax = max(T.kmax, k);
+  L.n1++;
+  L.n2++;
+  f16_any(L, __half2float(__ushort_as_half((unsigned short)r)));
+}
+
+// one piece [a, b) inside this CTA's range
+__device__ void ts_piece_f16(const TsParams& p, int64_t a, int64_t b, long long* lim, TsLane<PEAT_F16>& T) {
+  constexpr int VEC = 8, U = 4;  // vectors per thread in a round, loaded before any is used
+  int64_t a0 = b, nv = 0;
+  if (p.p0 >= 0 && p.p0 < p.n_total) {
+    a0 = a <= p.p0 ? p.p0 : p.p0 + ((a - p.p0 + VEC - 1) / VEC) * VEC;
+    if (a0 < b) nv = (b - a0) / VEC;
+    else a0 = b;
+  }
+  F16Sum L;
+  __half2 mx = as_h2(0xFC00FC00u), mn = as_h2(0x7C007C00u);  // -inf, +inf: no element yet
+  const __half2 quarter = as_h2(0x34003400u), nquarter = as_h2(0xB400B400u);
+  const char* base = reinterpret_cast<const char*>(p.x) + a0 * 2 + (int64_t)threadIdx.x * 16;
+  for (int64_t k0 = 0; k0 < nv; k0 += (int64_t)U * TB, base += U * TB * 16) {
+    uint4 v[U];
+    const int left = (int)min((int64_t)U * TB, nv - k0) - (int)threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      v[u] = u * TB < left ? ts_vec(base, (int64_t)u * TB * 16) : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    if (__any_sync(0xFFFFFFFFu, L.since > (1u << 18) - U * VEC)) f16_flush(L, T, lim);
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const bool on = u * TB < left;
+      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+      const __half2 hx = __hmax2_nan(__hmax2_nan(as_h2(w[0]), as_h2(w[1])), __hmax2_nan(as_h2(w[2]), as_h2(w[3])));
+      const __half2 hn = __hmin2_nan(__hmin2_nan(as_h2(w[0]), as_h2(w[1])), __hmin2_nan(as_h2(w[2]), as_h2(w[3])));
+      // (a lane past the end holds NaN: it joins none of the two vector paths)
+      if (__all_sync(0xFFFFFFFFu, __hblt2(hx, quarter) && __hbgt2(hn, nquarter))) {
+        mx = __hmax2(mx, hx);
+        mn = __hmin2(mn, hn);
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          f16_small(L, __low2float(as_h2(w[i])));
+          f16_small(L, __high2float(as_h2(w[i])));
+        }
+        L.n2 += VEC;
+      } else if (__all_sync(0xFFFFFFFFu, __hblt2(hx, as_h2(0x7C007C00u)) && __hbgt2(hn, as_h2(0xFC00FC00u)))) {
+        mx = __hmax2(mx, hx);
+        mn = __hmin2(mn, hn);
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          f16_any(L, __low2float(as_h2(w[i])));
+          f16_any(L, __high2float(as_h2(w[i])));
+        }
+        L.n1 += VEC;
+        L.n2 += VEC;
+      } else if (on) {  // some lane holds NaN or an infinity, or is past the end
+#pragma unroll 1
+        for (int j = 0; j < VEC; j++) f16_one(L, T, ((j & 4 ? (j & 2 ? w[3] : w[2]) : (j & 2 ? w[1] : w[0])) >> (16 * (j & 1))) & 0xFFFFu);
+      }
+    }
+    L.since += U * VEC;
+    f16_fold(L);
+  }
+  // the elements outside the vector grid: [a, a0) and [a0 + nv VEC, b)
+  const int64_t h = a0 - a, t0 = a0 + nv * VEC, ns = h + (b - t0);
+  for (int64_t i0 = 0; i0 < ns; i0 += TB) {
+    if (__any_sync(0xFFFFFFFFu, L.since >= (1u << 18))) f16_flush(L, T, lim);
+    const int64_t i = i0 + threadIdx.x;
+    if (i < ns) f16_one(L, T, ts_load<PEAT_F16>(p.x, i < h ? a + i : t0 + (i - h)));
+    L.since++;
+    f16_fold(L);
+  }
+  f16_flush(L, T, lim);
+  // the packed extremes into the lane's keys
+  const uint32_t bx = *reinterpret_cast<const uint32_t*>(&mx), bn = *reinterpret_cast<const uint32_t*>(&mn);
+  if (__hbgt2(mx, as_h2(0xFC00FC00u))) {
+    T.kmax = max(T.kmax, max(raw_key<PEAT_F16>(bx & 0xFFFFu), raw_key<PEAT_F16>(bx >> 16)));
+    T.kmin = min(T.kmin, min(raw_key<PEAT_F16>(bn & 0xFFFFu), raw_key<PEAT_F16>(bn >> 16)));
+  }
 }
 
 template <int DT>
@@ -338,8 +459,12 @@ __global__ void __launch_bounds__(TB) tstats_stage1(TsParams p) {
     }
     __syncthreads();
     TsLane<DT> L;
-    ts_piece<DT>(p, a, b, lim, lb, L);
-    ts_flush<DT>(L, lb, lim);
+    if constexpr (DT == PEAT_F16) {
+      ts_piece_f16(p, a, b, lim, L);
+    } else {
+      ts_piece<DT>(p, a, b, lim, lb, L);
+      ts_flush<DT>(L, lb, lim);
+    }
     // finite = the piece's elements less the NaN and infinite ones
     const uint32_t nn = __reduce_add_sync(0xFFFFFFFFu, L.nnan), ni = __reduce_add_sync(0xFFFFFFFFu, L.ninf);
     // the lanes' extremes as float32 order keys (a lane with no finite element keeps neutral keys)
@@ -893,10 +1018,9 @@ cudaError_t hist_prepare() {
 
 // Stage 1 by element type: the bit-pattern histogram for bf16 (a window of 32
 // of its 254 binades holds nearly every tensor's bulk); the per-thread integer
-// window for float32 and fp16 (fp16 has only 30 binades, and the histogram's
-// 8-binade window leaves a wide distribution largely to the exact path:
-// Laplace-distributed fp16 checkpoint values took 11.9 ms for 355 M elements,
-// the register window of 16 binades takes them all but the tiniest)
+// window for float32; the fixed-point sums for fp16 (a histogram's 8-binade
+// window left a wide distribution largely to the exact path: 355 M
+// Laplace-distributed checkpoint values took 11.9 ms)
 template <int DT>
 cudaError_t launch_t(const TsParams& p, cudaStream_t s) {
   if constexpr (DT != PEAT_BF16) {
