@@ -847,7 +847,8 @@ peat_status_t peat_isclose_grid(peat_handle_t h, const void* golden, const void*
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemsetAsync(counts)");
   if (n == 0) return PEAT_OK;
   const int64_t want = (n + 4095) / 4096;
-  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->nsm * 8, want));
+  // one wave of the kernel's resident CTAs (64 registers a thread), so that its tables are made once per SM and CTA
+  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->nsm * (dtype == PEAT_F64 ? 8 : 4), want));
   // per-CTA counts are 32-bit
   if (n / nctas >= ((int64_t)1 << 31)) return fail(h, PEAT_ERR_UNSUPPORTED, "more than 2^31 elements per CTA");
   e = dtype == PEAT_F64 ? peat::launch_isclose64(p, nctas, st) : peat::launch_isclose(dtype, p, nctas, st);
