@@ -663,7 +663,8 @@ peat_status_t peat_signature_create(peat_handle_t* out, const peat_config_t* cfg
     delete h;
     return PEAT_ERR_CUDA;
   }
-  if (peat::compare_prepare() != cudaSuccess || peat::compare8_prepare() != cudaSuccess) {
+  if (peat::compare_prepare() != cudaSuccess || peat::compare8_prepare() != cudaSuccess ||
+      peat::topk_prepare() != cudaSuccess) {
     cudaGetLastError();
     g_create_error = "could not configure the compare kernels";
     delete h;
@@ -781,6 +782,7 @@ peat_status_t peat_topk_mean(peat_handle_t h, const void* golden, const void* ca
   // streaming passes: one wave of resident CTAs, about one CTA per 1K elements
   const int64_t want = (n + 1023) / 1024;
   const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>(peat::topk_max_ctas(h->nsm), want));
+  if (p.nvec * vec >= peat::TK_TABLE_MIN) p.tabled = h->nsm;
   // per-thread integer sums in the sum pass stay below 2^64
   if (n / ((int64_t)nctas * 256) >= ((int64_t)1 << 24) - 16)
     return fail(h, PEAT_ERR_UNSUPPORTED, "n is too large for one call (more than 2^24 elements per thread)");

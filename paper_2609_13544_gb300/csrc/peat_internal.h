@@ -147,6 +147,10 @@ cudaError_t launch_bounds_on_device(int dtype, int64_t* offsets, int64_t* bounds
 // the window miss, an exact pass over key >> 21 replaces the sample.
 constexpr int TK_NB0 = 1024, TK_NB1 = 2048, TK_NB2 = 1024, TK_WIN = 3;
 constexpr int64_t TK_SAMPLE = 1 << 18;  // pairs in the sample
+// pairs from which the table pass is offered: at 2^20 the call takes 44 us
+// with it and 48 without; below, the launches are all there is (41 us at 1e5
+// pairs and at 5e3)
+constexpr int64_t TK_TABLE_MIN = 1 << 20;
 constexpr unsigned TK_LCAP = 65536;     // listed pairs whose |d| is not a float32 value
 constexpr int TK_NBL = 65536;           // bins of each 16-bit digit of the order key of a rounding error
 
@@ -165,6 +169,9 @@ struct TopkState {
   unsigned int nlist, nlist2;   // list entries from the last pass and the optional extra one
   unsigned int lowor, inexact;  // over the window pairs of pass 1: OR of the keys' low 10 bits, any |d| not a float32
   unsigned int skip2;           // pass 1 resolved the last digit itself (passes 2 and 3 return at once)
+  unsigned int table;           // pass 1 counts in a table: 1 one cell per value, 2 one per value and lane
+  unsigned int Tlo;             // first digit of the table
+  unsigned int low[TK_NB0];     // of the sample, per digit: OR of the keys' low bits, bit 31: some |d| not a float32
   long long limbs[NLIMB];       // exact sum of the |d| resolved above the prefix
   // only when T's bucket has more than TK_LCAP pairs whose |d| is not a
   // float32 value: a radix select over the order key of their rounding
@@ -184,12 +191,14 @@ struct TopkParams {
   int64_t p0;     // first element of the 16-byte vector grid; -1: none
   int64_t nvec;   // vectors on the grid
   uint64_t num, den;
+  int tabled;     // CTAs of the table pass; 0: not offered
   TopkState* st;
   TopkListEntry* list;
   peat_topk_t* out;
 };
 // CTAs of the streaming passes that fit on the device at once
 int topk_max_ctas(int nsm);
+cudaError_t topk_prepare();
 cudaError_t launch_topk(int dtype, const TopkParams& p, int nctas, cudaStream_t s);
 
 // ---- context statistics (tstats.cu) ----

@@ -13,7 +13,8 @@
 //           top fraction ends; the window [Plo, Phi] is that digit +- 1;
 //   pass 1  every pair: those with key >> 21 above the window counted and
 //           summed, those inside counted by key >> 10; the last CTA checks
-//           that the window holds the k-th largest and resolves P1 = T >> 10;
+//           that the window holds the k-th largest and resolves P1 = T >> 10
+//           (where the sample's keys are short, all in one shared table);
 //   (pass 0 and pass 1 again on the exact digit, only if the window missed)
 //   pass 2  every pair: digit histogram of bits 9..0 for key >> 10 = P1, the
 //           exact sum of the window's pairs with key >> 10 > P1, and a list
@@ -36,6 +37,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "exact.cuh"
 #include "peat_internal.h"
@@ -46,6 +48,14 @@ namespace {
 constexpr int TB = 256;                    // threads per CTA
 constexpr unsigned KEY_OVF = 0x7F800000u;  // keys from here up: c - g overflowed float32
 constexpr int NO_FAST = 1000;              // binade floor that disables the integer path
+
+// the table pass (below): one CTA of TT threads per SM, a shared table of
+// TAB_DIGITS digits of key >> 21, 2048 cells each, behind 32 cells for the
+// pairs below the window
+constexpr int TT = 1024, TAB_DIGITS = 24, TAB_CELLS = TAB_DIGITS * TK_NB1;
+constexpr size_t TAB_SMEM = sizeof(uint32_t) * (32 + TAB_CELLS);
+constexpr uint32_t COPY_MASK = 0x7FFFu;  // low key bits that are zero when every lane has its own copy of a cell
+static_assert(TAB_CELLS % TT == 0 && TK_WIN <= TAB_DIGITS && (TK_WIN * TK_NB1) % TT == 0, "table layout");
 
 template <int DT>
 struct TK;
@@ -138,6 +148,15 @@ __device__ __forceinline__ void tk_exact(float gf, float cf, float& hi, float& l
   lo = s < 0.0f ? -t : t;
 }
 
+// 0 if and only if c - g is a float32 value: s = RN(c - g) is exact exactly
+// when s - c and s + g both give the other operand back (the one taken with
+// the larger operand is exact and tells; when s is exact both do).  NaN for a
+// NaN or an infinity.
+__device__ __forceinline__ float inexactness(float gf, float cf) {
+  const float s = __fsub_rn(cf, gf);
+  return fabsf(__fadd_rn(__fsub_rn(s, cf), gf)) + fabsf(__fsub_rn(__fadd_rn(s, gf), cf));
+}
+
 // the value a key stands for: v 2^sc
 __device__ __forceinline__ float key_value(unsigned key, int& sc) {
   sc = key >= KEY_OVF ? 1 : 0;
@@ -216,7 +235,7 @@ __device__ __forceinline__ void tk_visit(const TopkParams& p, F&& f) {
 // pass needs) reaches proc(G, C), which makes the exact decision.  Pairs that
 // pass are queued in the warp's ring and handed to proc 32 at a time, so the
 // rarely taken work runs on full warps.
-template <int DT, class Pred, class Proc>
+template <int DT, int NT = TB, class Pred, class Proc>
 __device__ __forceinline__ void tk_filtered(const TopkParams& p, typename QT<DT>::T* ring, Pred&& isint,
                                             Proc&& proc) {
   constexpr int VEC = TK<DT>::VEC, B = TK<DT>::BYTES, CAP = ring_cap<DT>();
@@ -250,8 +269,8 @@ __device__ __forceinline__ void tk_filtered(const TopkParams& p, typename QT<DT>
     }
     __syncwarp();
   };
-  const int64_t stride = (int64_t)gridDim.x * TB;
-  const int64_t gt = (int64_t)blockIdx.x * TB + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  const int64_t gt = (int64_t)blockIdx.x * NT + threadIdx.x;
   // rounds of two vectors; every lane of the warp takes every round
   for (int64_t v = gt; __any_sync(0xFFFFFFFFu, v < p.nvec); v += 2 * stride) {
     const bool ok0 = v < p.nvec, ok1 = v + stride < p.nvec;
@@ -355,14 +374,15 @@ struct ExactAcc {
 
 // The CTA's shared histogram and digits into the global state; true in the
 // last CTA of the grid to get here (which then sees every CTA's totals).
+template <int NT = TB>
 __device__ __forceinline__ bool pass_end(const uint32_t* h, int nb, unsigned long long* gh, const long long* lim,
                                          TopkState* st, int pass, unsigned* last_s) {
   __syncthreads();
   if (h)
-    for (int b = threadIdx.x; b < nb; b += TB)
+    for (int b = threadIdx.x; b < nb; b += NT)
       if (h[b]) atomicAdd(&gh[b], (unsigned long long)h[b]);
   if (lim)
-    for (int j = threadIdx.x; j < NLIMB; j += TB)
+    for (int j = threadIdx.x; j < NLIMB; j += NT)
       if (lim[j]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->limbs[j]), (unsigned long long)lim[j]);
   __threadfence();
   __syncthreads();
@@ -386,13 +406,13 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long x) {
   return t;
 }
 
-// One CTA: the digit d of a histogram of TB PER bins with count(bins above
+// One CTA of NT threads: the digit d of a histogram of NT PER bins with count(bins above
 // d) < krem <= count(bins at or above d); krem becomes krem - count(bins
 // above d); the histogram's total is returned.  Thread t owns bins
 // [t PER, t PER + PER); every loop is unrolled so the loads go out together.
-template <int PER>
+template <int PER, int NT = TB>
 __device__ unsigned long long select_digit(const unsigned long long* gh, unsigned long long& krem, unsigned& digit) {
-  __shared__ unsigned long long wsum[TB / 32];
+  __shared__ unsigned long long wsum[NT / 32];
   __shared__ unsigned long long sk;
   __shared__ unsigned sd;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -416,7 +436,7 @@ __device__ unsigned long long select_digit(const unsigned long long* gh, unsigne
   __syncthreads();
   unsigned long long above = suf - mine, total = 0;
 #pragma unroll
-  for (int w = 0; w < TB / 32; w++) {
+  for (int w = 0; w < NT / 32; w++) {
     total += wsum[w];
     if (w > warp) above += wsum[w];
   }
@@ -455,10 +475,11 @@ template <int DT>
 __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
   constexpr int VEC = TK<DT>::VEC, B = TK<DT>::BYTES;
   __shared__ uint32_t h[TK_NB0];
+  __shared__ uint32_t low[TK_NB0];  // per digit: the OR of the keys' low 15 bits; bit 31: some |d| is not a float32 value
   __shared__ unsigned last_s;
   pdl_trigger();
   TopkState* st = p.st;
-  for (int b = threadIdx.x; b < TK_NB0; b += TB) h[b] = 0;
+  for (int b = threadIdx.x; b < TK_NB0; b += TB) h[b] = low[b] = 0;
   __syncthreads();
   RunCount rc;
   auto count = [&](uint32_t G, uint32_t C) {
@@ -466,6 +487,9 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
     if (key >= KEY_OVF) {
       if (!tk_finite<DT>(G, C)) return;
       key = tk_key(tk_f32<DT>(G), tk_f32<DT>(C));
+    } else if (p.tabled) {
+      const uint32_t l = (key & COPY_MASK) | (inexactness(tk_f32<DT>(G), tk_f32<DT>(C)) == 0.0f ? 0u : 0x80000000u);
+      if (l & ~low[key >> 21]) atomicOr(&low[key >> 21], l);
     }
     rc.add(h, key >> 21);
   };
@@ -487,6 +511,9 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
     for (int64_t j = w * 32 + lane; j < ns; j += nw * 32) count(tk_load<DT>(p.g, j * step), tk_load<DT>(p.c, j * step));
   }
   rc.flush(h);
+  __syncthreads();
+  for (int b = threadIdx.x; b < TK_NB0; b += TB)
+    if (low[b]) atomicOr(&st->low[b], low[b]);
   if (!pass_end(h, TK_NB0, st->hist0, nullptr, st, 0, &last_s)) return;
   // the sample's own count of finite pairs is the histogram's total
   unsigned d = 0;
@@ -497,11 +524,95 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
     select_digit<TK_NB0 / TB>(st->hist0, kr, d);
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < TK_NB0; b += TB) st->hist0[b] = 0;
+  const unsigned Plo = d > 0 ? d - 1 : 0, Phi = min(d + 1, (unsigned)TK_NB0 - 1);
+  uint32_t mode = 0;
+  unsigned Tlo = Plo;
+  if (tot > 0) {  // the same in every thread
+    // The table starts at the window.  When the window starts at zero (most
+    // pairs equal) the few that differ lie far above it: the table then ends
+    // at the sample's largest digit, all but one pair in 4096, and only zeros
+    // may lie below it.
+    const unsigned long long few = tot >> 12;
+    if (Plo == 0) {
+      unsigned long long r = few + 1;
+      unsigned most = 0;
+      select_digit<TK_NB0 / TB>(st->hist0, r, most);
+      Tlo = max(Phi + 1, most > (unsigned)TAB_DIGITS - 1 ? most - (TAB_DIGITS - 1) : 0u);
+      __syncthreads();
+    }
+    // the table pass takes the call when the sample's pairs in the table have
+    // short keys and exact differences and (but for one in 2048, which it does
+    // pair by pair) the others lie where they share a cell
+    uint32_t l = 0;
+    unsigned long long out = 0;
+    for (unsigned b = threadIdx.x; b < (unsigned)TK_NB0; b += TB) {
+      if (b >= Tlo) l |= __ldcg(&st->low[b]);
+      if (b >= Tlo + TAB_DIGITS || (Plo == 0 && b > 0 && b < Tlo)) out += __ldcg(&st->hist0[b]);
+    }
+    out = block_sum(out);
+    const bool any15 = __syncthreads_or((int)(l & (0x80000000u | COPY_MASK)));
+    const bool any10 = __syncthreads_or((int)(l & 0x800003FFu));
+    mode = !p.tabled || any10 || out > 2 * few ? 0u : any15 ? 1u : 2u;
+  }
+  for (int b = threadIdx.x; b < TK_NB0; b += TB) st->hist0[b] = st->low[b] = 0;
   if (threadIdx.x == 0) {
-    st->Plo = d > 0 ? d - 1 : 0;
-    st->Phi = min(d + 1, (unsigned)TK_NB0 - 1);
+    st->Plo = Plo;
+    st->Phi = Phi;
+    st->Tlo = Tlo;
+    st->table = mode;
     st->done[0] = 0;
+  }
+}
+
+// The last CTA of a pass over the window: whether it holds the k-th largest,
+// and if so key >> 10 of that pair (and, with TRACK, perhaps its last digit).
+template <int NT, bool TRACK>
+__device__ __forceinline__ void resolve_window(const TopkParams& p, long long* lim, uint32_t Plo) {
+  TopkState* st = p.st;
+  const unsigned long long nfin = (unsigned long long)p.n - __ldcg(&st->nonfin);
+  const unsigned long long k = take_count(nfin, p), above = __ldcg(&st->above);
+  // krem in range: the digit is selected as the window's total comes back
+  unsigned long long krem = k > above ? k - above : 0;
+  unsigned d = 0;
+  const unsigned long long wt = select_digit<TK_WIN * TK_NB1 / NT, NT>(st->hist1, krem, d);
+  const bool hit = k == 0 || (above < k && k <= above + wt);
+  // TRACK: lowor and inexact were kept.  Window keys that are all multiples of 2^10 with float32
+  // |d|: every window bucket then holds one value, so the last digit is 0, the
+  // k-th largest is P1 2^10, and the buckets above P1 add count x value
+  // exactly; pass 2 (and 3) then have nothing to do
+  bool skip = false;
+  if constexpr (TRACK) skip = hit && k > 0 && __ldcg(&st->lowor) == 0 && __ldcg(&st->inexact) == 0;
+  if (skip) {
+    for (int j = threadIdx.x; j < NLIMB; j += NT) lim[j] = 0;
+    __syncthreads();
+    for (int b = d + 1 + threadIdx.x; b < TK_WIN * TK_NB1; b += NT) {
+      const unsigned long long cnt = __ldcg(&st->hist1[b]);
+      if (cnt) {
+        int sc;
+        const float v = key_value(((Plo << 11) + (uint32_t)b) << 10, sc);
+        digits_of_n(lim, v, sc, cnt);
+      }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < NLIMB; j += NT)
+      if (lim[j]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->limbs[j]), (unsigned long long)lim[j]);
+  }
+  if (threadIdx.x == 0) {
+    st->nfin = nfin;
+    st->k = k;
+    st->ok = hit ? 1u : 0u;
+    if (hit && k > 0) {
+      const uint32_t P1 = (Plo << 11) + d;
+      st->P1 = P1;
+      st->P0 = P1 >> 11;
+      st->krem = krem;
+      if (skip) {
+        st->hist2[0] = __ldcg(&st->hist1[d]);  // P1's bucket: every key is P1 2^10 (last digit 0)
+        st->T = P1 << 10;
+        st->skip2 = 1u;
+      }
+    }
+    st->done[1] = 0;
   }
 }
 
@@ -510,24 +621,20 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
 // infinity counted.  The last CTA checks that the window holds the k-th
 // largest and, if so, resolves key >> 10.  As the fallback (FB) it runs only
 // when the sampled window missed, on the exact window from topk_pass0.
-template <int DT, bool FB>
-__global__ void __launch_bounds__(TB) topk_pass1(TopkParams p) {
-  __shared__ uint32_t h[TK_WIN * TK_NB1];
-  __shared__ long long lim[NLIMB];
-  __shared__ typename QT<DT>::T ring[(TB / 32) * ring_cap<DT>()];
-  __shared__ unsigned long long cnt_s[2];
-  __shared__ unsigned last_s;
-  pdl_wait();
-  pdl_trigger();
+template <int DT, int NT>
+__device__ __forceinline__ void pass1_general(const TopkParams& p, uint32_t* h, long long* lim,
+                                              typename QT<DT>::T* ring, unsigned long long* cnt_s, unsigned* last_s) {
   TopkState* st = p.st;
-  if (FB && st->ok) return;
-  for (int b = threadIdx.x; b < TK_WIN * TK_NB1; b += TB) h[b] = 0;
-  for (int j = threadIdx.x; j < NLIMB; j += TB) lim[j] = 0;
+  for (int b = threadIdx.x; b < TK_WIN * TK_NB1; b += NT) h[b] = 0;
+  for (int j = threadIdx.x; j < NLIMB; j += NT) lim[j] = 0;
   if (threadIdx.x < 2) cnt_s[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t Plo = st->Plo, Phi = st->Phi;
-  // every key above the window has a biased exponent of at least (Phi + 1) >> 2
-  ExactAcc acc(Phi + 1 >= (KEY_OVF >> 21) ? NO_FAST : max((int)((Phi + 1) >> 2), 1), lim);
+  // the floor of the integer sums: every key above the window has a biased
+  // exponent of at least (Phi + 1) >> 2, and when the window starts at zero
+  // most of them lie at Tlo or above
+  const uint32_t a0 = max(Phi + 1, st->Tlo);
+  ExactAcc acc(a0 >= (KEY_OVF >> 21) ? NO_FAST : max((int)(a0 >> 2), 1), lim);
   RunCount rc;
   uint32_t nab = 0, nnf = 0;
   // 16-bit operands: whether the window's keys all have zero low 10 bits and
@@ -536,7 +643,7 @@ __global__ void __launch_bounds__(TB) topk_pass1(TopkParams p) {
   // a pair whose raw key is below KEY_OVF is finite with that key: inside
   // the window it is only counted, here; everything above the window, and
   // every pair with a NaN, an infinity or an overflow, is queued
-  tk_filtered<DT>(
+  tk_filtered<DT, NT>(
       p, ring + (threadIdx.x >> 5) * ring_cap<DT>(),
       [&](uint32_t G, uint32_t C) {
         const uint32_t u = raw_key<DT>(G, C), k0 = u >> 21;
@@ -586,52 +693,202 @@ __global__ void __launch_bounds__(TB) topk_pass1(TopkParams p) {
     if (cnt_s[0]) atomicAdd(&st->above, cnt_s[0]);
     if (cnt_s[1]) atomicAdd(&st->nonfin, cnt_s[1]);
   }
-  if (!pass_end(h, TK_WIN * TK_NB1, st->hist1, lim, st, 1, &last_s)) return;
-  const unsigned long long nfin = (unsigned long long)p.n - __ldcg(&st->nonfin);
-  const unsigned long long k = take_count(nfin, p), above = __ldcg(&st->above);
-  // krem in range: the digit is selected as the window's total comes back
-  unsigned long long krem = k > above ? k - above : 0;
-  unsigned d = 0;
-  const unsigned long long wt = select_digit<TK_WIN * TK_NB1 / TB>(st->hist1, krem, d);
-  const bool hit = k == 0 || (above < k && k <= above + wt);
-  // 16-bit operands whose window keys are all multiples of 2^10 with float32
-  // |d|: every window bucket holds one value, so the last digit is 0, the
-  // k-th largest is P1 2^10, and the buckets above P1 add count x value
-  // exactly; pass 2 (and 3) then have nothing to do
-  bool skip = false;
-  if constexpr (TK<DT>::BYTES == 2) skip = hit && k > 0 && __ldcg(&st->lowor) == 0 && __ldcg(&st->inexact) == 0;
-  if (skip) {
-    for (int j = threadIdx.x; j < NLIMB; j += TB) lim[j] = 0;
-    __syncthreads();
-    for (int b = d + 1 + threadIdx.x; b < TK_WIN * TK_NB1; b += TB) {
-      const unsigned long long cnt = __ldcg(&st->hist1[b]);
-      if (cnt) {
-        int sc;
-        const float v = key_value(((Plo << 11) + (uint32_t)b) << 10, sc);
-        digits_of_n(lim, v, sc, cnt);
+  if (!pass_end<NT>(h, TK_WIN * TK_NB1, st->hist1, lim, st, 1, last_s)) return;
+  resolve_window<NT, TK<DT>::BYTES == 2>(p, lim, Plo);
+}
+
+template <int DT, bool FB>
+__global__ void __launch_bounds__(TB) topk_pass1(TopkParams p) {
+  __shared__ uint32_t h[TK_WIN * TK_NB1];
+  __shared__ long long lim[NLIMB];
+  __shared__ typename QT<DT>::T ring[(TB / 32) * ring_cap<DT>()];
+  __shared__ unsigned long long cnt_s[2];
+  __shared__ unsigned last_s;
+  pdl_wait();
+  pdl_trigger();
+  if (FB && p.st->ok) return;
+  pass1_general<DT, TB>(p, h, lim, ring, cnt_s, &last_s);
+}
+
+// A pair of the table pass that its table does not take, and the elements
+// outside the vector grid: exactly, one at a time.
+template <int DT>
+__device__ __noinline__ void table_pair(const TopkParams* p, uint32_t G, uint32_t C, uint32_t Plo, uint32_t Phi,
+                                        long long* lim, unsigned long long* cnt_s) {
+  TopkState* st = p->st;
+  if (!tk_finite<DT>(G, C)) {
+    atomicAdd(&cnt_s[1], 1ull);
+    return;
+  }
+  const float gf = tk_f32<DT>(G), cf = tk_f32<DT>(C);
+  const uint32_t key = tk_key(gf, cf), k0 = key >> 21;
+  if (k0 < Plo) return;
+  float hi, lo;
+  int sc;
+  tk_exact(gf, cf, hi, lo, sc);
+  if (k0 > Phi) {
+    atomicAdd(&cnt_s[0], 1ull);
+    digits_of(lim, hi, sc);
+    digits_of(lim, lo, sc);
+    return;
+  }
+  atomicAdd(&st->hist1[((k0 - Plo) << 11) | ((key >> 10) & 0x7FFu)], 1ull);
+  if (key & 0x3FFu) atomicOr(&st->lowor, key & 0x3FFu);
+  if (lo != 0.0f) atomicOr(&st->inexact, 1u);
+}
+
+template <int DT>
+__device__ __noinline__ void table_vec_slow(const TopkParams* p, uint4 g, uint4 c, uint32_t Plo, uint32_t Phi,
+                                            long long* lim, unsigned long long* cnt_s) {
+  constexpr int PW = 4 / TK<DT>::BYTES;  // pairs per word
+#pragma unroll 1
+  for (int w = 0; w < 4; w++) {
+    uint32_t a = g.x, b = c.x;
+    g = make_uint4(g.y, g.z, g.w, 0);
+    c = make_uint4(c.y, c.z, c.w, 0);
+#pragma unroll 1
+    for (int j = 0; j < PW; j++) {
+      if constexpr (PW == 1) {
+        table_pair<DT>(p, a, b, Plo, Phi, lim, cnt_s);
+      } else {
+        table_pair<DT>(p, a & 0xFFFFu, b & 0xFFFFu, Plo, Phi, lim, cnt_s);
+        a >>= 16;
+        b >>= 16;
       }
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < NLIMB; j += TB)
-      if (lim[j]) atomicAdd(reinterpret_cast<unsigned long long*>(&st->limbs[j]), (unsigned long long)lim[j]);
   }
+}
+
+// Pass 1 when every |d| from the window up is a float32 value whose key has
+// zero low bits and lies within TAB_DIGITS digits of the window's start: one
+// shared counter per key >> 10.  All pairs below the window share a cell (the
+// magnitude is clamped to a value just below it), so the loop has no branch
+// but one per vector: s = c - g, the clamp, the checks, an increment by the
+// constant one at (bits >> 8).  At the end the cells above the window are
+// summed as count x value and the window's cells go to hist1.  A vector with
+// a pair that fails a check (a NaN, an infinity, a longer key, an inexact
+// difference, a value beyond the table) is done pair by pair.
+//
+// When the keys have only 9 significant bits, every lane counts in its own
+// copy of a cell (the 32 words after a value's first are then no value's):
+// the increments of a warp fall on 32 banks whatever the values.
+//
+// About 14 instructions per pair against 55 with a queue of the pairs above
+// the window, which leaves the loads as the bound.  67.1 M bf16 pairs,
+// truncated against rounded: the pass 150 us with the queue, 57 now (40 at
+// the copy rate), the call 171 -> 82; 33.6 M float32 pairs against noise: the
+// call 162 -> 80.  One CTA of 1024 threads: two vectors of both operands in
+// flight per thread keep 64 KB outstanding per SM.
+template <int DT>
+__global__ void __launch_bounds__(TT, 1) topk_table(const __grid_constant__ TopkParams p) {
+  constexpr int VEC = TK<DT>::VEC, B = TK<DT>::BYTES;
+  extern __shared__ __align__(16) uint32_t tab[];  // 32 cells for the pairs below the window, then TAB_CELLS
+  __shared__ long long lim[NLIMB];
+  __shared__ unsigned long long cnt_s[2];
+  __shared__ unsigned last_s;
+  for (int b = threadIdx.x; b < (32 + TAB_CELLS) / 4; b += TT) reinterpret_cast<uint4*>(tab)[b] = make_uint4(0, 0, 0, 0);
+  for (int j = threadIdx.x; j < NLIMB; j += TT) lim[j] = 0;
+  if (threadIdx.x < 2) cnt_s[threadIdx.x] = 0;
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  TopkState* st = p.st;
+  const uint32_t mode = st->table;
+  if (mode == 0) {
+    constexpr int W = TK_WIN * TK_NB1;
+    using Q = typename QT<DT>::T;
+    static_assert(W * 4 + (TT / 32) * ring_cap<DT>() * sizeof(Q) <= TAB_SMEM, "shared memory of the general pass");
+    pass1_general<DT, TT>(p, tab, lim, reinterpret_cast<Q*>(tab + W), cnt_s, &last_s);
+    return;
+  }
+  const uint32_t Plo = st->Plo, Phi = st->Phi, lane = threadIdx.x & 31;
+  const uint32_t Tlo = st->Tlo, lo = Tlo << 21, mask = mode == 2 ? COPY_MASK : 0x3FFu;
+  const uint32_t top = min(lo + ((uint32_t)TAB_DIGITS << 21), KEY_OVF);  // Tlo < 1024: no wrap
+  // the magnitude that pairs below the table are clamped to (Tlo >= 1)
+  const float vlo = __uint_as_float(lo - (mask + 1));
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab) + 128u + (mode == 2 ? lane * 4u : 0u) - (lo >> 8);
+  auto vec = [&](auto zero, const uint4& g, const uint4& c) {
+    constexpr bool ZERO = decltype(zero)::value;  // only zeros may lie below the table
+    uint32_t m[VEC], orv = 0, mx = 0, mn = 0xFFFFFFFFu;
+    float err = 0.0f;
+#pragma unroll
+    for (int j = 0; j < VEC; j++) {
+      const float gf = tk_f32<DT>(tk_lane<DT>(g, j)), cf = tk_f32<DT>(tk_lane<DT>(c, j));
+      const float s = __fsub_rn(cf, gf);
+      err = __fadd_rn(err, fabsf(__fadd_rn(__fsub_rn(s, cf), gf)));
+      err = __fadd_rn(err, fabsf(__fsub_rn(__fadd_rn(s, gf), cf)));
+      m[j] = __float_as_uint(fmaxf(fabsf(s), vlo));
+      orv |= m[j];
+      mx = max(mx, m[j]);
+      if (ZERO) mn = min(mn, (__float_as_uint(s) & 0x7FFFFFFFu) - 1u);
+    }
+    if (err == 0.0f && mx < top && !(orv & mask) && (!ZERO || mn >= lo - 1u)) {
+#pragma unroll
+      for (int j = 0; j < VEC; j++)
+        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(base + (m[j] >> 8)) : "memory");
+    } else {
+      table_vec_slow<DT>(&p, g, c, Plo, Phi, lim, cnt_s);
+    }
+  };
+  const int64_t stride = (int64_t)gridDim.x * TT, gt = (int64_t)blockIdx.x * TT + threadIdx.x;
+  auto all = [&](auto zero) {
+    int64_t v = gt;
+    for (; v + stride < p.nvec; v += 2 * stride) {
+      const int64_t o0 = (p.p0 + v * VEC) * B, o1 = o0 + stride * VEC * B;
+      const uint4 g0 = tk_vec(p.g, o0), c0 = tk_vec(p.c, o0);
+      const uint4 g1 = tk_vec(p.g, o1), c1 = tk_vec(p.c, o1);
+      vec(zero, g0, c0);
+      vec(zero, g1, c1);
+    }
+    if (v < p.nvec) {
+      const int64_t o0 = (p.p0 + v * VEC) * B;
+      vec(zero, tk_vec(p.g, o0), tk_vec(p.c, o0));
+    }
+  };
+  if (Plo == 0) all(std::true_type{});
+  else all(std::false_type{});
+  const int64_t tail = p.p0 + p.nvec * VEC, ns = p.p0 + (p.n - tail);  // elements outside the vector grid
+  if (gt < ns) {
+    const int64_t i = gt < p.p0 ? gt : tail + (gt - p.p0);
+    table_pair<DT>(&p, tk_load<DT>(p.g, i), tk_load<DT>(p.c, i), Plo, Phi, lim, cnt_s);
+  }
+  __syncthreads();
+  // cells above the window: values of at most 14 significant bits, less than
+  // 7 binades above the floor, at most n / 152 pairs per CTA: sums below 2^60
+  const unsigned a0 = max(Phi + 1, Tlo);
+  ExactAcc acc(a0 >= (KEY_OVF >> 21) ? NO_FAST : max((int)(a0 >> 2), 1), lim);
+  unsigned long long nab = 0;
+  if (Plo == 0 && threadIdx.x < 32) {
+    const uint32_t zeros = __reduce_add_sync(0xFFFFFFFFu, tab[lane]);
+    if (lane == 0 && zeros) atomicAdd(&st->hist1[0], (unsigned long long)zeros);
+  }
+  for (int i = threadIdx.x; i < TAB_CELLS; i += TT) {
+    uint32_t cnt = tab[32 + i];
+    if (mode == 2) {  // the 32 copies of one cell
+      cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+      if (lane) cnt = 0;
+    }
+    if (!cnt) continue;
+    const uint32_t key = lo + ((uint32_t)i << 10);
+    if ((key >> 21) <= Phi) {
+      atomicAdd(&st->hist1[i], (unsigned long long)cnt);
+    } else {
+      nab += cnt;
+      const int e = max((int)(key >> 23), 1);
+      acc.V += (unsigned long long)cnt * ((uint64_t)((key & 0x7FFFFFu) | ((key >> 23) ? 0x800000u : 0u)) << (e - acc.eb));
+    }
+  }
+  __syncwarp();
+  acc.flush();
+  const unsigned hi32 = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(nab >> 16)), lo32 = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(nab & 0xFFFFu));
+  if (lane == 0 && (hi32 | lo32)) atomicAdd(&cnt_s[0], ((unsigned long long)hi32 << 16) + lo32);
+  __syncthreads();
   if (threadIdx.x == 0) {
-    st->nfin = nfin;
-    st->k = k;
-    st->ok = hit ? 1u : 0u;
-    if (hit && k > 0) {
-      const uint32_t P1 = (Plo << 11) + d;
-      st->P1 = P1;
-      st->P0 = P1 >> 11;
-      st->krem = krem;
-      if (skip) {
-        st->hist2[0] = __ldcg(&st->hist1[d]);  // P1's bucket: every key is P1 2^10 (last digit 0)
-        st->T = P1 << 10;
-        st->skip2 = 1u;
-      }
-    }
-    st->done[1] = 0;
+    if (cnt_s[0]) atomicAdd(&st->above, cnt_s[0]);
+    if (cnt_s[1]) atomicAdd(&st->nonfin, cnt_s[1]);
   }
+  if (!pass_end<TT>(nullptr, 0, nullptr, lim, st, 1, &last_s)) return;
+  resolve_window<TT, true>(p, lim, Plo);
 }
 
 // Only when the sampled window missed: the exact digit of key >> 21 (k and
@@ -971,10 +1228,10 @@ __global__ void __launch_bounds__(TB) topk_finalize(TopkParams p) {
     st->nonfin = st->above = st->nfin = st->k = st->krem = 0;
     st->kreml[0] = st->kreml[1] = 0;
     st->dl[0] = st->dl[1] = 0;
-    st->Plo = st->Phi = st->P0 = st->P1 = st->T = 0;
+    st->Plo = st->Phi = st->P0 = st->P1 = st->T = st->Tlo = 0;
     st->ok = 0;
     st->nlist = st->nlist2 = 0;
-    st->lowor = st->inexact = st->skip2 = 0;
+    st->lowor = st->inexact = st->skip2 = st->table = 0;
   }
 }
 
@@ -1006,7 +1263,9 @@ cudaError_t launch_t(const TopkParams& p, int nctas, cudaStream_t s) {
   topk_sample<DT><<<sctas, TB, 0, s>>>(p);
   cudaError_t e = cudaGetLastError();
   const unsigned g = (unsigned)nctas;
-  if (e == cudaSuccess) e = launch_dependent(topk_pass1<DT, false>, g, TB, 0, s, p);
+  if (e == cudaSuccess)
+    e = p.tabled ? launch_dependent(topk_table<DT>, (unsigned)p.tabled, TT, TAB_SMEM, s, p)
+                 : launch_dependent(topk_pass1<DT, false>, g, TB, 0, s, p);
   if (e == cudaSuccess) e = launch_dependent(topk_pass0<DT>, g, TB, 0, s, p);
   if (e == cudaSuccess) e = launch_dependent(topk_pass1<DT, true>, g, TB, 0, s, p);
   if (e == cudaSuccess) e = launch_dependent(topk_pass2<DT>, g, TB, 0, s, p);
@@ -1018,6 +1277,16 @@ cudaError_t launch_t(const TopkParams& p, int nctas, cudaStream_t s) {
 }
 
 }  // namespace
+
+// once per device, before the first launch
+cudaError_t topk_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(topk_table<PEAT_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAB_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(topk_table<PEAT_F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAB_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(topk_table<PEAT_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, TAB_SMEM);
+  return e;
+}
 
 int topk_max_ctas(int nsm) {
   static const int per_sm = [] {
