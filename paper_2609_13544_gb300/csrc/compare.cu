@@ -362,6 +362,39 @@ __device__ __forceinline__ int cmp_ratio_f(float a1, float g1, float a2, float g
   return P1 > P2 ? 1 : (P1 < P2 ? -1 : 0);
 }
 
+// log2-like key of the ratio (hi + lo) 2^sc / g, within 8 of an increasing
+// function of its exact value (2^22 units per binade): the quotient of the
+// significands, rounded, under the difference of the exponents.
+__device__ __forceinline__ int ratio_key(float h, int sc, float g) {
+  if (h == 0.0f) return -0x7FFFFFFF;
+  if (g == 0.0f) return 0x7FFFFFFF;
+  int e = sc;
+  if (h < 1.17549435e-38f) h = __fmul_rn(h, 1.8446744e19f), e -= 64;  // subnormals scaled by 2^64
+  if (g < 1.17549435e-38f) g = __fmul_rn(g, 1.8446744e19f), e += 64;
+  const uint32_t bh = __float_as_uint(h), bg = __float_as_uint(g);
+  e += (int)(bh >> 23) - (int)(bg >> 23);
+  const float q = __fdividef(__uint_as_float((bh & 0x7FFFFFu) | 0x3F800000u), __uint_as_float((bg & 0x7FFFFFu) | 0x3F800000u));
+  return ((int)(__float_as_uint(q) - 0x3F800000u) >> 1) + e * (1 << 22);
+}
+constexpr int RATIO_MARGIN = 32;  // keys further apart decide (the key's error, and lo against hi, below 8 each)
+
+// sign((h1 + l1) 2^s1 / g1 - (h2 + l2) 2^s2 / g2): by the keys when they
+// differ clearly, by the exact products otherwise
+__device__ __forceinline__ int cmp_rel_close(float h1, float l1, int s1, float g1, float h2, float l2, int s2, float g2) {
+  const float tiny = 1.17549435e-38f;
+  if (h1 == h2 && l1 == l2 && s1 == s2 && g1 == g2) return 0;
+  if (l1 == 0.0f && l2 == 0.0f && s1 == 0 && s2 == 0 && h1 >= tiny && h2 >= tiny && g1 >= tiny && g2 >= tiny)
+    return cmp_ratio_f(h1, g1, h2, g2);
+  return cmp_rel_exact(h1, l1, s1, g1, h2, l2, s2, g2);
+}
+__device__ __forceinline__ int cmp_rel_rec(float h1, float l1, int s1, float g1, float h2, float l2, int s2, float g2) {
+  const int k1 = ratio_key(h1, s1, g1), k2 = ratio_key(h2, s2, g2);
+  const long long d = (long long)k1 - k2;
+  if (d > RATIO_MARGIN) return 1;
+  if (d < -RATIO_MARGIN) return -1;
+  return cmp_rel_close(h1, l1, s1, g1, h2, l2, s2, g2);
+}
+
 // float32 filter for a rel best: a value <= rel with a margin for the
 // approximate per-lane ratio a * rcp(|g|)
 __device__ __forceinline__ float rel_filter(float hi, int sc, float g) {
@@ -407,8 +440,8 @@ static_assert(LIMB_LSB % 32 == 0, "the S2 shift is a whole number of digits");
 struct FinScratch {
   unsigned long long cnt[8];
   long long limbs[NSUM * NLIMB];
-  Partial wbest[16];
-  double sums[NSUM];
+  Partial wbest[16], best;
+  double sums[NSUM], max_abs, max_rel;
 };
 constexpr int NSTAGE = 2;  // a power of two: stage and phase are bit fields of the use count
 constexpr int RWMAX = 6;   // window moves per warp and piece (float32)
@@ -472,7 +505,7 @@ struct Common {
   uint32_t gn;                     // entries appended in this piece (may exceed GCAP)
   uint32_t nfe;                    // bitwise-equal pairs holding NaN or Inf
   int last;                        // this CTA finished the last piece of a one-segment call
-  unsigned pieces;                 // a one-segment call's pieces: the CTAs whose ranges are not empty
+  int first, final;                // a one-segment call's pieces: the CTAs first .. final
   int lb, ub;
   // the CTA's window maxima of the piece: value in the high word, the
   // complement of the pair's offset in the low one (the larger key is the
@@ -493,7 +526,7 @@ struct Common {
   // the general path's totals, one copy per warp (fewer threads contend for an
   // address), folded into hist and sacc at the end of a piece that used them
   unsigned long long ghist[NW][HBINS];
-  unsigned long long gsacc[NW][NSUM][NLIMB];
+  int gsacc[NW][NSUM * NLIMB][2];  // sums of the low and the high 16 bits of each digit (gen_flush)
 };
 
 template <int DT>
@@ -519,43 +552,36 @@ template <int DT>
 __device__ __forceinline__ void sacc_add(Smem<DT>& sm, int which, unsigned __int128 m, int e, bool neg) {
   for_digits(m, e, neg, [&](int j, int64_t v) { atomicAdd(&sm.k.sacc[which][j], (unsigned long long)v); });
 }
-// General-path terms, one per lane of a converged warp, into the warp's copy
-// of the sum digits: lanes whose digit indices agree are summed in registers
-// first (__match_any_sync groups them; the 32-bit reductions take each signed
-// digit value as a signed 16-bit high part and an unsigned 16-bit low part,
-// so that no group sum overflows), and one lane per group adds the total.
-// Without this, the lanes of a warp would serialise on 64-bit shared atomics
-// to the same few digits.
-template <int DT>
-__device__ __forceinline__ void wsacc_add(Smem<DT>& sm, int which, uint64_t m, int e, bool neg, bool on) {
-  on = on && m != 0;
-  if (!__any_sync(0xFFFFFFFFu, on)) return;
-  const int lane = threadIdx.x & 31;
+// A general-path term +-m 2^e into the warp's copy of a sum's digits.  A copy
+// holds each digit's 32-bit contributions as two sums of 16-bit halves in
+// signed 32-bit words, which shared memory adds natively (64-bit adds there
+// are compare-and-swap loops, and grouping the lanes by digit first, match
+// and reductions, took 6 us for the terms of one round; this takes 1.3).
+// gen_flush empties the words before they can overflow.
+__device__ __forceinline__ void wsacc_add(int* d, uint64_t m, int e, bool neg) {
   const int p = e - LIMB_LSB, j = p >> 5, r = p & 31;
   const uint32_t m0 = (uint32_t)m, m1 = (uint32_t)(m >> 32);
   const uint32_t out[3] = {m0 << r, (m1 << r) | (r ? m0 >> (32 - r) : 0u), r ? m1 >> (32 - r) : 0u};
-  unsigned long long* d = sm.k.gsacc[threadIdx.x >> 5][which];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
-    const bool ok = on && out[k] != 0u && (unsigned)(j + k) < (unsigned)NLIMB;
-    const unsigned grp = __match_any_sync(0xFFFFFFFFu, ok ? j + k : -1);
-    const int64_t v = ok ? (neg ? -(int64_t)out[k] : (int64_t)out[k]) : 0;
-    const uint32_t slo = __reduce_add_sync(grp, (uint32_t)v & 0xFFFFu);
-    const int32_t shi = (int32_t)__reduce_add_sync(grp, (uint32_t)(int32_t)(v >> 16));
-    if (ok && lane == __ffs(grp) - 1) atomicAdd(d + j + k, (unsigned long long)((int64_t)shi * 65536 + slo));
+    if (out[k] == 0u || (unsigned)(j + k) >= (unsigned)NLIMB) continue;
+    const int lo = (int)(out[k] & 0xFFFFu), hi = (int)(out[k] >> 16);
+    atomicAdd(d + 2 * (j + k), neg ? -lo : lo);
+    atomicAdd(d + 2 * (j + k) + 1, neg ? -hi : hi);
   }
 }
+// Three terms of a round go to one sum: 256 rounds of 32 lanes stay below 2^31.
+constexpr int GEN_FLUSH = 256;
 template <int DT>
-__device__ __forceinline__ void wsacc_add_f(Smem<DT>& sm, int which, float x, int sc, bool on) {
-  int e = 0;
-  const uint32_t m = x != 0.0f ? split_float(x, e) : 0u;
-  wsacc_add(sm, which, m, e + sc, x < 0.0f, on);
-}
-template <int DT>
-__device__ __forceinline__ void wsacc_add_prod_f(Smem<DT>& sm, int which, float x, float y, int sc, bool on) {
-  int ex = 0, ey = 0;
-  const uint32_t mx = x != 0.0f ? split_float(x, ex) : 0u, my = y != 0.0f ? split_float(y, ey) : 0u;
-  wsacc_add(sm, which, (uint64_t)mx * my, ex + ey + sc, (x < 0.0f) != (y < 0.0f), on);
+__device__ __noinline__ void gen_flush(Smem<DT>& sm) {
+  __syncwarp();
+  int(*d)[2] = sm.k.gsacc[threadIdx.x >> 5];
+  for (int j = threadIdx.x & 31; j < NSUM * NLIMB; j += 32) {
+    const int64_t v = (int64_t)d[j][1] * 65536 + d[j][0];
+    d[j][0] = d[j][1] = 0;
+    if (v) atomicAdd(&sm.k.sacc[0][0] + j, (unsigned long long)v);
+  }
+  __syncwarp();
 }
 // one histogram bin per lane (bin < 0: none), counted once per distinct bin
 template <int DT>
@@ -672,7 +698,7 @@ __device__ __forceinline__ void general_pair(GenRec& cd, GenOut& o, uint32_t G, 
     bool maybe = cd.rel_idx < 0 || ag == 0.0f || sc ||
                  __fmul_rn(__fmul_rn(hi, rcp_approx(ag)), 1.00001f) >= cd.rel_f;
     if (maybe) {
-      int c = cd.rel_idx < 0 ? 1 : cmp_rel_exact(hi, lo, sc, ag, cd.rel_hi, cd.rel_lo, cd.rel_sc, cd.rel_g);
+      int c = cd.rel_idx < 0 ? 1 : cmp_rel_rec(hi, lo, sc, ag, cd.rel_hi, cd.rel_lo, cd.rel_sc, cd.rel_g);
       if (c > 0 || (c == 0 && idx < cd.rel_idx)) {
         cd.rel_hi = hi;
         cd.rel_lo = lo;
@@ -699,15 +725,22 @@ __device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, uint32_t 
   whist_add(sm, o.hb0);
   whist_add(sm, o.hb1);
   const bool on = o.s != 0.0f;
-  const bool neg = o.s < 0.0f;
-  const float hi = neg ? -o.s : o.s, lo = neg ? -o.t : o.t;
-  wsacc_add_f(sm, 0, o.s, o.sc, on);
-  wsacc_add_f(sm, 0, o.t, o.sc, on);
-  wsacc_add_f(sm, 1, hi, o.sc, on);
-  wsacc_add_f(sm, 1, lo, o.sc, on);
-  wsacc_add_prod_f(sm, 2, o.s, o.s, 2 * o.sc, on);
-  wsacc_add_prod_f(sm, 2, o.s, o.t, 2 * o.sc + 1, on);
-  wsacc_add_prod_f(sm, 2, o.t, o.t, 2 * o.sc, on);
+  // the seven terms through one copy of the code: a piece with few general
+  // pairs spends most of this path's time on fetching it
+  int* d = &sm.k.gsacc[threadIdx.x >> 5][0][0];
+#pragma unroll 1
+  for (int k = 0; k < 7; k++) {
+    // s, t | |d|'s parts, s and t with the sign of s | s^2, 2 s t, t^2
+    float x = k == 1 || k == 3 || k == 6 ? o.t : o.s;
+    const float y = k < 4 ? 1.0f : (k == 4 ? o.s : o.t);
+    if ((k == 2 || k == 3) && o.s < 0.0f) x = -x;
+    if (on && x != 0.0f && y != 0.0f) {
+      int ex = 0, ey = 0;
+      const uint32_t mx = split_float(x, ex), my = split_float(y, ey);
+      wsacc_add(d + min(k >> 1, 2) * (2 * NLIMB), (uint64_t)mx * my, ex + ey + (k < 4 ? o.sc : 2 * o.sc + (k == 5)),
+                (x < 0.0f) != (y < 0.0f));
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1517,13 +1550,6 @@ __device__ __forceinline__ int64_t min_idx(int64_t a, int64_t b) {
   return a < b ? a : b;
 }
 
-__device__ __forceinline__ int cmp_rel_rec(float h1, float l1, int s1, float g1, float h2, float l2, int s2, float g2) {
-  const float tiny = 1.17549435e-38f;
-  if (l1 == 0.0f && l2 == 0.0f && s1 == 0 && s2 == 0 && h1 >= tiny && h2 >= tiny && g1 >= tiny && g2 >= tiny)
-    return cmp_ratio_f(h1, g1, h2, g2);
-  return cmp_rel_exact(h1, l1, s1, g1, h2, l2, s2, g2);
-}
-
 // x <- the better of x and y, field by field; ties to the lower index
 __device__ __forceinline__ void part_merge(Partial& x, const Partial& y) {
   if (y.abs_idx >= 0) {
@@ -1553,35 +1579,87 @@ __device__ __forceinline__ void part_merge(Partial& x, const Partial& y) {
   x.first_ulp = min_idx(x.first_ulp, y.first_ulp);
 }
 
-__device__ __forceinline__ int64_t shfl_i64(int64_t v, int o) {
-  return (int64_t)((uint64_t)__shfl_down_sync(0xFFFFFFFFu, (uint32_t)v, o) |
-                   ((uint64_t)__shfl_down_sync(0xFFFFFFFFu, (uint32_t)((uint64_t)v >> 32), o) << 32));
+__device__ __forceinline__ uint64_t warp_min64(uint64_t v) {
+  const uint32_t h = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)(v >> 32));
+  const uint32_t l = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)(v >> 32) == h ? (uint32_t)v : 0xFFFFFFFFu);
+  return ((uint64_t)h << 32) | l;
 }
-__device__ __forceinline__ float shfl_f(float v, int o) { return __shfl_down_sync(0xFFFFFFFFu, v, o); }
-__device__ __forceinline__ int shfl_int(int v, int o) { return __shfl_down_sync(0xFFFFFFFFu, v, o); }
 
-// warp tournament; lane 0 ends with the warp's best
-__device__ __forceinline__ void part_warp_reduce(Partial& x) {
+// The best of the warp's 32 records, field by field, into *out (shared or
+// global; the warp synchronises afterwards).  Each maximum goes by 32-bit
+// warp reductions over keys (value, then rounding error, then index), and the
+// lane that holds it stores it: no record travels between lanes.  A ratio's
+// key is approximate; the lanes within its margin of the best are compared
+// exactly with one of them, all at once, until none is greater.  Out of line
+// and by value: its four callers run once each, so the fetch of the code is
+// most of its time and they share it (a tournament of whole records over
+// shuffles took 2 to 10 us at each place, this 0.7 to 2).
+__device__ __noinline__ void warp_best(float ah, float al, int as, int64_t ai, float rh, float rl, float rg, int rs,
+                                       int64_t ri, uint64_t u, int64_t ui, int64_t ff, int64_t fu, Partial* out) {
+  const uint32_t all = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31;
-  for (int o = 16; o > 0; o >>= 1) {
-    Partial y;
-    y.abs_hi = shfl_f(x.abs_hi, o);
-    y.abs_lo = shfl_f(x.abs_lo, o);
-    y.abs_sc = shfl_int(x.abs_sc, o);
-    y.abs_idx = shfl_i64(x.abs_idx, o);
-    y.rel_hi = shfl_f(x.rel_hi, o);
-    y.rel_lo = shfl_f(x.rel_lo, o);
-    y.rel_g = shfl_f(x.rel_g, o);
-    y.rel_sc = shfl_int(x.rel_sc, o);
-    y.rel_idx = shfl_i64(x.rel_idx, o);
-    y.ulp = (uint64_t)shfl_i64((int64_t)x.ulp, o);
-    y.ulp_idx = shfl_i64(x.ulp_idx, o);
-    y.first_fin = shfl_i64(x.first_fin, o);
-    y.first_ulp = shfl_i64(x.first_ulp, o);
-    if (lane + o < 32) part_merge(x, y);
+  {
+    // (scaled values exceed every unscaled float32)
+    const uint32_t k = ai < 0 ? 0u : __float_as_uint(ah) + ((uint32_t)as << 23) + 1u;
+    const uint32_t m = __reduce_max_sync(all, k);
+    const uint32_t b = __float_as_uint(al);
+    const uint32_t kl = k != m ? 0u : (al == 0.0f ? 0x80000000u : ((b & 0x80000000u) ? ~b : (b | 0x80000000u)));
+    const uint32_t ml = __reduce_max_sync(all, kl);
+    const bool c = k == m && kl == ml;
+    const uint64_t i = warp_min64(c ? (uint64_t)ai : ~0ull);
+    if (m ? (c && (uint64_t)ai == i) : lane == 0) {
+      out->abs_hi = ah;
+      out->abs_lo = al;
+      out->abs_sc = as;
+      out->pad0 = 0;
+      out->abs_idx = ai;
+    }
   }
+  {
+    constexpr int NONE = (int)0x80000000;
+    const int k = ri < 0 ? NONE : ratio_key(rh, rs, rg);
+    const int m = __reduce_max_sync(all, k);
+    uint32_t cand = __ballot_sync(all, ri >= 0 && (long long)k >= (long long)m - RATIO_MARGIN);
+    while (cand & (cand - 1)) {
+      const int w = __ffs(cand) - 1;
+      const float wh = __shfl_sync(all, rh, w), wl = __shfl_sync(all, rl, w), wg = __shfl_sync(all, rg, w);
+      const int ws = __shfl_sync(all, rs, w);
+      const int c = lane == w ? 0 : ((cand >> lane) & 1u) ? cmp_rel_close(rh, rl, rs, rg, wh, wl, ws, wg) : -1;
+      const uint32_t gt = __ballot_sync(all, c > 0), eq = __ballot_sync(all, c == 0);
+      cand = gt ? gt : eq;
+      if (!gt) break;
+    }
+    const bool c = ((cand >> lane) & 1u) != 0;
+    const uint64_t i = warp_min64(c ? (uint64_t)ri : ~0ull);
+    if (cand ? (c && (uint64_t)ri == i) : lane == 0) {
+      out->rel_hi = rh;
+      out->rel_lo = rl;
+      out->rel_g = rg;
+      out->rel_sc = rs;
+      out->rel_idx = ri;
+    }
+  }
+  {
+    const uint64_t v = ui < 0 ? 0ull : u;  // a recorded distance is positive
+    const uint64_t m = ~warp_min64(~v);
+    const uint64_t i = warp_min64(m && v == m ? (uint64_t)ui : ~0ull);
+    if (m ? (v == m && (uint64_t)ui == i) : lane == 0) {
+      out->ulp = u;
+      out->ulp_idx = ui;
+    }
+  }
+  // -1 (none) is the largest unsigned value
+  const uint64_t f = warp_min64((uint64_t)ff), g = warp_min64((uint64_t)fu);
+  if (lane == 0) {
+    out->first_fin = (int64_t)f;
+    out->first_ulp = (int64_t)g;
+  }
+  __syncwarp();
 }
-
+__device__ __forceinline__ void warp_best(const Partial& x, Partial* out) {
+  warp_best(x.abs_hi, x.abs_lo, x.abs_sc, x.abs_idx, x.rel_hi, x.rel_lo, x.rel_g, x.rel_sc, x.rel_idx, x.ulp, x.ulp_idx,
+            x.first_fin, x.first_ulp, out);
+}
 
 // warp sums of the general path's class counters into the CTA counters
 template <int DT>
@@ -1616,7 +1694,7 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
   const int64_t lo = sm.k.lo;
   GenRec cd;
   gen_init(cd);
-  // whole warps in every round (general_lane adds with the whole warp)
+  // whole warps in every round (general_lane counts with the whole warp)
   const uint32_t lane = threadIdx.x & 31u, w0 = threadIdx.x & ~31u;
   if (n <= (uint32_t)GCAP) {
     for (uint32_t b = w0; b < n; b += NT) {
@@ -1631,9 +1709,12 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
         C = cand_at<DT, INJ>(p, i, G);
       }
       general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, valid);
-    }
+    }  // (at most GCAP / NT rounds: no flush)
+    static_assert(GCAP / NT <= GEN_FLUSH, "rounds of the list");
   } else {
+    int rounds = 0;
     for (int64_t b = pb + w0; b < pe; b += NT) {
+      if (++rounds > GEN_FLUSH) gen_flush<DT>(sm), rounds = 1;
       const int64_t i = b + lane;
       bool want = false;
       uint32_t G = 0, C = 0;
@@ -1671,21 +1752,8 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
     }
   }
   gen_counts<DT>(cd, sm);
-  Partial x;
-  part_none(x);
-  x.abs_hi = cd.abs_hi;
-  x.abs_lo = cd.abs_lo;
-  x.abs_sc = cd.abs_sc;
-  x.abs_idx = cd.abs_idx;
-  x.rel_hi = cd.rel_hi;
-  x.rel_lo = cd.rel_lo;
-  x.rel_g = cd.rel_g;
-  x.rel_sc = cd.rel_sc;
-  x.rel_idx = cd.rel_idx;
-  x.ulp = cd.ulp;
-  x.ulp_idx = cd.ulp_idx;
-  part_warp_reduce(x);
-  if ((threadIdx.x & 31) == 0) sm.k.wbest[threadIdx.x >> 5] = x;
+  warp_best(cd.abs_hi, cd.abs_lo, cd.abs_sc, cd.abs_idx, cd.rel_hi, cd.rel_lo, cd.rel_g, cd.rel_sc, cd.rel_idx, cd.ulp,
+            cd.ulp_idx, -1, -1, &sm.k.wbest[threadIdx.x >> 5]);
   __syncthreads();
   // the per-warp totals into the CTA's
   for (int b = threadIdx.x; b < HBINS; b += NT) {
@@ -1698,13 +1766,13 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
     if (v) atomicAdd(&sm.k.hist[b], v);
   }
   for (int j = threadIdx.x; j < NSUM * NLIMB; j += NT) {
-    unsigned long long v = 0;
+    int64_t v = 0;
 #pragma unroll
     for (int w = 0; w < NW; w++) {
-      v += (&sm.k.gsacc[w][0][0])[j];
-      (&sm.k.gsacc[w][0][0])[j] = 0;
+      v += (int64_t)sm.k.gsacc[w][j][1] * 65536 + sm.k.gsacc[w][j][0];
+      sm.k.gsacc[w][j][0] = sm.k.gsacc[w][j][1] = 0;
     }
-    if (v) atomicAdd(&sm.k.sacc[0][0] + j, v);
+    if (v) atomicAdd(&sm.k.sacc[0][0] + j, (unsigned long long)v);
   }
 }
 
@@ -1898,7 +1966,7 @@ __device__ __forceinline__ void window_best(Smem<DT>& sm, Partial& x) {
 }
 
 template <int NT>
-__device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, FinScratch& f, MV& mv);
+__device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, int b0, int b1, FinScratch& f, MV& mv);
 __device__ void write_empty_segments(const CompareParams& p);
 
 // the window maxima, class counters and list of a new piece
@@ -1940,22 +2008,20 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
   if (warp == 0) {
     Partial x;
     window_best<DT>(sm, x);
-    if (gen) {
-      Partial y;
-      if (lane < NW) y = sm.k.wbest[lane];
-      else part_none(y);
-      part_warp_reduce(y);
-      if (lane == 0) part_merge(x, y);
-    }
+    const bool ok = PEAT_CHECK(seg >= 0 && seg < p.nseg && seg + (int64_t)blockIdx.x < p.nseg + p.nctas && pb <= pe &&
+                               pe <= p.n_total);
     if (lane == 0) {
       constexpr long long NONE = 0x7FFFFFFFFFFFFFFFll;
       x.first_fin = sm.k.ff == NONE ? -1 : sm.k.ff;
       x.first_ulp = sm.k.fu == NONE ? -1 : sm.k.fu;
-      if (PEAT_CHECK(seg >= 0 && seg < p.nseg && seg + (int64_t)blockIdx.x < p.nseg + p.nctas && pb <= pe &&
-                     pe <= p.n_total))
-        *out = x;
+      if (!gen && ok) *out = x;
       atomicAdd(&sm.k.cnt[0], (unsigned long long)(pe - pb));
       atomicAdd(&sm.k.cnt[3], (unsigned long long)sm.k.nfe);
+    }
+    if (gen) {  // the window's records and each warp's general ones
+      if (lane >= 1 && lane <= NW) x = sm.k.wbest[lane - 1];
+      else if (lane > NW) part_none(x);
+      if (ok) warp_best(x, out);
     }
   }
   fold_tables<DT>(sm, W);
@@ -1976,11 +2042,11 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
   if (p.nseg == 1) {
     __threadfence();
     __syncthreads();
-    if (tid == 0) sm.k.last = atomicAdd(&acc->done, 1u) == sm.k.pieces - 1u;
+    if (tid == 0) sm.k.last = atomicAdd(&acc->done, 1u) == (unsigned)(sm.k.final - sm.k.first);
     __syncthreads();
     if (sm.k.last) {
       __threadfence();
-      finalize_segment<NT>(p, seg, sm.k.fin, sm.mv);
+      finalize_segment<NT>(p, seg, sm.k.first, sm.k.final, sm.k.fin, sm.mv);
     }
   } else {
     __syncthreads();
@@ -2039,7 +2105,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
     for (int j = tid; j < Tab<DT>::N1 / 4; j += NT) tz[j] = make_uint4(0, 0, 0, 0);
   }
   for (int j = tid; j < NW * HBINS; j += NT) (&sm.k.ghist[0][0])[j] = 0;
-  for (int j = tid; j < NW * NSUM * NLIMB; j += NT) (&sm.k.gsacc[0][0][0])[j] = 0;
+  for (int j = tid; j < NW * NSUM * NLIMB * 2; j += NT) (&sm.k.gsacc[0][0][0])[j] = 0;
   const int64_t lo = p.bounds[blockIdx.x], hi = p.bounds[blockIdx.x + 1];
   if (tid == 0) {
     sm.k.lo = lo;
@@ -2058,7 +2124,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
   lane_init(L);
   if (p.nseg == 1 && p.n_total > 0 && warp == 0) {  // (counted here, off the tail of the last piece)
     const int b1 = cta_of_warp(p.n_total - 1, p), b0 = cta_of_warp(0, p);
-    if (lane == 0) sm.k.pieces = (unsigned)(b1 - b0 + 1);
+    if (lane == 0) sm.k.first = b0, sm.k.final = b1;
   }
   __syncthreads();
   if (blockIdx.x == 0 && p.has_empty) write_empty_segments(p);
@@ -2306,53 +2372,59 @@ __device__ __forceinline__ Partial load_partial(const Partial* src) {
   return x;
 }
 
-// The whole CTA, once every piece of segment s is in: merge the pieces'
-// maxima in CTA order, round the exact sums once, write the outputs and clear
-// the accumulator for the next call.  Uses the CTA's totals in shared memory
-// as scratch (they are zero on entry and on exit).
+// The whole CTA, once every piece of segment s (those of CTAs b0 .. b1) is in:
+// merge the pieces' maxima, round the exact sums once, write the outputs and clear the
+// accumulator for the next call.  Latency is all that matters here (one CTA,
+// at the end of the call): the last step of the maxima and the rounding of
+// the three sums run on warps of their own beside the mean and the variance.
 template <int NT>
-__device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, FinScratch& f, MV& mv) {
+__device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s, int b0, int b1, FinScratch& f, MV& mv) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t s0 = p.offsets[s], s1 = p.offsets[s + 1];
   SegAcc* acc = p.acc + s;
-  long long* limbs = f.limbs;
   unsigned long long hv = 0;
   if (tid < HBINS) {
     hv = __ldcg(&acc->hist[tid]);
     acc->hist[tid] = 0;
+  } else if (tid < HBINS + NSUM * NLIMB) {
+    f.limbs[tid - HBINS] = __ldcg(&acc->limbs[0][0] + (tid - HBINS));
+    (&acc->limbs[0][0])[tid - HBINS] = 0;
+  } else if (tid < HBINS + NSUM * NLIMB + 8) {
+    const int j = tid - HBINS - NSUM * NLIMB;
+    f.cnt[j] = __ldcg(&acc->cnt[j]);
+    acc->cnt[j] = 0;
+  } else if (tid == HBINS + NSUM * NLIMB + 8) {
+    acc->done = 0;
   }
-  if (tid >= HBINS && tid < HBINS + 8) {
-    f.cnt[tid - HBINS] = __ldcg(&acc->cnt[tid - HBINS]);
-    acc->cnt[tid - HBINS] = 0;
-  }
-  if (tid >= 160 && tid < 160 + NSUM * NLIMB) {
-    const int j = tid - 160;
-    limbs[j] = __ldcg(&acc->limbs[0][0] + j);
-    (&acc->limbs[0][0])[j] = 0;
-  }
-  if (tid == 0) acc->done = 0;
-  // maxima over the segment's pieces
-  Partial x;
-  part_none(x);
   {
-    const int b0 = cta_of_warp(s0, p), b1 = cta_of_warp(s1 - 1, p);
+    Partial x;
+    part_none(x);
+#pragma unroll 1
     for (int b = b0 + tid; b <= b1; b += NT) part_merge(x, load_partial(p.partials + s + b));
+    warp_best(x, &f.wbest[warp]);
   }
-  part_warp_reduce(x);
-  if (lane == 0) f.wbest[warp] = x;
   __syncthreads();
-  if (warp == 1 && lane < NSUM) f.sums[lane] = limbs_to_double(limbs + lane * NLIMB);
-  if (warp == 0) {
-    if (lane < NT / 32) x = f.wbest[lane];
-    else part_none(x);
-    part_warp_reduce(x);
-  }
-  if (tid == 64) carry_to_digits(limbs + 1 * NLIMB, NLIMB, mv.A);  // S1 = sum |d|
-  if (tid == 96) carry_to_digits(limbs + 2 * NLIMB, NLIMB, mv.B);  // S2 = sum d^2
-  // the mean and variance of |d| over the finite pairs (synchronises the block)
-  mean_var_block(mv, (uint64_t)(s1 - s0) - f.cnt[3], LIMB_LSB);
+  if (tid == 0) carry_to_digits(f.limbs + 1 * NLIMB, NLIMB, mv.A);   // S1 = sum |d|
+  if (tid == 32) carry_to_digits(f.limbs + 2 * NLIMB, NLIMB, mv.B);  // S2 = sum d^2
+  // the mean and variance of |d| over the finite pairs
+  mean_var_block(mv, (uint64_t)(s1 - s0) - f.cnt[3], LIMB_LSB, [&] {
+    if (warp == 2) {
+      Partial x;
+      if (lane < NT / 32) x = f.wbest[lane];
+      else part_none(x);
+      warp_best(x, &f.best);
+      if (lane == 0) {
+        const Partial& y = f.best;
+        f.max_abs = y.abs_idx >= 0 ? __dadd_rn((double)y.abs_hi, (double)y.abs_lo) * (y.abs_sc ? 2.0 : 1.0) : 0.0;
+        f.max_rel = y.rel_idx >= 0 ? rel_value(y.rel_hi, y.rel_lo, y.rel_sc, y.rel_g) : 0.0;
+      }
+    } else if (warp == 3 && lane < NSUM) {
+      f.sums[lane] = limbs_to_double(f.limbs + lane * NLIMB);
+    }
+  });
   if (tid == 0) {
     const unsigned long long* cnt = f.cnt;
+    const Partial& x = f.best;
     peat_stats_t r;
     const uint64_t n = (uint64_t)(s1 - s0);
     r.n = n;
@@ -2362,20 +2434,11 @@ __device__ __noinline__ void finalize_segment(const CompareParams& p, int64_t s,
     r.count[PEAT_NAN_INF_ASYM] = cnt[6];
     r.count[PEAT_SIGN_FLIP] = cnt[7];
     r.n_finite = n - cnt[3];
-    if (x.abs_idx >= 0) {
-      r.max_abs = __dadd_rn((double)x.abs_hi, (double)x.abs_lo) * (x.abs_sc ? 2.0 : 1.0);
-      r.argmax_abs = x.abs_idx - s0;
-    } else {
-      r.max_abs = 0.0;
-      r.argmax_abs = x.first_fin >= 0 ? x.first_fin - s0 : -1;
-    }
-    if (x.rel_idx >= 0) {
-      r.max_rel = rel_value(x.rel_hi, x.rel_lo, x.rel_sc, x.rel_g);
-      r.argmax_rel = x.rel_idx - s0;
-    } else {
-      r.max_rel = 0.0;
-      r.argmax_rel = x.first_fin >= 0 ? x.first_fin - s0 : -1;
-    }
+    const int64_t first = x.first_fin >= 0 ? x.first_fin - s0 : -1;
+    r.max_abs = f.max_abs;
+    r.argmax_abs = x.abs_idx >= 0 ? x.abs_idx - s0 : first;
+    r.max_rel = f.max_rel;
+    r.argmax_rel = x.rel_idx >= 0 ? x.rel_idx - s0 : first;
     if (x.ulp_idx >= 0) {
       r.max_ulp = x.ulp;
       r.argmax_ulp = x.ulp_idx - s0;
@@ -2403,7 +2466,8 @@ __global__ void __launch_bounds__(BLOCK) compare_finalize(CompareParams p) {
   __shared__ FinScratch f;
   __shared__ MV mv;
   pdl_wait();  // stage 1 complete
-  if (p.offsets[blockIdx.x] < p.offsets[blockIdx.x + 1]) finalize_segment<BLOCK>(p, blockIdx.x, f, mv);
+  const int64_t s0 = p.offsets[blockIdx.x], s1 = p.offsets[blockIdx.x + 1];
+  if (s0 < s1) finalize_segment<BLOCK>(p, blockIdx.x, cta_of_warp(s0, p), cta_of_warp(s1 - 1, p), f, mv);
 }
 
 // The outputs of every empty segment (no pairs): zero counts and sums, argmax -1.

@@ -203,35 +203,30 @@ __device__ inline void carry_to_digits(const long long* src, int n, uint32_t* ou
   out[n + 1] = (uint32_t)((unsigned long long)carry >> 32);
 }
 
-// A barrier of nt threads (a multiple of 32): the block's own barrier for
-// id 0, else the named barrier id (only the group's threads take part).
-__device__ __forceinline__ void group_sync(int id, int nt) {
-  if (id == 0) __syncthreads();
-  else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nt) : "memory");
-}
-
-// Called by every thread of a group of nt threads (t = 0 .. nt - 1, barrier
-// id bar) once s.A and s.B hold S1 and S2 (written by threads of the group);
-// leaves s.mean and s.var for every thread of the group.  n_f S2 - S1^2 is
-// never negative (Cauchy-Schwarz over the n_f values |d|), so the carry
-// propagation below ends without a borrow.  The mean (thread 32) and the
-// carries and the variance (thread 0) run side by side on two warps.
-template <int NA, int NB, int SHB>
-__device__ void mean_var_group(MeanVarScratch<NA, NB, SHB>& s, uint64_t nf, int e1, int t, int nt, int bar) {
+// Called by every thread of the block once s.A and s.B hold S1 and S2
+// (written by threads of the block); leaves s.mean and s.var for all of them.
+// n_f S2 - S1^2 is never negative (Cauchy-Schwarz over the n_f values |d|),
+// so the carry propagation below ends without a borrow.  The mean (thread 32)
+// and the carries and the variance (thread 0) run side by side on two warps,
+// and side() beside them on the others (it synchronises no more than a warp).
+template <int NA, int NB, int SHB, class Side>
+__device__ void mean_var_block(MeanVarScratch<NA, NB, SHB>& s, uint64_t nf, int e1, Side&& side) {
+  const int t = (int)threadIdx.x, nt = (int)blockDim.x;
   constexpr int ND = MeanVarScratch<NA, NB, SHB>::ND;
-  group_sync(bar, nt);
+  __syncthreads();
   // the nonzero digit ranges: the loops below skip the zeros around them
   int la = NA, ta = -1, lb = NB, tb = -1;
-  for (int i = 0; i < NA; i++)
-    if (s.A[i]) {
-      la = min(la, i);
-      ta = i;
-    }
-  for (int i = 0; i < NB; i++)
-    if (s.B[i]) {
-      lb = min(lb, i);
-      tb = i;
-    }
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int b = 0; b < NA; b += 32) {
+    const unsigned nz = __ballot_sync(0xFFFFFFFFu, b + lane < NA && s.A[b + lane] != 0u);
+    if (nz) la = min(la, b + __ffs(nz) - 1), ta = b + 31 - __clz(nz);
+  }
+#pragma unroll
+  for (int b = 0; b < NB; b += 32) {
+    const unsigned nz = __ballot_sync(0xFFFFFFFFu, b + lane < NB && s.B[b + lane] != 0u);
+    if (nz) lb = min(lb, b + __ffs(nz) - 1), tb = b + 31 - __clz(nz);
+  }
   for (int c = 2 * la + t; c <= 2 * ta; c += nt) {
     unsigned __int128 acc = 0;
     const int i0 = max(la, c - ta), i1 = min(ta, c - la);
@@ -245,7 +240,7 @@ __device__ void mean_var_group(MeanVarScratch<NA, NB, SHB>& s, uint64_t nf, int 
   // on (past the last carry).
   const int j0 = ta < 0 ? 0 : (tb >= 0 ? min(2 * la, SHB + lb) : 2 * la);
   const int j1 = ta < 0 ? 0 : min(ND, max(2 * ta + 4, tb >= 0 ? SHB + tb + 4 : 0));
-  group_sync(bar, nt);
+  __syncthreads();
   for (int j = j0 + t; j < j1; j += nt) {
     long long v = 0;
 #pragma unroll
@@ -257,32 +252,36 @@ __device__ void mean_var_group(MeanVarScratch<NA, NB, SHB>& s, uint64_t nf, int 
     }
     s.t[j] = v;
   }
-  group_sync(bar, nt);
-  const int tmean = nt > 32 ? 32 : 0;
-  if (t == tmean) s.mean = (nf == 0 || ta < 0) ? 0.0 : digits_quot_rn(s.A, ta + 1, nf, e1);
+  for (int j = t; j < j0; j += nt) s.N[j] = 0;  // (the digits from j1 on are not read)
+  __syncthreads();
+  if (t >= 64) side();
+  if (t == 32) s.mean = (nf == 0 || ta < 0) ? 0.0 : digits_quot_rn(s.A, ta + 1, nf, e1);
   if (t == 0) {
     if (nf == 0 || ta < 0) {
       s.var = 0.0;
     } else {
       // carry propagation (64-bit arithmetic shifts; the final carry is 0 as N >= 0)
-      for (int j = 0; j < j0; j++) s.N[j] = 0;
       long long carry = 0;
-      for (int j = j0; j < j1; j++) {
-        const long long v = s.t[j] + carry;
-        s.N[j] = (uint32_t)v;
-        carry = v >> 32;
+      for (int j = j0; j < j1; j += 8) {  // eight loads at a time, then their chain
+        long long v[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) v[q] = j + q < j1 ? s.t[j + q] : 0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          const long long x = v[q] + carry;
+          if (j + q < j1) s.N[j + q] = (uint32_t)x;
+          carry = x >> 32;
+        }
       }
-      for (int j = j1; j < ND; j++) s.N[j] = 0;
       s.var = nf < (1ull << 32) ? digits_quot_rn(s.N, j1, nf * nf, 2 * e1) : digits_div_rn(s.N, j1, nf, 2, 2 * e1);
     }
   }
-  group_sync(bar, nt);
+  __syncthreads();
 }
 
-// the same with the whole block as the group (every thread calls it)
 template <int NA, int NB, int SHB>
 __device__ void mean_var_block(MeanVarScratch<NA, NB, SHB>& s, uint64_t nf, int e1) {
-  mean_var_group(s, nf, e1, (int)threadIdx.x, (int)blockDim.x, 0);
+  mean_var_block(s, nf, e1, [] {});
 }
 
 }  // namespace peat
