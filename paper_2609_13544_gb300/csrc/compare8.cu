@@ -426,6 +426,96 @@ __device__ __forceinline__ void eval_cell(const unsigned long long* amax, Tot& t
   atomicAdd(H + 64 + ulpbin, n);
 }
 
+// Every pair evaluated by itself: the whole of a call with fewer than
+// C8_TABLE_MIN pairs, where the passes over the table and the search for the
+// maxima's first pairs would cost more than they save.
+constexpr int DTB = 256;
+template <int DT>
+__global__ void __launch_bounds__(DTB) compare8_direct(Cmp8Params p) {
+  __shared__ unsigned H[PEAT_HIST_BINS];
+  __shared__ Tot warp_tot[DTB / 32];
+  __shared__ unsigned long long AM[128];
+  pdl_trigger();  // the finalize kernel may start launching (it waits for this grid)
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x; k < 128; k += DTB) AM[k] = p.amax[k];
+  for (long long item = blockIdx.x; item < p.nitems; item += gridDim.x) {
+    const long long b = p.item_b[item], e = p.item_e[item], seg = p.item_seg[item];
+    const long long base = p.offsets[seg];  // indices are reported within the segment
+    for (int k = threadIdx.x; k < PEAT_HIST_BINS; k += DTB) H[k] = 0u;
+    __syncthreads();
+    Acc8<DT> acc;
+    acc_init(acc);
+    uint32_t nsame = 0;  // pairs of the equal-group fast path (rel and ULP bin 0)
+    // groups of 16 elements on the absolute index grid, whole warps in every round
+    const long long q0 = b >> 4, q1 = (e + 15) >> 4;
+    for (long long q = q0 + threadIdx.x; __any_sync(0xFFFFFFFFu, q < q1); q += DTB) {
+      const bool okq = q < q1;
+      const long long i0 = q << 4;
+      uint32_t w[4] = {0u, 0u, 0u, 0u}, x[4] = {0u, 0u, 0u, 0u};
+      if (okq && p.vec && i0 >= b && i0 + 16 <= e) {
+        const uint4 gv = __ldg(reinterpret_cast<const uint4*>(p.g) + q);
+        const uint4 cv = __ldg(reinterpret_cast<const uint4*>(p.c) + q);
+        w[0] = gv.x, w[1] = gv.y, w[2] = gv.z, w[3] = gv.w;
+        x[0] = cv.x, x[1] = cv.y, x[2] = cv.z, x[3] = cv.w;
+      } else if (okq) {
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+          const long long i = i0 + j;
+          if (i >= b && i < e) {
+            w[j >> 2] |= (uint32_t)__ldg(reinterpret_cast<const unsigned char*>(p.g) + i) << (8 * (j & 3));
+            x[j >> 2] |= (uint32_t)__ldg(reinterpret_cast<const unsigned char*>(p.c) + i) << (8 * (j & 3));
+          }
+        }
+      }
+      // a warp slot of bitwise-equal, finite whole groups (decided for the whole warp):
+      // 16 EXACT pairs per lane with |d| = 0 and u = 0
+      bool fast = !okq;
+      if (okq && p.vec && i0 >= b && i0 + 16 <= e && w[0] == x[0] && w[1] == x[1] && w[2] == x[2] && w[3] == x[3]) {
+        bool fin = true;
+#pragma unroll
+        for (int j = 0; j < 16; j++) fin &= f8_kind<DT>((w[j >> 2] >> (8 * (j & 3))) & 0x7Fu) == 0;
+        fast = fin;
+      }
+      if (__all_sync(0xFFFFFFFFu, fast)) {
+        if (okq) {
+          const uint32_t off = (uint32_t)(i0 - b);
+          acc.cnt[PEAT_EXACT] += 16;
+          acc.nfin += 16;
+          if (acc.ia == 0) acc.ma = 0, acc.ia = off + 1;
+          if (acc.ir == 0) acc.ra = 0, acc.rb = 1, acc.ir = off + 1, acc.rt = 0.0f;
+          if (acc.iu == 0) acc.mu = 0, acc.iu = off + 1;
+          nsame += 16;
+        }
+        continue;
+      }
+      // one copy of the pair code: the loop stays rolled (the body is long)
+#pragma unroll 1
+      for (int j = 0; j < 16; j++) {
+        const long long i = i0 + j;
+        const bool ok = okq && i >= b && i < e;
+        const uint32_t gw = j < 8 ? (j < 4 ? w[0] : w[1]) : (j < 12 ? w[2] : w[3]);
+        const uint32_t cw = j < 8 ? (j < 4 ? x[0] : x[1]) : (j < 12 ? x[2] : x[3]);
+        pair8<DT>(AM, acc, H, (gw >> (8 * (j & 3))) & 0xFFu, (cw >> (8 * (j & 3))) & 0xFFu, ok, (uint32_t)(i - b));
+      }
+    }
+    {
+      const uint32_t ns = __reduce_add_sync(0xFFFFFFFFu, nsame);
+      if (lane == 0 && ns) {
+        atomicAdd(&H[0], ns);
+        atomicAdd(&H[64], ns);
+      }
+    }
+    Tot t;
+    acc_to_tot<DT>(t, acc, b - base);
+    block_total(t, warp_tot);
+    if (threadIdx.x == 0) store_tot(p.parts + item, t);
+    if (p.hist)
+      for (int k = threadIdx.x; k < PEAT_HIST_BINS; k += DTB)
+        if (H[k]) atomicAdd(p.hist + seg * PEAT_HIST_BINS + k, (unsigned long long)H[k]);
+    __syncthreads();
+  }
+}
+
 template <int DT>
 __global__ void __launch_bounds__(TB, 1) compare8_stage1(Cmp8Params p) {
   extern __shared__ __align__(16) uint32_t T[];  // CELLS counters, then the list
@@ -477,9 +567,10 @@ __global__ void __launch_bounds__(TB, 1) compare8_stage1(Cmp8Params p) {
       load(v + TB, gn, cn);
       const int o = o0 + 16 * v;
       const uint32_t w[4] = {gc.x, gc.y, gc.z, gc.w}, x[4] = {cc.x, cc.y, cc.z, cc.w};
-      const bool odd = (((w[0] ^ x[0]) | (w[1] ^ x[1]) | (w[2] ^ x[2]) | (w[3] ^ x[3])) & 0x80808080u) != 0u || o < 0 ||
-                       o + 16 > len;
-      if (!__any_sync(0xFFFFFFFFu, odd)) {
+      const bool edge = o < 0 || o + 16 > len;
+      const bool odd = (((w[0] ^ x[0]) | (w[1] ^ x[1]) | (w[2] ^ x[2]) | (w[3] ^ x[3])) & 0x80808080u) != 0u || edge;
+      const bool odd_w = __any_sync(0xFFFFFFFFu, odd);
+      if (!odd_w || !__any_sync(0xFFFFFFFFu, edge)) {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
           const uint32_t c0 = cells2(w[i], x[i]), c1 = cells2(w[i] >> 8, x[i] >> 8);
@@ -488,9 +579,27 @@ __global__ void __launch_bounds__(TB, 1) compare8_stage1(Cmp8Params p) {
           inc_cell(table, c1 & 0xFFFFu);
           inc_cell(table, c1 >> 16);
         }
+        if (!odd_w) continue;
+        // pairs of opposite signs: taken back from the table and done one by
+        // one, the lanes that still have some together
+        uint32_t todo = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) todo |= ((((w[i] ^ x[i]) >> 7 & 0x01010101u) * 0x01020408u) >> 24 & 0xFu) << (4 * i);
+        any_slow = 1;
+#pragma unroll 1
+        while (__any_sync(0xFFFFFFFFu, todo != 0u)) {
+          const bool ok = todo != 0u;
+          const int j = ok ? __ffs(todo) - 1 : 0;
+          todo &= todo - 1u;
+          const uint32_t gw = j < 8 ? (j < 4 ? w[0] : w[1]) : (j < 12 ? w[2] : w[3]);
+          const uint32_t cw = j < 8 ? (j < 4 ? x[0] : x[1]) : (j < 12 ? x[2] : x[3]);
+          const uint32_t G = (gw >> (8 * (j & 3))) & 0xFFu, C = (cw >> (8 * (j & 3))) & 0xFFu;
+          if (ok) atomicSub(T + (G * 128u + (C & 0x7Fu)), 1u);
+          pair8_slow<DT>(AM, acc, H, G, C, ok, (uint32_t)(o + j));
+        }
         continue;
       }
-      // a group at an item's edge, or with a pair of opposite signs
+      // groups at an item's edge
 #pragma unroll 1
       for (int j = 0; j < 16; j++) {
         const uint32_t gw = j < 8 ? (j < 4 ? w[0] : w[1]) : (j < 12 ? w[2] : w[3]);
@@ -566,6 +675,44 @@ __device__ double u128_to_double(u128 x) {
   return ldexp(__ull2double_rn(top), 64 - sh);
 }
 
+// The segment's totals (thread 0's t) rounded and written (every thread calls it).
+template <int DT>
+__device__ void write_stats(const Cmp8Params& p, long long seg, const Tot& t, MeanVarScratch<4, 4, 0>& mv,
+                            unsigned long long& nfin) {
+  constexpr int S = F8<DT>::S;
+  if (threadIdx.x == 0) {
+    for (int j = 0; j < 4; j++) {
+      mv.A[j] = (uint32_t)(t.s1 >> (32 * j));
+      mv.B[j] = (uint32_t)(t.s2 >> (32 * j));
+    }
+    nfin = t.nfin;
+  }
+  __syncthreads();
+  mean_var_block(mv, nfin, -S);
+  if (threadIdx.x != 0) return;
+  peat_stats_t r;
+  r.n = (uint64_t)(p.offsets[seg + 1] - p.offsets[seg]);
+  for (int k = 0; k < PEAT_NCLASS; k++) r.count[k] = t.cnt[k];
+  r.n_finite = t.nfin;
+  r.max_abs = t.ia >= 0 ? ldexp((double)t.ma, -S) : 0.0;
+  r.argmax_abs = t.ia;
+  if (t.ir < 0 || t.ra == 0) r.max_rel = 0.0;
+  else if (t.rb == 0) r.max_rel = __longlong_as_double(0x7FF0000000000000ll);
+  else r.max_rel = __ddiv_rn((double)t.ra, (double)t.rb);  // both exact in binary64: one rounding
+  r.argmax_rel = t.ir;
+  r.max_ulp = t.iu >= 0 ? t.mu : 0;
+  r.argmax_ulp = t.iu;
+  r.sum_abs = ldexp(u128_to_double(t.s1), -S);
+  r.sum_sq = ldexp(u128_to_double(t.s2), -2 * S);
+  const double sdm = ldexp(u128_to_double(t.sd < 0 ? (u128)(-t.sd) : (u128)t.sd), -S);
+  r.sum_signed = t.sd < 0 ? -sdm : sdm;
+  r.rtol_eff = (double)p.rtol;
+  r.atol_eff = (double)p.atol;
+  r.mean_abs = mv.mean;
+  r.var_abs = mv.var;
+  p.stats[seg] = r;
+}
+
 // One cluster of CL CTAs per segment: every CTA merges the items (a few KB), and
 // the search for the first pair of a maximum is split over them.
 constexpr int CL = 8;
@@ -579,7 +726,6 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(FB) compare8_finali
   __shared__ MeanVarScratch<4, 4, 0> mv;
   __shared__ unsigned long long nfin;
   pdl_wait();  // stage 1 complete
-  constexpr int S = F8<DT>::S;
   const long long seg = blockIdx.x / CL;
   const unsigned rank = blockIdx.x % CL;
   // the items' table values (their index: the item, so that the first one wins
@@ -720,44 +866,39 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(FB) compare8_finali
     o.ia = where[0], o.ir = where[1], o.iu = where[2];
     tot_merge(t, o);
   }
-  if (threadIdx.x == 0) {
-    for (int j = 0; j < 4; j++) {
-      mv.A[j] = (uint32_t)(t.s1 >> (32 * j));
-      mv.B[j] = (uint32_t)(t.s2 >> (32 * j));
-    }
-    nfin = t.nfin;
+  write_stats<DT>(p, seg, t, mv, nfin);
+}
+
+// the same for items of compare8_direct, one record each
+template <int DT>
+__global__ void __launch_bounds__(DTB) compare8_finalize_direct(Cmp8Params p) {
+  __shared__ Tot warp_tot[DTB / 32];
+  __shared__ MeanVarScratch<4, 4, 0> mv;
+  __shared__ unsigned long long nfin;
+  pdl_wait();
+  const long long seg = blockIdx.x;
+  Tot t;
+  tot_init(t);
+  for (long long it = p.seg_first[seg] + threadIdx.x; it < p.seg_first[seg + 1]; it += DTB) {
+    Tot o;
+    load_tot(o, p.parts + it);
+    tot_merge(t, o);
   }
-  __syncthreads();
-  mean_var_block(mv, nfin, -S);
-  if (threadIdx.x != 0) return;
-  peat_stats_t r;
-  r.n = (uint64_t)(p.offsets[seg + 1] - p.offsets[seg]);
-  for (int k = 0; k < PEAT_NCLASS; k++) r.count[k] = t.cnt[k];
-  r.n_finite = t.nfin;
-  r.max_abs = t.ia >= 0 ? ldexp((double)t.ma, -S) : 0.0;
-  r.argmax_abs = t.ia;
-  if (t.ir < 0 || t.ra == 0) r.max_rel = 0.0;
-  else if (t.rb == 0) r.max_rel = __longlong_as_double(0x7FF0000000000000ll);
-  else r.max_rel = __ddiv_rn((double)t.ra, (double)t.rb);  // both exact in binary64: one rounding
-  r.argmax_rel = t.ir;
-  r.max_ulp = t.iu >= 0 ? t.mu : 0;
-  r.argmax_ulp = t.iu;
-  r.sum_abs = ldexp(u128_to_double(t.s1), -S);
-  r.sum_sq = ldexp(u128_to_double(t.s2), -2 * S);
-  const double sdm = ldexp(u128_to_double(t.sd < 0 ? (u128)(-t.sd) : (u128)t.sd), -S);
-  r.sum_signed = t.sd < 0 ? -sdm : sdm;
-  r.rtol_eff = (double)p.rtol;
-  r.atol_eff = (double)p.atol;
-  r.mean_abs = mv.mean;
-  r.var_abs = mv.var;
-  p.stats[seg] = r;
+  block_total(t, warp_tot);
+  write_stats<DT>(p, seg, t, mv, nfin);
 }
 
 template <int DT>
 cudaError_t launch_t(const Cmp8Params& p, int nctas, cudaStream_t s) {
   if (p.nitems == 0) {
-    compare8_finalize<DT><<<(unsigned)p.nseg * CL, FB, 0, s>>>(p);
+    compare8_finalize_direct<DT><<<(unsigned)p.nseg, DTB, 0, s>>>(p);
     return cudaGetLastError();
+  }
+  if (p.direct) {
+    compare8_direct<DT><<<nctas, DTB, 0, s>>>(p);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_dependent(compare8_finalize_direct<DT>, (unsigned)p.nseg, DTB, 0, s, p);
   }
   compare8_stage1<DT><<<nctas, TB, SMEM8, s>>>(p);
   const cudaError_t e = cudaGetLastError();

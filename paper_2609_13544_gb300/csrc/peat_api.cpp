@@ -346,7 +346,9 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
                                    int64_t nseg, int dtype, float rtol, float atol, peat_stats_t* stats,
                                    uint64_t* hist, cudaStream_t st) {
   Items it;
-  peat_status_t ps = stage_items(h, offsets, nseg, 2 * sizeof(peat::Part8), 1, (int64_t)1 << 20, st, &it);
+  const bool direct = offsets[nseg] < peat::C8_TABLE_MIN;  // (a rule on the size, see there)
+  peat_status_t ps = direct ? stage_items(h, offsets, nseg, sizeof(peat::Part8), 4, (int64_t)1 << 20, st, &it)
+                            : stage_items(h, offsets, nseg, 2 * sizeof(peat::Part8), 1, (int64_t)1 << 20, st, &it);
   if (ps != PEAT_OK) return ps;
   cudaError_t e;
   if (hist) {
@@ -383,7 +385,8 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
   p.parts = static_cast<peat::Part8*>(it.parts);
   p.stats = stats;
   p.hist = reinterpret_cast<unsigned long long*>(hist);
-  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>(it.nitems, (int64_t)h->nsm));
+  p.direct = direct ? 1 : 0;
+  const int nctas = (int)std::max<int64_t>(1, std::min<int64_t>(it.nitems, (int64_t)h->nsm * (direct ? 4 : 1)));
   e = peat::launch_compare8(dtype, p, nctas, st);
   if (e != cudaSuccess) return cuda_fail(h, e, "8-bit compare launch");
   return PEAT_OK;

@@ -262,10 +262,17 @@ struct Cmp8Params {
   // floor(rtol |g| 2^S + atol 2^S) (2^40 when it exceeds every possible difference)
   unsigned long long amax[128];
   int vec;                   // both bases 16-byte aligned
-  Part8* parts;              // 2 nitems: the table's totals, and those of the pairs of opposite signs
+  int direct;                // fewer than C8_TABLE_MIN pairs: no table
+  Part8* parts;              // direct: nitems; else 2 nitems: the table's totals, and those of the other pairs
   peat_stats_t* stats;       // nseg
   unsigned long long* hist;  // nseg x 128, zero before the launch; NULL: none
 };
+// Pairs from which a call counts combinations in tables (measured, E4M3 noise
+// of one spacing): 3.0 M 72 us pair by pair, 56 with tables; 1.3 M 42 and 58;
+// E5M2 with 0.2 % of opposite signs at 4.2 M 84 and 71.  The line is higher
+// than those need because pairs of opposite signs are evaluated one by one
+// beside the table (4.3 M E5M2 with 5 % of them: 98 with tables, 86 without).
+constexpr int64_t C8_TABLE_MIN = 1 << 22;
 cudaError_t compare8_prepare();  // once per device, before the first launch
 cudaError_t launch_compare8(int dtype, const Cmp8Params& p, int nctas, cudaStream_t s);
 

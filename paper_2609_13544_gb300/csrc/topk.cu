@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
   const unsigned Plo = d > 0 ? d - 1 : 0, Phi = min(d + 1, (unsigned)TK_NB0 - 1);
   uint32_t mode = 0;
   unsigned Tlo = Plo;
-  if (tot > 0) {  // the same in every thread
+  if (tot > 0 && p.tabled) {  // the same in every thread
     // The table starts at the window.  When the window starts at zero (most
     // pairs equal) the few that differ lie far above it: the table then ends
     // at the sample's largest digit, all but one pair in 4096, and only zeros
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(TB) topk_sample(TopkParams p) {
     out = block_sum(out);
     const bool any15 = __syncthreads_or((int)(l & (0x80000000u | COPY_MASK)));
     const bool any10 = __syncthreads_or((int)(l & 0x800003FFu));
-    mode = !p.tabled || any10 || out > 2 * few ? 0u : any15 ? 1u : 2u;
+    mode = any10 || out > 2 * few ? 0u : any15 ? 1u : 2u;
   }
   for (int b = threadIdx.x; b < TK_NB0; b += TB) st->hist0[b] = st->low[b] = 0;
   if (threadIdx.x == 0) {

@@ -1,5 +1,6 @@
-"""The 8-bit compare's table of (golden, candidate) combinations against the
-oracle: every pair of patterns, ties of the maxima in many places, item and
+"""The 8-bit compare, short items pair by pair and longer ones (from about
+4 M elements) through a table of (golden, candidate) combinations, against
+the oracle: every pair of patterns, ties of the maxima in many places, item and
 vector edges, opposite signs, all-equal tensors and segments."""
 import numpy as np
 import pytest
@@ -31,24 +32,29 @@ def check(peat_gpu, oracle, g, c, dtype, rtol, atol, ctx, offsets=None, shift=0)
 
 @pytest.mark.parametrize("dtype", TDT)
 @pytest.mark.parametrize("rtol,atol", ((0.125, 0.0), (0.0, 0.0), (0.1, 0.01)))
-def test_every_pair(peat_gpu, oracle, dtype, rtol, atol):
-    """All 65536 combinations in a random order, twice; then those of one sign, and without the non-finite ones."""
+@pytest.mark.parametrize("least", (131_072, 1 << 22))
+def test_every_pair(peat_gpu, oracle, dtype, rtol, atol, least):
+    """All 65536 combinations in a random order; then those of one sign, and without the non-finite ones; those of
+    opposite signs, and a few of them among the others."""
     rng = np.random.default_rng(1)
-    idx = rng.permutation(np.tile(np.arange(65536), 2))
+    idx = np.arange(65536)
     g, c = (idx >> 8).astype(np.uint8), (idx & 255).astype(np.uint8)
-    check(peat_gpu, oracle, g, c, dtype, rtol, atol, "all")
-    k = ((g ^ c) & 0x80) == 0
-    check(peat_gpu, oracle, g[k], c[k], dtype, rtol, atol, "one sign")
-    k &= ((g & 0x7F) < 0x78) & ((c & 0x7F) < 0x78)
-    check(peat_gpu, oracle, g[k], c[k], dtype, rtol, atol, "finite")
-    k &= (g & 0x7F) != 0
-    check(peat_gpu, oracle, g[k], c[k], dtype, rtol, atol, "no zero golden")
-    k = ((g ^ c) & 0x80) != 0
-    check(peat_gpu, oracle, g[k], c[k], dtype, rtol, atol, "opposite signs")
+
+    def run(k, ctx):
+        i = rng.permutation(np.tile(idx[k], -(-least // int(k.sum()))))
+        check(peat_gpu, oracle, g[i], c[i], dtype, rtol, atol, ctx)
+    run(idx >= 0, "all")
+    one = ((g ^ c) & 0x80) == 0
+    run(~one, "opposite signs")
+    run(one | (idx % 101 == 0), "few of opposite signs")
+    run(one, "one sign")
+    one &= ((g & 0x7F) < 0x78) & ((c & 0x7F) < 0x78)
+    run(one, "finite")
+    run(one & ((g & 0x7F) != 0), "no zero golden")
 
 
 @pytest.mark.parametrize("dtype", TDT)
-@pytest.mark.parametrize("n", (1, 15, 16, 17, 4095, 4096, 4097, 16385, 700_001))
+@pytest.mark.parametrize("n", (1, 15, 16, 17, 4095, 4096, 4097, 16385, 700_001, (1 << 22) - 1, (1 << 22) + 77))
 @pytest.mark.parametrize("shift", (0, 5))
 def test_edges(peat_gpu, oracle, dtype, n, shift):
     rng = np.random.default_rng(n)
@@ -59,14 +65,15 @@ def test_edges(peat_gpu, oracle, dtype, n, shift):
 
 
 @pytest.mark.parametrize("dtype", TDT)
-def test_segments_and_ties(peat_gpu, oracle, dtype):
+@pytest.mark.parametrize("scale", (1, 15))
+def test_segments_and_ties(peat_gpu, oracle, dtype, scale):
     rng = np.random.default_rng(3)
-    n = 300_000
+    n = 300_000 * scale
     g = np.full(n, 0x41, np.uint8)
     c = g.copy()
-    c[100_001:] = 0x42
-    c[250_000:] = 0xC1
-    off = [0, 0, 7, 100_000, 100_003, 250_000, 250_000, n]
+    c[100_001 * scale:] = 0x42
+    c[250_000 * scale:] = 0xC1
+    off = [0, 0, 7, 100_000 * scale, 100_003 * scale, 250_000 * scale, 250_000 * scale, n]
     check(peat_gpu, oracle, g, c, dtype, 0.01, 0.0, "constant", off)
     g = rng.integers(0, 256, n).astype(np.uint8)
     check(peat_gpu, oracle, g, rng.permutation(g), dtype, 0.01, 0.0, "random", off)
