@@ -1025,6 +1025,12 @@ __device__ __forceinline__ Bounds read_bounds(const Smem<DT>& sm, uint32_t tli, 
   return b;
 }
 
+// atomicMax of a 64-bit shared key (a compare-and-swap loop that every warp of
+// a CTA would run for every vector here) only where it raises the key
+__device__ __forceinline__ void raise_key(unsigned long long* k, unsigned long long v) {
+  if (v > *reinterpret_cast<volatile unsigned long long*>(k)) atomicMax(k, v);
+}
+
 // One vector position of a staged tile, all lanes of the warp, when some pair
 // of it is out of the window or above a bound: pairs out of the window go to
 // the general list, the window maxima into the CTA's records, and the tile's
@@ -1045,6 +1051,7 @@ __device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, ui
   E* g = reinterpret_cast<E*>(gt);
   E* c = reinterpret_cast<E*>(ct);
   float ba = 0.0f, rq = 0.0f, ra = 0.0f, rg = 1.0f;
+  const float qlow = __uint_as_float((uint32_t)(*reinterpret_cast<volatile unsigned long long*>(&sm.k.krel) >> 32));
   uint32_t ai = 0, bu = 0, ui = 0, ri = 0, nd = 0, ne = 0, nf = 0, em = 0, um0 = 0;
   {
 #pragma unroll 1
@@ -1076,6 +1083,8 @@ __device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, ui
       const float ag = fabsf(gf);
       if (a > ba) ba = a, ai = li0 + j;
       if (u > bu) bu = u, ui = li0 + j;
+      // the ratio only where it can reach the CTA's best (the margin covers the reciprocal's error)
+      if (__fmul_rn(__fmul_rn(a, rcp_approx(ag)), 1.00001f) < qlow) continue;
       if constexpr (DT == PEAT_F32) {
         if (rel_greater(a, ag, ra, rg)) ra = a, rg = ag, ri = li0 + j;
       } else {
@@ -1097,14 +1106,14 @@ __device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, ui
   const uint32_t am = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(ba));
   if (am) {
     const unsigned who = __ballot_sync(0xFFFFFFFFu, __float_as_uint(ba) == am);
-    if (lane == __ffs(who) - 1) atomicMax(&sm.k.kabs, ((unsigned long long)am << 32) | (uint32_t)~ai);
+    if (lane == __ffs(who) - 1) raise_key(&sm.k.kabs, ((unsigned long long)am << 32) | (uint32_t)~ai);
   }
   const uint32_t um = __reduce_max_sync(0xFFFFFFFFu, bu);
   if (um) {
     const unsigned who = __ballot_sync(0xFFFFFFFFu, bu == um);
-    if (lane == __ffs(who) - 1) atomicMax(&sm.k.kulp, ((unsigned long long)um << 32) | (uint32_t)~ui);
+    if (lane == __ffs(who) - 1) raise_key(&sm.k.kulp, ((unsigned long long)um << 32) | (uint32_t)~ui);
   }
-  if (am) {
+  if (__any_sync(0xFFFFFFFFu, ra > 0.0f)) {
     RelRec& R = sm.k.wrel[warp];
     if constexpr (DT == PEAT_F32) {
       // the lanes near the best approximate ratio, in order, compared exactly
