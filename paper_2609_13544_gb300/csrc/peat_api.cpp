@@ -149,14 +149,18 @@ bool round_tol(peat_tol_t tol, float* r, float* a) {
 }
 
 // CTA ranges of a segmented call.  A CTA pays for its elements and, per
-// segment piece it meets, a fixed CTA-wide merge worth about PIECE_COST
-// elements.  For a capacity C, a greedy walk over the segments gives the
+// segment piece it meets, a fixed CTA-wide merge (its tables, its maxima, its
+// sums) worth about piece_cost elements.  For a capacity C, a greedy walk over the segments gives the
 // fewest CTAs with cost <= C each (cutting a segment where a CTA fills up);
 // a bisection on C finds the smallest capacity that fits in max_ctas CTAs,
 // i.e. one wave.  Writes out[0..nctas] and returns nctas (0: no split fits).
-constexpr int64_t PIECE_COST = 8192;
+// Measured (GPT-2 list, binary16, 292 tensors / 151 tensors of 22.9 M binary16
+// elements / ResNet-50 list, float32, 161 tensors): 8192 elements a piece 470 /
+// 160 / 116 us, 24 576 458 / 119 / 111, 40 960 446 / 85 / 112, 57 344 435 / 78 /
+// 114, 81 920 443 / 75 / 121.
+int64_t piece_cost(int dtype) { return dtype == PEAT_F32 ? 24576 : 57344; }
 
-int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t C, int cap, int64_t* out) {
+int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t C, int cap, int64_t* out) {
   int nct = 0;
   out[0] = 0;
   int64_t cost = 0;
@@ -164,13 +168,13 @@ int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t C, int cap
     int64_t pos = off[s];
     const int64_t s1 = off[s + 1];
     while (pos < s1) {
-      if (cost > 0 && cost + PIECE_COST >= C) {  // no room for another piece: close the CTA
+      if (cost > 0 && cost + pc >= C) {  // no room for another piece: close the CTA
         if (nct == cap) return 0;
         out[++nct] = pos;
         cost = 0;
       }
-      const int64_t take = std::min(s1 - pos, std::max<int64_t>(1, C - cost - PIECE_COST));
-      cost += PIECE_COST + take;
+      const int64_t take = std::min(s1 - pos, std::max<int64_t>(1, C - cost - pc));
+      cost += pc + take;
       pos += take;
       if (pos < s1) {  // the segment goes on in the next CTA
         if (nct == cap) return 0;
@@ -186,14 +190,14 @@ int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t C, int cap
   return nct;
 }
 
-int segment_split(const int64_t* off, int64_t nseg, int64_t n, int max_ctas, int64_t* out) {
-  int64_t lo = n / max_ctas, hi = n + (nseg + 1) * PIECE_COST;  // hi always fits in one CTA
+int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int max_ctas, int64_t* out) {
+  int64_t lo = n / max_ctas, hi = n + (nseg + 1) * pc;  // hi always fits in one CTA
   for (int it = 0; it < 40 && lo + 1 < hi; it++) {
     const int64_t mid = lo + (hi - lo) / 2;
-    if (greedy_split(off, nseg, n, mid, max_ctas, out) > 0) hi = mid;
+    if (greedy_split(off, nseg, n, pc, mid, max_ctas, out) > 0) hi = mid;
     else lo = mid;
   }
-  return greedy_split(off, nseg, n, hi, max_ctas, out);
+  return greedy_split(off, nseg, n, pc, hi, max_ctas, out);
 }
 
 // wait until the pinned staging buffers may be rewritten
@@ -486,8 +490,10 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
     p.p0 = (int64_t)(((16 - ag % 16) % 16) / B);
   else
     p.p0 = -1;
-  // persistent grid; small inputs get about one CTA per 4K elements
-  int64_t want = (n + 4095) / 4096;
+  // persistent grid; small inputs get about one CTA per 4K elements, and one
+  // per segment, as a piece takes 3 to 8 us however short it is (38 055
+  // bfloat16 elements in 308 segments: 10 CTAs 300 us, 152 CTAs 46)
+  const int64_t want = std::max<int64_t>((n + 4095) / 4096, nseg);
   p.nctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)h->nsm * peat::compare_ctas_per_sm(dtype), want));
   // stage 1 keeps element offsets within a CTA's range in 32 bits
   if (n / p.nctas >= ((int64_t)1 << 31) - 64)
@@ -506,7 +512,7 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
     if (ps != PEAT_OK) return ps;
     std::memcpy(h->h_offsets, offsets, sizeof(int64_t) * (size_t)(nseg + 1));
     int64_t* hb = h->h_offsets + nseg + 1;
-    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, p.nctas, hb) : 0;
+    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, piece_cost(dtype), p.nctas, hb) : 0;
     if (nsplit > 0)
       p.nctas = nsplit;
     else
