@@ -310,9 +310,9 @@ peat_status_t peat_topk_mean(peat_handle_t h, const void* golden, const void* ca
  *                      rtols non-decreasing after the rounding.
  *   nr, na             1 <= nr, na and nr * na <= 64.
  *   counts_out         device pointer to nr * na uint64 (overwritten).
- * About 15 na log2(nr) operations per differing pair (a binary search per
- * atol, bounded by the previous atol's result; bitwise-equal warp slots cost
- * a vote).  Asynchronous on `stream`.
+ * About 20 na operations per differing pair (a table gives the first
+ * accepting rtol per atol, one exact test decides; binary64: a binary search
+ * per atol); bitwise-equal warp slots cost a vote.  Asynchronous on `stream`.
  * Errors: INVALID_ARG (bad dtype, pointers, tolerances or grid size), CUDA. */
 peat_status_t peat_isclose_grid(peat_handle_t h, const void* golden, const void* candidate, int64_t n,
                                 peat_dtype_t dtype, const double* rtols, int nr, const double* atols, int na,
@@ -408,7 +408,7 @@ const char* peat_last_error(peat_handle_t h);
  * bounds, a status word and one accumulator).  Nothing is allocated by a
  * call, on the device or on the host.
  *   - Each CTA's range must stay below 2^31 - 64 elements (at most 320
- *     CTAs, two per SM): a larger n is rejected with PEAT_ERR_UNSUPPORTED.
+ *     CTAs: two per SM for float32, one for the 16-bit types): a larger n is rejected with PEAT_ERR_UNSUPPORTED.
  *   - The block's accumulator must be zero when a call starts.  It is zero
  *     when the code loads and every call that runs to completion leaves it
  *     zero; a call that fails to launch clears it with cudaMemsetAsync.

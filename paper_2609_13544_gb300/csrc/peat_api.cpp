@@ -150,9 +150,9 @@ bool round_tol(peat_tol_t tol, float* r, float* a) {
 
 // CTA ranges of a segmented call.  A CTA pays for its elements and, per
 // segment piece it meets, a fixed CTA-wide merge (its tables, its maxima, its
-// sums) worth about piece_cost elements.  For a capacity C, a greedy walk over the segments gives the
-// fewest CTAs with cost <= C each (cutting a segment where a CTA fills up);
-// a bisection on C finds the smallest capacity that fits in max_ctas CTAs,
+// sums) worth about piece_cost elements.  For a capacity C, a greedy walk over
+// the segments gives the fewest CTAs with cost <= C each (cutting a segment
+// where a CTA fills up); a bisection on C finds the smallest capacity that fits in max_ctas CTAs,
 // i.e. one wave.  Writes out[0..nctas] and returns nctas (0: no split fits).
 // Measured (GPT-2 list, binary16, 292 tensors / 151 tensors of 22.9 M binary16
 // elements / ResNet-50 list, float32, 161 tensors): 8192 elements a piece 470 /
@@ -260,7 +260,9 @@ static peat_status_t stage_items(peat_handle_t h, const int64_t* offsets, int64_
     h->h_f8 = nullptr;
     h->d_f8 = nullptr;
     h->f8_hcap = h->f8_dcap = 0;
-    const size_t hc = std::max(hbytes, (size_t)65536), dc = std::max(dbytes, (size_t)1 << 20);
+    // (256 KB: holds one tensor's 8-bit items and lies in memory already mapped; a
+    // block of 1 MB was mapped anew, 90 us of a handle's first 8-bit call)
+    const size_t hc = std::max(hbytes, (size_t)65536), dc = std::max(dbytes, (size_t)1 << 18);
     if (cudaMallocHost(&h->h_f8, hc) != cudaSuccess || cudaMalloc(&h->d_f8, dc) != cudaSuccess) {
       cudaGetLastError();
       return fail(h, PEAT_ERR_ALLOC, "compare workspace allocation failed");
