@@ -77,3 +77,19 @@ def test_table(peat_gpu, oracle, dtype, kind, n, shift, bad):
             want = oracle.topk_mean(g, c, dtype, num, den)
             for k in ("n_finite", "k", "threshold", "sum", "mean"):
                 assert got[k] == want[k], (num, den, k, got[k], want[k])
+
+
+@pytest.mark.parametrize("n", (65_535, 65_536, 65_537))
+def test_inexact_pairs_up_to_the_list(peat_gpu, oracle, n):
+    """Every pair tied in float32 and inexact, at the length of the list of rounding errors: up to it the passes
+    for an overflowing list are not launched."""
+    rng = np.random.default_rng(n)
+    g = -(rng.integers(1, 3000, n).astype(np.float32) * np.float32(2.0 ** -12))
+    c = np.full(n, np.float32(2 ** 24 + 2), np.float32)
+    gb, cb = g.view(np.uint32), c.view(np.uint32)
+    with peat.Handle(0) as h:
+        for num, den in ((1, 10), (1, 1), (1, 1000)):
+            got = peat.peat_topk_mean(h, to_device(gb, "f32"), to_device(cb, "f32"), num, den)
+            want = oracle.topk_mean(gb, cb, "f32", num, den)
+            for k in ("n_finite", "k", "threshold", "sum", "mean"):
+                assert got[k] == want[k], (num, den, k, got[k], want[k])
