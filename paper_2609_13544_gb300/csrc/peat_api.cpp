@@ -352,7 +352,11 @@ static peat_status_t compare8_impl(peat_handle_t h, const void* g, const void* c
                                    int64_t nseg, int dtype, float rtol, float atol, peat_stats_t* stats,
                                    uint64_t* hist, cudaStream_t st) {
   Items it;
-  const bool direct = offsets[nseg] < peat::C8_TABLE_MIN;  // (a rule on the size, see there)
+  // pair by pair below C8_TABLE_MIN pairs (see there) per round of one item per
+  // SM: many segments make short items (1000 segments of 8000 E4M3 pairs: 1065 us
+  // through tables, 123 without)
+  const int64_t rounds = std::max<int64_t>((nseg + h->nsm - 1) / h->nsm, 1);
+  const bool direct = offsets[nseg] < peat::C8_TABLE_MIN * rounds;
   peat_status_t ps = direct ? stage_items(h, offsets, nseg, sizeof(peat::Part8), 4, (int64_t)1 << 20, st, &it)
                             : stage_items(h, offsets, nseg, 2 * sizeof(peat::Part8), 1, (int64_t)1 << 20, st, &it);
   if (ps != PEAT_OK) return ps;

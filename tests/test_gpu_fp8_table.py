@@ -77,3 +77,15 @@ def test_segments_and_ties(peat_gpu, oracle, dtype, scale):
     check(peat_gpu, oracle, g, c, dtype, 0.01, 0.0, "constant", off)
     g = rng.integers(0, 256, n).astype(np.uint8)
     check(peat_gpu, oracle, g, rng.permutation(g), dtype, 0.01, 0.0, "random", off)
+
+
+@pytest.mark.parametrize("dtype", TDT)
+def test_many_segments(peat_gpu, oracle, dtype):
+    """More segments than CTAs and more pairs than a table call needs: short items, evaluated pair by pair."""
+    rng = np.random.default_rng(5)
+    off = np.concatenate([[0], np.cumsum(rng.integers(0, 20_000, 460))])
+    n = int(off[-1])
+    assert n > 1 << 22
+    g = rng.integers(0x20, 0x50, n).astype(np.uint8) | (rng.integers(0, 2, n).astype(np.uint8) << 7)
+    c = g + rng.integers(-2, 3, n).astype(np.uint8)
+    check(peat_gpu, oracle, g, c, dtype, 0.125, 0.0, "many segments", list(map(int, off)))
