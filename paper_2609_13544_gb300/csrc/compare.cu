@@ -1795,8 +1795,12 @@ __device__ __noinline__ void first_pairs(Smem<DT>& sm, const CompareParams& p, i
   using Ty = Tr<DT>;
   constexpr long long NONE = 0x7FFFFFFFFFFFFFFFll;
   for (int64_t base = pb;; base += Geo<DT>::NT) {
+    // read between two barriers, where no warp lowers them: every thread leaves
+    // after the same round
     __syncthreads();
-    if (base >= pe || (sm.k.ff != NONE && sm.k.fu != NONE)) break;
+    const bool found = sm.k.ff != NONE && sm.k.fu != NONE;
+    __syncthreads();
+    if (base >= pe || found) break;
     const int64_t i = base + threadIdx.x;
     if (i < pe) {
       const uint32_t Gi = load_scalar<DT>(p.g, i);
@@ -1805,7 +1809,6 @@ __device__ __noinline__ void first_pairs(Smem<DT>& sm, const CompareParams& p, i
       if (ag <= Ty::INF && ac <= Ty::INF) atomicMin(&sm.k.fu, (long long)i);
     }
   }
-  __syncthreads();
 }
 
 // Add n pairs of log2-relative exponent k, each lane its own (n = 0: none; the
