@@ -1036,9 +1036,9 @@ __device__ __forceinline__ void raise_key(unsigned long long* k, unsigned long l
 // of it is out of the window or above a bound: pairs out of the window go to
 // the general list, the window maxima into the CTA's records, and the tile's
 // pairs that the table phase must not see (general pairs, equal pairs holding
-// NaN or Inf) are zeroed in the stage.  Returns the lane's general pairs and
-// (high half) unequal pairs.  Out of line: it runs a few times per warp on
-// ordinary data.
+// NaN, Inf or a golden above the window) are zeroed in the stage.  Returns the
+// lane's general pairs and (high half) unequal pairs.  Out of line: it runs a
+// few times per warp on ordinary data.
 template <int DT>
 __device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t li0, int lb, int fe) {
   using Ty = Tr<DT>;
@@ -1064,8 +1064,11 @@ __device__ __noinline__ uint32_t slow_vec(Smem<DT>& sm, uint4* gt, uint4* ct, ui
         if (((G ^ C) & Ty::SIGN) == 0u && mg < Ty::INF && (C & Ty::MAG) < Ty::INF) um0 = max(um0, G > C ? G - C : C - G);
       }
       if (G == C) {
-        if ((G & Ty::MAG) >= Ty::INF) {
-          nf++;
+        // binary16: an equal pair whose scaled golden overflows would count
+        // d = -inf in T1
+        const uint32_t over = DT == PEAT_F16 ? min((uint32_t)(31 - fe) << 10, Ty::INF) : Ty::INF;
+        if ((G & Ty::MAG) >= over) {
+          if ((G & Ty::MAG) >= Ty::INF) nf++;
           g[j] = 0;
           c[j] = 0;
         }

@@ -5,7 +5,7 @@ ends of the window, and a nonzero atol.  Everything exact against the oracle."""
 import numpy as np
 import pytest
 
-from parity_util import NP_BITS, assert_hist_equal, assert_stats_equal, to_device
+from parity_util import NP_BITS, assert_hist_equal, assert_stats_equal, oracle_segmented, to_device
 
 pytestmark = pytest.mark.gpu
 DTYPES = ("f32", "f16", "bf16")
@@ -94,3 +94,24 @@ def test_tolerances(peat_gpu, oracle, dtype, rtol, atol):
     gb = encode(rng.standard_normal(n), dtype)
     cb = steps(gb, rng.integers(-9, 10, n))
     check(peat_gpu, oracle, gb, cb, dtype, rtol, atol, f"{dtype} rtol={rtol} atol={atol}")
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("share", (0.02, 0.6))
+@pytest.mark.parametrize("lead", (0.0, 1e-3))
+def test_magnitudes_above_the_first_ones(peat_gpu, oracle, dtype, share, lead):
+    """Equal and unequal pairs far above the elements that a CTA's range starts with: each segment, one CTA's work,
+    begins with zeros or small values, as a padded batch does, then holds data over many binades."""
+    rng = np.random.default_rng(int(share * 100) + int(lead * 1e4))
+    m, nseg = 18_000, 200
+    x = np.exp2(rng.uniform(-3, 15, (nseg, m))) * rng.choice([-1.0, 1.0], (nseg, m))
+    x[:, :9000] = lead * rng.standard_normal((nseg, 9000))
+    gb = encode(x.reshape(-1), dtype)
+    cb = steps(gb, np.where(rng.random(gb.size) < share, rng.integers(-2, 3, gb.size), 0))
+    off = np.arange(nseg + 1, dtype=np.int64) * m
+    with peat_gpu.Handle(0, max_segments=nseg) as h:
+        st, hist = peat_gpu.peat_compare_segmented(h, to_device(gb, dtype), to_device(cb, dtype), off, 1e-3, 0.0)
+    ost, oh = oracle_segmented(gb, cb, off, dtype, 1e-3, 0.0)
+    for s in range(nseg):
+        assert_stats_equal(st[s], ost[s], f"{dtype} share={share} lead={lead} segment {s}")
+        assert_hist_equal(hist[s], oh[s], f"{dtype} share={share} lead={lead} segment {s}")
