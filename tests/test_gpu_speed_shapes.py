@@ -1,0 +1,58 @@
+"""Calls whose data is laid out in a way that once cost many times an ordinary
+call of the same size: each against that ordinary call, timed in turn on the
+same GPU.  The limits lie between the two and leave room for noise."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+EPS = {"f16": 2.0 ** -10, "bf16": 2.0 ** -7}
+
+
+def median_us(torch, f):
+    f()
+    torch.cuda.synchronize()
+    a, b, t = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True), []
+    for _ in range(9):
+        a.record()
+        for _ in range(5):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        t.append(a.elapsed_time(b) * 200.0)
+    return sorted(t)[4]
+
+
+def compare_us(peat, golden, candidate, rtol=1e-3, atol=0.0):
+    import torch
+    stats = torch.zeros(peat.STATS_BYTES, dtype=torch.uint8, device="cuda")
+    hist = torch.zeros(peat.HIST_BINS, dtype=torch.int64, device="cuda")
+    with peat.Handle(0) as h:
+        return median_us(torch, lambda: peat.peat_compare_raw(h, golden, candidate, rtol, atol, stats, hist))
+
+
+def activation(dtype, rows=1 << 13, cols=1 << 12):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    dt = getattr(torch, {"f16": "float16", "bf16": "bfloat16"}[dtype])
+    return dt, torch.randn(rows, cols, generator=gen, device="cuda"), torch.randn(rows, cols, generator=gen, device="cuda")
+
+
+def noisy(x, noise, dtype, dt):
+    g = x.to(dt)
+    return g.view(-1), (g.float() * (1.0 + EPS[dtype] * noise)).to(dt).view(-1)
+
+
+@pytest.mark.parametrize("dtype", ("f16", "bf16"))
+def test_zero_padding(peat_gpu, dtype):
+    """Rows and parts of rows of zeros before the data (25 and 4 times the ordinary call, with a window placed by
+    the first elements of a CTA's range)."""
+    dt, x, noise = activation(dtype)
+    plain = compare_us(peat_gpu, *noisy(x, noise, dtype, dt))
+    for pad in ("sequences", "rows"):
+        y = x.clone()
+        if pad == "sequences":
+            y.view(8, -1)[:, : y.numel() // 16] = 0.0
+        else:
+            y[:, :2048] = 0.0
+        t = compare_us(peat_gpu, *noisy(y, noise, dtype, dt))
+        assert t < 1.7 * plain, f"{dtype} {pad}: {t:.1f} us against {plain:.1f}"
