@@ -526,7 +526,7 @@ struct Common {
   FinScratch fin;
   // the general path's totals, one copy per warp (fewer threads contend for an
   // address), folded into hist and sacc at the end of a piece that used them
-  unsigned long long ghist[NW][HBINS];
+  uint32_t ghist[NW][HBINS];  // (a piece has below 2^31 pairs)
   int gsacc[NW][NSUM * NLIMB][2];  // sums of the low and the high 16 bits of each digit (gen_flush)
 };
 
@@ -589,7 +589,7 @@ template <int DT>
 __device__ __forceinline__ void whist_add(Smem<DT>& sm, int bin) {
   const unsigned grp = __match_any_sync(0xFFFFFFFFu, bin);
   if (bin >= 0 && (threadIdx.x & 31) == __ffs(grp) - 1 && PEAT_CHECK(bin < HBINS))
-    atomicAdd(&sm.k.ghist[threadIdx.x >> 5][bin], (unsigned long long)__popc(grp));
+    atomicAdd(&sm.k.ghist[threadIdx.x >> 5][bin], (uint32_t)__popc(grp));
 }
 
 // floor(log2(a / g)) for a = (hi + lo) 2^sc > 0 and g > 0 (float32 pair, any range)
@@ -735,7 +735,9 @@ __device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, uint32_t 
     float x = k == 1 || k == 3 || k == 6 ? o.t : o.s;
     const float y = k < 4 ? 1.0f : (k == 4 ? o.s : o.t);
     if ((k == 2 || k == 3) && o.s < 0.0f) x = -x;
-    if (on && x != 0.0f && y != 0.0f) {
+    const bool use = on && x != 0.0f && y != 0.0f;
+    if (!__any_sync(0xFFFFFFFFu, use)) continue;  // (t is zero where c - g is a float32 value, most often)
+    if (use) {
       int ex = 0, ey = 0;
       const uint32_t mx = split_float(x, ex), my = split_float(y, ey);
       wsacc_add(d + min(k >> 1, 2) * (2 * NLIMB), (uint64_t)mx * my, ex + ey + (k < 4 ? o.sc : 2 * o.sc + (k == 5)),
@@ -1694,6 +1696,93 @@ __device__ __forceinline__ void gen_counts(const GenRec& g, Smem<DT>& sm) {
   }
 }
 
+// The rescan of a piece whose general pairs overflowed its list: slot k of the
+// warp's, its general pairs added to the cnt entries of the warp's queue (in its
+// part of the staging ring, idle now), so that general_lane runs on full warps.
+// Slot 0 is the head, then 32 x VEC elements of the body each, the last one the
+// tail.  With one round of general_lane per 32 elements, whatever they held: 67 M
+// binary16 pairs of which 5 % are general 2520 us, float32 pairs of which a third
+// are 3250; now 765 and 1085.
+template <int DT>
+struct Queue {
+  static constexpr uint32_t SLOT = 32 * Tr<DT>::VEC;
+  uint32_t *i, *g, *c;  // offsets from the CTA's first element; goldens (16-bit types: with the candidate); candidates
+  __device__ __forceinline__ Queue(Smem<DT>& sm) {
+    i = reinterpret_cast<uint32_t*>(sm.ring.g[threadIdx.x >> 5]);
+    c = reinterpret_cast<uint32_t*>(sm.ring.c[threadIdx.x >> 5]);
+    g = DT == PEAT_F32 ? i + CHV * 4 * NSTAGE / 2 : c;
+  }
+};
+static_assert(Queue<PEAT_F16>::SLOT + 31 <= CHV * 4 * NSTAGE && Queue<PEAT_F32>::SLOT + 31 <= CHV * 4 * NSTAGE / 2,
+              "the queue fits the ring");
+template <int DT, bool INJ>
+__device__ __noinline__ uint32_t scan_slot(Win W, Smem<DT>& sm, const CompareParams& p, int64_t pb, int64_t pe, int64_t vb,
+                                           int64_t ve, int64_t k, uint32_t cnt) {
+  constexpr int VEC = Tr<DT>::VEC, B = Tr<DT>::BYTES, NW = Geo<DT>::NW;
+  constexpr uint32_t SLOT = Queue<DT>::SLOT;
+  const uint32_t lane = threadIdx.x & 31u;
+  const Queue<DT> q(sm);
+  const int64_t b = k == 0 ? pb : vb + (k - 1) * (int64_t)SLOT;
+  const int64_t e = k == 0 ? vb : b < ve ? min(b + SLOT, ve) : pe, b1 = k == 0 || b < ve ? b : ve;
+  if constexpr (DT == PEAT_F32) {
+    // the window this slot was tested with: the head ran with the initial
+    // window, a body chunk with its warp's window of that time, the tail with
+    // warp 0's last window
+    int w = 0;
+    uint32_t ik = 0;
+    if (vb < ve && k > 0) {
+      if (b >= ve) {
+        ik = 0xFFFFFFFFu;
+      } else {
+        const int64_t t = (b - vb) / (CHV * VEC);
+        w = (int)(t % NW);
+        ik = (uint32_t)(t / NW);
+      }
+    }
+    int r = (int)sm.k.nwin[w];
+    while (r > 0 && sm.k.wstart[w][r] > ik) r--;
+    set_window_lb<DT>(W, sm.k.wlb[w][r]);
+  }
+  uint32_t G[VEC], C[VEC];
+  // whole vectors where the slot holds them on their grid, else elements lane + 32 j
+  const uintptr_t ob = (uintptr_t)b1 * B;
+  const bool vec = e - b1 == SLOT && ((((uintptr_t)p.g + ob) | (INJ ? 0 : (uintptr_t)p.c + ob)) & 15u) == 0;
+  if (vec) {
+    const int64_t i0 = b1 + (int64_t)lane * VEC;
+    const uint4 gv = load_vec(p.g, i0 * B);
+    const uint4 cv = INJ ? inj_one<DT>(p, gv, i0) : load_vec(p.c, i0 * B);
+    unpack_vec<DT>(gv, G);
+    unpack_vec<DT>(cv, C);
+  } else {
+#pragma unroll
+    for (int j = 0; j < VEC; j++) {
+      const int64_t i = b1 + lane + 32 * j;
+      G[j] = C[j] = 0;
+      if (i < e) {
+        G[j] = load_scalar<DT>(p.g, i);
+        C[j] = cand_at<DT, INJ>(p, i, G[j]);
+      }
+    }
+  }
+  const uint32_t li = (uint32_t)(b1 - sm.k.lo);
+#pragma unroll
+  for (int j = 0; j < VEC; j++) {
+    uint32_t u;
+    float gf, a;
+    const bool want = G[j] != C[j] && !pair_window<DT>(G[j], C[j], W, u, gf, a);
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, want);
+    if (want) {
+      const uint32_t at = cnt + __popc(m & ((1u << lane) - 1u));
+      q.i[at] = li + (vec ? lane * VEC + j : lane + 32 * j);
+      q.g[at] = DT == PEAT_F32 ? G[j] : G[j] | (C[j] << 16);
+      if constexpr (DT == PEAT_F32) q.c[at] = C[j];
+    }
+    cnt += __popc(m);
+  }
+  __syncwarp();
+  return cnt;
+}
+
 // The general pairs of a piece [pb, pe), evaluated exactly by every thread of
 // the CTA: from the list when it held them all, else found again by a rescan
 // of the piece with the same window test.  Out of line, so that the hot loop
@@ -1708,62 +1797,44 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
   GenRec cd;
   gen_init(cd);
   // whole warps in every round (general_lane counts with the whole warp)
-  const uint32_t lane = threadIdx.x & 31u, w0 = threadIdx.x & ~31u;
-  if (n <= (uint32_t)GCAP) {
-    for (uint32_t b = w0; b < n; b += NT) {
-      const uint32_t e = b + lane;
-      const bool valid = e < n;
-      int64_t i = 0;
-      uint32_t G = 0, C = 0;
+  const uint32_t lane = threadIdx.x & 31u;
+  const bool listed = n <= (uint32_t)GCAP;
+  uint32_t b = threadIdx.x & ~31u, cnt = 0;  // the warp's place in the list; its queue
+  int64_t k = threadIdx.x >> 5;
+  const int64_t slots = (ve - vb + Queue<DT>::SLOT - 1) / Queue<DT>::SLOT + 2;
+  for (int rounds = 0;; rounds++) {
+    int64_t i = 0;
+    uint32_t G = 0, C = 0;
+    bool valid;
+    if (listed) {
+      if (b >= n) break;
+      valid = b + lane < n;
       if (valid) {
-        i = lo + sm.k.glist[e];
+        i = lo + sm.k.glist[b + lane];
         if (!PEAT_CHECK(i >= 0 && i < p.n_total)) i = lo;  // a listed offset outside the tensor
         G = load_scalar<DT>(p.g, i);
         C = cand_at<DT, INJ>(p, i, G);
       }
-      general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, valid);
-    }  // (at most GCAP / NT rounds: no flush)
-    static_assert(GCAP / NT <= GEN_FLUSH, "rounds of the list");
-  } else {
-    int rounds = 0;
-    for (int64_t b = pb + w0; b < pe; b += NT) {
-      if (++rounds > GEN_FLUSH) gen_flush<DT>(sm), rounds = 1;
-      const int64_t i = b + lane;
-      bool want = false;
-      uint32_t G = 0, C = 0;
-      if (i < pe) {
-        G = load_scalar<DT>(p.g, i);
-        C = cand_at<DT, INJ>(p, i, G);
-        want = G != C;
+      b += NT;
+    } else {
+      for (; cnt < 32u && k < slots; k += NW) cnt = scan_slot<DT, INJ>(W, sm, p, pb, pe, vb, ve, k, cnt);
+      if (cnt == 0u) break;
+      const uint32_t take = min(cnt, 32u);
+      const Queue<DT> q(sm);
+      cnt -= take;
+      valid = lane < take;
+      if (valid) {
+        i = lo + q.i[cnt + lane];
+        G = q.g[cnt + lane];
+        if constexpr (DT == PEAT_F32) C = q.c[cnt + lane];
+        else C = G >> 16, G &= 0xFFFFu;
       }
-      if (want) {
-        Win Wi = W;
-        if constexpr (DT == PEAT_F32) {
-          // the window this pair was tested with: the head ran with the
-          // initial window, a body chunk with its warp's window of that time,
-          // the tail with warp 0's last window
-          int w = 0;
-          uint32_t ik = 0;
-          if (vb < ve && i >= vb) {
-            if (i >= ve) {
-              ik = 0xFFFFFFFFu;
-            } else {
-              const int64_t k = (i - vb) / (CHV * Tr<DT>::VEC);
-              w = (int)(k % NW);
-              ik = (uint32_t)(k / NW);
-            }
-          }
-          int r = (int)sm.k.nwin[w];
-          while (r > 0 && sm.k.wstart[w][r] > ik) r--;
-          set_window_lb<DT>(Wi, sm.k.wlb[w][r]);
-        }
-        uint32_t u;
-        float gf, a;
-        want = !pair_window<DT>(G, C, Wi, u, gf, a);
-      }
-      general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, want);
+      __syncwarp();
     }
+    if (rounds == GEN_FLUSH) gen_flush<DT>(sm), rounds = 0;
+    general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, valid);
   }
+  fence_proxy_async();  // the queue, before the next piece's bulk copies into the ring
   gen_counts<DT>(cd, sm);
   warp_best(cd.abs_hi, cd.abs_lo, cd.abs_sc, cd.abs_idx, cd.rel_hi, cd.rel_lo, cd.rel_g, cd.rel_sc, cd.rel_idx, cd.ulp,
             cd.ulp_idx, -1, -1, &sm.k.wbest[threadIdx.x >> 5]);

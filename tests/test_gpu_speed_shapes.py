@@ -4,7 +4,7 @@ same GPU.  The limits lie between the two and leave room for noise."""
 import pytest
 
 pytestmark = pytest.mark.gpu
-EPS = {"f16": 2.0 ** -10, "bf16": 2.0 ** -7}
+EPS = {"f32": 2.0 ** -23, "f16": 2.0 ** -10, "bf16": 2.0 ** -7}
 
 
 def median_us(torch, f):
@@ -33,7 +33,7 @@ def activation(dtype, rows=1 << 13, cols=1 << 12):
     import torch
     gen = torch.Generator(device="cuda")
     gen.manual_seed(1)
-    dt = getattr(torch, {"f16": "float16", "bf16": "bfloat16"}[dtype])
+    dt = getattr(torch, {"f32": "float32", "f16": "float16", "bf16": "bfloat16"}[dtype])
     return dt, torch.randn(rows, cols, generator=gen, device="cuda"), torch.randn(rows, cols, generator=gen, device="cuda")
 
 
@@ -56,3 +56,13 @@ def test_zero_padding(peat_gpu, dtype):
             y[:, :2048] = 0.0
         t = compare_us(peat_gpu, *noisy(y, noise, dtype, dt))
         assert t < 1.7 * plain, f"{dtype} {pad}: {t:.1f} us against {plain:.1f}"
+
+
+@pytest.mark.parametrize("dtype,limit", (("f32", 6.5), ("f16", 17), ("bf16", 11)))
+def test_most_pairs_outside_the_window(peat_gpu, dtype, limit):
+    """Additive noise of a tenth of the scale: a third of the pairs and more are general, every piece is rescanned
+    (20 times the ordinary 16-bit call when the rescan ran a round for every 32 elements)."""
+    dt, x, noise = activation(dtype)
+    plain = compare_us(peat_gpu, *noisy(x, noise, dtype, dt))
+    t = compare_us(peat_gpu, x.to(dt).view(-1), (x + 0.1 * noise).to(dt).view(-1))
+    assert t < limit * plain, f"{dtype}: {t:.1f} us against {plain:.1f}"
