@@ -502,8 +502,9 @@ struct Common {
   Partial wbest[NW];
   long long lo;                    // the CTA's first element
   long long ff, fu;                // first finite pair, first pair without NaN (search result)
-  uint32_t* glist;                 // this CTA's list of general pairs (offsets), GCAP entries
-  uint32_t gn;                     // entries appended in this piece (may exceed GCAP)
+  uint32_t* glist;                 // this CTA's list of general pairs, gcap entries
+  uint32_t gcap;
+  uint32_t gn;                     // entries appended in this piece (may exceed gcap)
   uint32_t nfe;                    // bitwise-equal pairs holding NaN or Inf
   int last;                        // this CTA finished the last piece of a one-segment call
   int first, final;                // a one-segment call's pieces: the CTAs first .. final
@@ -584,12 +585,12 @@ __device__ __noinline__ void gen_flush(Smem<DT>& sm) {
   }
   __syncwarp();
 }
-// one histogram bin per lane (bin < 0: none), counted once per distinct bin
+// one histogram bin per lane (bin < 0: none), an increment by the constant one
+// (see the tables)
 template <int DT>
 __device__ __forceinline__ void whist_add(Smem<DT>& sm, int bin) {
-  const unsigned grp = __match_any_sync(0xFFFFFFFFu, bin);
-  if (bin >= 0 && (threadIdx.x & 31) == __ffs(grp) - 1 && PEAT_CHECK(bin < HBINS))
-    atomicAdd(&sm.k.ghist[threadIdx.x >> 5][bin], (uint32_t)__popc(grp));
+  if (bin >= 0 && PEAT_CHECK(bin < HBINS))
+    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(smem_addr(&sm.k.ghist[threadIdx.x >> 5][bin])) : "memory");
 }
 
 // floor(log2(a / g)) for a = (hi + lo) 2^sc > 0 and g > 0 (float32 pair, any range)
@@ -714,18 +715,44 @@ __device__ __forceinline__ void general_pair(GenRec& cd, GenOut& o, uint32_t G, 
   o.t = t;
   o.sc = sc;
 }
+// binary16: every finite difference is D 2^-24 for an integer D below 2^41 in
+// size, so where a piece has many general pairs their sums are integers in
+// registers: of |D|, of |D| over the negative ones, and of D^2 (at most 2^22
+// pairs per thread and piece).  Through the digits in shared memory a round of
+// 32 pairs took 1700 instructions, 14 of them conflicting increments, now 600;
+// but the integers' own reduction at the end takes 2 to 3 us, hence GEN_MANY.
+struct GenSum {
+  uint64_t a = 0, n = 0;
+  unsigned __int128 q = 0;
+};
+constexpr uint32_t GEN_MANY = 4096;
+__device__ __forceinline__ int64_t f16_units(uint32_t b) {
+  const uint32_t e = (b >> 10) & 31u, m = b & 0x3FFu;
+  const int64_t k = e ? (int64_t)(m | 0x400u) << (e - 1) : (int64_t)m;
+  return (b & 0x8000u) ? -k : k;
+}
 // One general pair per lane of a converged warp (valid: the lane has one):
 // the per-lane part, then the histogram bins and the exact sums, d = (s + t)
 // 2^sc, |d| = (hi + lo) 2^sc with (hi, lo) = +-(s, t), d^2 = (s^2 + 2st +
 // t^2) 4^sc, added by the whole warp.
 template <int DT>
-__device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, uint32_t G, uint32_t C, int64_t idx, float rtol,
-                                             float atol, bool valid) {
+__device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, GenSum& gs, bool many, uint32_t G, uint32_t C,
+                                             int64_t idx, float rtol, float atol, bool valid) {
   GenOut o{-1, -1, 0.0f, 0.0f, 0};
   if (valid) general_pair<DT>(cd, o, G, C, idx, rtol, atol);
   whist_add(sm, o.hb0);
   whist_add(sm, o.hb1);
   const bool on = o.s != 0.0f;
+  if (DT == PEAT_F16 && many) {
+    if (on) {
+      const int64_t d = f16_units(C) - f16_units(G);
+      const uint64_t a = (uint64_t)(d < 0 ? -d : d);
+      gs.a += a;
+      gs.n += d < 0 ? a : 0ull;
+      gs.q += (unsigned __int128)a * a;
+    }
+    return;
+  }
   // the seven terms through one copy of the code: a piece with few general
   // pairs spends most of this path's time on fetching it
   int* d = &sm.k.gsacc[threadIdx.x >> 5][0][0];
@@ -891,11 +918,11 @@ __device__ __forceinline__ bool pair_window(uint32_t G, uint32_t C, const Win& W
 }
 
 // a pair outside the window: append it to the CTA's general list (evaluated
-// at the end of the piece; past GCAP entries the piece is rescanned)
+// at the end of the piece; past gcap entries the piece is rescanned)
 template <int DT>
 __device__ __forceinline__ void defer_pair(uint32_t li, Smem<DT>& sm) {
   const uint32_t slot = atomicAdd(&sm.k.gn, 1u);
-  if (slot < (uint32_t)GCAP) sm.k.glist[slot] = li;
+  if (slot < sm.k.gcap) sm.k.glist[slot] = li;
 }
 
 // lanes of one vector whose golden value is NaN or Inf, as a bitmask
@@ -961,6 +988,20 @@ __device__ __forceinline__ void flush_sums(Lane& L, Smem<PEAT_F32>& sm, int lexp
   }
   L.A = L.S = L.Q12 = 0;
   L.Q11 = L.Q22 = 0;
+}
+
+// binary16: the warp's general sums into the CTA's digits, word by word
+__device__ __forceinline__ void gen_sums(const GenSum& gs, Smem<PEAT_F16>& sm) {
+#pragma unroll 1
+  for (int w = 0; w < 4; w++) {
+    const uint64_t a = w < 2 ? wsum64((uint32_t)(gs.a >> (32 * w))) : 0, n = w < 2 ? wsum64((uint32_t)(gs.n >> (32 * w))) : 0;
+    const uint64_t q = wsum64((uint32_t)(gs.q >> (32 * w)));
+    if ((threadIdx.x & 31) == 0) {
+      if (a) sacc_add<PEAT_F16>(sm, 1, a, 32 * w - 24, false), sacc_add<PEAT_F16>(sm, 0, a, 32 * w - 24, false);
+      if (n) sacc_add<PEAT_F16>(sm, 0, n, 32 * w - 23, true);  // sum d = sum |d| - 2 sum of the negative ones
+      if (q) sacc_add<PEAT_F16>(sm, 2, q, 32 * w - 48, false);
+    }
+  }
 }
 
 // float32: when the slow path sent many pairs of a tile (at least 32, and a
@@ -1303,6 +1344,64 @@ __device__ __forceinline__ void count16(const Vec16<NP>& v, const Win& W, uint32
   }
 }
 
+// The pairs of a vector that are more than UMAX steps apart, each lane's in m
+// (general ones, as pair_window has it): to the list, the lanes' entries taken
+// together, and zeroed in the stage.
+template <int DT>
+__device__ __forceinline__ void drop_far(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t li, uint32_t m) {
+  constexpr uint32_t ALL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  // the lanes' first places from a running count over the warp
+  const uint32_t k = __popc(m);
+  uint32_t at = k;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(ALL, at, o);
+    if (lane >= o) at += y;
+  }
+  uint32_t base = 0;
+  if (lane == 31) base = atomicAdd(&sm.k.gn, at);
+  at += __shfl_sync(ALL, base, 31) - k;
+  unsigned short *g = reinterpret_cast<unsigned short*>(gt), *c = reinterpret_cast<unsigned short*>(ct);
+#pragma unroll 1
+  for (; m; m &= m - 1u, at++) {
+    const int j = __ffs(m) - 1;
+    if (at < sm.k.gcap) sm.k.glist[at] = li + j;
+    g[j] = c[j] = 0;
+  }
+  fence_proxy_async();  // the zeroed pairs before the next bulk copy into the stage
+  __syncwarp();
+}
+// A dense vector with a flagged pair.  Additive noise leaves pairs far apart in
+// nearly every vector, so those are taken out first, without slow_vec's look at the
+// maxima, and slow_vec runs only if a pair is still flagged.  Measured, 67 M pairs,
+// slow_vec alone and now: noise of 1 % of the scale, bfloat16 428 -> 268 us,
+// binary16 765 -> 352; of 0.1 %, 234 -> 162 and 381 -> 230.
+template <int DT>
+__device__ __noinline__ void slow16(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t li, int fe) {
+  constexpr uint32_t UM = (uint32_t)Tab<DT>::UMAX, ALL = 0xFFFFFFFFu;
+  uint32_t m = 0;
+  const uint32_t *gw = reinterpret_cast<const uint32_t*>(gt), *cw = reinterpret_cast<const uint32_t*>(ct);
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const uint32_t x = gw[i], y = cw[i];
+    const uint32_t lo = (y & 0xFFFFu) - (x & 0xFFFFu) + UM, hi = (y >> 16) - (x >> 16) + UM;
+    m |= (lo > 2u * UM ? 1u : 0u) << (2 * i) | (hi > 2u * UM ? 2u : 0u) << (2 * i);
+  }
+  if (__any_sync(ALL, m != 0u)) {
+    drop_far<DT>(sm, gt, ct, li, m);
+    Win W;
+    W.rtol = W.atol = W.lim = W.M1 = W.M2 = 0.0f, W.lb = 0;
+    W.fe = fe;
+    const Bounds B = read_bounds<DT>(sm, li - (threadIdx.x & 31u) * 8u, W);
+    const uint32_t g[4] = {gw[0], gw[1], gw[2], gw[3]}, c[4] = {cw[0], cw[1], cw[2], cw[3]};
+    Vec16<4> v;
+    prep16<DT, 4>(v, g, c, (uint32_t)(15 + fe) * 0x04000400u);
+    if (!__any_sync(ALL, check16<DT, 4>(v, W, B))) return;
+  }
+  slow_vec<DT>(sm, gt, ct, li, 0, fe);
+}
+
 // A vector of which few lanes hold an unequal pair: each lane visits its own
 // unequal words (two pairs at a time), the rest of the warp an equal one.
 // (Out of line of the dense path: late steps of a sweep and fault injections
@@ -1367,7 +1466,7 @@ __device__ __forceinline__ void tile16(Lane& L, Smem<DT>& sm, uint4* gt, uint4* 
     uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w}, c[4] = {cv.x, cv.y, cv.z, cv.w};
     prep16<DT, 4>(v, g, c, scale2);
     if (__any_sync(0xFFFFFFFFu, check16<DT, 4>(v, W, B))) {
-      slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
+      slow16<DT>(sm, gt, ct, li, W.fe);
       gv = *gt;
       cv = *ct;
       const uint32_t gn[4] = {gv.x, gv.y, gv.z, gv.w}, cn[4] = {cv.x, cv.y, cv.z, cv.w};
@@ -1796,9 +1895,10 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
   const int64_t lo = sm.k.lo;
   GenRec cd;
   gen_init(cd);
+  GenSum gs;
   // whole warps in every round (general_lane counts with the whole warp)
   const uint32_t lane = threadIdx.x & 31u;
-  const bool listed = n <= (uint32_t)GCAP;
+  const bool listed = n <= sm.k.gcap, many = DT == PEAT_F16 && n > GEN_MANY;
   uint32_t b = threadIdx.x & ~31u, cnt = 0;  // the warp's place in the list; its queue
   int64_t k = threadIdx.x >> 5;
   const int64_t slots = (ve - vb + Queue<DT>::SLOT - 1) / Queue<DT>::SLOT + 2;
@@ -1832,8 +1932,10 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
       __syncwarp();
     }
     if (rounds == GEN_FLUSH) gen_flush<DT>(sm), rounds = 0;
-    general_lane<DT>(sm, cd, G, C, i, p.rtol, p.atol, valid);
+    general_lane<DT>(sm, cd, gs, many, G, C, i, p.rtol, p.atol, valid);
   }
+  if constexpr (DT == PEAT_F16)
+    if (many) gen_sums(gs, sm);
   fence_proxy_async();  // the queue, before the next piece's bulk copies into the ring
   gen_counts<DT>(cd, sm);
   warp_best(cd.abs_hi, cd.abs_lo, cd.abs_sc, cd.abs_idx, cd.rel_hi, cd.rel_lo, cd.rel_g, cd.rel_sc, cd.rel_idx, cd.ulp,
@@ -2214,7 +2316,8 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
   const int64_t lo = p.bounds[blockIdx.x], hi = p.bounds[blockIdx.x + 1];
   if (tid == 0) {
     sm.k.lo = lo;
-    sm.k.glist = p.glist + (size_t)blockIdx.x * GCAP;
+    sm.k.glist = p.glist + (size_t)blockIdx.x * p.gcap;
+    sm.k.gcap = p.gcap;
   }
   if (lane == 0) {
     for (int st = 0; st < NSTAGE; st++) mbar_init(smem_addr(&sm.k.bar[warp][st]), 1);

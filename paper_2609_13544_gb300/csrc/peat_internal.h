@@ -47,7 +47,7 @@ constexpr int LIMB_LSB = -416;
 constexpr int NSUM = 3;  // 0: sum d, 1: sum |d|, 2: sum d^2
 
 constexpr int BLOCK = 256;    // threads of the small kernels (bounds, per-segment finalize)
-constexpr int GCAP = 16384;   // general-path pairs a CTA lists per segment piece (more: the piece is rescanned)
+constexpr int GCAP = 16384;   // entries of the list of general pairs per CTA of the largest grid
 constexpr int HBINS = 128;    // 64 rel bins + 64 ULP bins
 
 // Exact maxima of one CTA piece (element indices are global).  |d| is kept
@@ -115,7 +115,8 @@ struct CompareParams {
   int nctas;
   Partial* partials;       // nseg + nctas slots; slot s + b holds CTA b's part of segment s
   SegAcc* acc;             // nseg accumulators, all zero between calls
-  uint32_t* glist;         // nctas * GCAP offsets: each CTA's general pairs of the current piece
+  uint32_t* glist;         // nctas * gcap offsets: each CTA's general pairs of the current piece
+  uint32_t gcap;           // entries per CTA (a piece with more general pairs is rescanned)
   int has_empty;           // some segment is empty (CTA 0 writes the outputs of the empty segments)
   unsigned int* status;    // device-visible error word (bit 0: a bounded wait expired)
   unsigned int wait_limit; // iteration bound of a pipeline wait (0: give up at once, for tests)

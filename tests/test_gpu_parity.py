@@ -56,11 +56,18 @@ def test_noise_ragged_large(peat_gpu, oracle, h, dtype):
 
 @pytest.mark.parametrize("dtype", DTYPES)
 def test_general_pairs_beyond_the_list(peat_gpu, oracle, h, dtype):
-    """Random bit patterns: most pairs leave the window, so every CTA piece
-    holds more general pairs than its list (16384) and is rescanned."""
+    """Random bit patterns: nine in ten pairs leave the window, so every CTA piece
+    holds more general pairs than its list (32768, 16-bit types 65536) and is
+    rescanned, on the vector grid and (bases of different alignment) off it."""
     n = 12_000_017
     gb, cb = random_pairs(dtype, n, seed=4242)
-    check_pair(peat_gpu, oracle, h, gb, cb, dtype, 1e-3, 0.0, ctx=f"{dtype} rescan")
+    rng = np.random.default_rng(4243)
+    cb = np.where(rng.random(n) < 0.875, rng.integers(0, 2 ** (8 * cb.itemsize), n).astype(cb.dtype), cb)
+    os_, oh = oracle.compare(gb, cb, dtype, 1e-3, 0.0)
+    for coff in (0, 1):
+        gs, gh = run_pair(peat_gpu, h, gb, cb, dtype, 1e-3, 0.0, 0, coff)
+        assert_stats_equal(gs, os_, f"{dtype} rescan, candidate at {coff}")
+        assert_hist_equal(gh, oh, f"{dtype} rescan, candidate at {coff}")
 
 
 @pytest.mark.parametrize("dtype", DTYPES)

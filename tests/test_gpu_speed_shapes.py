@@ -58,7 +58,7 @@ def test_zero_padding(peat_gpu, dtype):
         assert t < 1.7 * plain, f"{dtype} {pad}: {t:.1f} us against {plain:.1f}"
 
 
-@pytest.mark.parametrize("dtype,limit", (("f32", 6.5), ("f16", 17), ("bf16", 11)))
+@pytest.mark.parametrize("dtype,limit", (("f16", 15), ("bf16", 12)))
 def test_most_pairs_outside_the_window(peat_gpu, dtype, limit):
     """Additive noise of a tenth of the scale: a third of the pairs and more are general, every piece is rescanned
     (20 times the ordinary 16-bit call when the rescan ran a round for every 32 elements)."""
@@ -66,3 +66,14 @@ def test_most_pairs_outside_the_window(peat_gpu, dtype, limit):
     plain = compare_us(peat_gpu, *noisy(x, noise, dtype, dt))
     t = compare_us(peat_gpu, x.to(dt).view(-1), (x + 0.1 * noise).to(dt).view(-1))
     assert t < limit * plain, f"{dtype}: {t:.1f} us against {plain:.1f}"
+
+
+@pytest.mark.parametrize("dtype", ("f16", "bf16"))
+def test_additive_noise(peat_gpu, dtype):
+    """Errors of absolute size: small values differ by hundreds of steps, nearly every vector holds such a pair, and
+    1 to 8 % of all are general (25 times the ordinary binary16 call when each went the slow path)."""
+    dt, x, noise = activation(dtype)
+    plain = compare_us(peat_gpu, *noisy(x, noise, dtype, dt))
+    for sigma, limit in ((0.001, 2.7), (0.01, 4.5)):
+        t = compare_us(peat_gpu, x.to(dt).view(-1), (x + sigma * noise).to(dt).view(-1))
+        assert t < limit * plain, f"{dtype} {sigma}: {t:.1f} us against {plain:.1f}"
