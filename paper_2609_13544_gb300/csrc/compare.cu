@@ -1044,20 +1044,27 @@ __device__ __forceinline__ Bounds read_bounds(const Smem<DT>& sm, uint32_t tli, 
   const unsigned long long ku = *(volatile const unsigned long long*)&sm.k.kulp;
   const unsigned long long kr = *(volatile const unsigned long long*)&sm.k.krel;
   Bounds b;
-  b.ab = (uint32_t)(ka >> 32);
+  // (a record above what the window can hold, a general pair's in the sample,
+  // bounds every window pair as it is; the general path has that pair)
+  const uint32_t av = (uint32_t)(ka >> 32), uv = (uint32_t)(ku >> 32);
+  uint32_t cap;
   if constexpr (DT == PEAT_BF16) {
-    b.ab = min(b.ab, ((uint32_t)(W.fe + 64) << 23) - 0x10000u) >> 16;
+    cap = (((uint32_t)(W.fe + 64) << 23) - 0x10000u) >> 16;
+    b.ab = av >> 16;
   } else if constexpr (DT == PEAT_F16) {
-    const float sc = __fmul_rn(__uint_as_float(b.ab), __uint_as_float((uint32_t)(127 + W.fe) << 23));
-    b.ab = sc < 65504.0f ? (uint32_t)__half_as_ushort(__float2half_rn(sc)) : 0x7BFFu;
+    cap = 0x7BFFu;
+    const float sc = __fmul_rn(__uint_as_float(av), __uint_as_float((uint32_t)(127 + W.fe) << 23));
+    b.ab = sc < 65536.0f ? (uint32_t)__half_as_ushort(__float2half_rn(sc)) : 0x7C00u;
   } else {
-    b.ab = min(b.ab, __float_as_uint(W.lim) - 1u);
+    cap = __float_as_uint(W.lim) - 1u;
+    b.ab = av;
   }
-  b.low = ~(uint32_t)ka >= tli && b.ab != 0u;
+  b.low = ~(uint32_t)ka >= tli && b.ab != 0u && b.ab <= cap;
+  b.ab = min(b.ab, cap);
   if (b.low) b.ab--;
   if constexpr (DT != PEAT_F32) b.ab |= b.ab << 16;
-  b.ub = min((uint32_t)(ku >> 32), (uint32_t)Tab<DT>::UMAX);
-  const bool lu = ~(uint32_t)ku >= tli && b.ub != 0u, lr = ~(uint32_t)kr >= tli;
+  b.ub = min(uv, (uint32_t)Tab<DT>::UMAX);
+  const bool lu = ~(uint32_t)ku >= tli && b.ub != 0u && uv <= (uint32_t)Tab<DT>::UMAX, lr = ~(uint32_t)kr >= tli;
   if (lu) b.ub--;
   b.low = b.low || lu || (DT != PEAT_F32 && lr && kr != 0ull);
   const float q = __uint_as_float((uint32_t)(kr >> 32));
@@ -2415,7 +2422,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
       if (emax) atomicMax(&sm.k.lb, (int)emax);
       if (umax) atomicMax(&sm.k.ub, (int)(32 - __clz(umax)));
       if (ab) atomicMax(&sm.k.kabs, (unsigned long long)ab << 32);
-      if (umax) atomicMax(&sm.k.kulp, (unsigned long long)min(umax, (1u << 23) - 1u) << 32);
+      if (umax) atomicMax(&sm.k.kulp, (unsigned long long)umax << 32);
       if (qb) atomicMax(&sm.k.krel, (unsigned long long)qb << 32);
     }
     if (tid == 0) {

@@ -115,3 +115,21 @@ def test_magnitudes_above_the_first_ones(peat_gpu, oracle, dtype, share, lead):
     for s in range(nseg):
         assert_stats_equal(st[s], ost[s], f"{dtype} share={share} lead={lead} segment {s}")
         assert_hist_equal(hist[s], oh[s], f"{dtype} share={share} lead={lead} segment {s}")
+
+
+@pytest.mark.parametrize("dtype,umax", (("f32", 2 ** 23 - 1), ("f16", 127), ("bf16", 63)))
+@pytest.mark.parametrize("flip", (None, 5, 150_000))
+def test_steps_at_the_limit(peat_gpu, oracle, dtype, umax, flip):
+    """Pairs exactly as many steps apart as the window allows, tied all over the tensor, beside none or one that is far
+    outside of it (in the window's sample or not): the largest ULP distance and difference and their first indices."""
+    n = 200_001
+    rng = np.random.default_rng(umax)
+    gb = encode(1.0 + rng.random(n), dtype)
+    cb = gb.copy()
+    for i in rng.integers(300, n, 2000):
+        cb[i] += umax if rng.random() < 0.5 else umax - 1
+    if flip is not None:
+        cb[flip] ^= 1 << (8 * gb.itemsize - 3)
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} flip={flip}")
+    cb[-1] = gb[-1] + umax + 1  # one step more, at the very end
+    check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} flip={flip}, one past the limit")
