@@ -566,7 +566,11 @@ __device__ __forceinline__ void wsacc_add(int* d, uint64_t m, int e, bool neg) {
   const uint32_t out[3] = {m0 << r, (m1 << r) | (r ? m0 >> (32 - r) : 0u), r ? m1 >> (32 - r) : 0u};
 #pragma unroll
   for (int k = 0; k < 3; k++) {
-    if (out[k] == 0u || (unsigned)(j + k) >= (unsigned)NLIMB) continue;
+    if (out[k] == 0u) continue;
+    if ((unsigned)(j + k) >= (unsigned)NLIMB) {  // (excluded by the bounds on the terms, see for_digits)
+      digit_dropped();
+      continue;
+    }
     const int lo = (int)(out[k] & 0xFFFFu), hi = (int)(out[k] >> 16);
     atomicAdd(d + 2 * (j + k), neg ? -lo : lo);
     atomicAdd(d + 2 * (j + k) + 1, neg ? -hi : hi);
