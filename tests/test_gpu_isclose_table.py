@@ -9,7 +9,7 @@ from parity_util import to_device
 pytestmark = pytest.mark.gpu
 RTOLS = {"decades": [10.0 ** -k for k in range(8, 0, -1)], "powers": [2.0 ** -k for k in range(14, -2, -2)],
          "near": [1e-4, 1.1e-4, 1.2e-4, 1.21e-4], "same": [1e-3, 1e-3, 1e-2], "zero": [0.0, 1e-6, 1.0], "one": [1e-4],
-         "huge": [1e-30, 1.0, 1e30]}
+         "huge": [1e-30, 1.0, 1e30], "close": [0.0, 0.0, 1.0, 1.0, 1.1, 1.2, 1.3, 1.7]}
 
 
 @pytest.mark.parametrize("rtols", RTOLS)

@@ -77,3 +77,22 @@ def test_additive_noise(peat_gpu, dtype):
     for sigma, limit in ((0.001, 2.7), (0.01, 4.5)):
         t = compare_us(peat_gpu, x.to(dt).view(-1), (x + sigma * noise).to(dt).view(-1))
         assert t < limit * plain, f"{dtype} {sigma}: {t:.1f} us against {plain:.1f}"
+
+
+@pytest.mark.parametrize("rtols", ("decades", "close"))
+def test_isclose_large_noise(peat_gpu, rtols):
+    """An isclose grid over errors as large as the values, most of which are not float32 numbers, with rtols a decade
+    or a tenth apart (4.5 times the grid over small errors when each test of such a difference took the margins of two roundings)."""
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    decades = [10.0 ** -k for k in range(8, 0, -1)]
+    g = torch.randn(1 << 24, generator=gen, device="cuda")
+    c = g + torch.randn(1 << 24, generator=gen, device="cuda")
+    counts = torch.zeros(64, dtype=torch.int64, device="cuda")
+    atols = [0.0] + [10.0 ** -k for k in range(8, 1, -1)]
+    with peat_gpu.Handle(0) as h:
+        plain = median_us(torch, lambda: peat_gpu.peat_isclose_grid_raw(h, g, g.half().float(), decades, atols, counts))
+        rt = decades if rtols == "decades" else [1.0 + 0.1 * k for k in range(8)]
+        t = median_us(torch, lambda: peat_gpu.peat_isclose_grid_raw(h, g, c, rt, atols, counts))
+    assert t < 3.7 * plain, f"{t:.1f} us against {plain:.1f}"
