@@ -191,13 +191,19 @@ int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_
 }
 
 int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int max_ctas, int64_t* out) {
-  int64_t lo = n / max_ctas, hi = n + (nseg + 1) * pc;  // hi always fits in one CTA
-  for (int it = 0; it < 40 && lo + 1 < hi; it++) {
+  // no smaller capacity fits all pieces; the larger one fits the greedy walk,
+  // which leaves less than a piece of a CTA empty and cuts each CTA's end once.
+  // To one part in 8192: bisecting to the last element took 1.3 ms of host
+  // time for 16 000 segments, longer than the GPU's part.
+  const int64_t cuts = nseg + max_ctas;
+  int64_t lo = std::max<int64_t>((n + pc) / max_ctas, 1), hi = (n + cuts * pc) / max_ctas + 2 * pc + 2;
+  while (hi - lo > 1 + hi / 8192) {
     const int64_t mid = lo + (hi - lo) / 2;
     if (greedy_split(off, nseg, n, pc, mid, max_ctas, out) > 0) hi = mid;
     else lo = mid;
   }
-  return greedy_split(off, nseg, n, pc, hi, max_ctas, out);
+  const int k = greedy_split(off, nseg, n, pc, hi, max_ctas, out);
+  return k > 0 ? k : greedy_split(off, nseg, n, pc, n + (nseg + 1) * pc, max_ctas, out);  // (one CTA holds everything)
 }
 
 // wait until the pinned staging buffers may be rewritten
