@@ -1895,21 +1895,21 @@ __device__ __noinline__ uint32_t scan_slot(Win W, Smem<DT>& sm, const ComparePar
 
 // The general pairs of a piece [pb, pe), evaluated exactly by every thread of
 // the CTA: from the list when it held them all, else found again by a rescan
-// of the piece with the same window test.  Out of line, so that the hot loop
+// of the piece with the same window test.  all: every pair of the piece.  Out of line, so that the hot loop
 // carries no call.  Leaves each warp's general maxima in sm.k.wbest[warp].
 template <int DT, bool INJ>
 __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParams& p, int64_t pb, int64_t pe,
-                                         int64_t vb, int64_t ve) {
+                                         int64_t vb, int64_t ve, bool all) {
   constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   // entered only after a barrier and with at least one general pair (finish_piece)
-  const uint32_t n = sm.k.gn;
+  const uint32_t n = all ? (uint32_t)(pe - pb) : sm.k.gn;
   const int64_t lo = sm.k.lo;
   GenRec cd;
   gen_init(cd);
   GenSum gs;
   // whole warps in every round (general_lane counts with the whole warp)
   const uint32_t lane = threadIdx.x & 31u;
-  const bool listed = n <= sm.k.gcap, many = DT == PEAT_F16 && n > GEN_MANY;
+  const bool listed = all || n <= sm.k.gcap, many = DT == PEAT_F16 && n > GEN_MANY;
   uint32_t b = threadIdx.x & ~31u, cnt = 0;  // the warp's place in the list; its queue
   int64_t k = threadIdx.x >> 5;
   const int64_t slots = (ve - vb + Queue<DT>::SLOT - 1) / Queue<DT>::SLOT + 2;
@@ -1921,7 +1921,7 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
       if (b >= n) break;
       valid = b + lane < n;
       if (valid) {
-        i = lo + sm.k.glist[b + lane];
+        i = all ? pb + b + lane : lo + sm.k.glist[b + lane];
         if (!PEAT_CHECK(i >= 0 && i < p.n_total)) i = lo;  // a listed offset outside the tensor
         G = load_scalar<DT>(p.g, i);
         C = cand_at<DT, INJ>(p, i, G);
@@ -2188,7 +2188,7 @@ __device__ __forceinline__ void piece_init(Smem<DT>& sm) {
 // CTA that finishes the segment's last piece then finalizes the segment.
 template <int DT, bool INJ>
 __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm, const CompareParams& p,
-                                             int64_t seg, int64_t pb, int64_t pe, int64_t vb, int64_t ve) {
+                                             int64_t seg, int64_t pb, int64_t pe, int64_t vb, int64_t ve, bool all) {
   constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   Partial* out = p.partials + seg + blockIdx.x;
   SegAcc* acc = p.acc + seg;
@@ -2202,8 +2202,8 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
   __syncthreads();  // every tile is in the tables, the list and the records
   // the piece's general pairs, if any: the out-of-line call (and its register
   // traffic) only when there is one
-  const bool gen = sm.k.gn != 0;
-  if (gen) run_general<DT, INJ>(W, sm, p, pb, pe, vb, ve);
+  const bool gen = all || sm.k.gn != 0;
+  if (gen) run_general<DT, INJ>(W, sm, p, pb, pe, vb, ve, all);
   if (sm.k.ff == 0x7FFFFFFFFFFFFFFFll || sm.k.fu == 0x7FFFFFFFFFFFFFFFll) first_pairs<DT, INJ>(sm, p, pb, pe);
   if (warp == 0) {
     Partial x;
@@ -2224,7 +2224,7 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
       if (ok) warp_best(x, out);
     }
   }
-  fold_tables<DT>(sm, W);
+  if (!all) fold_tables<DT>(sm, W);
   __syncthreads();  // the totals are complete
   for (int b = tid; b < HBINS; b += NT) {
     if (sm.k.hist[b]) atomicAdd(&acc->hist[b], sm.k.hist[b]);
@@ -2256,6 +2256,14 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
 // ---------------------------------------------------------------------------
 // stage 1
 // ---------------------------------------------------------------------------
+// Pieces of at most a pair per thread are evaluated on the general path by all
+// warps: their window, tables and copies, and one warp's partial tile, take 13 us
+// whatever the piece holds.  Measured, 16-bit types: 16 000 segments of 100 pairs
+// 1370 -> 960 us, 4000 of 500 399 -> 288 (of 1000, two pairs per thread, no
+// gain; of 2000 a third slower).
+template <int DT>
+constexpr int64_t SHORT_PIECE = Geo<DT>::NT;
+
 // The window sample: VEC (or one) pairs per thread, from the start of the
 // piece (float32) or from places all over it, give the largest finite golden
 // exponent (16-bit types: of the unequal pairs that a window can take, if there
@@ -2368,6 +2376,8 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
     }
     const bool body_scalar = scalar || vb >= ve;  // also a piece inside one vector
     if (body_scalar) vb = pb, ve = pe;
+    const bool all = pe - pb <= SHORT_PIECE<DT>;
+    if (all) vb = ve = pe;  // nothing for the tiles
     const int64_t nvec = (ve - vb + VEC - 1) / VEC;
     const int64_t nchunk = (nvec + CHV - 1) / CHV;
     // this warp's chunks: warp + NW i, i < nmy; only the piece's last chunk is partial
@@ -2463,7 +2473,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
       }
       B.low = true;
     };
-    if (warp == 0 && pb < vb) {
+    if (warp == 0 && pb < vb && !all) {
       stage_scalar<DT, INJ>(p, sm.k.edge_g, sm.k.edge_c, pb, vb);
       run_cold(sm.k.edge_g, sm.k.edge_c, (uint32_t)(pb - lo), -1);
     }
@@ -2535,7 +2545,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
         mbar_wait(bar0 + 8u * (sq % NSTAGE), (sq / NSTAGE) & 1u, DRAIN_LIMIT);
       }
     }
-    finish_piece<DT, INJ>(L, W, sm, p, s, pb, pe, vb, ve);
+    finish_piece<DT, INJ>(L, W, sm, p, s, pb, pe, vb, ve, all);
     pb = pe;
   }
 }

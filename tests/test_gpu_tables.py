@@ -5,7 +5,7 @@ ends of the window, and a nonzero atol.  Everything exact against the oracle."""
 import numpy as np
 import pytest
 
-from parity_util import NP_BITS, assert_hist_equal, assert_stats_equal, oracle_segmented, to_device
+from parity_util import NP_BITS, assert_hist_equal, assert_stats_equal, oracle_segmented, random_pairs, to_device
 
 pytestmark = pytest.mark.gpu
 DTYPES = ("f32", "f16", "bf16")
@@ -133,3 +133,24 @@ def test_steps_at_the_limit(peat_gpu, oracle, dtype, umax, flip):
     check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} flip={flip}")
     cb[-1] = gb[-1] + umax + 1  # one step more, at the very end
     check(peat_gpu, oracle, gb, cb, dtype, 1e-3, 0.0, f"{dtype} flip={flip}, one past the limit")
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("seed", (1, 2))
+def test_short_segments(peat_gpu, oracle, dtype, seed):
+    """Segments of about as many pairs as a CTA has threads (at most a pair per thread is a path of its own), of any
+    bit patterns and of close pairs, between longer and empty ones, at odd offsets."""
+    rng = np.random.default_rng(seed)
+    sizes = rng.choice([0, 1, 2, 31, 33, 255, 256, 257, 511, 512, 513, 700, 5000], 300)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    gb, cb = random_pairs(dtype, n, seed) if seed == 1 else (None, None)
+    if gb is None:
+        gb = encode(rng.standard_normal(n), dtype)
+        cb = steps(gb, np.where(rng.random(n) < 0.6, rng.integers(-3, 4, n), 0))
+    with peat_gpu.Handle(0, max_segments=300) as h:
+        st, hist = peat_gpu.peat_compare_segmented(h, to_device(gb, dtype, 1), to_device(cb, dtype, 1), off, 1e-3, 1e-6)
+    ost, oh = oracle.compare_segmented(gb, cb, off, dtype, 1e-3, 1e-6)
+    for s in range(300):
+        assert_stats_equal(st[s], ost[s], f"{dtype} segment {s} of {sizes[s]}")
+        assert_hist_equal(hist[s], oh[s], f"{dtype} segment {s} of {sizes[s]}")
