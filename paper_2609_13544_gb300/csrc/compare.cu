@@ -1895,21 +1895,21 @@ __device__ __noinline__ uint32_t scan_slot(Win W, Smem<DT>& sm, const ComparePar
 
 // The general pairs of a piece [pb, pe), evaluated exactly by every thread of
 // the CTA: from the list when it held them all, else found again by a rescan
-// of the piece with the same window test.  all: every pair of the piece.  Out of line, so that the hot loop
+// of the piece with the same window test.  ALL: every pair of the piece.  Out of line, so that the hot loop
 // carries no call.  Leaves each warp's general maxima in sm.k.wbest[warp].
-template <int DT, bool INJ>
+template <int DT, bool INJ, bool ALL>
 __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParams& p, int64_t pb, int64_t pe,
-                                         int64_t vb, int64_t ve, bool all) {
+                                         int64_t vb, int64_t ve) {
   constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   // entered only after a barrier and with at least one general pair (finish_piece)
-  const uint32_t n = all ? (uint32_t)(pe - pb) : sm.k.gn;
+  const uint32_t n = ALL ? (uint32_t)(pe - pb) : sm.k.gn;
   const int64_t lo = sm.k.lo;
   GenRec cd;
   gen_init(cd);
   GenSum gs;
   // whole warps in every round (general_lane counts with the whole warp)
   const uint32_t lane = threadIdx.x & 31u;
-  const bool listed = all || n <= sm.k.gcap, many = DT == PEAT_F16 && n > GEN_MANY;
+  const bool listed = ALL || n <= sm.k.gcap, many = !ALL && DT == PEAT_F16 && n > GEN_MANY;
   uint32_t b = threadIdx.x & ~31u, cnt = 0;  // the warp's place in the list; its queue
   int64_t k = threadIdx.x >> 5;
   const int64_t slots = (ve - vb + Queue<DT>::SLOT - 1) / Queue<DT>::SLOT + 2;
@@ -1921,7 +1921,7 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
       if (b >= n) break;
       valid = b + lane < n;
       if (valid) {
-        i = all ? pb + b + lane : lo + sm.k.glist[b + lane];
+        i = ALL ? pb + b + lane : lo + sm.k.glist[b + lane];
         if (!PEAT_CHECK(i >= 0 && i < p.n_total)) i = lo;  // a listed offset outside the tensor
         G = load_scalar<DT>(p.g, i);
         C = cand_at<DT, INJ>(p, i, G);
@@ -2183,18 +2183,19 @@ __device__ __forceinline__ void piece_init(Smem<DT>& sm) {
   if (tid >= 64 && tid < 72) sm.k.cnt[tid - 64] = 0;
 }
 
-// End of one segment piece [pb, pe): the integer totals go to the segment's
+// End of one segment piece [pb, pe) (ALL: of which nothing has been done yet, see
+// compare_short): the integer totals go to the segment's
 // accumulator (global atomics), the maxima to the CTA's partial slot.  The
 // CTA that finishes the segment's last piece then finalizes the segment.
-template <int DT, bool INJ>
+template <int DT, bool INJ, bool ALL>
 __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm, const CompareParams& p,
-                                             int64_t seg, int64_t pb, int64_t pe, int64_t vb, int64_t ve, bool all) {
+                                             int64_t seg, int64_t pb, int64_t pe, int64_t vb, int64_t ve) {
   constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
   Partial* out = p.partials + seg + blockIdx.x;
   SegAcc* acc = p.acc + seg;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if constexpr (DT == PEAT_F32) flush_sums(L, sm, win_lexp<DT>(W));
-  {
+  if constexpr (DT == PEAT_F32 && !ALL) flush_sums(L, sm, win_lexp<DT>(W));
+  if constexpr (!ALL) {
     const uint32_t over = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)L.mism);
     if (lane == 0 && over) atomicAdd(&sm.k.cnt[2], 0ull - (unsigned long long)over);
   }
@@ -2202,8 +2203,8 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
   __syncthreads();  // every tile is in the tables, the list and the records
   // the piece's general pairs, if any: the out-of-line call (and its register
   // traffic) only when there is one
-  const bool gen = all || sm.k.gn != 0;
-  if (gen) run_general<DT, INJ>(W, sm, p, pb, pe, vb, ve, all);
+  const bool gen = ALL || sm.k.gn != 0;
+  if (gen) run_general<DT, INJ, ALL>(W, sm, p, pb, pe, vb, ve);
   if (sm.k.ff == 0x7FFFFFFFFFFFFFFFll || sm.k.fu == 0x7FFFFFFFFFFFFFFFll) first_pairs<DT, INJ>(sm, p, pb, pe);
   if (warp == 0) {
     Partial x;
@@ -2224,7 +2225,7 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
       if (ok) warp_best(x, out);
     }
   }
-  if (!all) fold_tables<DT>(sm, W);
+  if constexpr (!ALL) fold_tables<DT>(sm, W);
   __syncthreads();  // the totals are complete
   for (int b = tid; b < HBINS; b += NT) {
     if (sm.k.hist[b]) atomicAdd(&acc->hist[b], sm.k.hist[b]);
@@ -2256,14 +2257,6 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
 // ---------------------------------------------------------------------------
 // stage 1
 // ---------------------------------------------------------------------------
-// Pieces of at most a pair per thread are evaluated on the general path by all
-// warps: their window, tables and copies, and one warp's partial tile, take 13 us
-// whatever the piece holds.  Measured, 16-bit types: 16 000 segments of 100 pairs
-// 1370 -> 960 us, 4000 of 500 399 -> 288 (of 1000, two pairs per thread, no
-// gain; of 2000 a third slower).
-template <int DT>
-constexpr int64_t SHORT_PIECE = Geo<DT>::NT;
-
 // The window sample: VEC (or one) pairs per thread, from the start of the
 // piece (float32) or from places all over it, give the largest finite golden
 // exponent (16-bit types: of the unequal pairs that a window can take, if there
@@ -2376,8 +2369,6 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
     }
     const bool body_scalar = scalar || vb >= ve;  // also a piece inside one vector
     if (body_scalar) vb = pb, ve = pe;
-    const bool all = pe - pb <= SHORT_PIECE<DT>;
-    if (all) vb = ve = pe;  // nothing for the tiles
     const int64_t nvec = (ve - vb + VEC - 1) / VEC;
     const int64_t nchunk = (nvec + CHV - 1) / CHV;
     // this warp's chunks: warp + NW i, i < nmy; only the piece's last chunk is partial
@@ -2473,7 +2464,7 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
       }
       B.low = true;
     };
-    if (warp == 0 && pb < vb && !all) {
+    if (warp == 0 && pb < vb) {
       stage_scalar<DT, INJ>(p, sm.k.edge_g, sm.k.edge_c, pb, vb);
       run_cold(sm.k.edge_g, sm.k.edge_c, (uint32_t)(pb - lo), -1);
     }
@@ -2545,11 +2536,53 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
         mbar_wait(bar0 + 8u * (sq % NSTAGE), (sq / NSTAGE) & 1u, DRAIN_LIMIT);
       }
     }
-    finish_piece<DT, INJ>(L, W, sm, p, s, pb, pe, vb, ve, all);
+    finish_piece<DT, INJ, false>(L, W, sm, p, s, pb, pe, vb, ve);
     pb = pe;
   }
 }
 
+
+// Stage 1 of a list of short segments, at most a pair per thread each: every pair
+// on the general path, all warps of the CTA at a segment, without the window,
+// copies and tables, which take 13 us a piece whatever it holds.  Measured (16 000
+// segments of 100 and 4000 of 500 bfloat16 pairs): 1370 -> 831 us and 399 -> 255; with two
+// pairs per thread there is no gain, with four it is a third slower.  A kernel of its own: the
+// same choice inside compare_stage1 cost every 16-bit call 1.5 to 2 us.
+template <int DT>
+__global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_short(CompareParams p) {
+  constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;
+  Smem<DT>& sm = *reinterpret_cast<Smem<DT>*>(smem_raw);
+  pdl_trigger();
+  const int tid = threadIdx.x;
+  for (int b = tid; b < HBINS; b += NT) sm.k.hist[b] = 0;
+  for (int j = tid; j < NSUM * NLIMB; j += NT) (&sm.k.sacc[0][0])[j] = 0;
+  for (int j = tid; j < NW * HBINS; j += NT) (&sm.k.ghist[0][0])[j] = 0;
+  for (int j = tid; j < NW * NSUM * NLIMB * 2; j += NT) (&sm.k.gsacc[0][0][0])[j] = 0;
+  const int64_t lo = p.bounds[blockIdx.x], hi = p.bounds[blockIdx.x + 1];
+  if (tid == 0) sm.k.lo = lo;
+  Win W;
+  W.rtol = p.rtol;
+  W.atol = p.atol;
+  W.lim = W.M1 = W.M2 = 0.0f;
+  W.lb = W.fe = 0;
+  Lane L;
+  lane_init(L);
+  __syncthreads();
+  if (blockIdx.x == 0 && p.has_empty) write_empty_segments(p);
+  int64_t s = seg_of(lo, p.offsets, p.nseg);
+  for (int64_t pb = lo; pb < hi;) {
+    while (p.offsets[s + 1] <= pb) s++;  // skip empty segments
+    const int64_t pe = min(hi, p.offsets[s + 1]);
+    piece_init<DT>(sm);
+    if (tid == 0) {
+      const uint32_t G = load_scalar<DT>(p.g, pb), C = load_scalar<DT>(p.c, pb);
+      const bool fin = (G & Tr<DT>::MAG) < Tr<DT>::INF && (C & Tr<DT>::MAG) < Tr<DT>::INF;
+      sm.k.ff = sm.k.fu = fin ? pb : 0x7FFFFFFFFFFFFFFFll;
+    }
+    finish_piece<DT, false, true>(L, W, sm, p, s, pb, pe, pe, pe);
+    pb = pe;
+  }
+}
 
 // ---------------------------------------------------------------------------
 // stage 2: one CTA per segment: merge the maxima of the segment's pieces,
@@ -2724,7 +2757,8 @@ template <int DT>
 cudaError_t launch_t(const CompareParams& p, cudaStream_t st) {
   // NVTX ranges (host-side enqueue of each stage) for profilers; no cost without one attached
   nvtxRangePushA(p.inj_n > 0 ? "peat inject+compare stage 1" : "peat compare stage 1");
-  if (p.inj_n > 0) compare_stage1<DT, true><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
+  if (p.shorts) compare_short<DT><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
+  else if (p.inj_n > 0) compare_stage1<DT, true><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
   else compare_stage1<DT, false><<<p.nctas, Geo<DT>::NT, sizeof(Smem<DT>), st>>>(p);
   cudaError_t e = cudaGetLastError();
   nvtxRangePop();
@@ -2798,18 +2832,17 @@ int64_t compare_cta_bound(int dtype, int64_t b, int nctas, int64_t n, int64_t p0
 }
 
 // once per device, before the first launch
-template <int DT, bool INJ>
-cudaError_t prepare_one() {
-  cudaError_t e =
-      cudaFuncSetAttribute(compare_stage1<DT, INJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<DT>));
+cudaError_t prepare_one(void (*kernel)(CompareParams), size_t smem) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)  // as much shared memory as the SM offers: Geo<DT>::CTAS CTAs of sizeof(Smem<DT>) each
-    e = cudaFuncSetAttribute(compare_stage1<DT, INJ>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 template <int DT>
 cudaError_t prepare_t() {
-  cudaError_t e = prepare_one<DT, false>();
-  return e == cudaSuccess ? prepare_one<DT, true>() : e;
+  cudaError_t e = prepare_one(compare_stage1<DT, false>, sizeof(Smem<DT>));
+  if (e == cudaSuccess) e = prepare_one(compare_stage1<DT, true>, sizeof(Smem<DT>));
+  return e == cudaSuccess ? prepare_one(compare_short<DT>, sizeof(Smem<DT>)) : e;
 }
 
 cudaError_t compare_prepare() {
@@ -2819,6 +2852,7 @@ cudaError_t compare_prepare() {
   return e;
 }
 
+int compare_short_pairs(int dtype) { return dtype == PEAT_F32 ? Geo<PEAT_F32>::NT : Geo<PEAT_BF16>::NT; }
 int compare_ctas_per_sm(int dtype) { return dtype == PEAT_F32 ? Geo<PEAT_F32>::CTAS : Geo<PEAT_BF16>::CTAS; }
 size_t compare_partial_bytes() { return sizeof(Partial); }
 size_t compare_segacc_bytes() { return sizeof(SegAcc); }

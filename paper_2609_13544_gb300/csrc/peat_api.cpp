@@ -546,7 +546,12 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
   // a rescan past 32 768 entries took 100 us)
   p.gcap = (uint32_t)((int64_t)peat::GCAP * 2 * h->max_ctas / ((int64_t)h->nsm * peat::compare_ctas_per_sm(dtype)));
   p.has_empty = 0;
-  for (int64_t s = 0; s < nseg && !p.has_empty; s++) p.has_empty = offsets[s + 1] == offsets[s];
+  int64_t longest = 0;
+  for (int64_t s = 0; s < nseg; s++) {
+    p.has_empty |= offsets[s + 1] == offsets[s];
+    longest = std::max(longest, offsets[s + 1] - offsets[s]);
+  }
+  p.shorts = nseg > 1 && !inj && longest <= peat::compare_short_pairs(dtype);
   p.status = h->status_dev;
   p.stage1_event = h->stage1_event;
   p.wait_limit = h->wait_limit;

@@ -117,6 +117,7 @@ struct CompareParams {
   SegAcc* acc;             // nseg accumulators, all zero between calls
   uint32_t* glist;         // nctas * gcap offsets: each CTA's general pairs of the current piece
   uint32_t gcap;           // entries per CTA (a piece with more general pairs is rescanned)
+  int shorts;              // several segments, none of more than compare_short_pairs pairs
   int has_empty;           // some segment is empty (CTA 0 writes the outputs of the empty segments)
   unsigned int* status;    // device-visible error word (bit 0: a bounded wait expired)
   unsigned int wait_limit; // iteration bound of a pipeline wait (0: give up at once, for tests)
@@ -128,6 +129,7 @@ struct CompareParams {
 
 // Host-side launchers (compare.cu / inject.cu).
 cudaError_t launch_compare(int dtype, const CompareParams& p, cudaStream_t s);
+int compare_short_pairs(int dtype);
 int compare_ctas_per_sm(int dtype);  // resident CTAs of the element type's stage 1 (at most 2)
 cudaError_t compare_prepare();
 // CTA b of a grid of nctas owns elements [bound(b), bound(b+1)); boundaries
