@@ -1279,12 +1279,13 @@ __device__ __forceinline__ void prep16(Vec16<NP>& v, const uint32_t (&g)[NP], co
     }
   }
 }
-// true when a pair of the vector is flagged
+// true when a pair of the vector is flagged; um: the largest step count of each
+// half, above UMAX or NaN when a pair is too far apart
 template <int DT, int NP>
-__device__ __forceinline__ bool check16(const Vec16<NP>& v, const Win& W, const Bounds& B) {
+__device__ __forceinline__ bool check16(const Vec16<NP>& v, const Win& W, const Bounds& B, __half2& um) {
   // the biased step counts are binary16 subnormals: exact sums in units of 2^-24
   constexpr uint32_t NBIAS = (uint32_t)(Tab<DT>::UMAX + 1) * 0x10001u | 0x80008000u;
-  __half2 um = h2(0u);
+  um = h2(0u);
   float xm = 0.0f;
   bool bad;
 #pragma unroll
@@ -1383,8 +1384,8 @@ __device__ __forceinline__ void drop_far(Smem<DT>& sm, uint4* gt, uint4* ct, uin
   fence_proxy_async();  // the zeroed pairs before the next bulk copy into the stage
   __syncwarp();
 }
-// A dense vector with a flagged pair.  Additive noise leaves pairs far apart in
-// nearly every vector, so those are taken out first, without slow_vec's look at the
+// A dense vector with a pair too far apart.  Additive noise leaves such pairs in
+// nearly every vector, so they are taken out first, without slow_vec's look at the
 // maxima, and slow_vec runs only if a pair is still flagged.  Measured, 67 M pairs,
 // slow_vec alone and now: noise of 1 % of the scale, bfloat16 428 -> 268 us,
 // binary16 765 -> 352; of 0.1 %, 234 -> 162 and 381 -> 230.
@@ -1408,7 +1409,8 @@ __device__ __noinline__ void slow16(Smem<DT>& sm, uint4* gt, uint4* ct, uint32_t
     const uint32_t g[4] = {gw[0], gw[1], gw[2], gw[3]}, c[4] = {cw[0], cw[1], cw[2], cw[3]};
     Vec16<4> v;
     prep16<DT, 4>(v, g, c, (uint32_t)(15 + fe) * 0x04000400u);
-    if (!__any_sync(ALL, check16<DT, 4>(v, W, B))) return;
+    __half2 um;
+    if (!__any_sync(ALL, check16<DT, 4>(v, W, B, um))) return;
   }
   slow_vec<DT>(sm, gt, ct, li, 0, fe);
 }
@@ -1429,7 +1431,8 @@ __device__ __forceinline__ void sparse16(Smem<DT>& sm, uint4* gt, uint4* ct, uin
     if (m == 0u) cw[0] = gw[0] = 0u;
     Vec16<1> v;
     prep16<DT, 1>(v, gw, cw, scale2);
-    if (!checked && __any_sync(0xFFFFFFFFu, check16<DT, 1>(v, W, B))) {
+    __half2 um;
+    if (!checked && __any_sync(0xFFFFFFFFu, check16<DT, 1>(v, W, B, um))) {
       slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
       B = read_bounds<DT>(sm, next, W);
       checked = true;  // the whole vector
@@ -1476,8 +1479,12 @@ __device__ __forceinline__ void tile16(Lane& L, Smem<DT>& sm, uint4* gt, uint4* 
     Vec16<4> v;
     uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w}, c[4] = {cv.x, cv.y, cv.z, cv.w};
     prep16<DT, 4>(v, g, c, scale2);
-    if (__any_sync(0xFFFFFFFFu, check16<DT, 4>(v, W, B))) {
-      slow16<DT>(sm, gt, ct, li, W.fe);
+    __half2 um;
+    if (__any_sync(0xFFFFFFFFu, check16<DT, 4>(v, W, B, um))) {
+      // (a vector flagged for its maxima alone goes straight to slow_vec: the few
+      // of them at the start of a piece are a chain, 1.5 us more each through slow16)
+      if (__any_sync(0xFFFFFFFFu, !__hble2(um, h2((uint32_t)Tab<DT>::UMAX * 0x10001u)))) slow16<DT>(sm, gt, ct, li, W.fe);
+      else slow_vec<DT>(sm, gt, ct, li, 0, W.fe);
       gv = *gt;
       cv = *ct;
       const uint32_t gn[4] = {gv.x, gv.y, gv.z, gv.w}, cn[4] = {cv.x, cv.y, cv.z, cv.w};
