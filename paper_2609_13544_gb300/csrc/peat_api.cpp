@@ -160,7 +160,7 @@ bool round_tol(peat_tol_t tol, float* r, float* a) {
 // 114, 81 920 443 / 75 / 121.
 int64_t piece_cost(int dtype) { return dtype == PEAT_F32 ? 24576 : 57344; }
 
-int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t C, int cap, int64_t* out) {
+int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t p0, int64_t C, int cap, int64_t* out) {
   int nct = 0;
   out[0] = 0;
   int64_t cost = 0;
@@ -173,7 +173,9 @@ int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_
         out[++nct] = pos;
         cost = 0;
       }
-      const int64_t take = std::min(s1 - pos, std::max<int64_t>(1, C - cost - pc));
+      int64_t take = std::min(s1 - pos, std::max<int64_t>(1, C - cost - pc));
+      // a cut lies on the vector grid: a piece's ends off it take a step each
+      if (take < s1 - pos && take > 8) take -= (pos + take - p0) & 7;
       cost += pc + take;
       pos += take;
       if (pos < s1) {  // the segment goes on in the next CTA
@@ -190,7 +192,7 @@ int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_
   return nct;
 }
 
-int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int max_ctas, int64_t* out) {
+int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t p0, int max_ctas, int64_t* out) {
   // no smaller capacity fits all pieces; the larger one fits the greedy walk,
   // which leaves less than a piece of a CTA empty and cuts each CTA's end once.
   // To one part in 8192: bisecting to the last element took 1.3 ms of host
@@ -199,11 +201,11 @@ int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int m
   int64_t lo = std::max<int64_t>((n + pc) / max_ctas, 1), hi = (n + cuts * pc) / max_ctas + 2 * pc + 2;
   while (hi - lo > 1 + hi / 8192) {
     const int64_t mid = lo + (hi - lo) / 2;
-    if (greedy_split(off, nseg, n, pc, mid, max_ctas, out) > 0) hi = mid;
+    if (greedy_split(off, nseg, n, pc, p0, mid, max_ctas, out) > 0) hi = mid;
     else lo = mid;
   }
-  const int k = greedy_split(off, nseg, n, pc, hi, max_ctas, out);
-  return k > 0 ? k : greedy_split(off, nseg, n, pc, n + (nseg + 1) * pc, max_ctas, out);  // (one CTA holds everything)
+  const int k = greedy_split(off, nseg, n, pc, p0, hi, max_ctas, out);
+  return k > 0 ? k : greedy_split(off, nseg, n, pc, p0, n + (nseg + 1) * pc, max_ctas, out);  // (one CTA holds everything)
 }
 
 // wait until the pinned staging buffers may be rewritten
@@ -524,7 +526,7 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
     if (ps != PEAT_OK) return ps;
     std::memcpy(h->h_offsets, offsets, sizeof(int64_t) * (size_t)(nseg + 1));
     int64_t* hb = h->h_offsets + nseg + 1;
-    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, piece_cost(dtype), p.nctas, hb) : 0;
+    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, piece_cost(dtype), std::max<int64_t>(p.p0, 0), p.nctas, hb) : 0;
     if (nsplit > 0)
       p.nctas = nsplit;
     else
