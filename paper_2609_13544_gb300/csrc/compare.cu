@@ -767,7 +767,7 @@ __device__ __forceinline__ void general_lane(Smem<DT>& sm, GenRec& cd, GenSum& g
     const float y = k < 4 ? 1.0f : (k == 4 ? o.s : o.t);
     if ((k == 2 || k == 3) && o.s < 0.0f) x = -x;
     const bool use = on && x != 0.0f && y != 0.0f;
-    if (!__any_sync(0xFFFFFFFFu, use)) continue;  // (t is zero where c - g is a float32 value, most often)
+    if (many && !__any_sync(0xFFFFFFFFu, use)) continue;  // (t is zero where c - g is a float32 value, most often)
     if (use) {
       int ex = 0, ey = 0;
       const uint32_t mx = split_float(x, ex), my = split_float(y, ey);
@@ -1916,7 +1916,7 @@ __device__ __noinline__ void run_general(Win W, Smem<DT>& sm, const CompareParam
   GenSum gs;
   // whole warps in every round (general_lane counts with the whole warp)
   const uint32_t lane = threadIdx.x & 31u;
-  const bool listed = ALL || n <= sm.k.gcap, many = !ALL && DT == PEAT_F16 && n > GEN_MANY;
+  const bool listed = ALL || n <= sm.k.gcap, many = !ALL && n > GEN_MANY;
   uint32_t b = threadIdx.x & ~31u, cnt = 0;  // the warp's place in the list; its queue
   int64_t k = threadIdx.x >> 5;
   const int64_t slots = (ve - vb + Queue<DT>::SLOT - 1) / Queue<DT>::SLOT + 2;
