@@ -824,7 +824,7 @@ def run_gpu(args) -> None:
                "us_per_call": ms * 1e3, "pairs_per_s": w.n / (ms * 1e-3),
                "roofline": {"bound": "alu", "achieved": gbs64, "peak": peak, "unit": "GB/s", "frac": gbs64 / peak,
                             "algorithmic_bytes_per_call": 16 * w.n,
-                            "note": "FP64 TwoSum per pair and the three sums as digit atomics in shared memory"}}
+                            "note": "integer arithmetic on the patterns, the sums as 64-bit digit columns in shared memory"}}
         del g64, c64
 
     # end to end through the C ABI with host buffers: every step copies both

@@ -998,7 +998,8 @@ __device__ __forceinline__ void flush_sums(Lane& L, Smem<PEAT_F32>& sm, int lexp
 __device__ __forceinline__ void gen_sums(const GenSum& gs, Smem<PEAT_F16>& sm) {
 #pragma unroll 1
   for (int w = 0; w < 4; w++) {
-    const uint64_t a = w < 2 ? wsum64((uint32_t)(gs.a >> (32 * w))) : 0, n = w < 2 ? wsum64((uint32_t)(gs.n >> (32 * w))) : 0;
+    const uint64_t a = w < 2 ? wsum64((uint32_t)(gs.a >> (32 * w))) : 0;
+    const uint64_t n = w < 2 ? wsum64((uint32_t)(gs.n >> (32 * w))) : 0;
     const uint64_t q = wsum64((uint32_t)(gs.q >> (32 * w)));
     if ((threadIdx.x & 31) == 0) {
       if (a) sacc_add<PEAT_F16>(sm, 1, a, 32 * w - 24, false), sacc_add<PEAT_F16>(sm, 0, a, 32 * w - 24, false);
@@ -2268,8 +2269,8 @@ __device__ __forceinline__ void finish_piece(Lane& L, const Win& W, Smem<DT>& sm
 // piece (float32) or from places all over it, give the largest finite golden
 // exponent (16-bit types: of the unequal pairs that a window can take, if there
 // are any, plus 256) and the largest ULP distance of a pair of one sign (they
-// place the window), and starting bounds for the three maxima.  A starting bound is the value of some pair of the piece, so
-// no maximum lies below it.
+// place the window), and starting bounds for the three maxima.  A starting bound
+// is the value of some pair of the piece, so no maximum lies below it.
 template <int DT, int NV>
 __device__ __forceinline__ void sample_pairs(const uint32_t (&g)[NV], const uint32_t (&c)[NV], uint32_t& emax,
                                              uint32_t& umax, uint32_t& ab, uint32_t& qb) {
@@ -2548,13 +2549,13 @@ __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_stage1(Com
   }
 }
 
-
 // Stage 1 of a list of short segments, at most a pair per thread each: every pair
 // on the general path, all warps of the CTA at a segment, without the window,
 // copies and tables, which take 13 us a piece whatever it holds.  Measured (16 000
-// segments of 100 and 4000 of 500 bfloat16 pairs): 1370 -> 831 us and 399 -> 255; with two
-// pairs per thread there is no gain, with four it is a third slower.  A kernel of its own: the
-// same choice inside compare_stage1 cost every 16-bit call 1.5 to 2 us.
+// segments of 100 and 4000 of 500 bfloat16 pairs): 1370 -> 831 us and 399 -> 255;
+// with two pairs per thread there is no gain, with four it is a third slower.  A
+// kernel of its own: the same choice inside compare_stage1 cost every 16-bit call
+// 1.5 to 2 us.
 template <int DT>
 __global__ void __launch_bounds__(Geo<DT>::NT, Geo<DT>::CTAS) compare_short(CompareParams p) {
   constexpr int NT = Geo<DT>::NT, NW = Geo<DT>::NW;

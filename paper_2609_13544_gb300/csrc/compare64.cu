@@ -375,8 +375,9 @@ __device__ __forceinline__ uint64_t wsum_u64(uint64_t v) {
 //   - the two bins from shared counters by (floor(log2(|d| / |g|)) mod 64,
 //     min(ULP distance, 63)) (increments by one merge equal addresses; column
 //     0 takes the lanes without an unequal pair and is left out);
-//   - the tolerance (atol = 0) and the relative maximum from the ratio in
-//     float32, within 2^-21: closer calls take the slow path.
+//   - the tolerance (atol = 0; with another atol every unequal pair goes to
+//     pair64) and the relative maximum from the ratio in float32, within 2^-21:
+//     closer calls take the slow path.
 // A pair outside the window, non-finite, or above one of the warp's maxima so
 // far goes to pair64.  The warp's iterations visit its pairs in index order, so a
 // pair equal to a maximum of an earlier round cannot win.
@@ -384,7 +385,8 @@ __device__ __forceinline__ uint64_t wsum_u64(uint64_t v) {
 // What bounds it: integer instruction issue (no FP64 instruction, whose pipe
 // takes 64 cycles per warp here, and no local memory): about 250 instructions
 // per pair slot of a warp.  12.3 M pairs (a float32 rounding widened, rtol
-// 1e-7), one call: 2200 -> 207 us, of which the finalization 32; before, every
+// 1e-7), one call: 2200 -> 207 us, of which the finalization 32 (atol 1e-8: 2210 -> 870);
+// before, every
 // term went through binary64 Fast2Sum and local-memory windows (1070
 // instructions and 1.9 GB of local-memory traffic).
 constexpr int WS = 56, QD = 8;

@@ -152,15 +152,18 @@ bool round_tol(peat_tol_t tol, float* r, float* a) {
 // segment piece it meets, a fixed CTA-wide merge (its tables, its maxima, its
 // sums) worth about piece_cost elements.  For a capacity C, a greedy walk over
 // the segments gives the fewest CTAs with cost <= C each (cutting a segment
-// where a CTA fills up); a bisection on C finds the smallest capacity that fits in max_ctas CTAs,
-// i.e. one wave.  Writes out[0..nctas] and returns nctas (0: no split fits).
+// where a CTA fills up); a bisection on C finds the smallest capacity, to one part
+// in 8192, that fits in max_ctas CTAs, i.e. one wave.  Writes out[0..nctas] and
+// returns nctas (0: no split fits).
 // Measured (GPT-2 list, binary16, 292 tensors / 151 tensors of 22.9 M binary16
 // elements / ResNet-50 list, float32, 161 tensors): 8192 elements a piece 470 /
 // 160 / 116 us, 24 576 458 / 119 / 111, 40 960 446 / 85 / 112, 57 344 435 / 78 /
-// 114, 81 920 443 / 75 / 121.
+// 114, 81 920 443 / 75 / 121 (one cost per type for every list: the middle one is
+// best at 81 920).
 int64_t piece_cost(int dtype) { return dtype == PEAT_F32 ? 24576 : 57344; }
 
-int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t p0, int64_t C, int cap, int64_t* out) {
+int greedy_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64_t p0, int64_t C, int cap,
+                 int64_t* out) {
   int nct = 0;
   out[0] = 0;
   int64_t cost = 0;
@@ -205,7 +208,8 @@ int segment_split(const int64_t* off, int64_t nseg, int64_t n, int64_t pc, int64
     else lo = mid;
   }
   const int k = greedy_split(off, nseg, n, pc, p0, hi, max_ctas, out);
-  return k > 0 ? k : greedy_split(off, nseg, n, pc, p0, n + (nseg + 1) * pc, max_ctas, out);  // (one CTA holds everything)
+  // (the last one holds everything in one CTA)
+  return k > 0 ? k : greedy_split(off, nseg, n, pc, p0, n + (nseg + 1) * pc, max_ctas, out);
 }
 
 // wait until the pinned staging buffers may be rewritten
@@ -526,7 +530,8 @@ peat_status_t compare_impl(peat_handle_t h, const void* g, const void* c, const 
     if (ps != PEAT_OK) return ps;
     std::memcpy(h->h_offsets, offsets, sizeof(int64_t) * (size_t)(nseg + 1));
     int64_t* hb = h->h_offsets + nseg + 1;
-    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, piece_cost(dtype), std::max<int64_t>(p.p0, 0), p.nctas, hb) : 0;
+    const int64_t p0 = std::max<int64_t>(p.p0, 0);
+    const int nsplit = n > 0 ? segment_split(offsets, nseg, n, piece_cost(dtype), p0, p.nctas, hb) : 0;
     if (nsplit > 0)
       p.nctas = nsplit;
     else

@@ -46,8 +46,8 @@ constexpr int NLIMB = 24;
 constexpr int LIMB_LSB = -416;
 constexpr int NSUM = 3;  // 0: sum d, 1: sum |d|, 2: sum d^2
 
-constexpr int BLOCK = 256;    // threads of the small kernels (bounds, per-segment finalize)
-constexpr int GCAP = 16384;   // entries of the list of general pairs per CTA of the largest grid
+constexpr int BLOCK = 256;    // threads of compare_bounds (compare_finalize: FIN_NT)
+constexpr int GCAP = 16384;   // unit of the CTAs' lists of general pairs (CompareParams::gcap entries each)
 constexpr int HBINS = 128;    // 64 rel bins + 64 ULP bins
 
 // Exact maxima of one CTA piece (element indices are global).  |d| is kept
@@ -151,8 +151,8 @@ cudaError_t launch_bounds_on_device(int dtype, int64_t* offsets, int64_t* bounds
 constexpr int TK_NB0 = 1024, TK_NB1 = 2048, TK_NB2 = 1024, TK_WIN = 3;
 constexpr int64_t TK_SAMPLE = 1 << 18;  // pairs in the sample
 // pairs from which the table pass is offered: at 2^20 the call takes 44 us
-// with it and 48 without; below, the launches are all there is (41 us at 1e5
-// pairs and at 5e3)
+// with it and 48 without; below, the launches are most of it (41 us at 1e5
+// pairs, 35 at 5e3)
 constexpr int64_t TK_TABLE_MIN = 1 << 20;
 constexpr unsigned TK_LCAP = 65536;     // listed pairs whose |d| is not a float32 value
 constexpr int TK_NBL = 65536;           // bins of each 16-bit digit of the order key of a rounding error
