@@ -38,10 +38,13 @@
 // rate.  The kernel before it compacted unequal pairs into a queue and kept
 // histogram rows per thread, about 60 instructions per unequal pair and 30 per
 // pair.  Measured (back-to-back calls, one GB300): 67 M bfloat16 pairs of
-// which half differ 182 -> 89 us, 355 M binary16 pairs in 292 segments 1007 ->
-// 441 us, 268 M bfloat16 pairs of which 0.3 % differ 264 -> 201 us, 25.6 M
-// float32 pairs in 161 segments 222 -> 109 us.  What a small call takes (20 to
-// 30 us) is latency: the window sample, the piece end, the finalization.
+// which half differ 182 -> 88 us, 355 M binary16 pairs in 292 segments 1007 ->
+// 445 us, 268 M bfloat16 pairs of which 0.3 % differ 264 -> 202 us, 25.6 M
+// float32 pairs in 161 segments 222 -> 110 us.  What a small call takes (20 to
+// 40 us) is latency: the window sample, the piece end, the finalization.  The
+// 16-bit window does not move within a piece: 67 M binary16 pairs whose rows lie
+// over eight decades, most of them general then, take 882 us, with the kernel
+// before 534; over two decades 124 and 409.
 // Binary64 arithmetic is avoided per element (GB300 runs it at a small
 // fraction of float32 rate); binary64 values appear only as containers and
 // in the once-per-segment rounding.

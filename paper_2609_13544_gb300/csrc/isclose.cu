@@ -21,10 +21,10 @@
 // goes to integer digits only where the part of |d| below a float32 could decide.
 // Cell (i, j) is the histogram's prefix over f <= i.
 //
-// What bounds it: instruction issue, about 29 warp instructions per 32 pairs and atol.
+// What bounds it: instruction issue, about 30 warp instructions per 32 pairs and atol.
 // Measured: an 8 x 8 grid over 16.8 M float32 pairs (a binary16 rounding) took
 // 535 us with a binary search of margin tests per atol and a match-based
-// histogram (894 instructions per 32 pairs), 139 us now.
+// histogram (894 instructions per 32 pairs), 141 us now.
 #include <cuda_fp16.h>
 
 #include <cstdint>
@@ -163,7 +163,7 @@ __device__ __forceinline__ int classify(uint32_t G, uint32_t C, float& hi, float
 // down) and the next float32, and lo is at most half a step of hi, so hi decides
 // unless it is one of the two.  (With the integer digits for every |d| that is
 // not a float32, 16.8 M float32 pairs against noise as large as the values took
-// 917 us, now 526.)
+// 917 us, now 506.)
 __device__ __forceinline__ bool within(float hi, float lo, float ag, float r, float at) {
   const float v = __fmaf_rd(r, ag, at);
   if (lo != 0.0f && __float_as_uint(hi) - __float_as_uint(v) <= 1u) return close_test(hi, lo, 0, ag, r, at);
