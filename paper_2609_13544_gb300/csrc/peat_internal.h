@@ -274,7 +274,7 @@ struct Cmp8Params {
 // of one spacing): 3.0 M 72 us pair by pair, 56 with tables; 1.3 M 42 and 58;
 // E5M2 with 0.2 % of opposite signs at 4.2 M 84 and 71.  The line is higher
 // than those need because pairs of opposite signs are evaluated one by one
-// beside the table (4.3 M E5M2 with 16 % of them: 98 with tables, 97 without).
+// beside the table (4.3 M E5M2 with 16 % of them: 99 with tables, 97 without).
 constexpr int64_t C8_TABLE_MIN = 1 << 22;
 cudaError_t compare8_prepare();  // once per device, before the first launch
 cudaError_t launch_compare8(int dtype, const Cmp8Params& p, int nctas, cudaStream_t s);
